@@ -28,9 +28,10 @@ struct ulisse_ctx {
   size_t esz = 4;
   long long ld128 = 0;        // rows of the tensor-core operand images (multiple of 128)
   float* bneg = nullptr;      // -log2(e)/2 |x^|^2 per input (tensor-core path)
-  void *Vt_hi = nullptr, *Vt_lo = nullptr;
+  void* Vt = nullptr;         // BF16 operand tiles of K V, high | low part per tile
   void *Gt_hi = nullptr, *Gt_lo = nullptr;   // packed operands of the tensor-core gradient
-  float *Xt_hi = nullptr, *Xt_lo = nullptr;  // TF32 images A | B (tensor-core cross term)
+  float *Xt_hi = nullptr, *Xt_lo = nullptr;  // TF32 images of the A rows (tensor-core cross term)
+  float* Xt_b = nullptr;      // ... and the tiles of the B rows, see launch_pack_x_tf32
 
   float* X = nullptr;         // raw inputs, n x d row-major
   void* y = nullptr;          // labels, ldn (element type T)
@@ -332,7 +333,7 @@ static ulisse_status prescale(ulisse_ctx* ctx) {
     CK(launch_prescale_tc((const float*)ctx->xhat, ctx->DP, ctx->d, ctx->n, ctx->ld128,
                           ctx->bneg, ctx->num_sms, ctx->stream));
     CK(launch_pack_x_tf32((const float*)ctx->xhat, ctx->bneg, ctx->params, ctx->DP, ctx->n,
-                          ctx->ld128, ctx->Xt_hi, ctx->Xt_lo, ctx->ld128 * 24, ctx->num_sms,
+                          ctx->ld128, ctx->Xt_hi, ctx->Xt_lo, ctx->Xt_b, ctx->num_sms,
                           ctx->stream, !ctx->tc_no_aug));
     if (!ctx->capturing) ctx->launches += 2;
   }
@@ -367,8 +368,7 @@ static ulisse_status run_kmv_tc(ulisse_ctx* ctx, const void* V, const int* vmap,
     TcLaunch L{};
     L.xhat = (const float*)ctx->xhat;
     L.bneg = ctx->bneg;
-    L.V_hi = ctx->Vt_hi;
-    L.V_lo = ctx->Vt_lo;
+    L.Vp = ctx->Vt;
     L.V = V;
     L.ldv = ctx->ldn;
     L.vmap = vmap + c0;
@@ -383,7 +383,7 @@ static ulisse_status run_kmv_tc(ulisse_ctx* ctx, const void* V, const int* vmap,
     L.num_sms = ctx->num_sms;
     L.X_hi = ctx->Xt_hi;
     L.X_lo = ctx->Xt_lo;
-    L.X_off = ctx->ld128 * 24;
+    L.X_b = ctx->Xt_b;
     // where the cross term is formed: the tuned choice, else the configured one (default:
     // tensor cores)
     int cross = ctx->cfg.tc_cross_term != 0 ? ctx->cfg.tc_cross_term : kCrossTensor;
@@ -837,7 +837,7 @@ static ulisse_status ensure_grad_maps(ulisse_ctx* ctx, int nr) {
 static void set_grad_images(GradLaunch& L, const ulisse_ctx* c) {
   L.X_hi = c->Xt_hi;
   L.X_lo = c->Xt_lo;
-  L.X_off = c->ld128 * 24;
+  L.X_b = c->Xt_b;
   L.c_has_bj = c->DP < 8 && !c->tc_no_aug;
 }
 
@@ -1045,12 +1045,13 @@ static ulisse_status create_impl(ulisse_ctx** out, const float* X, const float* 
     return bail(s);
   if (ctx->mixed) {
     if ((s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->bneg), sizeof(float) * ctx->ld128)) ||
-        (s = dev_alloc(ctx, &ctx->Vt_hi, 2 * ctx->ld128 * 64)) ||
-        (s = dev_alloc(ctx, &ctx->Vt_lo, 2 * ctx->ld128 * 64)) ||
+        (s = dev_alloc(ctx, &ctx->Vt, 2 * 2 * ctx->ld128 * 64)) ||
         (s = dev_alloc(ctx, &ctx->Gt_hi, 2 * ctx->ld128 * kGtScratchRows)) ||
         (s = dev_alloc(ctx, &ctx->Gt_lo, 2 * ctx->ld128 * kGtScratchRows)) ||
-        (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->Xt_hi), 4 * ctx->ld128 * 48)) ||
-        (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->Xt_lo), 4 * ctx->ld128 * 48)))
+        (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->Xt_hi), 4 * ctx->ld128 * 16)) ||
+        (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->Xt_lo), 4 * ctx->ld128 * 16)) ||
+        (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->Xt_b),
+                       4 * (ctx->ld128 / 32) * tc2_b_stride(16))))
       return bail(s);
   }
   if (cudaMallocHost(&ctx->h_n_live, sizeof(int)) != cudaSuccess ||
@@ -2283,8 +2284,7 @@ static ulisse_status batch_tc_upload(ulisse_ctx* ctx, int k, Fn cols) {
     l.ldu = sub->ldn;
     l.xhat = (const float*)sub->xhat;
     l.bneg = sub->bneg;
-    l.V_hi = sub->Vt_hi;
-    l.V_lo = sub->Vt_lo;
+    l.Vp = sub->Vt;
     l.n = sub->n;
     l.DP = sub->DP;
     l.params = sub->params;
@@ -2294,7 +2294,7 @@ static ulisse_status batch_tc_upload(ulisse_ctx* ctx, int k, Fn cols) {
     l.status = ctx->status_dev;
     l.X_hi = sub->Xt_hi;
     l.X_lo = sub->Xt_lo;
-    l.X_off = sub->ld128 * 24;
+    l.X_b = sub->Xt_b;
     L[b] = l;
   }
   CK(tc2_batch_upload_args(L.data(), B, (char*)ctx->b_tc_args + k * tc2_batch_args_bytes(B),
@@ -3065,8 +3065,9 @@ void ulisse_destroy(ulisse_ctx* ctx) {
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
   for (void** p : {reinterpret_cast<void**>(&ctx->st_next), reinterpret_cast<void**>(&ctx->part1),
                    reinterpret_cast<void**>(&ctx->part2), reinterpret_cast<void**>(&ctx->bneg),
-                   &ctx->Vt_hi, &ctx->Vt_lo, &ctx->Gt_hi, &ctx->Gt_lo,
+                   &ctx->Vt, &ctx->Gt_hi, &ctx->Gt_lo,
                    reinterpret_cast<void**>(&ctx->Xt_hi), reinterpret_cast<void**>(&ctx->Xt_lo),
+                   reinterpret_cast<void**>(&ctx->Xt_b),
                    reinterpret_cast<void**>(&ctx->q_map), &ctx->q_sa, &ctx->pcg_buf, &ctx->pred_xs,
                    reinterpret_cast<void**>(&ctx->pcg_aux), reinterpret_cast<void**>(&ctx->pcg_live)})
     dev_free(*p);

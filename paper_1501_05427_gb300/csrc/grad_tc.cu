@@ -143,8 +143,7 @@ struct GtDevArgs {
   // B_j = [2 c1 x^_j, b_j?]; c_has_bj when the augmented column carries b_j
   const float* XA_hi;
   const float* XA_lo;
-  const float* XB_hi;
-  const float* XB_lo;
+  const float* XB;     // tiles of B_J: high part | remainder | b_J (tc2_b_stride floats)
   int c_has_bj;
   double* partials;
   int* counter;
@@ -324,12 +323,11 @@ __device__ __forceinline__ void gt_body(const GtDevArgs& a, const int rb, const 
         unsigned char* st = stage(s);
         mbar_arrive_expect_tx(&full[s], S::STAGE_BYTES);
         if constexpr (S::XC) {
-          bulk_g2s(st, a.XB_hi + t * kGtBN * S::K8, S::XB_BYTES, &full[s]);
-          bulk_g2s(st + S::XB_BYTES, a.XB_lo + t * kGtBN * S::K8, S::XB_BYTES, &full[s]);
+          bulk_g2s(st, a.XB + t * tc2_b_stride(S::K8), S::X_BYTES + S::BN_BYTES, &full[s]);
         } else {
           bulk_g2s(st, a.xhat + t * kGtBN * DP, S::X_BYTES, &full[s]);
+          bulk_g2s(st + S::OFF_BN, a.bneg + t * kGtBN, S::BN_BYTES, &full[s]);
         }
-        bulk_g2s(st + S::OFF_BN, a.bneg + t * kGtBN, S::BN_BYTES, &full[s]);
         unsigned char* bt = st + S::OFF_BT;
         bulk_g2s(bt, a.Bt_hi + t * kGtBN * K1, S::BT_BYTES, &full[s]);
         bulk_g2s(bt + S::BT_BYTES, a.Bt_lo + t * kGtBN * K1, S::BT_BYTES, &full[s]);
@@ -699,12 +697,11 @@ static int plan_gt_split(long long n_rb, long long ntiles, int num_sms, int occ)
   return best_s;
 }
 
-// The TF32 row images of the K V pass (A rows at X_hi / X_lo, B rows X_off floats on).
+// The TF32 row images of the K V pass (A rows at X_hi / X_lo, B tiles at X_b).
 static void gt_set_images(GtDevArgs& a, const GradLaunch& L) {
   a.XA_hi = L.X_hi;
   a.XA_lo = L.X_lo;
-  a.XB_hi = L.X_hi ? L.X_hi + L.X_off : nullptr;
-  a.XB_lo = L.X_lo ? L.X_lo + L.X_off : nullptr;
+  a.XB = L.X_b;
   a.c_has_bj = L.c_has_bj ? 1 : 0;
 }
 
@@ -813,7 +810,7 @@ cudaError_t gt_batch_upload_args(const GradLaunch* L, const int* nsplit, int B, 
     const long long ntiles = (l.n + kGtBN - 1) / kGtBN;
     const long long n_rb = (l.n + kGtBM - 1) / kGtBM;
     if (l.M < 1 || l.M > kMaxM || nsplit[b] < 1 || l.DP != L[0].DP || !l.tc_hi || !l.tc_lo ||
-        !l.X_hi || !l.X_lo ||
+        !l.X_hi || !l.X_lo || !l.X_b ||
         (ntiles + nsplit[b] - 1) / nsplit[b] > kTcMaxSplitTiles)
       return cudaErrorInvalidValue;
     GtDevArgs& a = h[b];
@@ -896,7 +893,7 @@ cudaError_t launch_grad_tc_batch(const void* args_dev, int B, const int4* items,
 
 cudaError_t launch_grad_tc(GradLaunch& L, cudaStream_t s) {
   if (L.M < 1 || L.M > kMaxM || !L.tc_hi || !L.tc_lo || !L.bneg) return cudaErrorInvalidValue;
-  if (L.DP <= 8 && (!L.X_hi || !L.X_lo)) return cudaErrorInvalidValue;
+  if (L.DP <= 8 && (!L.X_hi || !L.X_lo || !L.X_b)) return cudaErrorInvalidValue;
   switch (L.DP) {
     case 2: return grad_tc_dispatch_m<2>(L, s);
     case 4: return grad_tc_dispatch_m<4>(L, s);

@@ -51,12 +51,12 @@ __global__ void prescale_tc_kernel(const float* __restrict__ xhat, int DP, int d
   }
 }
 
-// V columns vmap[0..R) -> BF16 high and low parts, one K-major canonical image of N rows
-// (right-hand sides) x 32 points per j-tile; rows r >= R and points >= n are zero.
+// V columns vmap[0..R) -> BF16 high and low parts, a K-major canonical image of N rows
+// (right-hand sides) x 32 points each, back to back per j-tile (one bulk copy); rows r >= R and
+// points >= n are zero.
 __global__ void pack_v_kernel(const float* __restrict__ V, long long ldv,
                               const int* __restrict__ vmap, int R, int N, long long n,
-                              long long ntiles, __nv_bfloat16* __restrict__ Vhi,
-                              __nv_bfloat16* __restrict__ Vlo) {
+                              long long ntiles, __nv_bfloat16* __restrict__ Vp) {
   const long long per_tile = (long long)N * kTcBN;
   for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < ntiles * per_tile;
        idx += (long long)gridDim.x * blockDim.x) {
@@ -67,9 +67,9 @@ __global__ void pack_v_kernel(const float* __restrict__ V, long long ldv,
     const float v = (r < R && j < n) ? V[(long long)vmap[r] * ldv + j] : 0.f;
     const __nv_bfloat16 h = __float2bfloat16_rn(v);
     const __nv_bfloat16 l = __float2bfloat16_rn(v - __bfloat162float(h));
-    const long long off = t * per_tile + tc::canon_offset(r, jj, 2, kTcBN / 8) / 2;
-    Vhi[off] = h;
-    Vlo[off] = l;
+    const long long off = t * 2 * per_tile + tc::canon_offset(r, jj, 2, kTcBN / 8) / 2;
+    Vp[off] = h;
+    Vp[off + per_tile] = l;
   }
 }
 
@@ -79,8 +79,7 @@ __global__ void pack_v_kernel(const float* __restrict__ V, long long ldv,
 struct TcDevArgs {
   const float* xhat;     // x^ rows (ld x DP, row-major)
   const float* bneg;     // -c1 |x^|^2
-  const __nv_bfloat16* V_hi;
-  const __nv_bfloat16* V_lo;
+  const __nv_bfloat16* Vp;   // BF16 tiles of V: high | low part
   const float* V;        // FP32 operand columns (diagonal term)
   long long ldv;
   const int* vmap;
@@ -187,9 +186,7 @@ __global__ void __launch_bounds__(kTcThreads, 3) kmv_tc_kernel(const TcDevArgs a
         mbar_arrive_expect_tx(&full[s], S::STAGE_BYTES);
         bulk_g2s(st, a.xhat + t * kTcBN * DP, S::X_BYTES, &full[s]);
         bulk_g2s(st + S::X_BYTES, a.bneg + t * kTcBN, S::B_BYTES, &full[s]);
-        bulk_g2s(st + S::X_BYTES + S::B_BYTES, a.V_hi + t * N * kTcBN, S::V_BYTES, &full[s]);
-        bulk_g2s(st + S::X_BYTES + S::B_BYTES + S::V_BYTES, a.V_lo + t * N * kTcBN,
-                 S::V_BYTES, &full[s]);
+        bulk_g2s(st + S::X_BYTES + S::B_BYTES, a.Vp + t * 2 * N * kTcBN, 2 * S::V_BYTES, &full[s]);
       }
     }
   } else if (warp == 1) {
@@ -355,8 +352,7 @@ void launch_pack_v(const TcLaunch& L, int N, long long ntiles, cudaStream_t s) {
   const long long total = ntiles * N * kTcBN;
   const int blocks = (int)std::min<long long>((total + 255) / 256, 8LL * L.num_sms);
   pack_v_kernel<<<blocks, 256, 0, s>>>(static_cast<const float*>(L.V), L.ldv, L.vmap, L.R, N,
-                                       L.n, ntiles, static_cast<__nv_bfloat16*>(L.V_hi),
-                                       static_cast<__nv_bfloat16*>(L.V_lo));
+                                       L.n, ntiles, static_cast<__nv_bfloat16*>(L.Vp));
 }
 
 template <int DP, int N>
@@ -402,8 +398,7 @@ struct TcInst {
     TcDevArgs a;
     a.xhat = L.xhat;
     a.bneg = L.bneg;
-    a.V_hi = static_cast<const __nv_bfloat16*>(L.V_hi);
-    a.V_lo = static_cast<const __nv_bfloat16*>(L.V_lo);
+    a.Vp = static_cast<const __nv_bfloat16*>(L.Vp);
     a.V = static_cast<const float*>(L.V);
     a.ldv = L.ldv;
     a.vmap = L.vmap;

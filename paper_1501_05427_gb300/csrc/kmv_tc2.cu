@@ -19,13 +19,24 @@
 //      products), FP32 accumulation in tensor memory, as in the FP32-pipe variant.
 // The TF32 images of A and B (high and low parts, K-major canonical, 32-point tiles back to
 // back so that four tiles form the 128-row A operand) are written once per parameter value by
-// pack_x_tf32_kernel.  Roles: warp 0 streams the A image once, then the B_J image and V_J
-// into a 3- or 4-stage ring with bulk copies; one thread of warp 1 issues the MMAs; eight
-// epilogue warps make the kernel values, in two sets of four (one per tensor-memory lane
-// quadrant) that take alternate tiles whole, so that each wait and hand-off covers 32
-// entries per thread.  Three C/K buffers (two when the accumulator takes 64 columns); a buffer
-// is refilled only after the MMAs that read it have completed.  Every wait is bounded.  The split j range, the fixed-order fix-up of the
-// partial sums and the FP32 diagonal term lambda V are those of the FP32-pipe variant.
+// pack_x_tf32_kernel; B's tiles and V's tiles each lie contiguously with all their parts, so
+// that a tile is two bulk copies.  Roles: warp 0 copies (the A image once, then B_J, b_J and
+// V_J into a ring of 3 to 8 stages) and issues the MMAs; eight epilogue warps make the kernel
+// values, in two sets of four (one per tensor-memory lane quadrant) that take alternate tiles
+// whole, so that each wait and hand-off covers 32 entries per thread.  Three C/K buffers (two
+// when the accumulator takes 64 columns); a buffer is refilled only after the MMAs that read it
+// have completed, and the stage of that tile is refilled at the same moment, so the copies need
+// no barrier and no warp of their own.  Every wait is bounded.  The split j range, the
+// fixed-order fix-up of the partial sums and the FP32 diagonal term lambda V are those of the
+// FP32-pipe variant.
+//
+// What bounds it: the issue slots of the epilogue's instruction stream and, next to them, the
+// chain C -> epilogue -> contraction -> refill, whose middle is one warp's instructions.  That
+// warp runs its loop warp-uniformly and elects a lane only for the issuing instructions: the
+// descriptors then live in uniform registers.  With a separate copying warp and one divergent
+// lane issuing (moving every descriptor to uniform registers per MMA) a product at n = 50,000,
+// d = 8, 17 columns took 1.046 ms; nine warps instead of ten also raise the register budget from
+// 48 to 56, so that the high and low parts get registers of their own.  Now 0.78 ms.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -39,19 +50,20 @@ namespace ulisse {
 
 constexpr int kT2BN = 32;
 constexpr int kT2BM = 128;
-constexpr int kT2Threads = 320;    // warp 0 producer, warp 1 MMA issuer, warps 2-9 epilogue
+constexpr int kT2Threads = 288;    // warp 0 copies and MMAs, warps 1-8 epilogue
 constexpr uint32_t kT2Cols = 128;  // tensor-memory columns per CTA
 
 // The rows A_j = [x^_j, 1, 0...] and B_j = [2 c1 x^_j, b_j, 0...] for j in [0, rows) as TF32
 // high part and remainder, K8 columns, in 32-row K-major canonical tiles; rows >= n are zero.
 // When K8 == DP there is no slot for the augmented column (A_j = x^_j, B_j = 2 c1 x^_j); the
 // batched launches leave it out for every d (aug = 0) and add b_j in the epilogue.
-// b_j = -c1 |x^_j|^2 is read from the row norms of launch_prescale_tc.
+// b_j = -c1 |x^_j|^2 is read from the row norms of launch_prescale_tc.  A's parts are two
+// arrays; B's tiles hold high part, remainder and the tile's 32 b_j back to back
+// (tc2_b_stride floats each), so that a tile is one bulk copy.
 __global__ void pack_x_tf32_kernel(const float* __restrict__ xhat, const float* __restrict__ bneg,
                                    const DevParams* __restrict__ params, int DP, int K8, int aug,
                                    long long n, long long rows, float* __restrict__ Ahi,
-                                   float* __restrict__ Alo, float* __restrict__ Bhi,
-                                   float* __restrict__ Blo) {
+                                   float* __restrict__ Alo, float* __restrict__ Bt) {
   const float two_c1 = 2.f * params->c1f;
   for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < rows * K8;
        idx += (long long)gridDim.x * blockDim.x) {
@@ -69,23 +81,24 @@ __global__ void pack_x_tf32_kernel(const float* __restrict__ xhat, const float* 
     }
     const long long t = j / kT2BN;
     const int jj = (int)(j - t * kT2BN);
-    const long long off = t * kT2BN * K8 + tc::canon_offset(jj, k, 4, K8 / 4) / 4;
+    const uint32_t in_tile = tc::canon_offset(jj, k, 4, K8 / 4) / 4;
+    const long long off = t * kT2BN * K8 + in_tile;
     const float ha = tc::tf32_round(va), hb = tc::tf32_round(vb);
     Ahi[off] = ha;
     Alo[off] = va - ha;
-    Bhi[off] = hb;
-    Blo[off] = vb - hb;
+    float* bt = Bt + t * tc2_b_stride(K8);
+    bt[in_tile] = hb;
+    bt[kT2BN * K8 + in_tile] = vb - hb;
+    if (k == 0) bt[2 * kT2BN * K8 + jj] = bneg[j];
   }
 }
 
 struct Tc2DevArgs {
   const float* A_hi;     // TF32 image of the augmented A rows (high part)
   const float* A_lo;     // remainder
-  const float* B_hi;     // TF32 image of the augmented B rows
-  const float* B_lo;
+  const float* B;        // TF32 tiles of the augmented B rows: high part | remainder | b_j
   const float* bneg;     // -c1 |x^|^2
-  const __nv_bfloat16* V_hi;
-  const __nv_bfloat16* V_lo;
+  const __nv_bfloat16* Vp;   // BF16 tiles of V: high | low part
   const float* V;        // FP32 operand columns (diagonal term)
   long long ldv;
   const int* vmap;
@@ -109,29 +122,29 @@ struct Tc2Shape {
   static constexpr uint32_t XB_BYTES = kT2BN * K8 * 4;  // one part of the B_J image
   static constexpr uint32_t V_BYTES = N * kT2BN * 2;    // one part of the BF16 V_J tile
   static constexpr uint32_t BN_BYTES = BJ ? kT2BN * 4 : 0;   // b_J
-  static constexpr uint32_t OFF_BN = 2 * XB_BYTES + 2 * V_BYTES;   // within a stage
-  static constexpr uint32_t STAGE_BYTES = 2 * XB_BYTES + 2 * V_BYTES + BN_BYTES;
-  // four stages while four CTAs still fit in shared memory (~54 KB each), else three
-  static constexpr int ST = (2 * A_BYTES + 4 * STAGE_BYTES <= 54 * 1024) ? 4 : 3;
+  static constexpr uint32_t X_COPY = 2 * XB_BYTES + BN_BYTES;   // B_J high | remainder | b_J
+  static constexpr uint32_t OFF_BN = 2 * XB_BYTES;              // within a stage
+  static constexpr uint32_t OFF_V = X_COPY;
+  static constexpr uint32_t STAGE_BYTES = X_COPY + 2 * V_BYTES;
+  // as many stages (at most 8) as let four CTAs fit in shared memory (~54 KB each), at least 3
+  static constexpr int ST_FIT = (int)((54u * 1024u - 2 * A_BYTES) / STAGE_BYTES);
+  static constexpr int ST = ST_FIT > 8 ? 8 : ST_FIT < 3 ? 3 : ST_FIT;
   static constexpr uint32_t OFF_STAGES = 2 * A_BYTES;
   static constexpr uint32_t OFF_BARS = OFF_STAGES + ST * STAGE_BYTES;
   // C/K buffers of 32 columns: three while they fit beside the accumulator, else two
   static constexpr int NB = (3 * 32 + N <= (int)kT2Cols) ? 3 : 2;
-  // full, empty per stage; a_full; c_full per tile mod 6 (so that each barrier serves one
+  // full per stage; a_full; c_full per tile mod 6 (so that each barrier serves one
   // epilogue set and its phases are waited in order); k_full, b_free per buffer; done
   static constexpr int NCF = 6;
-  static constexpr int NBARS = 2 * ST + 1 + NCF + 2 * NB + 1;
+  static constexpr int NBARS = ST + 1 + NCF + 2 * NB + 1;
   static constexpr uint32_t SMEM = OFF_BARS + NBARS * 8 + 64;
   static constexpr uint32_t COL_U = NB * 32;   // after the C/K buffers
   static_assert(COL_U + N <= kT2Cols, "tensor memory layout exceeds the allocation");
-  static_assert(STAGE_BYTES % 16 == 0 && A_BYTES % 16 == 0 && XB_BYTES % 16 == 0,
+  static_assert(STAGE_BYTES % 16 == 0 && A_BYTES % 16 == 0 && XB_BYTES % 16 == 0 &&
+                    X_COPY % 16 == 0,
                 "bulk copies and descriptors need 16-byte alignment");
+  static_assert(NCF % NB == 0, "a c_full barrier belongs to one buffer");
 };
-
-__device__ inline bool t2_warp_wait(uint64_t* bar, uint32_t parity) {
-  const bool ok = mbar_wait_spin(bar, parity);
-  return __all_sync(0xffffffffu, ok);
-}
 
 template <int NH>
 __device__ inline void t2_ld_cols(uint32_t taddr, float (&v)[NH]) {
@@ -162,12 +175,10 @@ __device__ __forceinline__ void tc2_body(const Tc2DevArgs& a, const int rb, cons
   constexpr int NB = S::NB;
   constexpr int NH = N / 2;
   extern __shared__ __align__(1024) unsigned char smem[];
-  unsigned char* sAh = smem;
-  unsigned char* sAl = smem + S::A_BYTES;
+  const uint32_t smem0 = smem_u32(smem);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S::OFF_BARS);
   uint64_t* full = bars;
-  uint64_t* empty = bars + ST;
-  uint64_t* a_full = bars + 2 * ST;
+  uint64_t* a_full = bars + ST;
   uint64_t* c_full = a_full + 1;
   uint64_t* k_full = c_full + S::NCF;
   uint64_t* b_free = k_full + NB;
@@ -175,19 +186,18 @@ __device__ __forceinline__ void tc2_body(const Tc2DevArgs& a, const int rb, cons
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + S::OFF_BARS + S::NBARS * 8);
   volatile int* s_fail = reinterpret_cast<volatile int*>(s_tmem + 1);
   int* s_last = reinterpret_cast<int*>(s_tmem + 2);
-  auto stage = [&](int s) -> unsigned char* { return smem + S::OFF_STAGES + s * S::STAGE_BYTES; };
+  const uint32_t full0 = smem_u32(full), c_full0 = smem_u32(c_full), k_full0 = smem_u32(k_full),
+                 b_free0 = smem_u32(b_free);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform for the compiler
   const long long slot = (long long)rb * a.nsplit + sp;   // this CTA's partial-sum slot
   const long long row0 = (long long)rb * kT2BM;
   const int tile_begin = sp * a.tiles_per_split;
   const int nt = max(0, min(tile_begin + a.tiles_per_split, a.ntiles) - tile_begin);
 
   if (tid == 0) {
-    for (int s = 0; s < ST; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);   // the MMA commit: only the tensor cores read a stage
-    }
+    for (int s = 0; s < ST; ++s) mbar_init(&full[s], 1);
     mbar_init(a_full, 1);
     for (int c = 0; c < S::NCF; ++c) mbar_init(&c_full[c], 1);
     for (int b = 0; b < NB; ++b) {
@@ -198,73 +208,72 @@ __device__ __forceinline__ void tc2_body(const Tc2DevArgs& a, const int rb, cons
     fence_barrier_init();
     *s_fail = 0;
   }
-  if (warp == 1) tc::tmem_alloc(s_tmem, kT2Cols);
+  if (warp == 0) tc::tmem_alloc(s_tmem, kT2Cols);
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
-  const uint32_t tbase = *s_tmem;
-  int issued = 0;   // tiles whose copies the producer started (lane 0 of warp 0)
+  const uint32_t tbase = __shfl_sync(0xffffffffu, *s_tmem, 0);
+  int issued = 0;   // tiles whose copies were started (warp 0)
 
   if (warp == 0) {
-    // ---------------- producer: the x^_I image, then x^_J, b_J, V_J into the ring ----------
-    if (lane == 0) {
-      mbar_arrive_expect_tx(a_full, 2 * S::A_BYTES);
-      bulk_g2s(sAh, a.A_hi + row0 * K8, S::A_BYTES, a_full);
-      bulk_g2s(sAl, a.A_lo + row0 * K8, S::A_BYTES, a_full);
-      for (int lt = 0; lt < nt; ++lt) {
-        const int s = lt % ST;
-        if (lt >= ST && !mbar_wait_backoff(&empty[s], (uint32_t)(((lt / ST) - 1) & 1))) {
-          *s_fail = 1;
-          break;
-        }
-        if (*s_fail) break;
-        const long long t = tile_begin + lt;
-        unsigned char* st = stage(s);
-        mbar_arrive_expect_tx(&full[s], S::STAGE_BYTES);
-        bulk_g2s(st, a.B_hi + t * kT2BN * K8, S::XB_BYTES, &full[s]);
-        bulk_g2s(st + S::XB_BYTES, a.B_lo + t * kT2BN * K8, S::XB_BYTES, &full[s]);
-        unsigned char* sv = st + 2 * S::XB_BYTES;
-        bulk_g2s(sv, a.V_hi + t * N * kT2BN, S::V_BYTES, &full[s]);
-        bulk_g2s(sv + S::V_BYTES, a.V_lo + t * N * kT2BN, S::V_BYTES, &full[s]);
-        if constexpr (BJ) bulk_g2s(st + S::OFF_BN, a.bneg + t * kT2BN, S::BN_BYTES, &full[s]);
-        issued = lt + 1;
+    // ------ copies and MMAs: C = x^_I x^_J^T, then U += K V; one elected lane issues, the
+    //        whole warp runs the loop, so that descriptors and addresses stay warp-uniform ------
+    constexpr uint32_t idesc_c = tc::instr_desc(2, kT2BM, kT2BN);   // TF32
+    constexpr uint32_t idesc_u = tc::instr_desc(1, kT2BM, N);       // BF16
+    constexpr uint32_t sbo_x = (K8 / 4) * 128;
+    const uint64_t dAh = tc::smem_desc(smem0, 128, sbo_x);
+    const uint64_t dAl = tc::smem_desc(smem0 + S::A_BYTES, 128, sbo_x);
+    const uint64_t dB0 = tc::smem_desc(smem0 + S::OFF_STAGES, 128, sbo_x);
+    const uint64_t dV0 = tc::smem_desc(smem0 + S::OFF_STAGES + S::OFF_V, 128, 512);
+    const float* srcX = a.B + (long long)tile_begin * tc2_b_stride(K8);
+    const __nv_bfloat16* srcV = a.Vp + (long long)tile_begin * 2 * N * kT2BN;
+    auto copy_tile = [&](int p, int s) {   // elected lane: tile p's B_J (with b_J) and V_J
+      unsigned char* st = smem + S::OFF_STAGES + s * S::STAGE_BYTES;
+      mbar_arrive_expect_tx(&full[s], S::STAGE_BYTES);
+      bulk_g2s(st, srcX + (long long)p * tc2_b_stride(K8), S::X_COPY, &full[s]);
+      bulk_g2s(st + S::OFF_V, srcV + (long long)p * 2 * N * kT2BN, 2 * S::V_BYTES, &full[s]);
+    };
+    auto mma_c = [&](int s, int b, int cf) {   // elected lane: C into buffer b
+      const uint64_t dBh = dB0 + (uint64_t)s * (S::STAGE_BYTES >> 4), dBl = dBh + (S::XB_BYTES >> 4);
+      const uint32_t dC = tbase + (uint32_t)(b * 32);
+#pragma unroll
+      for (int term = 0; term < 3; ++term) {
+        const uint64_t A = term == 2 ? dAl : dAh;
+        const uint64_t B = term == 1 ? dBl : dBh;
+#pragma unroll
+        for (int ks = 0; ks < K8 / 8; ++ks)
+          tc::mma_tf32(dC, A + 16u * ks, B + 16u * ks, idesc_c, (term | ks) != 0);
       }
+      tc::commit(&c_full[cf]);
+    };
+    const int pre = min(ST, nt);
+    if (tc::elect_one()) {
+      mbar_arrive_expect_tx(a_full, 2 * S::A_BYTES);
+      bulk_g2s(smem, a.A_hi + row0 * K8, S::A_BYTES, a_full);
+      bulk_g2s(smem + S::A_BYTES, a.A_lo + row0 * K8, S::A_BYTES, a_full);
+      for (int p = 0; p < pre; ++p) copy_tile(p, p);
     }
-  } else if (warp == 1) {
-    // ---------------- MMA issuer: C = x^_I x^_J^T, then U += K V ----------------
-    if (lane == 0) {
-      constexpr uint32_t idesc_c = tc::instr_desc(2, kT2BM, kT2BN);   // TF32
-      constexpr uint32_t idesc_u = tc::instr_desc(1, kT2BM, N);       // BF16
-      constexpr uint32_t sbo_x = (K8 / 4) * 128;
-      const uint32_t aH = smem_u32(sAh), aL = smem_u32(sAl);
-      const uint64_t dAh = tc::smem_desc(aH, 128, sbo_x), dAl = tc::smem_desc(aL, 128, sbo_x);
-      const uint64_t dB0 = tc::smem_desc(smem_u32(stage(0)), 128, sbo_x);
-      const uint64_t dV0 = tc::smem_desc(smem_u32(stage(0)) + 2 * S::XB_BYTES, 128, 512);
-      bool ok = mbar_wait_spin(a_full, 0);
-      auto issue_c = [&](int p) -> bool {
-        const int s = p % ST, b = p % NB;
-        if (!mbar_wait_spin(&full[s], (uint32_t)((p / ST) & 1))) return false;
-        tc::fence_after();
-        const uint64_t dBh = dB0 + (uint64_t)s * (S::STAGE_BYTES >> 4), dBl = dBh + (S::XB_BYTES >> 4);
-        const uint32_t dC = tbase + (uint32_t)(b * 32);
-#pragma unroll
-        for (int term = 0; term < 3; ++term) {
-          const uint64_t A = term == 2 ? dAl : dAh;
-          const uint64_t B = term == 1 ? dBl : dBh;
-#pragma unroll
-          for (int ks = 0; ks < K8 / 8; ++ks)
-            tc::mma_tf32(dC, A + 16u * ks, B + 16u * ks, idesc_c, (term | ks) != 0);
-        }
-        tc::commit(&c_full[p % S::NCF]);
-        return true;
-      };
-      if (ok) tc::fence_after();
-      for (int p = 0; p < min(NB, nt) && ok; ++p) ok = issue_c(p);
-      for (int p = 0; p < nt && ok; ++p) {
-        if (*s_fail) { ok = false; break; }
-        const int s = p % ST, b = p % NB;
-        if (!mbar_wait_spin(&k_full[b], (uint32_t)((p / NB) & 1))) { ok = false; break; }
-        tc::fence_after();
+    issued = pre;
+    bool ok = tc::warp_wait_uniform(smem_u32(a_full), 0);
+    // s_c, cf: stage and c_full barrier of the next tile whose C is issued; s, b: stage and
+    // buffer of tile p
+    int s_c = 0, ph_c = 0, cf = 0;
+    for (int p = 0; p < NB && p < nt && ok; ++p) {
+      ok = tc::warp_wait_uniform(full0 + 8u * s_c, ph_c);
+      tc::fence_after();
+      if (ok && tc::elect_one()) mma_c(s_c, p, cf);
+      __syncwarp();
+      if (++s_c == ST) { s_c = 0; ph_c ^= 1; }
+      if (++cf == S::NCF) cf = 0;
+    }
+    int s = 0, b = 0, ph_b = 0;
+#pragma unroll 1
+    for (int p = 0; p < nt && ok; ++p) {
+      ok = tc::warp_wait_uniform(k_full0 + 8u * b, ph_b);
+      if (!ok) break;
+      tc::fence_after();
+      const bool more_c = p + NB < nt, more_v = p + ST < nt;
+      if (tc::elect_one()) {
         const uint64_t dVh = dV0 + (uint64_t)s * (S::STAGE_BYTES >> 4), dVl = dVh + (S::V_BYTES >> 4);
         const uint32_t kcol = tbase + (uint32_t)(b * 32);
 #pragma unroll
@@ -275,38 +284,54 @@ __device__ __forceinline__ void tc2_body(const Tc2DevArgs& a, const int rb, cons
           for (int ks = 0; ks < kT2BN / 16; ++ks)
             tc::mma_bf16_ts(tbase + S::COL_U, A + ks * 16, B + 16u * ks, idesc_u, (p | term | ks) != 0);
         }
-        tc::commit(&empty[s]);
-        if (p + NB < nt) {
-          // buffer b takes tile p + NB's C only after these MMAs have read its K
-          tc::commit(&b_free[b]);
-          if (!mbar_wait_spin(&b_free[b], (uint32_t)((p / NB) & 1))) { ok = false; break; }
+        // buffer b takes tile p + NB's C, and stage s tile p + ST's operands, only after these
+        // MMAs have read its K and V
+        if (more_c || more_v) tc::commit(&b_free[b]);
+      }
+      __syncwarp();
+      if (more_c || more_v) {
+        ok = tc::warp_wait_uniform(b_free0 + 8u * b, ph_b);
+        if (ok && more_c) {
+          ok = tc::warp_wait_uniform(full0 + 8u * s_c, ph_c);
           tc::fence_after();
-          ok = issue_c(p + NB);
+          if (ok && tc::elect_one()) mma_c(s_c, b, cf);
+          __syncwarp();
+          if (++s_c == ST) { s_c = 0; ph_c ^= 1; }
+          if (++cf == S::NCF) cf = 0;
+        }
+        if (ok && more_v) {
+          if (tc::elect_one()) copy_tile(p + ST, s);
+          __syncwarp();
+          issued = p + ST + 1;
         }
       }
-      if (!ok) *s_fail = 1;
-      tc::commit(done);
+      if (++s == ST) s = 0;
+      if (++b == NB) { b = 0; ph_b ^= 1; }
     }
+    if (!ok) *s_fail = 1;
+    if (tc::elect_one()) tc::commit(done);
+    __syncwarp();
   } else {
     // ------ epilogue: 8 warps; warp (lane quadrant eq, set h) takes the tiles h, h + 2, ...
-    //        with all 32 of their columns, in two 16-column halves ------
+    //        with all 32 of their columns ------
     const int eq = warp & 3;
-    const int half = (warp - 2) >> 2;   // tile set; also the half of U it reads back
+    const int half = (warp - 1) >> 2;   // tile set; also the half of U it reads back
     const int il = eq * 32 + lane;
     const long long i = row0 + il;
     const uint32_t lane_base = (uint32_t)(eq * 32) << 16;
     const float ai = a.params->c0f + a.bneg[i];   // bneg covers the padded rows (zero there)
     bool ok = true;
+    int s = half % ST, ph_s = 0, b = half % NB, cf = half, ph_cf = 0;
+#pragma unroll 1
     for (int lt = half; lt < nt; lt += 2) {
-      const int b = lt % NB;
+      ok = tc::warp_wait_uniform(c_full0 + 8u * cf, ph_cf);
       // b_J is read from the stage: wait for its copy too (the stage is refilled only after
       // this tile's contraction, which waits for this warp's K)
-      const bool ready =
-          t2_warp_wait(&c_full[lt % S::NCF], (uint32_t)((lt / S::NCF) & 1)) &&
-          (!BJ || t2_warp_wait(&full[lt % ST], (uint32_t)((lt / ST) & 1)));
-      if (!__all_sync(0xffffffffu, ready && !*s_fail)) { ok = false; break; }
+      if constexpr (BJ) ok = ok && tc::warp_wait_uniform(full0 + 8u * s, ph_s);
+      if (!ok) break;
       tc::fence_after();
-      const float* bj = reinterpret_cast<const float*>(stage(lt % ST) + S::OFF_BN);
+      const float4* bj = reinterpret_cast<const float4*>(smem + S::OFF_STAGES + s * S::STAGE_BYTES +
+                                                         S::OFF_BN);
       // all 32 columns of C in one tensor-memory round trip; each pair's K high and low parts
       // are written back into the pair's own registers (no extra registers live)
       const uint32_t ccol = tbase + lane_base + (uint32_t)(b * 32);
@@ -317,26 +342,29 @@ __device__ __forceinline__ void tc2_body(const Tc2DevArgs& a, const int rb, cons
       const float2 ai2 = make_float2(ai, ai);
       const float2 minus1 = make_float2(-1.f, -1.f);
 #pragma unroll
-      for (int q = 0; q < 16; ++q) {
-        // the exponent is <= log2 sigma^2 up to rounding (about 1e-6 relative in k)
-        float2 e = ai2;
-        if constexpr (BJ) e = __fadd2_rn(e, *reinterpret_cast<const float2*>(bj + 2 * q));
-        e = __fadd2_rn(e, make_float2(__uint_as_float(c[2 * q]), __uint_as_float(c[2 * q + 1])));
-        const float2 k = make_float2(ex2_approx(e.x), ex2_approx(e.y));
-        const __nv_bfloat162 h = __floats2bfloat162_rn(k.x, k.y);
-        const float2 r = __ffma2_rn(__bfloat1622float2(h), minus1, k);   // k - high part
-        const __nv_bfloat162 l = __floats2bfloat162_rn(r.x, r.y);
-        c[2 * q] = *reinterpret_cast<const uint32_t*>(&h);
-        c[2 * q + 1] = *reinterpret_cast<const uint32_t*>(&l);
-      }
-#pragma unroll
       for (int hh = 0; hh < 2; ++hh) {
+        uint32_t hi[8], lo[8];
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
+          if constexpr (BJ) b4 = bj[4 * hh + g];
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            const int e0 = 16 * hh + 4 * g + 2 * q;
+            // the exponent is <= log2 sigma^2 up to rounding (about 1e-6 relative in k)
+            float2 e = ai2;
+            if constexpr (BJ) e = __fadd2_rn(e, q == 0 ? make_float2(b4.x, b4.y) : make_float2(b4.z, b4.w));
+            e = __fadd2_rn(e, make_float2(__uint_as_float(c[e0]), __uint_as_float(c[e0 + 1])));
+            const float2 k = make_float2(ex2_approx(e.x), ex2_approx(e.y));
+            const __nv_bfloat162 h = __floats2bfloat162_rn(k.x, k.y);
+            const float2 r = __ffma2_rn(__bfloat1622float2(h), minus1, k);   // k - high part
+            const __nv_bfloat162 l = __floats2bfloat162_rn(r.x, r.y);
+            hi[2 * g + q] = *reinterpret_cast<const uint32_t*>(&h);
+            lo[2 * g + q] = *reinterpret_cast<const uint32_t*>(&l);
+          }
+        }
         // columns [16 hh, 16 hh + 16): high parts, then low parts (the A operand of the
         // contraction's k-step hh)
-        const uint32_t hi[8] = {c[16 * hh + 0], c[16 * hh + 2], c[16 * hh + 4], c[16 * hh + 6],
-                                c[16 * hh + 8], c[16 * hh + 10], c[16 * hh + 12], c[16 * hh + 14]};
-        const uint32_t lo[8] = {c[16 * hh + 1], c[16 * hh + 3], c[16 * hh + 5], c[16 * hh + 7],
-                                c[16 * hh + 9], c[16 * hh + 11], c[16 * hh + 13], c[16 * hh + 15]};
         tc::tmem_st8(ccol + 16 * hh, hi);
         tc::tmem_st8(ccol + 16 * hh + 8, lo);
       }
@@ -344,9 +372,15 @@ __device__ __forceinline__ void tc2_body(const Tc2DevArgs& a, const int rb, cons
       tc::fence_before();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&k_full[b]);
+      s += 2;
+      if (s >= ST) { s -= ST; ph_s ^= 1; }
+      b += 2;
+      if (b >= NB) b -= NB;
+      cf += 2;
+      if (cf >= S::NCF) { cf -= S::NCF; ph_cf ^= 1; }
     }
     if (!ok) *s_fail = 1;
-    const bool fin = ok && t2_warp_wait(done, 0);
+    const bool fin = ok && tc::warp_wait_uniform(smem_u32(done), 0);
     ok = __all_sync(0xffffffffu, fin && !*s_fail);
     if (ok && nt > 0) {
       tc::fence_after();
@@ -376,21 +410,18 @@ __device__ __forceinline__ void tc2_body(const Tc2DevArgs& a, const int rb, cons
   }
 
   // -------- all roles: release tensor memory; last CTA of the row block reduces --------
-  if (warp == 1) {
-    if (lane == 0) (void)mbar_wait_backoff(done, 0);
-    __syncwarp();
-  }
+  if (warp == 0) (void)tc::warp_wait_uniform(smem_u32(done), 0);
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
-  if (warp == 1) tc::tmem_dealloc(tbase, kT2Cols);
+  if (warp == 0) tc::tmem_dealloc(tbase, kT2Cols);
   if (*s_fail) {
     if (tid == 0) {
       atomicOr(a.status, kStatusTimeout);
       // let the copies still in flight land before the CTA's shared memory goes away
       (void)mbar_wait_bounded(a_full, 0);
-      for (int lt2 = max(0, issued - S::ST); lt2 < issued; ++lt2)
-        (void)mbar_wait_bounded(&full[lt2 % S::ST], (uint32_t)((lt2 / S::ST) & 1));
+      for (int lt2 = max(0, issued - ST); lt2 < issued; ++lt2)
+        (void)mbar_wait_bounded(&full[lt2 % ST], (uint32_t)((lt2 / ST) & 1));
     }
     return;
   }
@@ -442,8 +473,7 @@ __global__ void pack_v_batch_kernel(const Tc2DevArgs* __restrict__ args, int N) 
   if (R <= 0) return;
   const long long ntiles = a.ntiles;
   const long long per_tile = (long long)N * kT2BN;
-  __nv_bfloat16* Vhi = const_cast<__nv_bfloat16*>(a.V_hi);
-  __nv_bfloat16* Vlo = const_cast<__nv_bfloat16*>(a.V_lo);
+  __nv_bfloat16* Vp = const_cast<__nv_bfloat16*>(a.Vp);
   for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < ntiles * per_tile;
        idx += (long long)gridDim.x * blockDim.x) {
     const long long t = idx / per_tile;
@@ -453,9 +483,9 @@ __global__ void pack_v_batch_kernel(const Tc2DevArgs* __restrict__ args, int N) 
     const float v = (r < R && j < a.n) ? a.V[(long long)a.vmap[r] * a.ldv + j] : 0.f;
     const __nv_bfloat16 h = __float2bfloat16_rn(v);
     const __nv_bfloat16 l = __float2bfloat16_rn(v - __bfloat162float(h));
-    const long long off = t * per_tile + tc::canon_offset(r, jj, 2, kT2BN / 8) / 2;
-    Vhi[off] = h;
-    Vlo[off] = l;
+    const long long off = t * 2 * per_tile + tc::canon_offset(r, jj, 2, kT2BN / 8) / 2;
+    Vp[off] = h;
+    Vp[off + per_tile] = l;
   }
 }
 
@@ -501,11 +531,9 @@ struct Tc2Inst {
     Tc2DevArgs a;
     a.A_hi = L.X_hi;
     a.A_lo = L.X_lo;
-    a.B_hi = L.X_hi + L.X_off;
-    a.B_lo = L.X_lo + L.X_off;
+    a.B = L.X_b;
     a.bneg = L.bneg;
-    a.V_hi = static_cast<const __nv_bfloat16*>(L.V_hi);
-    a.V_lo = static_cast<const __nv_bfloat16*>(L.V_lo);
+    a.Vp = static_cast<const __nv_bfloat16*>(L.Vp);
     a.V = static_cast<const float*>(L.V);
     a.ldv = L.ldv;
     a.vmap = L.vmap;
@@ -544,7 +572,7 @@ static cudaError_t tc2_dispatch_n(TcLaunch& L, cudaStream_t s) {
 static int tc2_k8(int DP) { return DP >= 8 ? DP : 8; }
 
 cudaError_t launch_kmv_tc2(TcLaunch& L, cudaStream_t s) {
-  if (L.R < 1 || L.R > 64 || !L.X_hi || !L.X_lo) return cudaErrorInvalidValue;
+  if (L.R < 1 || L.R > 64 || !L.X_hi || !L.X_lo || !L.X_b) return cudaErrorInvalidValue;
   switch (L.DP) {
     case 2:
     case 4: return tc2_dispatch_n<8, false>(L, s);
@@ -556,12 +584,12 @@ cudaError_t launch_kmv_tc2(TcLaunch& L, cudaStream_t s) {
 
 cudaError_t launch_pack_x_tf32(const float* xhat, const float* bneg, const DevParams* params,
                                int DP, long long n, long long ld128, float* X_hi, float* X_lo,
-                               long long X_off, int num_sms, cudaStream_t s, bool aug) {
+                               float* X_b, int num_sms, cudaStream_t s, bool aug) {
   const int K8 = tc2_k8(DP);
   const long long total = ld128 * K8;
   const int blocks = (int)std::min<long long>((total + 255) / 256, 8LL * num_sms);
   pack_x_tf32_kernel<<<blocks, 256, 0, s>>>(xhat, bneg, params, DP, K8, aug ? 1 : 0, n, ld128,
-                                            X_hi, X_lo, X_hi + X_off, X_lo + X_off);
+                                            X_hi, X_lo, X_b);
   return cudaGetLastError();
 }
 
@@ -580,11 +608,9 @@ cudaError_t tc2_batch_upload_args(const TcLaunch* L, int B, void* args_dev, cuda
     const long long ntiles = (l.n + kT2BN - 1) / kT2BN;
     a.A_hi = l.X_hi;
     a.A_lo = l.X_lo;
-    a.B_hi = l.X_hi + l.X_off;
-    a.B_lo = l.X_lo + l.X_off;
+    a.B = l.X_b;
     a.bneg = l.bneg;
-    a.V_hi = static_cast<const __nv_bfloat16*>(l.V_hi);
-    a.V_lo = static_cast<const __nv_bfloat16*>(l.V_lo);
+    a.Vp = static_cast<const __nv_bfloat16*>(l.Vp);
     a.V = static_cast<const float*>(l.V);
     a.ldv = l.ldv;
     a.vmap = l.vmap;

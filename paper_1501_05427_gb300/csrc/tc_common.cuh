@@ -184,6 +184,32 @@ __device__ inline float tf32_round(float x) {
   return __uint_as_float(y);
 }
 
+// One lane of a converged warp (the same one each time): the lane that issues MMAs, commits
+// and bulk copies while the whole warp keeps the loop's control flow uniform.
+__device__ inline bool elect_one() {
+  uint32_t p;
+  asm volatile("{ .reg .pred q; elect.sync _|q, 0xffffffff; selp.u32 %0, 1, 0, q; }" : "=r"(p));
+  return p != 0;
+}
+
+// Bounded wait of a whole converged warp, with a warp-uniform result (about a second at most,
+// then false).  The first poll is inline: most waits of a full pipeline end there.
+__device__ __forceinline__ bool warp_wait_uniform(uint32_t bar, uint32_t parity) {
+#pragma unroll 1
+  for (int it = 0; it < (1 << 25); ++it) {
+    uint32_t ok;
+    asm volatile(
+        "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; "
+        "selp.u32 %0, 1, 0, p; }"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (__all_sync(0xffffffffu, ok != 0)) return true;
+    if (it > (1 << 16)) __nanosleep(32);
+  }
+  return false;
+}
+
 // mbarrier arrive (count one) from a generic thread.
 __device__ inline void mbar_arrive(uint64_t* bar) {
   asm volatile("{ .reg .b64 st; mbarrier.arrive.shared::cta.b64 st, [%0]; }" ::"r"(smem_u32(bar))

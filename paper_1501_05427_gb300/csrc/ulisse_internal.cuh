@@ -265,12 +265,12 @@ struct GradLaunch {
   void* tc_hi;
   void* tc_lo;
   long long tc_ld;
-  // padded d <= 8: the TF32 row images of launch_pack_x_tf32 (A rows at X_hi / X_lo, B rows
-  // X_off floats further on), from which the pass forms the exponent's cross term on the
-  // tensor cores; c_has_bj when they were packed with the augmented column (b_j in C)
+  // padded d <= 8: the TF32 row images of launch_pack_x_tf32, from which the pass forms the
+  // exponent's cross term on the tensor cores; c_has_bj when they were packed with the
+  // augmented column (b_j in C)
   const float* X_hi;
   const float* X_lo;
-  long long X_off;
+  const float* X_b;
   bool c_has_bj;
 };
 
@@ -278,8 +278,8 @@ struct GradLaunch {
 struct TcLaunch {
   const float* xhat;     // prescaled inputs, ld x DP row-major (the SIMT layout)
   const float* bneg;     // -c1 |x^|^2 (launch_prescale_tc), ld128
-  void* V_hi;            // BF16 packed operand tiles (written by the launch), ld128 x 64
-  void* V_lo;
+  void* Vp;              // BF16 packed operand tiles, high | low part per tile (written by the
+                         // launch), ld128 x 128
   const void* V;         // FP32 operand columns
   long long ldv;
   const int* vmap;
@@ -304,10 +304,10 @@ struct TcLaunch {
   int need_counters;
   bool plan_only;        // only fill need_* (no launch): sizing scratch ahead of a capture
   // tensor-core cross term (launch_kmv_tc2): TF32 images of the augmented rows
-  // (launch_pack_x_tf32): A rows at X_hi / X_lo, B rows X_off floats further on
+  // (launch_pack_x_tf32): A rows at X_hi / X_lo, B tiles at X_b
   const float* X_hi;
   const float* X_lo;
-  long long X_off;
+  const float* X_b;
 };
 
 // Launchers (return cudaSuccess or the launch error).
@@ -323,11 +323,14 @@ cudaError_t launch_kmv_tc(TcLaunch& L, cudaStream_t s);
 cudaError_t launch_grad_tc(GradLaunch& L, cudaStream_t s);
 cudaError_t launch_kmv_tc2(TcLaunch& L, cudaStream_t s);
 void launch_pack_v(const TcLaunch& L, int N, long long ntiles, cudaStream_t s);
+// A rows: high part X_hi and remainder X_lo, ld128 x K8 floats each (K8 = max(8, DP)); B rows:
+// tiles of 32 points, high part | remainder | b_j, tc2_b_stride(K8) floats each, ld128 / 32 tiles.
+__host__ __device__ constexpr int tc2_b_stride(int K8) { return 2 * 32 * K8 + 32; }
 // aug: rows carry the column term b_j (padded d 2 and 4 of the single-problem launches);
 // false for the batched launches, whose epilogue adds it for every d.
 cudaError_t launch_pack_x_tf32(const float* xhat, const float* bneg, const DevParams* params,
                                int DP, long long n, long long ld128, float* X_hi, float* X_lo,
-                               long long X_off, int num_sms, cudaStream_t s, bool aug);
+                               float* X_b, int num_sms, cudaStream_t s, bool aug);
 // Batched tensor-core K V (padded d <= 8): per problem a TcLaunch with the operand pointers,
 // R or R_dev, and the forced split nsplit >= 1 (tiles per split <= kTcMaxSplitTiles);
 // items: (problem, 128-row block, split) per CTA; R_max: the largest live column count.
