@@ -29,7 +29,7 @@ struct ulisse_ctx {
   long long ld128 = 0;        // rows of the tensor-core operand images (multiple of 128)
   float* bneg = nullptr;      // -log2(e)/2 |x^|^2 per input (tensor-core path)
   void* Vt = nullptr;         // BF16 operand tiles of K V, high | low part per tile
-  void *Gt_hi = nullptr, *Gt_lo = nullptr;   // packed operands of the tensor-core gradient
+  void* Gt = nullptr;         // packed operand blocks of the tensor-core gradient
   float *Xt_hi = nullptr, *Xt_lo = nullptr;  // TF32 images of the A rows (tensor-core cross term)
   float* Xt_b = nullptr;      // ... and the tiles of the B rows, see launch_pack_x_tf32
 
@@ -864,9 +864,7 @@ static ulisse_status run_grad(ulisse_ctx* ctx, int M, const int* amap = nullptr,
   L.status = ctx->status_dev;
   L.num_sms = ctx->num_sms;
   L.bneg = ctx->bneg;
-  L.tc_hi = ctx->Gt_hi;
-  L.tc_lo = ctx->Gt_lo;
-  L.tc_ld = ctx->ld128;
+  L.tc_tiles = ctx->Gt;
   set_grad_images(L, ctx);
   for (int attempt = 0; attempt < 2; ++attempt) {
     L.partials = ctx->gpart;
@@ -890,7 +888,7 @@ static ulisse_status run_grad(ulisse_ctx* ctx, int M, const int* amap = nullptr,
         ctx->free_events.push_back({ea, eb});
     }
     if (e == cudaSuccess && !ctx->planning) {
-      if (!ctx->capturing) ctx->launches += ctx->mixed ? 3 : 1;   // tensor cores: 2 packings
+      if (!ctx->capturing) ctx->launches += ctx->mixed ? 2 : 1;   // tensor cores: the packing
       break;
     }
     if (e != cudaSuccess && (e != cudaErrorMemoryAllocation || attempt == 1 || ctx->capturing))
@@ -1046,8 +1044,7 @@ static ulisse_status create_impl(ulisse_ctx** out, const float* X, const float* 
   if (ctx->mixed) {
     if ((s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->bneg), sizeof(float) * ctx->ld128)) ||
         (s = dev_alloc(ctx, &ctx->Vt, 2 * 2 * ctx->ld128 * 64)) ||
-        (s = dev_alloc(ctx, &ctx->Gt_hi, 2 * ctx->ld128 * kGtScratchRows)) ||
-        (s = dev_alloc(ctx, &ctx->Gt_lo, 2 * ctx->ld128 * kGtScratchRows)) ||
+        (s = dev_alloc(ctx, &ctx->Gt, 2 * 2 * ctx->ld128 * kGtScratchRows)) ||
         (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->Xt_hi), 4 * ctx->ld128 * 16)) ||
         (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->Xt_lo), 4 * ctx->ld128 * 16)) ||
         (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->Xt_b),
@@ -1646,7 +1643,7 @@ static ulisse_status graph_build(ulisse_ctx* ctx, int s0_cols) {
   // prescale (+ the tensor-core images), probes, the CG start, the gradient pass (+ its
   // operand images), the update, the learned start's two kernels, the product K s_0
   ctx->graph_launches_fixed = (ctx->mixed ? 3 : 1) + 1 + cg_init_launch_count(ctx->n, R, ctx->num_sms) +
-      (ctx->mixed ? 3 : 1) + 1 + (s0_cols > 0 ? 2 : 0) +
+      (ctx->mixed ? 2 : 1) + 1 + (s0_cols > 0 ? 2 : 0) +
       (init_cols > 0 ? kmv_per * ((init_cols + kmv_cols - 1) / kmv_cols) : 0);
   ctx->graph_entries_fixed = (double)ctx->n * (double)ctx->n * (double)(R + init_cols);
   ctx->graph_rounds_fixed = init_cols > 0 ? 1 : 0;
@@ -2516,9 +2513,7 @@ static ulisse_status batch_prepare(ulisse_ctx* ctx) {
         L.g_out = ctx->b_g + (long long)b * kMaxP;
         L.status = ctx->status_dev;
         L.bneg = sub->bneg;
-        L.tc_hi = sub->Gt_hi;
-        L.tc_lo = sub->Gt_lo;
-        L.tc_ld = sub->ld128;
+        L.tc_tiles = sub->Gt;
         set_grad_images(L, sub);
         gl[li] = L;
         ns[li] = ctx->b_gt_nsplit[b];
@@ -3065,7 +3060,7 @@ void ulisse_destroy(ulisse_ctx* ctx) {
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
   for (void** p : {reinterpret_cast<void**>(&ctx->st_next), reinterpret_cast<void**>(&ctx->part1),
                    reinterpret_cast<void**>(&ctx->part2), reinterpret_cast<void**>(&ctx->bneg),
-                   &ctx->Vt, &ctx->Gt_hi, &ctx->Gt_lo,
+                   &ctx->Vt, &ctx->Gt,
                    reinterpret_cast<void**>(&ctx->Xt_hi), reinterpret_cast<void**>(&ctx->Xt_lo),
                    reinterpret_cast<void**>(&ctx->Xt_b),
                    reinterpret_cast<void**>(&ctx->q_map), &ctx->q_sa, &ctx->pcg_buf, &ctx->pred_xs,

@@ -29,13 +29,20 @@
 //   3. [S | G | H]_I += P_IJ Z_J on the tensor cores, Z_j = [x^_j, x^_j^2, 1] split the same
 //      way, accumulated in tensor memory across all tiles of the CTA's j range.
 // The per-row combination and the diagonal sum run in FP64 at the end; CTA partials are summed
-// in a fixed order by the last CTA to arrive (as in the SIMT gradient kernel).  Warp 0 streams
-// B_J's TF32 image (x^_J for d = 16), the row norms, B^_J and Z_J into a 3- or 4-stage ring
-// with bulk copies; one thread of warp 1 issues the MMAs; eight epilogue warps (a tensor-memory
-// lane quadrant and half of the tile's 32 columns each) make P.  W/P tiles are double-buffered;
-// a buffer is refilled only after the MMAs that read it have completed.  The single C buffer
-// takes the next tile's product as soon as the eight warps have read it, so those MMAs run
-// during the current tile's arithmetic.  Every wait is bounded.
+// in a fixed order by the last CTA to arrive (as in the SIMT gradient kernel).  Roles: warp 0
+// copies (B_J's TF32 image with b_J, or x^_J and b_J for d = 16, then B^_J and Z_J as one
+// block, into a ring of 3 to 6 stages) and issues the MMAs, its loop warp-uniform with a lane
+// elected for the issuing instructions; twelve epilogue warps make P in three sets of four (one
+// warp per tensor-memory lane quadrant): set h takes the tiles h, h + 3, ... whole and owns
+// the W/P and C buffers h, so that each wait and hand-off covers 32 entries per thread.  A
+// buffer pair is refilled, and the tile's stage with it, only after the MMAs that read P have
+// completed.  Every wait is bounded.
+//
+// What bounds it: the issue slots and the chain W, C -> epilogue -> P Z -> refill of each set.
+// Two CTAs per SM of three sets (256 tensor-memory columns each) took the place of three CTAs
+// whose eight epilogue warps shared every tile by column halves behind one C buffer: the waits,
+// fences and hand-offs are then paid once per 32 entries of a thread instead of once per 16, and
+// no set waits for another to read C.  n = 50,000, d = 8, M = 17: 1.224 -> 0.99 ms.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -49,58 +56,43 @@ namespace ulisse {
 
 constexpr int kGtBN = 32;
 constexpr int kGtBM = 128;
-constexpr int kGtThreads = 320;    // warp 0 producer, warp 1 MMA issuer, warps 2-9 epilogue
-constexpr uint32_t kGtCols = 128;  // tensor-memory columns per CTA
-constexpr int kGtZOff = 128;       // Z image offset in the packed scratch, in units of ld128
-static_assert(16 * 8 <= kGtZOff && kGtZOff + 48 <= kGtScratchRows,
-              "operand images exceed the gradient scratch");
+constexpr int kGtSets = 3;         // epilogue sets of four warps
+constexpr int kGtThreads = 32 * (1 + 4 * kGtSets);   // warp 0 copies and MMAs, then the epilogue
+constexpr uint32_t kGtCols = 256;  // tensor-memory columns per CTA (two CTAs per SM)
+static_assert(16 * 8 + 48 <= kGtScratchRows, "operand images exceed the gradient scratch");
 
 __device__ inline void split_bf16(float v, __nv_bfloat16& h, __nv_bfloat16& l) {
   h = __float2bfloat16_rn(v);
   l = __float2bfloat16_rn(v - __bfloat162float(h));
 }
 
-// Right operand [b_j | A^_j] of every 32-point tile as BF16 high and low parts: a K-major
-// canonical image of 32 points (rows) x K1 factor slots, slot m < M holding b_m[j] and slot
-// M + m holding sa[m] a_m[j]; slots >= 2M and points j >= n are zero.
-__global__ void pack_bt_kernel(const float* __restrict__ B, const int* __restrict__ bmap,
-                               const float* __restrict__ A, const int* __restrict__ amap,
-                               const float* __restrict__ sa, long long ld, int M, int K1,
-                               long long n, long long ntiles, __nv_bfloat16* __restrict__ Bhi,
-                               __nv_bfloat16* __restrict__ Blo) {
-  const long long per_tile = (long long)kGtBN * K1;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < ntiles * per_tile;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const long long t = idx / per_tile;
-    const int rem = (int)(idx - t * per_tile);
-    const int m = rem / kGtBN, j = rem - m * kGtBN;
-    const long long jj = t * kGtBN + j;
-    float v = 0.f;
+// One element of a tile's operand block: [b_j | A^_j] as a K-major canonical image of 32 points
+// (rows) x K1 factor slots (slot m < M holding b_m[j], slot M + m holding sa[m] a_m[j], slots
+// >= 2M zero), then Z_j = [x^_j (DP), x^_j^2 (DP), 1, 0...] as an image of N2 rows (accumulator
+// columns) x 32 points; each as BF16 high part and low part, the four parts back to back, so
+// that a tile is one bulk copy.  Points j >= n are zero.
+__device__ inline void gt_pack_element(long long idx, int K1, int N2, int DP, int M, long long n,
+                                       const float* __restrict__ xhat, const float* __restrict__ A,
+                                       const int* __restrict__ amap, const float* __restrict__ sa,
+                                       const float* __restrict__ B, const int* __restrict__ bmap,
+                                       long long ld, __nv_bfloat16* __restrict__ tiles) {
+  const int per_b = kGtBN * K1, per_z = N2 * kGtBN, per = per_b + per_z;
+  const long long t = idx / per;
+  const int rem = (int)(idx - t * per);
+  const int j = rem % kGtBN;
+  const long long jj = t * kGtBN + j;
+  float v = 0.f;
+  uint32_t off, part;
+  if (rem < per_b) {
+    const int m = rem / kGtBN;
     if (jj < n) {
       if (m < M) v = B[(long long)bmap[m] * ld + jj];
       else if (m < 2 * M) v = sa[m - M] * A[(long long)amap[m - M] * ld + jj];
     }
-    __nv_bfloat16 h, l;
-    split_bf16(v, h, l);
-    const long long off = t * per_tile + tc::canon_offset(j, m, 2, K1 / 8) / 2;
-    Bhi[off] = h;
-    Blo[off] = l;
-  }
-}
-
-// Z_j = [x^_j (DP), x^_j^2 (DP), 1, 0...] for every tile as BF16 high and low parts: a
-// K-major canonical image of N2 rows (accumulator columns) x 32 points; points j >= n are zero.
-__global__ void pack_z_kernel(const float* __restrict__ xhat, int DP, long long n, int N2,
-                              long long ntiles, __nv_bfloat16* __restrict__ Zhi,
-                              __nv_bfloat16* __restrict__ Zlo) {
-  const long long per_tile = (long long)N2 * kGtBN;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < ntiles * per_tile;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const long long t = idx / per_tile;
-    const int rem = (int)(idx - t * per_tile);
-    const int c = rem / kGtBN, j = rem - c * kGtBN;
-    const long long jj = t * kGtBN + j;
-    float v = 0.f;
+    off = tc::canon_offset(j, m, 2, K1 / 8) / 2;
+    part = (uint32_t)per_b;
+  } else {
+    const int c = (rem - per_b) / kGtBN;
     if (jj < n) {
       if (c < DP) {
         v = xhat[jj * DP + c];
@@ -111,21 +103,31 @@ __global__ void pack_z_kernel(const float* __restrict__ xhat, int DP, long long 
         v = 1.f;
       }
     }
-    __nv_bfloat16 h, l;
-    split_bf16(v, h, l);
-    const long long off = t * per_tile + tc::canon_offset(c, j, 2, kGtBN / 8) / 2;
-    Zhi[off] = h;
-    Zlo[off] = l;
+    off = 2u * per_b + tc::canon_offset(c, j, 2, kGtBN / 8) / 2;
+    part = (uint32_t)per_z;
   }
+  __nv_bfloat16 h, l;
+  split_bf16(v, h, l);
+  __nv_bfloat16* o = tiles + t * (2LL * per) + off;
+  o[0] = h;
+  o[part] = l;
+}
+
+__global__ void pack_gt_kernel(int K1, int N2, int DP, int M, long long n, long long ntiles,
+                               const float* __restrict__ xhat, const float* __restrict__ A,
+                               const int* __restrict__ amap, const float* __restrict__ sa,
+                               const float* __restrict__ B, const int* __restrict__ bmap,
+                               long long ld, __nv_bfloat16* __restrict__ tiles) {
+  const long long total = ntiles * kGtBN * (K1 + N2);
+  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
+       idx += (long long)gridDim.x * blockDim.x)
+    gt_pack_element(idx, K1, N2, DP, M, n, xhat, A, amap, sa, B, bmap, ld, tiles);
 }
 
 struct GtDevArgs {
   const float* xhat;   // x^ rows (ld x DP, row-major)
   const float* bneg;   // -c1 |x^|^2
-  const __nv_bfloat16* Bt_hi;
-  const __nv_bfloat16* Bt_lo;
-  const __nv_bfloat16* Zt_hi;
-  const __nv_bfloat16* Zt_lo;
+  const __nv_bfloat16* tiles;   // per tile B^ high | low, Z high | low (gt_pack_element)
   const float* A;      // left factors: column amap[m], scaled by sa[m]
   const int* amap;
   const float* sa;
@@ -153,7 +155,7 @@ struct GtDevArgs {
 
 // XC (padded d <= 8): the exponent's cross term C = A_I B_J^T on the tensor cores from the
 // TF32 row images (three TF32 products, as the K V pass); the stage carries B_J's image instead
-// of x^_J.  Padded d = 16 keeps the FP32 cross term (its accumulator leaves no room for C).
+// of x^_J.  Padded d = 16 keeps the FP32 cross term.
 template <int DP, int KS>
 struct GtShape {
   static constexpr bool XC = DP <= 8;
@@ -167,29 +169,32 @@ struct GtShape {
   static constexpr uint32_t BN_BYTES = kGtBN * 4;
   static constexpr uint32_t BT_BYTES = kGtBN * K1 * 2;
   static constexpr uint32_t Z_BYTES = N2 * kGtBN * 2;
+  static constexpr uint32_t TILE_BYTES = 2 * BT_BYTES + 2 * Z_BYTES;   // the packed block
   // stage: x^_J (FP32) or B_J (TF32 high | remainder), b_J, B^_J high | low, Z_J high | low
   static constexpr uint32_t OFF_BN = X_BYTES;
   static constexpr uint32_t OFF_BT = OFF_BN + BN_BYTES;
   static constexpr uint32_t OFF_Z = OFF_BT + 2 * BT_BYTES;
   static constexpr uint32_t STAGE_BYTES = OFF_Z + 2 * Z_BYTES;
-  static constexpr int NBARS_FIXED = 2 + 2 + 2 + 1 + 2;  // w_full, p_full, free, done, c_full/free
-  static constexpr uint32_t FIXED = 2 * A_BYTES + 2 * XA_BYTES + (8 + NBARS_FIXED) * 8 + 64;
-  // four stages unless three keep one more CTA per SM (228 KB of shared memory per SM)
-  static constexpr int occ_with(int st) {
-    const int o = (int)((228u * 1024u) / (FIXED + st * STAGE_BYTES + 2048u));
-    const int cap = DP >= 16 ? 2 : 3;   // the launch bounds' CTAs per SM
-    return o < cap ? o : cap;
-  }
-  static constexpr int ST = occ_with(4) >= occ_with(3) ? 4 : 3;
+  // cw_full, p_full, b_free per set; done
+  static constexpr int NBARS_FIXED = 3 * kGtSets + 1;
+  static constexpr uint32_t FIXED = 2 * A_BYTES + 2 * XA_BYTES + (6 + NBARS_FIXED) * 8 + 64;
+  // as many stages (3 to 6) as let two CTAs share the SM's 228 KB, else as fit one
+  static constexpr int fit(uint32_t budget) { return (int)((budget - FIXED) / STAGE_BYTES); }
+  static constexpr uint32_t kHalfSm = 110u * 1024u, kWholeSm = 222u * 1024u;
+  static constexpr int ST_HALF = FIXED < kHalfSm ? fit(kHalfSm) : 0;
+  static constexpr int OCC = ST_HALF >= kGtSets ? 2 : 1;   // CTAs per SM
+  static constexpr int ST_ANY = OCC == 2 ? ST_HALF : fit(kWholeSm);
+  static constexpr int ST = ST_ANY > 6 ? 6 : ST_ANY;
+  static_assert(ST >= kGtSets, "each set's next tile needs a stage");
   static constexpr uint32_t OFF_XA = 2 * A_BYTES;
   static constexpr uint32_t OFF_STAGES = OFF_XA + 2 * XA_BYTES;
   static constexpr uint32_t OFF_BARS = OFF_STAGES + ST * STAGE_BYTES;
-  static constexpr int NBARS = 2 * ST + NBARS_FIXED;    // full, empty, then the fixed ones
+  static constexpr int NBARS = ST + NBARS_FIXED;    // full per stage, then the fixed ones
   static constexpr uint32_t SMEM = OFF_BARS + NBARS * 8 + 64;
-  // tensor-memory columns: two W/P buffers of 32, the C buffer of 32 (XC), then the
+  // tensor-memory columns: the sets' W/P buffers of 32, their C buffers of 32 (XC), then the
   // [G | H | S] accumulator
-  static constexpr uint32_t COL_C = 64;
-  static constexpr uint32_t COL_D2 = XC ? 96 : 64;
+  static constexpr uint32_t COL_C = 32 * kGtSets;
+  static constexpr uint32_t COL_D2 = XC ? 64 * kGtSets : 32 * kGtSets;
   static_assert(COL_D2 + N2 <= kGtCols, "tensor memory layout exceeds the allocation");
   static_assert(X_BYTES % 16 == 0 && STAGE_BYTES % 16 == 0 && A_BYTES % 16 == 0 &&
                     OFF_BT % 16 == 0 && OFF_Z % 16 == 0 && OFF_STAGES % 16 == 0,
@@ -213,11 +218,6 @@ __device__ inline void gt_tmem_ld16_two(uint32_t ta, uint32_t tb, uint32_t (&r)[
       : "memory");
 }
 
-__device__ inline bool gt_warp_wait(uint64_t* bar, uint32_t parity) {
-  const bool ok = mbar_wait_spin(bar, parity);
-  return __all_sync(0xffffffffu, ok);
-}
-
 // One CTA's work: row block rb, split sp of its tile range.  Shared by the single-problem
 // kernel and the batched one.
 template <int DP, int KS>
@@ -226,24 +226,24 @@ __device__ __forceinline__ void gt_body(const GtDevArgs& a, const int rb, const 
   constexpr int ST = S::ST, K1 = S::K1, N2 = S::N2;
   constexpr int NACC = DP + 2;
   extern __shared__ __align__(1024) unsigned char smem[];
-  __shared__ double s_red[8][NACC];
+  __shared__ double s_red[4 * kGtSets][NACC];
   unsigned char* sAh = smem;
   unsigned char* sAl = smem + S::A_BYTES;
+  const uint32_t smem0 = smem_u32(smem);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S::OFF_BARS);
   uint64_t* full = bars;
-  uint64_t* empty = bars + ST;
-  uint64_t* w_full = bars + 2 * ST;
-  uint64_t* p_full = w_full + 2;
-  uint64_t* b_free = p_full + 2;
-  uint64_t* done = b_free + 2;
-  uint64_t* c_full = done + 1;   // XC: C_J formed (MMA commit)
-  uint64_t* c_free = done + 2;   // XC: the eight epilogue warps have read C_J
+  uint64_t* cw_full = bars + ST;           // W (and C) of the set's tile formed (MMA commit)
+  uint64_t* p_full = cw_full + kGtSets;    // P written by the set's four warps
+  uint64_t* b_free = p_full + kGtSets;     // P Z of the set's tile done (MMA commit)
+  uint64_t* done = b_free + kGtSets;
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + S::OFF_BARS + S::NBARS * 8);
   volatile int* s_fail = reinterpret_cast<volatile int*>(s_tmem + 1);
   int* s_last = reinterpret_cast<int*>(s_tmem + 2);
-  auto stage = [&](int s) -> unsigned char* { return smem + S::OFF_STAGES + s * S::STAGE_BYTES; };
+  const uint32_t full0 = smem_u32(full), cw_full0 = smem_u32(cw_full),
+                 p_full0 = smem_u32(p_full), b_free0 = smem_u32(b_free);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform for the compiler
   // Row block rb visits the tiles [4 rb, ntiles) (its own four tiles, then every later
   // one), cut into nsplit equal ranges; CTAs start in row-block order, longest ranges first.
   constexpr int kTilesPerBlock = kGtBM / kGtBN;
@@ -283,150 +283,137 @@ __device__ __forceinline__ void gt_body(const GtDevArgs& a, const int rb, const 
   }
   tc::fence_async_smem();
   if (tid == 0) {
-    for (int s = 0; s < ST; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1 + 8);   // MMA commit + the eight epilogue warps
-    }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&w_full[b], 1);
-      mbar_init(&p_full[b], 8);
-      mbar_init(&b_free[b], 1);
+    for (int s = 0; s < ST; ++s) mbar_init(&full[s], 1);
+    for (int h = 0; h < kGtSets; ++h) {
+      mbar_init(&cw_full[h], 1);
+      mbar_init(&p_full[h], 4);
+      mbar_init(&b_free[h], 1);
     }
     mbar_init(done, 1);
-    mbar_init(c_full, 1);
-    mbar_init(c_free, 8);
     fence_barrier_init();
     *s_fail = 0;
   }
-  if (warp == 1) tc::tmem_alloc(s_tmem, kGtCols);
+  if (warp == 0) tc::tmem_alloc(s_tmem, kGtCols);
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
-  const uint32_t tbase = *s_tmem;
-  int issued = 0;   // tiles whose copies the producer started (lane 0 of warp 0)
+  const uint32_t tbase = __shfl_sync(0xffffffffu, *s_tmem, 0);
+  int issued = 0;   // tiles whose copies were started (warp 0)
 
   double acc[NACC];
 #pragma unroll
   for (int k = 0; k < NACC; ++k) acc[k] = 0.0;
 
   if (warp == 0) {
-    // ---------- producer: x^_J (or B_J's TF32 image), b_J, B^_J and Z_J into the ring ----------
-    if (lane == 0) {
-      for (int lt = 0; lt < nt; ++lt) {
-        const int s = lt % ST;
-        if (lt >= ST && !mbar_wait_spin(&empty[s], (uint32_t)(((lt / ST) - 1) & 1))) {
-          *s_fail = 1;
-          break;
-        }
-        if (*s_fail) break;
-        const long long t = tile_begin + lt;
-        unsigned char* st = stage(s);
-        mbar_arrive_expect_tx(&full[s], S::STAGE_BYTES);
-        if constexpr (S::XC) {
-          bulk_g2s(st, a.XB + t * tc2_b_stride(S::K8), S::X_BYTES + S::BN_BYTES, &full[s]);
-        } else {
-          bulk_g2s(st, a.xhat + t * kGtBN * DP, S::X_BYTES, &full[s]);
-          bulk_g2s(st + S::OFF_BN, a.bneg + t * kGtBN, S::BN_BYTES, &full[s]);
-        }
-        unsigned char* bt = st + S::OFF_BT;
-        bulk_g2s(bt, a.Bt_hi + t * kGtBN * K1, S::BT_BYTES, &full[s]);
-        bulk_g2s(bt + S::BT_BYTES, a.Bt_lo + t * kGtBN * K1, S::BT_BYTES, &full[s]);
-        unsigned char* zt = st + S::OFF_Z;
-        bulk_g2s(zt, a.Zt_hi + t * N2 * kGtBN, S::Z_BYTES, &full[s]);
-        bulk_g2s(zt + S::Z_BYTES, a.Zt_lo + t * N2 * kGtBN, S::Z_BYTES, &full[s]);
-        issued = lt + 1;
-      }
-    }
-  } else if (warp == 1) {
-    // ------------- MMA issuer: W = A^ B^T and C = A B^T, then [G | H | S] += P Z -------------
-    if (lane == 0) {
-      constexpr uint32_t idesc_w = tc::instr_desc(1, kGtBM, kGtBN);
-      constexpr uint32_t idesc_g = tc::instr_desc(1, kGtBM, N2);
-      constexpr uint32_t sbo_k1 = (K1 / 8) * 128;
-      const uint32_t aH = smem_u32(sAh), aL = smem_u32(sAl);
-      auto issue_w = [&](int p) -> bool {
-        const int s = p % ST, b = p & 1;
-        if (!mbar_wait_spin(&full[s], (uint32_t)((p / ST) & 1))) return false;
-        tc::fence_after();
-        const uint32_t bH = smem_u32(stage(s) + S::OFF_BT);
-        const uint32_t bL = bH + S::BT_BYTES;
-        const uint32_t dW = tbase + (uint32_t)(b * 32);
-#pragma unroll
-        for (int term = 0; term < 3; ++term) {
-          const uint32_t A = term == 2 ? aL : aH;
-          const uint32_t B = term == 1 ? bL : bH;
-#pragma unroll
-          for (int ks = 0; ks < KS; ++ks)
-            tc::mma_bf16(dW, tc::smem_desc(A + ks * 256, 128, sbo_k1),
-                         tc::smem_desc(B + ks * 256, 128, sbo_k1), idesc_w, (term | ks) != 0);
-        }
-        tc::commit(&w_full[b]);
-        return true;
-      };
-      // C_J = A_I B_J^T into the single C buffer (three TF32 products, K = 8)
-      auto issue_c = [&](int p) -> bool {
-        const int s = p % ST;
-        if (!mbar_wait_spin(&full[s], (uint32_t)((p / ST) & 1))) return false;
-        tc::fence_after();
-        constexpr uint32_t idesc_c = tc::instr_desc(2, kGtBM, kGtBN);   // TF32
-        constexpr uint32_t sbo_x = (S::K8 / 4) * 128;
-        const uint32_t xa = smem_u32(smem + S::OFF_XA), xb = smem_u32(stage(s));
-#pragma unroll
-        for (int term = 0; term < 3; ++term) {
-          const uint32_t A = term == 2 ? xa + S::XA_BYTES : xa;
-          const uint32_t B = term == 1 ? xb + S::XB_BYTES : xb;
-          tc::mma_tf32(tbase + S::COL_C, tc::smem_desc(A, 128, sbo_x),
-                       tc::smem_desc(B, 128, sbo_x), idesc_c, term != 0);
-        }
-        tc::commit(c_full);
-        return true;
-      };
-      bool ok = true;
-      for (int p = 0; p < min(2, nt) && ok; ++p) ok = issue_w(p);
+    // ------ copies and MMAs: W = A^ B^T and C = A B^T, then [G | H | S] += P Z ------
+    constexpr uint32_t idesc_w = tc::instr_desc(1, kGtBM, kGtBN);
+    constexpr uint32_t idesc_g = tc::instr_desc(1, kGtBM, N2);
+    constexpr uint32_t idesc_c = tc::instr_desc(2, kGtBM, kGtBN);   // TF32
+    constexpr uint32_t sbo_k1 = (K1 / 8) * 128;
+    constexpr uint32_t sbo_x = (S::K8 / 4) * 128;
+    const uint64_t dAh = tc::smem_desc(smem0, 128, sbo_k1);
+    const uint64_t dAl = tc::smem_desc(smem0 + S::A_BYTES, 128, sbo_k1);
+    const uint64_t dXAh = tc::smem_desc(smem0 + S::OFF_XA, 128, sbo_x);
+    const uint64_t dXAl = tc::smem_desc(smem0 + S::OFF_XA + S::XA_BYTES, 128, sbo_x);
+    const uint64_t dXB0 = tc::smem_desc(smem0 + S::OFF_STAGES, 128, sbo_x);
+    const uint64_t dBT0 = tc::smem_desc(smem0 + S::OFF_STAGES + S::OFF_BT, 128, sbo_k1);
+    const uint64_t dZ0 = tc::smem_desc(smem0 + S::OFF_STAGES + S::OFF_Z, 128, 512);
+    auto copy_tile = [&](int p, int s) {   // elected lane
+      const long long t = tile_begin + p;
+      unsigned char* st = smem + S::OFF_STAGES + s * S::STAGE_BYTES;
+      mbar_arrive_expect_tx(&full[s], S::STAGE_BYTES);
       if constexpr (S::XC) {
-        if (ok && nt > 0) ok = issue_c(0);
+        bulk_g2s(st, a.XB + t * tc2_b_stride(S::K8), S::X_BYTES + S::BN_BYTES, &full[s]);
+      } else {
+        bulk_g2s(st, a.xhat + t * kGtBN * DP, S::X_BYTES, &full[s]);
+        bulk_g2s(st + S::OFF_BN, a.bneg + t * kGtBN, S::BN_BYTES, &full[s]);
       }
-      for (int p = 0; p < nt && ok; ++p) {
-        if (*s_fail) { ok = false; break; }
-        const int s = p % ST, b = p & 1;
-        if constexpr (S::XC) {
-          // the C buffer takes tile p + 1 once the epilogue has read tile p's
-          if (p + 1 < nt) {
-            if (!mbar_wait_spin(c_free, (uint32_t)(p & 1))) { ok = false; break; }
-            tc::fence_after();
-            if (!issue_c(p + 1)) { ok = false; break; }
-          }
-        }
-        if (!mbar_wait_spin(&p_full[b], (uint32_t)((p / 2) & 1))) { ok = false; break; }
-        tc::fence_after();
-        const uint32_t zH = smem_u32(stage(s) + S::OFF_Z);
-        const uint32_t zL = zH + S::Z_BYTES;
-        const uint32_t pcol = tbase + (uint32_t)(b * 32);
+      bulk_g2s(st + S::OFF_BT, a.tiles + t * (S::TILE_BYTES / 2), S::TILE_BYTES, &full[s]);
+    };
+    auto mma_cw = [&](int s, int h) {   // elected lane: W and C of the tile in stage s
+      const uint64_t so = (uint64_t)s * (S::STAGE_BYTES >> 4);
+#pragma unroll
+      for (int term = 0; term < 3; ++term) {
+        const uint64_t A = term == 2 ? dAl : dAh;
+        const uint64_t B = dBT0 + so + (term == 1 ? (S::BT_BYTES >> 4) : 0u);
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks)
+          tc::mma_bf16(tbase + (uint32_t)(h * 32), A + 16u * ks, B + 16u * ks, idesc_w,
+                       (term | ks) != 0);
+      }
+      if constexpr (S::XC) {
+        // C_J = A_I B_J^T (three TF32 products, K = 8)
+#pragma unroll
+        for (int term = 0; term < 3; ++term)
+          tc::mma_tf32(tbase + S::COL_C + (uint32_t)(h * 32), term == 2 ? dXAl : dXAh,
+                       dXB0 + so + (term == 1 ? (S::XB_BYTES >> 4) : 0u), idesc_c, term != 0);
+      }
+      tc::commit(&cw_full[h]);
+    };
+    const int pre = min(ST, nt);
+    if (tc::elect_one())
+      for (int p = 0; p < pre; ++p) copy_tile(p, p);
+    __syncwarp();
+    issued = pre;
+    bool ok = true;
+    int s_c = 0, ph_c = 0;   // stage of the next tile whose W and C are issued
+    for (int p = 0; p < kGtSets && p < nt && ok; ++p) {
+      ok = tc::warp_wait_uniform(full0 + 8u * s_c, ph_c);
+      tc::fence_after();
+      if (ok && tc::elect_one()) mma_cw(s_c, p);
+      __syncwarp();
+      if (++s_c == ST) { s_c = 0; ph_c ^= 1; }
+    }
+    int s = 0, h = 0, ph_h = 0;
+#pragma unroll 1
+    for (int p = 0; p < nt && ok; ++p) {
+      ok = tc::warp_wait_uniform(p_full0 + 8u * h, ph_h);
+      if (!ok) break;
+      tc::fence_after();
+      const bool more_w = p + kGtSets < nt, more_t = p + ST < nt;
+      if (tc::elect_one()) {
+        const uint64_t dZ = dZ0 + (uint64_t)s * (S::STAGE_BYTES >> 4);
+        const uint32_t pcol = tbase + (uint32_t)(h * 32);
 #pragma unroll
         for (int term = 0; term < 3; ++term) {
           const uint32_t A = pcol + (term == 2 ? 8u : 0u);   // P high | P low per 16 points
-          const uint32_t B = term == 1 ? zL : zH;
+          const uint64_t B = dZ + (term == 1 ? (S::Z_BYTES >> 4) : 0u);
 #pragma unroll
           for (int ks = 0; ks < kGtBN / 16; ++ks)
-            tc::mma_bf16_ts(tbase + S::COL_D2, A + ks * 16, tc::smem_desc(B + ks * 256, 128, 512),
-                            idesc_g, (p | term | ks) != 0);
+            tc::mma_bf16_ts(tbase + S::COL_D2, A + ks * 16, B + 16u * ks, idesc_g,
+                            (p | term | ks) != 0);
         }
-        tc::commit(&empty[s]);
-        if (p + 2 < nt) {
-          // buffer b is rewritten by tile p + 2's W only after these MMAs have read P
-          tc::commit(&b_free[b]);
-          if (!mbar_wait_spin(&b_free[b], (uint32_t)((p / 2) & 1))) { ok = false; break; }
+        // the set's buffers take tile p + 3's W and C, and stage s tile p + ST's operands, only
+        // after these MMAs have read P and Z
+        if (more_w || more_t) tc::commit(&b_free[h]);
+      }
+      __syncwarp();
+      if (more_w || more_t) {
+        ok = tc::warp_wait_uniform(b_free0 + 8u * h, ph_h);
+        if (ok && more_w) {
+          ok = tc::warp_wait_uniform(full0 + 8u * s_c, ph_c);
           tc::fence_after();
-          ok = issue_w(p + 2);
+          if (ok && tc::elect_one()) mma_cw(s_c, h);
+          __syncwarp();
+          if (++s_c == ST) { s_c = 0; ph_c ^= 1; }
+        }
+        if (ok && more_t) {
+          if (tc::elect_one()) copy_tile(p + ST, s);
+          __syncwarp();
+          issued = p + ST + 1;
         }
       }
-      if (!ok) *s_fail = 1;
-      if (nt > 0) tc::commit(done);   // a CTA with an empty range issues nothing and waits on nothing
+      if (++s == ST) s = 0;
+      if (++h == kGtSets) { h = 0; ph_h ^= 1; }
     }
+    if (!ok) *s_fail = 1;
+    // a CTA with an empty range issues nothing and waits on nothing
+    if (nt > 0 && tc::elect_one()) tc::commit(done);
+    __syncwarp();
   } else {
-    // ------------- epilogue: 8 warps, (lane quadrant, column half) each -------------
+    // ------ epilogue: warp (lane quadrant eq, set h) takes the tiles h, h + 3, ... whole ------
     const int eq = warp & 3;
-    const int half = (warp - 2) >> 2;
+    const int set = (warp - 1) >> 2;
     const int il = eq * 32 + lane;
     const long long i = row0 + il;
     const uint32_t lane_base = (uint32_t)(eq * 32) << 16;
@@ -439,90 +426,100 @@ __device__ __forceinline__ void gt_body(const GtDevArgs& a, const int rb, const 
     }
     const float ai = c0 + ((i < a.n) ? a.bneg[i] : 0.f);
     const bool add_bj = !S::XC || !a.c_has_bj;   // else the augmented C carries b_j
+    const float2 minus1 = make_float2(-1.f, -1.f);
+    const float2 ai2 = make_float2(ai, ai);
     bool ok = true;
-    for (int lt = 0; lt < nt; ++lt) {
-      const int s = lt % ST, b = lt & 1;
-      bool ready = gt_warp_wait(&full[s], (uint32_t)((lt / ST) & 1)) &&
-                   gt_warp_wait(&w_full[b], (uint32_t)((lt / 2) & 1));
-      if constexpr (S::XC) ready = ready && gt_warp_wait(c_full, (uint32_t)(lt & 1));
-      if (!__all_sync(0xffffffffu, ready && !*s_fail)) { ok = false; break; }
+    int s = set, ph_s = 0, ph = 0;   // set < ST
+#pragma unroll 1
+    for (int lt = set; lt < nt; lt += kGtSets) {
+      // b_J (and x^_J) are read from the stage: wait for its copy too (the stage is refilled
+      // only after this tile's P Z, which waits for this warp's P)
+      ok = tc::warp_wait_uniform(cw_full0 + 8u * set, ph) &&
+           tc::warp_wait_uniform(full0 + 8u * s, ph_s);
+      if (!ok) break;
       tc::fence_after();
-      const uint32_t wcol = tbase + lane_base + (uint32_t)(b * 32 + half * 16);
-      float w[16], cx[16];
-      if constexpr (S::XC) {
-        uint32_t r[32];
-        gt_tmem_ld16_two(wcol, tbase + lane_base + S::COL_C + (uint32_t)(half * 16), r);
-        tc::fence_before();
-        __syncwarp();
-        if (lane == 0) tc::mbar_arrive(c_free);   // the C buffer may take the next tile
+      const bool own = tile_begin + lt < diag_end;   // a tile of I itself: weight 1/2
+      const float* tx = reinterpret_cast<const float*>(smem + S::OFF_STAGES + s * S::STAGE_BYTES);
+      const float* tb = reinterpret_cast<const float*>(smem + S::OFF_STAGES + s * S::STAGE_BYTES +
+                                                       S::OFF_BN);
 #pragma unroll
-        for (int q = 0; q < 16; ++q) {
-          w[q] = __uint_as_float(r[q]);
-          cx[q] = __uint_as_float(r[16 + q]);
-        }
-      } else {
-        tc::tmem_ld16(wcol, w);
-      }
-      if (tile_begin + lt < diag_end) {   // a tile of I itself: (i, j) and (j, i) both visited
-#pragma unroll
-        for (int q = 0; q < 16; ++q) w[q] *= 0.5f;
-      }
-      const float* tx = reinterpret_cast<const float*>(stage(s));
-      const float* tb = reinterpret_cast<const float*>(stage(s) + S::OFF_BN);
-      uint32_t hi[8], lo[8];
-      // packed FP32x2 instructions: the cross term two coordinates at a time (FP32 pipe) or
-      // the exponent two entries at a time (tensor-core C), the weight and the high/low split
-      // two entries at a time
-      const float2 minus1 = make_float2(-1.f, -1.f);
-      const float2 ai2 = make_float2(ai, ai);
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        float ex[2];
-        const float2 bj = *reinterpret_cast<const float2*>(tb + half * 16 + 2 * q);
+      for (int half = 0; half < 2; ++half) {   // 16 columns at a time
+        const uint32_t wcol = tbase + lane_base + (uint32_t)(set * 32 + half * 16);
+        float w[16], cx[S::XC ? 16 : 1];
         if constexpr (S::XC) {
-          // (a_i + b_j) + C_ij, the order of the K V pass
-          const float2 base = add_bj ? __fadd2_rn(ai2, bj) : ai2;
-          const float2 e2 = __fadd2_rn(base, make_float2(cx[2 * q], cx[2 * q + 1]));
-          ex[0] = e2.x;
-          ex[1] = e2.y;
+          uint32_t r[32];
+          gt_tmem_ld16_two(wcol, wcol + S::COL_C, r);
+#pragma unroll
+          for (int q = 0; q < 16; ++q) {
+            w[q] = __uint_as_float(r[q]);
+            cx[q] = __uint_as_float(r[16 + q]);
+          }
         } else {
+          tc::tmem_ld16(wcol, w);
+        }
+        if (own) {   // (i, j) and (j, i) are both visited
 #pragma unroll
-          for (int h2 = 0; h2 < 2; ++h2) {
-            const int j = half * 16 + 2 * q + h2;
-            float xj[DP];
-            load_row<float, DP>(tx + j * DP, xj);
-            float2 acc = make_float2(ai + (h2 == 0 ? bj.x : bj.y), 0.f);
+          for (int q = 0; q < 16; ++q) w[q] *= 0.5f;
+        }
+        uint32_t hi[8], lo[8];
+        // packed FP32x2 instructions: the cross term two coordinates at a time (FP32 pipe) or
+        // the exponent two entries at a time (tensor-core C), the weight and the high/low split
+        // two entries at a time
 #pragma unroll
-            for (int k = 0; k < DP; k += 2)
-              acc = __ffma2_rn(make_float2(xi[k], xi[k + 1]), make_float2(xj[k], xj[k + 1]), acc);
-            ex[h2] = acc.x + acc.y;
+        for (int q4 = 0; q4 < 4; ++q4) {
+          const float4 b4 = *reinterpret_cast<const float4*>(tb + half * 16 + 4 * q4);
+#pragma unroll
+          for (int q2 = 0; q2 < 2; ++q2) {
+            const int q = 2 * q4 + q2;
+            const float2 bj = q2 == 0 ? make_float2(b4.x, b4.y) : make_float2(b4.z, b4.w);
+            float ex[2];
+            if constexpr (S::XC) {
+              // (a_i + b_j) + C_ij, the order of the K V pass
+              const float2 base = add_bj ? __fadd2_rn(ai2, bj) : ai2;
+              const float2 e2 = __fadd2_rn(base, make_float2(cx[2 * q], cx[2 * q + 1]));
+              ex[0] = e2.x;
+              ex[1] = e2.y;
+            } else {
+#pragma unroll
+              for (int h2 = 0; h2 < 2; ++h2) {
+                const int j = half * 16 + 2 * q + h2;
+                float xj[DP];
+                load_row<float, DP>(tx + j * DP, xj);
+                float2 acc2 = make_float2(ai + (h2 == 0 ? bj.x : bj.y), 0.f);
+#pragma unroll
+                for (int k = 0; k < DP; k += 2)
+                  acc2 = __ffma2_rn(make_float2(xi[k], xi[k + 1]), make_float2(xj[k], xj[k + 1]), acc2);
+                ex[h2] = acc2.x + acc2.y;
+              }
+            }
+            const float2 pk = __fmul2_rn(make_float2(ex2_approx(fminf(ex[0], c0)),
+                                                     ex2_approx(fminf(ex[1], c0))),
+                                         make_float2(w[2 * q], w[2 * q + 1]));
+            const __nv_bfloat162 h = __floats2bfloat162_rn(pk.x, pk.y);
+            const float2 r = __ffma2_rn(__bfloat1622float2(h), minus1, pk);   // pk - high part
+            const __nv_bfloat162 l = __floats2bfloat162_rn(r.x, r.y);
+            hi[q] = *reinterpret_cast<const uint32_t*>(&h);
+            lo[q] = *reinterpret_cast<const uint32_t*>(&l);
           }
         }
-        const float2 pk = __fmul2_rn(make_float2(ex2_approx(fminf(ex[0], c0)),
-                                                 ex2_approx(fminf(ex[1], c0))),
-                                     make_float2(w[2 * q], w[2 * q + 1]));
-        const __nv_bfloat162 h = __floats2bfloat162_rn(pk.x, pk.y);
-        const float2 r = __ffma2_rn(__bfloat1622float2(h), minus1, pk);   // pk - high part
-        const __nv_bfloat162 l = __floats2bfloat162_rn(r.x, r.y);
-        hi[q] = *reinterpret_cast<const uint32_t*>(&h);
-        lo[q] = *reinterpret_cast<const uint32_t*>(&l);
+        // P over this warp's own W columns: high parts first, then low parts
+        tc::tmem_st8(wcol, hi);
+        tc::tmem_st8(wcol + 8, lo);
       }
-      __syncwarp();
-      if (lane == 0) tc::mbar_arrive(&empty[s]);   // x^_J (or nothing) and b_J consumed
-      // P over this warp's own 16 W columns: high parts first, then low parts
-      tc::tmem_st8(wcol, hi);
-      tc::tmem_st8(wcol + 8, lo);
       tc::tmem_wait_st();
       tc::fence_before();
       __syncwarp();
-      if (lane == 0) tc::mbar_arrive(&p_full[b]);
+      if (lane == 0) tc::mbar_arrive(&p_full[set]);
+      ph ^= 1;
+      s += kGtSets;
+      if (s >= ST) { s -= ST; ph_s ^= 1; }
     }
     if (!ok) *s_fail = 1;
-    const bool fin = ok && (nt == 0 || gt_warp_wait(done, 0));
+    const bool fin = ok && (nt == 0 || tc::warp_wait_uniform(smem_u32(done), 0));
     ok = __all_sync(0xffffffffu, fin && !*s_fail);
     if (ok && nt > 0) {
       tc::fence_after();
-      if (half == 0) {
+      if (set == 0) {
         float g[N2];
 #pragma unroll
         for (int c = 0; c < N2 / 16; ++c) {
@@ -540,7 +537,7 @@ __device__ __forceinline__ void gt_body(const GtDevArgs& a, const int rb, const 
           }
           acc[DP] = Ssum;
         }
-      } else if (sp == 0 && i < a.n) {
+      } else if (set == 1 && sp == 0 && i < a.n) {
         // diagonal W_ii for the lambda component, once per row
         float wii = 0.f;
         for (int m = 0; m < a.M; ++m)
@@ -552,14 +549,11 @@ __device__ __forceinline__ void gt_body(const GtDevArgs& a, const int rb, const 
   }
 
   // -------- all roles: release tensor memory; CTA reduction; last CTA sums the partials -------
-  if (warp == 1) {
-    if (lane == 0 && nt > 0) (void)mbar_wait_spin(done, 0);
-    __syncwarp();
-  }
+  if (warp == 0 && nt > 0) (void)tc::warp_wait_uniform(smem_u32(done), 0);
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
-  if (warp == 1) tc::tmem_dealloc(tbase, kGtCols);
+  if (warp == 0) tc::tmem_dealloc(tbase, kGtCols);
   if (*s_fail) {
     if (tid == 0) {
       atomicOr(a.status, kStatusTimeout);
@@ -569,18 +563,18 @@ __device__ __forceinline__ void gt_body(const GtDevArgs& a, const int rb, const 
     }
     return;
   }
-  if (warp >= 2) {
+  if (warp >= 1) {
 #pragma unroll
     for (int k = 0; k < NACC; ++k) {
       const double v = warp_sum(acc[k]);
-      if (lane == 0) s_red[warp - 2][k] = v;
+      if (lane == 0) s_red[warp - 1][k] = v;
     }
   }
   __syncthreads();
   double* part = a.partials + slot * kMaxP;
   if (tid < NACC) {
     double v = 0.0;
-    for (int ww = 0; ww < 8; ++ww) v += s_red[ww][tid];
+    for (int ww = 0; ww < 4 * kGtSets; ++ww) v += s_red[ww][tid];
     // slots: lengthscales 0..d-1, then sigma^2 at d, lambda at d+1
     if (tid < a.d) part[tid] = v;
     else if (tid == DP) part[a.d] = v;
@@ -602,7 +596,7 @@ __device__ __forceinline__ void gt_body(const GtDevArgs& a, const int rb, const 
 }
 
 template <int DP, int KS>
-__global__ void __launch_bounds__(kGtThreads, DP >= 16 ? 2 : 3) grad_tc_kernel(const GtDevArgs a) {
+__global__ void __launch_bounds__(kGtThreads, GtShape<DP, KS>::OCC) grad_tc_kernel(const GtDevArgs a) {
   const int rb = blockIdx.x / a.nsplit;
   gt_body<DP, KS>(a, rb, blockIdx.x - rb * a.nsplit);
 }
@@ -610,7 +604,7 @@ __global__ void __launch_bounds__(kGtThreads, DP >= 16 ? 2 : 3) grad_tc_kernel(c
 // Many problems of one input width in one launch: CTA b takes work item items[b] =
 // (problem, row block, split) with that problem's arguments.
 template <int DP, int KS>
-__global__ void __launch_bounds__(kGtThreads, DP >= 16 ? 2 : 3) grad_tc_batch_kernel(
+__global__ void __launch_bounds__(kGtThreads, GtShape<DP, KS>::OCC) grad_tc_batch_kernel(
     const GtDevArgs* __restrict__ args, const int4* __restrict__ items) {
   __shared__ GtDevArgs s_a;
   const int4 it = items[blockIdx.x];
@@ -619,65 +613,26 @@ __global__ void __launch_bounds__(kGtThreads, DP >= 16 ? 2 : 3) grad_tc_batch_ke
   gt_body<DP, KS>(s_a, it.y, it.z);
 }
 
-// The operand images of every problem of a batched launch (one problem per grid row), as
-// pack_bt_kernel and pack_z_kernel.
+// The operand blocks of every problem of a batched launch (one problem per grid row), as
+// pack_gt_kernel.
 template <int DP, int KS>
 __global__ void pack_gt_batch_kernel(const GtDevArgs* __restrict__ args) {
   using S = GtShape<DP, KS>;
-  constexpr int K1 = S::K1, N2 = S::N2;
   const GtDevArgs& a = args[blockIdx.y];
-  const long long ntiles = a.ntiles;
-  __nv_bfloat16* Bhi = const_cast<__nv_bfloat16*>(a.Bt_hi);
-  __nv_bfloat16* Blo = const_cast<__nv_bfloat16*>(a.Bt_lo);
-  __nv_bfloat16* Zhi = const_cast<__nv_bfloat16*>(a.Zt_hi);
-  __nv_bfloat16* Zlo = const_cast<__nv_bfloat16*>(a.Zt_lo);
-  const long long per_b = (long long)kGtBN * K1, per_z = (long long)N2 * kGtBN;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-       idx < ntiles * (per_b + per_z); idx += (long long)gridDim.x * blockDim.x) {
-    __nv_bfloat16 h, l;
-    if (idx < ntiles * per_b) {
-      const long long t = idx / per_b;
-      const int rem = (int)(idx - t * per_b);
-      const int m = rem / kGtBN, j = rem - m * kGtBN;
-      const long long jj = t * kGtBN + j;
-      float v = 0.f;
-      if (jj < a.n) {
-        if (m < a.M) v = a.B[(long long)a.bmap[m] * a.ld + jj];
-        else if (m < 2 * a.M) v = a.sa[m - a.M] * a.A[(long long)a.amap[m - a.M] * a.ld + jj];
-      }
-      split_bf16(v, h, l);
-      const long long off = t * per_b + tc::canon_offset(j, m, 2, K1 / 8) / 2;
-      Bhi[off] = h;
-      Blo[off] = l;
-    } else {
-      const long long z = idx - ntiles * per_b;
-      const long long t = z / per_z;
-      const int rem = (int)(z - t * per_z);
-      const int c = rem / kGtBN, j = rem - c * kGtBN;
-      const long long jj = t * kGtBN + j;
-      float v = 0.f;
-      if (jj < a.n) {
-        if (c < DP) {
-          v = a.xhat[jj * DP + c];
-        } else if (c < 2 * DP) {
-          const float x = a.xhat[jj * DP + (c - DP)];
-          v = x * x;
-        } else if (c == 2 * DP) {
-          v = 1.f;
-        }
-      }
-      split_bf16(v, h, l);
-      const long long off = t * per_z + tc::canon_offset(c, j, 2, kGtBN / 8) / 2;
-      Zhi[off] = h;
-      Zlo[off] = l;
-    }
-  }
+  const long long total = (long long)a.ntiles * kGtBN * (S::K1 + S::N2);
+  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
+       idx += (long long)gridDim.x * blockDim.x)
+    gt_pack_element(idx, S::K1, S::N2, DP, a.M, a.n, a.xhat, a.A, a.amap, a.sa, a.B, a.bmap, a.ld,
+                    const_cast<__nv_bfloat16*>(a.tiles));
 }
 
 // Split of each row block's tile range into s CTAs.  The SMs share the visited tiles plus a
 // fixed cost per CTA (the operand image, the pipeline fill and the reduction, about six
-// tiles' worth); a CTA shares its SM with occ - 1 others, so the longest range (row block 0,
-// ntiles / s tiles) takes about occ x its length and must not end the pass.
+// tiles' worth); a CTA shares its SM with others, so the longest range (row block 0, ntiles / s
+// tiles) takes about occ x its length and must not end the pass.  The ranges also bound the
+// rounding of the sums, which tensor memory accumulates in FP32 with truncation: occ is taken
+// as 3 (2 for four or more factor steps or padded d = 16, 1 for eight), not the two CTAs that
+// share an SM, because ranges 1.5 times as long would raise the error of the gradient 1.4 times.
 static int plan_gt_split(long long n_rb, long long ntiles, int num_sms, int occ) {
   const long long per_block = kGtBM / kGtBN;
   const long long visited = n_rb * ntiles - per_block * n_rb * (n_rb - 1) / 2;
@@ -708,28 +663,20 @@ static void gt_set_images(GtDevArgs& a, const GradLaunch& L) {
 template <int DP, int KS>
 struct GtInst {
   using S = GtShape<DP, KS>;
-  static int occupancy() {
-    static int occ = -1;
+  static constexpr int kPlanOcc = KS >= 8 ? 1 : (KS >= 4 || DP >= 16) ? 2 : 3;
+  static void prime() {
     static std::once_flag once;
     std::call_once(once, [] {
       auto fn = grad_tc_kernel<DP, KS>;
       cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
       cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-      int dev = 0, smem_sm = 0;
-      cudaGetDevice(&dev);
-      if (cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) !=
-          cudaSuccess)
-        smem_sm = 228 * 1024;
-      const int by_smem = smem_sm / (int)(S::SMEM + 2048);
-      occ = std::max(1, std::min({by_smem, (int)(512 / kGtCols), DP >= 16 ? 2 : 3}));
     });
-    return occ;
   }
   static cudaError_t launch(GradLaunch& L, cudaStream_t s) {
-    const int occ = occupancy();
+    prime();
     const long long ntiles = (L.n + kGtBN - 1) / kGtBN;
     const int n_rb = (int)((L.n + kGtBM - 1) / kGtBM);
-    const int nsplit = plan_gt_split(n_rb, ntiles, L.num_sms, occ);
+    const int nsplit = plan_gt_split(n_rb, ntiles, L.num_sms, kPlanOcc);
     const size_t need = (size_t)n_rb * nsplit * kMaxP;
     if (L.plan_only) {
       L.need_partials_len = need;
@@ -739,30 +686,19 @@ struct GtInst {
       L.need_partials_len = need;
       return cudaErrorMemoryAllocation;
     }
-    __nv_bfloat16* hi = static_cast<__nv_bfloat16*>(L.tc_hi);
-    __nv_bfloat16* lo = static_cast<__nv_bfloat16*>(L.tc_lo);
-    const long long zoff = (long long)kGtZOff * L.tc_ld;
+    __nv_bfloat16* tiles = static_cast<__nv_bfloat16*>(L.tc_tiles);
     {
-      const long long total = ntiles * kGtBN * S::K1;
+      const long long total = ntiles * kGtBN * (S::K1 + S::N2);
       const int blocks = (int)std::min<long long>((total + 255) / 256, 8LL * L.num_sms);
-      pack_bt_kernel<<<blocks, 256, 0, s>>>(static_cast<const float*>(L.B), L.bmap,
-                                            static_cast<const float*>(L.A), L.amap,
-                                            static_cast<const float*>(L.sa), L.ld, L.M, S::K1,
-                                            L.n, ntiles, hi, lo);
-    }
-    {
-      const long long total = ntiles * S::N2 * kGtBN;
-      const int blocks = (int)std::min<long long>((total + 255) / 256, 8LL * L.num_sms);
-      pack_z_kernel<<<blocks, 256, 0, s>>>(static_cast<const float*>(L.xhat), DP, L.n, S::N2,
-                                           ntiles, hi + zoff, lo + zoff);
+      pack_gt_kernel<<<blocks, 256, 0, s>>>(
+          S::K1, S::N2, DP, L.M, L.n, ntiles, static_cast<const float*>(L.xhat),
+          static_cast<const float*>(L.A), L.amap, static_cast<const float*>(L.sa),
+          static_cast<const float*>(L.B), L.bmap, L.ld, tiles);
     }
     GtDevArgs a;
     a.xhat = static_cast<const float*>(L.xhat);
     a.bneg = L.bneg;
-    a.Bt_hi = hi;
-    a.Bt_lo = lo;
-    a.Zt_hi = hi + zoff;
-    a.Zt_lo = lo + zoff;
+    a.tiles = tiles;
     a.A = static_cast<const float*>(L.A);
     a.amap = L.amap;
     a.sa = static_cast<const float*>(L.sa);
@@ -809,20 +745,14 @@ cudaError_t gt_batch_upload_args(const GradLaunch* L, const int* nsplit, int B, 
     const GradLaunch& l = L[b];
     const long long ntiles = (l.n + kGtBN - 1) / kGtBN;
     const long long n_rb = (l.n + kGtBM - 1) / kGtBM;
-    if (l.M < 1 || l.M > kMaxM || nsplit[b] < 1 || l.DP != L[0].DP || !l.tc_hi || !l.tc_lo ||
+    if (l.M < 1 || l.M > kMaxM || nsplit[b] < 1 || l.DP != L[0].DP || !l.tc_tiles ||
         !l.X_hi || !l.X_lo || !l.X_b ||
         (ntiles + nsplit[b] - 1) / nsplit[b] > kTcMaxSplitTiles)
       return cudaErrorInvalidValue;
     GtDevArgs& a = h[b];
-    __nv_bfloat16* hi = static_cast<__nv_bfloat16*>(l.tc_hi);
-    __nv_bfloat16* lo = static_cast<__nv_bfloat16*>(l.tc_lo);
-    const long long zoff = (long long)kGtZOff * l.tc_ld;
     a.xhat = static_cast<const float*>(l.xhat);
     a.bneg = l.bneg;
-    a.Bt_hi = hi;
-    a.Bt_lo = lo;
-    a.Zt_hi = hi + zoff;
-    a.Zt_lo = lo + zoff;
+    a.tiles = static_cast<const __nv_bfloat16*>(l.tc_tiles);
     a.A = static_cast<const float*>(l.A);
     a.amap = l.amap;
     a.sa = static_cast<const float*>(l.sa);
@@ -892,7 +822,7 @@ cudaError_t launch_grad_tc_batch(const void* args_dev, int B, const int4* items,
 }
 
 cudaError_t launch_grad_tc(GradLaunch& L, cudaStream_t s) {
-  if (L.M < 1 || L.M > kMaxM || !L.tc_hi || !L.tc_lo || !L.bneg) return cudaErrorInvalidValue;
+  if (L.M < 1 || L.M > kMaxM || !L.tc_tiles || !L.bneg) return cudaErrorInvalidValue;
   if (L.DP <= 8 && (!L.X_hi || !L.X_lo || !L.X_b)) return cudaErrorInvalidValue;
   switch (L.DP) {
     case 2: return grad_tc_dispatch_m<2>(L, s);
