@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "../../include/ulisse.h"
+#include "exp64.cuh"
 #include "solver_kernels.cuh"
 #include "pcg_kernels.cuh"
 #include "predict.cuh"
@@ -37,6 +38,7 @@ struct ulisse_ctx {
   void* y = nullptr;          // labels, ldn (element type T)
   void* xhat = nullptr;       // prescaled inputs, ldn x DP
   DevParams* params = nullptr;
+  double* exp_tab = nullptr;  // FP64: table of the exponential (exp64.cuh)
   double* psi_dev = nullptr;  // kMaxP
 
   int cap = 0;                // column capacity of B, S, E, D, KD
@@ -450,6 +452,7 @@ static ulisse_status run_kmv(ulisse_ctx* ctx, const void* V, const int* vmap, in
     L.ldu = ctx->ldn;
     L.umap = umap + c0;
     L.params = ctx->params;
+    L.exp_tab = ctx->exp_tab;
     L.mode = mode;
     L.which = which;
     L.tm = ctx->cfg.kmv_rows_per_thread;
@@ -859,6 +862,7 @@ static ulisse_status run_grad(ulisse_ctx* ctx, int M, const int* amap = nullptr,
   L.ld = ctx->ldn;
   L.M = M;
   L.params = ctx->params;
+  L.exp_tab = ctx->exp_tab;
   L.counter = ctx->gcounter;
   L.g_out = ctx->g_dev;
   L.status = ctx->status_dev;
@@ -1050,6 +1054,14 @@ static ulisse_status create_impl(ulisse_ctx** out, const float* X, const float* 
         (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->Xt_b),
                        4 * (ctx->ld128 / 32) * tc2_b_stride(16))))
       return bail(s);
+  }
+  if (ctx->f64) {
+    if ((s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->exp_tab), sizeof(double) * kExpTabN)))
+      return bail(s);
+    if (launch_fill_exp_tab(ctx->exp_tab, ctx->stream) != cudaSuccess) {
+      ctx->err = "table launch failed";
+      return bail(ULISSE_ERR_CUDA);
+    }
   }
   if (cudaMallocHost(&ctx->h_n_live, sizeof(int)) != cudaSuccess ||
       cudaMallocHost(&ctx->h_status, sizeof(int)) != cudaSuccess) {
@@ -3062,7 +3074,7 @@ void ulisse_destroy(ulisse_ctx* ctx) {
                    reinterpret_cast<void**>(&ctx->part2), reinterpret_cast<void**>(&ctx->bneg),
                    &ctx->Vt, &ctx->Gt,
                    reinterpret_cast<void**>(&ctx->Xt_hi), reinterpret_cast<void**>(&ctx->Xt_lo),
-                   reinterpret_cast<void**>(&ctx->Xt_b),
+                   reinterpret_cast<void**>(&ctx->Xt_b), reinterpret_cast<void**>(&ctx->exp_tab),
                    reinterpret_cast<void**>(&ctx->q_map), &ctx->q_sa, &ctx->pcg_buf, &ctx->pred_xs,
                    reinterpret_cast<void**>(&ctx->pcg_aux), reinterpret_cast<void**>(&ctx->pcg_live)})
     dev_free(*p);

@@ -31,6 +31,7 @@ struct GradDevArgs {
   long long ld;
   int M;
   const DevParams* params;
+  const double* exp_tab;   // FP64 only
   int nsplit, tiles_per_split, ntiles;
   double* partials;
   int* counter;
@@ -156,7 +157,7 @@ __global__ void __launch_bounds__(NT) grad_kernel(const GradDevArgs<T> a) {
               sq[k] = df * df;
               dist += sq[k];
             }
-            const T P = kernel_from_dist<T>(dist, c0, c1, sigma2) * W[t][q];
+            const T P = kernel_from_dist<T>(dist, c0, c1, sigma2, a.exp_tab) * W[t][q];
             gs += P;
 #pragma unroll
             for (int k = 0; k < DP; ++k) gl[k] = fma(P, sq[k], gl[k]);
@@ -269,6 +270,7 @@ struct GradInst {
     a.ld = L.ld;
     a.M = L.M;
     a.params = L.params;
+    a.exp_tab = L.exp_tab;
     a.nsplit = p.nsplit;
     a.tiles_per_split = p.tiles_per_split;
     a.ntiles = p.ntiles;

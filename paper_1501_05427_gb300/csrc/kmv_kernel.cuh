@@ -14,6 +14,7 @@
 // split order, adds the lambda V diagonal term and writes U: deterministic, one launch.
 #pragma once
 
+#include "exp64.cuh"
 #include "ulisse_internal.cuh"
 
 namespace ulisse {
@@ -30,6 +31,7 @@ struct KmvDevArgs {
   long long ldu;
   const int* umap;
   const DevParams* params;
+  const double* exp_tab;   // FP64 only
   int mode, which;
   int nsplit, tiles_per_split, ntiles;
   T* partials;
@@ -60,11 +62,12 @@ __device__ __forceinline__ void load_row(const T* __restrict__ p, T (&x)[DP]) {
 
 // Signal covariance from the squared prescaled distance.
 template <typename T>
-__device__ __forceinline__ T kernel_from_dist(T dist, float c0, float c1, double sigma2) {
+__device__ __forceinline__ T kernel_from_dist(T dist, float c0, float c1, double sigma2,
+                                              const double* __restrict__ exp_tab) {
   if constexpr (sizeof(T) == 4) {
     return ex2_approx(fmaf(-c1, dist, c0));
   } else {
-    return sigma2 * exp(-0.5 * dist);
+    return sigma2 * exp_neg_half(dist, exp_tab);
   }
 }
 
@@ -163,7 +166,7 @@ __global__ void __launch_bounds__(NT) kmv_kernel(const KmvDevArgs<T> a) {
               const T df = xi[t][k] - xj[k];
               dist = fma(df, df, dist);
             }
-            T kv = kernel_from_dist<T>(dist, c0, c1, sigma2);
+            T kv = kernel_from_dist<T>(dist, c0, c1, sigma2, a.exp_tab);
             if constexpr (MODE == kModeDLen) {
               const T dw = xiw[t] - tX[(jq + q) * DP + a.which];
               kv *= dw * dw;

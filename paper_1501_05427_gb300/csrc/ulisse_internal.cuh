@@ -221,6 +221,7 @@ struct KmvLaunch {
   const DevParams* params;
   int mode;              // KmvMode
   int which;             // dimension for kModeDLen
+  const double* exp_tab; // FP64: the exponential's table (exp64.cuh)
   int tm;                // rows per thread for K (0 = default)
   int r_min;             // compiled column count at least this (0: the smallest >= R)
   int nsplit;            // j-range split count (0: the launch plan's choice)
@@ -250,6 +251,7 @@ struct GradLaunch {
   long long ld;
   int M;
   const DevParams* params;
+  const double* exp_tab; // FP64: the exponential's table (exp64.cuh)
   double* partials;      // per-CTA FP64 partial sums, kMaxP each
   size_t partials_len;   // doubles
   int* counter;          // single counter, zero between launches
@@ -316,6 +318,8 @@ cudaError_t launch_kmv_f32_dp4(KmvLaunch& L, cudaStream_t s);
 cudaError_t launch_kmv_f32_dp8(KmvLaunch& L, cudaStream_t s);
 cudaError_t launch_kmv_f32_dp16(KmvLaunch& L, cudaStream_t s);
 cudaError_t launch_kmv_f64(KmvLaunch& L, cudaStream_t s);
+bool kmv_f64_sym_applies(const KmvLaunch& L);
+cudaError_t launch_kmv_f64_sym(KmvLaunch& L, cudaStream_t s);
 cudaError_t launch_grad_f32(GradLaunch& L, cudaStream_t s);
 cudaError_t launch_grad_f64(GradLaunch& L, cudaStream_t s);
 cudaError_t launch_kmv_tc(TcLaunch& L, cudaStream_t s);
