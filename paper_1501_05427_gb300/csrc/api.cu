@@ -40,6 +40,7 @@ struct ulisse_ctx {
   DevParams* params = nullptr;
   double* exp_tab = nullptr;  // FP64: table of the exponential (exp64.cuh)
   double* psi_dev = nullptr;  // kMaxP
+  PsiArg psi_arg{};           // by_value: psi of a host call, handed to the next prescale launch
 
   int cap = 0;                // column capacity of B, S, E, D, KD
   int cap_est = 0;            // column capacity of SE
@@ -312,34 +313,48 @@ static bool finite_psi(const double* psi, int p) {
   return true;
 }
 
-// psi (host) -> device, then the prescale kernel (a1).
+// psi of a host call: it travels by value with the next prescale launch.
 static ulisse_status set_psi_host(ulisse_ctx* ctx, const double* psi) {
   const int p = ctx->d + 2;
   if (!psi || !finite_psi(psi, p)) return fail(ctx, ULISSE_ERR_ARG, "psi is null or not finite");
-  CK(cudaMemcpyAsync(ctx->psi_dev, psi, sizeof(double) * p, cudaMemcpyHostToDevice,
-                     ctx->stream));
+  for (int i = 0; i < p; ++i) ctx->psi_arg.v[i] = psi[i];
+  ctx->psi_arg.by_value = 1;
+  return ULISSE_OK;
+}
+
+// ... or, where kernels of a captured step read it, to psi_dev.
+static ulisse_status psi_to_device(ulisse_ctx* ctx) {
+  CK(cudaMemcpyAsync(ctx->psi_dev, ctx->psi_arg.v, sizeof(double) * (ctx->d + 2),
+                     cudaMemcpyHostToDevice, ctx->stream));
+  ctx->psi_arg.by_value = 0;
+  return ULISSE_OK;
+}
+
+// The prescale launch (a1); TV columns of V (leading dimension n, may be null) are copied into D
+// by the same launch (FP32 and FP64 contexts).
+template <typename TV>
+static ulisse_status prescale_and_copy(ulisse_ctx* ctx, const TV* V, int R) {
+  PsiArg pa = ctx->psi_arg;
+  if (ctx->capturing) pa.by_value = 0;   // a captured step reads psi_dev
+  if (ctx->mixed)
+    CK(launch_prescale_mixed(pa, ctx->psi_dev, ctx->X, (float*)ctx->xhat, ctx->n, ctx->ld128, ctx->d,
+                             ctx->DP, !ctx->tc_no_aug, ctx->params, ctx->bneg, ctx->Xt_hi,
+                             ctx->Xt_lo, ctx->Xt_b, ctx->num_sms, ctx->stream));
+  else if (ctx->f64)
+    CK((launch_prescale<double, TV>(pa, ctx->psi_dev, ctx->X, (double*)ctx->xhat, ctx->n, ctx->d,
+                                    ctx->DP, ctx->params, V, (double*)ctx->D, ctx->ldn, R,
+                                    ctx->num_sms, ctx->stream)));
+  else
+    CK((launch_prescale<float, TV>(pa, ctx->psi_dev, ctx->X, (float*)ctx->xhat, ctx->n, ctx->d,
+                                   ctx->DP, ctx->params, V, (float*)ctx->D, ctx->ldn, R,
+                                   ctx->num_sms, ctx->stream)));
+  ctx->psi_arg.by_value = 0;
+  if (!ctx->capturing) ctx->launches++;
   return ULISSE_OK;
 }
 
 static ulisse_status prescale(ulisse_ctx* ctx) {
-  const int blocks = (int)std::min<long long>((ctx->n + 255) / 256, 4LL * ctx->num_sms);
-  if (ctx->f64)
-    prescale_kernel<double><<<blocks, 256, 0, ctx->stream>>>(
-        ctx->psi_dev, ctx->X, (double*)ctx->xhat, ctx->n, ctx->d, ctx->DP, ctx->params);
-  else
-    prescale_kernel<float><<<blocks, 256, 0, ctx->stream>>>(
-        ctx->psi_dev, ctx->X, (float*)ctx->xhat, ctx->n, ctx->d, ctx->DP, ctx->params);
-  CK(cudaGetLastError());
-  if (!ctx->capturing) ctx->launches++;
-  if (ctx->mixed) {
-    CK(launch_prescale_tc((const float*)ctx->xhat, ctx->DP, ctx->d, ctx->n, ctx->ld128,
-                          ctx->bneg, ctx->num_sms, ctx->stream));
-    CK(launch_pack_x_tf32((const float*)ctx->xhat, ctx->bneg, ctx->params, ctx->DP, ctx->n,
-                          ctx->ld128, ctx->Xt_hi, ctx->Xt_lo, ctx->Xt_b, ctx->num_sms,
-                          ctx->stream, !ctx->tc_no_aug));
-    if (!ctx->capturing) ctx->launches += 2;
-  }
-  return ULISSE_OK;
+  return prescale_and_copy<float>(ctx, nullptr, 0);
 }
 
 // U[:, umap[r]] = A V[:, vmap[r]] for r < R (chunks of kMaxRChunk columns per launch).
@@ -365,18 +380,18 @@ static ulisse_status grow_kmv_scratch(ulisse_ctx* ctx, size_t need_bytes, int ne
 
 // U[:, umap[r]] = A V[:, vmap[r]] for r < R (chunks of 64 columns per launch).
 static ulisse_status run_kmv_tc(ulisse_ctx* ctx, const void* V, const int* vmap, int R, void* U,
-                                const int* umap) {
+                                const int* umap, long long ldv, long long ldu) {
   for (int c0 = 0; c0 < R; c0 += 64) {
     TcLaunch L{};
     L.xhat = (const float*)ctx->xhat;
     L.bneg = ctx->bneg;
     L.Vp = ctx->Vt;
     L.V = V;
-    L.ldv = ctx->ldn;
+    L.ldv = ldv;
     L.vmap = vmap + c0;
     L.R = std::min(64, R - c0);
     L.U = U;
-    L.ldu = ctx->ldn;
+    L.ldu = ldu;
     L.umap = umap + c0;
     L.n = ctx->n;
     L.DP = ctx->DP;
@@ -434,9 +449,14 @@ static ulisse_status run_kmv_tc(ulisse_ctx* ctx, const void* V, const int* vmap,
   return ULISSE_OK;
 }
 
+// ldv, ldu: leading dimensions (0: the context's own, ldn); only the tensor-core products and
+// the FP64 pair form take a V that is not padded to whole tiles.
 static ulisse_status run_kmv(ulisse_ctx* ctx, const void* V, const int* vmap, int R, void* U,
-                             const int* umap, int mode, int which) {
-  if (ctx->mixed && mode == kModeK) return run_kmv_tc(ctx, V, vmap, R, U, umap);
+                             const int* umap, int mode, int which, long long ldv = 0,
+                             long long ldu = 0) {
+  if (ldv == 0) ldv = ctx->ldn;
+  if (ldu == 0) ldu = ctx->ldn;
+  if (ctx->mixed && mode == kModeK) return run_kmv_tc(ctx, V, vmap, R, U, umap, ldv, ldu);
   for (int c0 = 0; c0 < R; c0 += kMaxRChunk) {
     KmvLaunch L{};
     L.xhat = ctx->xhat;
@@ -445,11 +465,11 @@ static ulisse_status run_kmv(ulisse_ctx* ctx, const void* V, const int* vmap, in
     L.d = ctx->d;
     L.DP = ctx->DP;
     L.V = V;
-    L.ldv = ctx->ldn;
+    L.ldv = ldv;
     L.vmap = vmap + c0;
     L.R = std::min(kMaxRChunk, R - c0);
     L.U = U;
-    L.ldu = ctx->ldn;
+    L.ldu = ldu;
     L.umap = umap + c0;
     L.params = ctx->params;
     L.exp_tab = ctx->exp_tab;
@@ -1164,28 +1184,42 @@ static ulisse_status kmv_common(ulisse_ctx* ctx, const double* psi, int which, c
   if (f64_data && !ctx->f64)
     return fail(ctx, ULISSE_ERR_ARG, "double data needs a context created with FP64 precision");
   CKS(set_psi_host(ctx, psi));
-  CKS(prescale(ctx));
   CKS(ensure_columns(ctx, R, R));
   const long long n = ctx->n;
   const size_t ue = f64_data ? 8 : 4;
-  // caller's V (leading dimension n) -> context buffer D (leading dimension ldn)
-  if (ctx->esz == ue) {
-    CK(cudaMemcpy2DAsync(ctx->D, ctx->ldn * ctx->esz, V, n * ue, n * ue, R,
-                         cudaMemcpyDeviceToDevice, ctx->stream));
-  } else {
-    convert_cols_kernel<float, double><<<dim3(64, R), 256, 0, ctx->stream>>>(
-        (const float*)V, n, (double*)ctx->D, ctx->ldn, n);
-    CK(cudaGetLastError());
-  }
   int mode = kModeK, w = -1;
   if (which >= 0 && which < ctx->d) { mode = kModeDLen; w = which; }
   else if (which == ctx->d) mode = kModeDSig;
   else if (which == ctx->d + 1) mode = kModeDLam;
-  CKS(run_kmv(ctx, ctx->D, ctx->iota, R, ctx->KD, ctx->iota, mode, w));
-  if (ctx->esz == ue) {
-    CK(cudaMemcpy2DAsync(U, n * ue, ctx->KD, ctx->ldn * ctx->esz, n * ue, R,
-                         cudaMemcpyDeviceToDevice, ctx->stream));
+  // The tensor-core products and the FP64 pair form read the caller's V in place (unless U
+  // overlaps it); the other kernels copy whole 64-point tiles of padded columns, so their V goes
+  // into D with the prescale launch.  U is written in place when it has the context's type.
+  KmvLaunch probe{};
+  probe.n = n;
+  probe.R = std::min(R, kMaxRChunk);
+  probe.mode = mode;
+  probe.exp_tab = ctx->exp_tab;
+  const char *vb = (const char*)V, *ub = (const char*)U;
+  const size_t bytes = (size_t)n * R * ue;
+  const bool overlap = ub < vb + bytes && vb < ub + bytes;
+  const bool reads_direct = (ctx->mixed && mode == kModeK) ||
+                            (f64_data && kmv_f64_sym_applies(probe));
+  const bool in_place = reads_direct && !overlap;
+  if (in_place) {
+    CKS(prescale(ctx));
+  } else if (ctx->mixed) {
+    CKS(prescale(ctx));
+    CK(cudaMemcpy2DAsync(ctx->D, ctx->ldn * 4, V, n * 4, n * 4, R, cudaMemcpyDeviceToDevice,
+                         ctx->stream));
+  } else if (f64_data) {
+    CKS(prescale_and_copy(ctx, (const double*)V, R));
   } else {
+    CKS(prescale_and_copy(ctx, (const float*)V, R));
+  }
+  const bool out_direct = ctx->esz == ue;
+  CKS(run_kmv(ctx, in_place ? V : ctx->D, ctx->iota, R, out_direct ? U : ctx->KD, ctx->iota, mode, w,
+              in_place ? n : 0, out_direct ? n : 0));
+  if (!out_direct) {
     convert_cols_kernel<double, float><<<dim3(64, R), 256, 0, ctx->stream>>>(
         (const double*)ctx->KD, ctx->ldn, (float*)U, n, n);
     CK(cudaGetLastError());
@@ -1405,6 +1439,7 @@ ulisse_status ulisse_sgld_step(ulisse_ctx* ctx, double* psi_inout, double eps_t,
   if (ctx->batched) return fail(ctx, ULISSE_ERR_ARG, "batched context: use the ulisse_batch_* calls");
   if (!(eps_t >= 0.0) || !std::isfinite(eps_t)) return fail(ctx, ULISSE_ERR_ARG, "eps_t invalid");
   CKS(set_psi_host(ctx, psi_inout));
+  CKS(psi_to_device(ctx));
   const double *Md, *pd;
   CKS(upload_M_prior(ctx, M, prior_grad, &Md, &pd));
   CK(cudaMemsetAsync(ctx->status_dev, 0, sizeof(int), ctx->stream));
@@ -1652,9 +1687,9 @@ static ulisse_status graph_build(ulisse_ctx* ctx, int s0_cols) {
   // what one launch does outside the CG loop (the loop's share is counted on the device)
   const long long kmv_per = ctx->mixed ? 2 : 1, kmv_cols = ctx->mixed ? 64 : kMaxRChunk;
   const int init_cols = warm ? R : s0_cols;   // columns of the product K s_0
-  // prescale (+ the tensor-core images), probes, the CG start, the gradient pass (+ its
+  // prescale, probes, the CG start, the gradient pass (+ its
   // operand images), the update, the learned start's two kernels, the product K s_0
-  ctx->graph_launches_fixed = (ctx->mixed ? 3 : 1) + 1 + cg_init_launch_count(ctx->n, R, ctx->num_sms) +
+  ctx->graph_launches_fixed = 1 + 1 + cg_init_launch_count(ctx->n, R, ctx->num_sms) +
       (ctx->mixed ? 2 : 1) + 1 + (s0_cols > 0 ? 2 : 0) +
       (init_cols > 0 ? kmv_per * ((init_cols + kmv_cols - 1) / kmv_cols) : 0);
   ctx->graph_entries_fixed = (double)ctx->n * (double)ctx->n * (double)(R + init_cols);
@@ -1729,6 +1764,7 @@ ulisse_status ulisse_sgld_chain(ulisse_ctx* ctx, double* psi_dev, const double* 
   CK(cudaMemsetAsync(ctx->status_dev, 0, sizeof(int), ctx->stream));
   CK(cudaMemcpyAsync(ctx->psi_dev, psi_dev, sizeof(double) * p, cudaMemcpyDeviceToDevice,
                      ctx->stream));
+  ctx->psi_arg.by_value = 0;
   // Each step as one launch of the step graph, unless the event timing is on (it times
   // single launches) or warm-start pairs are being recorded (host-side bookkeeping).
   if (graph_usable(ctx) && n_steps > 0) {
@@ -2280,7 +2316,7 @@ static ulisse_status batch_clear_status(ulisse_ctx* ctx) {
 extern "C++" {
 // Kernel arguments of the batched tensor-core K V into slot k of b_tc_args (0: the CG
 // rounds, 1: K s_0 of warm-started solves, 2: ulisse_batch_kmv): cols(b, sub, L) sets each
-// problem's V, vmap, R or R_dev, U and umap; the rest is the problem's own operand buffers.
+// problem's V, vmap, R or R_dev, U and umap (and other leading dimensions); the rest is the problem's own operand buffers.
 template <typename Fn>
 static ulisse_status batch_tc_upload(ulisse_ctx* ctx, int k, Fn cols) {
   const int B = (int)ctx->subs.size();
@@ -2288,9 +2324,9 @@ static ulisse_status batch_tc_upload(ulisse_ctx* ctx, int k, Fn cols) {
   for (int b = 0; b < B; ++b) {
     ulisse_ctx* sub = ctx->subs[b];
     TcLaunch l{};
-    cols(b, sub, l);
     l.ldv = sub->ldn;
     l.ldu = sub->ldn;
+    cols(b, sub, l);
     l.xhat = (const float*)sub->xhat;
     l.bneg = sub->bneg;
     l.Vp = sub->Vt;
@@ -2336,45 +2372,63 @@ ulisse_status ulisse_batch_kmv(ulisse_ctx* ctx, const double* psi, const float* 
   CKS(batch_set_psi(ctx, psi));
   CKS(batch_clear_status(ctx));
   graph_release(ctx);   // the products below may reallocate the problems' buffers
+  // U is written in place.  The tensor-core products read V in place too, unless some U
+  // overlaps some V; the FP32 products copy whole tiles of padded columns, so there V goes into
+  // D with each problem's prescale launch.
+  const bool mixed = ctx->cfg.precision == ULISSE_PREC_MIXED;
+  bool in_place = mixed;
+  if (mixed) {
+    struct Span { const char *a, *b; bool out; };
+    std::vector<Span> sp;
+    for (int b = 0; b < B; ++b) {
+      const size_t bytes = (size_t)ctx->subs[b]->n * R * 4;
+      sp.push_back({(const char*)V[b], (const char*)V[b] + bytes, false});
+      sp.push_back({(const char*)U[b], (const char*)U[b] + bytes, true});
+    }
+    std::sort(sp.begin(), sp.end(), [](const Span& x, const Span& y) { return x.a < y.a; });
+    const char* end[2] = {nullptr, nullptr};   // furthest end of the inputs, of the outputs
+    for (const Span& x : sp) {
+      if (x.a < end[!x.out]) in_place = false;
+      end[x.out] = std::max(end[x.out], x.b);
+    }
+  }
   std::vector<BatchKmvDesc> desc(B);
   std::vector<int> rc(B, R);
   double entries = 0.0;
   for (int b = 0; b < B; ++b) {
     ulisse_ctx* sub = ctx->subs[b];
-    SUBS(ctx, sub, prescale(sub));
     SUBS(ctx, sub, ensure_columns(sub, R, R));
-    CK(cudaMemcpy2DAsync(sub->D, sub->ldn * 4, V[b], sub->n * 4, sub->n * 4, R,
-                         cudaMemcpyDeviceToDevice, ctx->stream));
+    SUBS(ctx, sub, mixed ? prescale(sub) : prescale_and_copy(sub, V[b], R));
+    if (mixed && !in_place)
+      CK(cudaMemcpy2DAsync(sub->D, sub->ldn * 4, V[b], sub->n * 4, sub->n * 4, R,
+                           cudaMemcpyDeviceToDevice, ctx->stream));
     desc[b] = BatchKmvDesc{(const float*)sub->xhat, sub->n, sub->DP, 0, sub->params,
-                           (const float*)sub->D, sub->ldn, sub->iota, (float*)sub->KD, sub->ldn,
+                           (const float*)sub->D, sub->ldn, sub->iota, U[b], sub->n,
                            sub->iota, ctx->b_rcount + b};
     entries += (double)sub->n * (double)sub->n * R;
   }
-  CK(cudaMemcpyAsync(ctx->b_kdesc, desc.data(), sizeof(BatchKmvDesc) * B, cudaMemcpyHostToDevice,
-                     ctx->stream));
-  CK(cudaMemcpyAsync(ctx->b_rcount, rc.data(), sizeof(int) * B, cudaMemcpyHostToDevice,
-                     ctx->stream));
-  if (ctx->cfg.precision == ULISSE_PREC_MIXED) {
-    CKS(batch_tc_upload(ctx, 2, [R](int, ulisse_ctx* sub, TcLaunch& l) {
-      l.V = sub->D;
+  if (mixed) {
+    CKS(batch_tc_upload(ctx, 2, [&](int b, ulisse_ctx* sub, TcLaunch& l) {
+      l.V = in_place ? V[b] : sub->D;
+      if (in_place) l.ldv = sub->n;
       l.vmap = sub->iota;
       l.R = R;
-      l.U = sub->KD;
+      l.U = U[b];
+      l.ldu = sub->n;
       l.umap = sub->iota;
     }));
     CK(batch_kv_launch(ctx, 2, nullptr, R, ctx->stream));
   } else {
+    CK(cudaMemcpyAsync(ctx->b_kdesc, desc.data(), sizeof(BatchKmvDesc) * B, cudaMemcpyHostToDevice,
+                       ctx->stream));
+    CK(cudaMemcpyAsync(ctx->b_rcount, rc.data(), sizeof(int) * B, cudaMemcpyHostToDevice,
+                       ctx->stream));
     CK(launch_kmv_batch(ctx->b_kdesc, ctx->b_items, ctx->b_n_items, ctx->b_queue, R,
                         ctx->num_sms, ctx->status_dev, ctx->stream));
   }
   ctx->launches++;
   ctx->mvp_rounds++;
   ctx->entry_rhs += entries;
-  for (int b = 0; b < B; ++b) {
-    ulisse_ctx* sub = ctx->subs[b];
-    CK(cudaMemcpy2DAsync(U[b], sub->n * 4, sub->KD, sub->ldn * 4, sub->n * 4, R,
-                         cudaMemcpyDeviceToDevice, ctx->stream));
-  }
   int st = 0;
   CKS(batch_read_status(ctx, &st));
   return status_to_result(ctx, st);
@@ -2555,6 +2609,7 @@ static ulisse_status batch_step_body(ulisse_ctx* ctx, bool sgld, bool in_graph) 
     const int p = sub->d + 2;
     CK(cudaMemcpyAsync(sub->psi_dev, ctx->b_psi + off, sizeof(double) * p,
                        cudaMemcpyDeviceToDevice, ctx->stream));
+    sub->psi_arg.by_value = 0;
     off += p;
     SUBS(ctx, sub, prescale(sub));
     CK(cudaMemcpyAsync(sub->B, sub->y, sub->ldn * 4, cudaMemcpyDeviceToDevice, ctx->stream));
@@ -2708,7 +2763,7 @@ static void batch_count_fixed(ulisse_ctx* ctx, int steps, bool sgld) {
   const long long grad_launches = mixed ? 2LL * (long long)ctx->b_gt_groups.size() : 2LL;
   long long init_launches = 0;   // the CG starts' (cg_init_launch_count) beyond one per problem
   for (ulisse_ctx* sub : ctx->subs) init_launches += cg_init_launch_count(sub->n, R, ctx->num_sms) - 1;
-  ctx->launches += (long long)steps * ((mixed ? 5LL : 3LL) * B + init_launches + grad_launches +
+  ctx->launches += (long long)steps * (3LL * B + init_launches + grad_launches +
                                        (sgld ? B + 1 : 0) + (warm ? (mixed ? 2 : 1) : 0));
   ctx->entry_rhs += steps * ent * (warm ? 2.0 : 1.0);
   if (warm) ctx->mvp_rounds += steps;

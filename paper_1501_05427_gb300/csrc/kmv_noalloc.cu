@@ -131,27 +131,25 @@ extern "C" ulisse_status ulisse_kmv_noalloc(const float* X, long long n, int d, 
     return e == cudaSuccess ? ULISSE_OK : fail(what, ULISSE_ERR_CUDA);
   };
   // The array keeps the previous call's contents: clear what must start at zero.
-  if ((st = ck(cudaMemcpyAsync(psi_dev, psi, sizeof(double) * (d + 2), cudaMemcpyHostToDevice, s),
-               "copy of psi failed")) != ULISSE_OK)
-    return st;
   if ((st = ck(cudaMemsetAsync(status, 0, sizeof(int), s), "memset failed")) != ULISSE_OK ||
       (st = ck(cudaMemsetAsync(counters, 0, (size_t)n_rb * sizeof(int), s), "memset failed")) !=
           ULISSE_OK ||
       (st = ck(cudaMemsetAsync(xhat + n * DP, 0, (size_t)(ldn - n) * DP * sizeof(float), s),
                "memset failed")) != ULISSE_OK)
     return st;
-  if ((st = ck(cudaMemcpy2DAsync(Vpad, ldn * sizeof(float), V, n * sizeof(float),
-                                 n * sizeof(float), R, cudaMemcpyDeviceToDevice, s),
-               "copy of V failed")) != ULISSE_OK)
-    return st;
   if (ldn > n &&
       (st = ck(cudaMemset2DAsync(Vpad + n, ldn * sizeof(float), 0, (ldn - n) * sizeof(float), R, s),
                "memset failed")) != ULISSE_OK)
     return st;
 
-  const int blocks = (int)std::min<long long>((n + 255) / 256, 4LL * sc->num_sms);
-  prescale_kernel<float><<<blocks, 256, 0, s>>>(psi_dev, X, xhat, n, d, DP, params);
-  if ((st = ck(cudaGetLastError(), "prescale launch failed")) != ULISSE_OK) return st;
+  // psi travels by value; the same launch copies V's columns into the padded scratch
+  PsiArg pa{};
+  for (int i = 0; i < d + 2; ++i) pa.v[i] = psi[i];
+  pa.by_value = 1;
+  if ((st = ck(launch_prescale<float, float>(pa, psi_dev, X, xhat, n, d, DP, params, V, Vpad, ldn, R,
+                                             sc->num_sms, s),
+               "prescale launch failed")) != ULISSE_OK)
+    return st;
 
   KmvLaunch L{};
   L.xhat = xhat;

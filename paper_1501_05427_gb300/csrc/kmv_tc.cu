@@ -36,21 +36,6 @@ constexpr uint32_t kTcCols = 128;  // tensor-memory columns per CTA (layout in T
 // ------------------------------------------------------------------------------------
 // Operand preparation
 // ------------------------------------------------------------------------------------
-// b_i = -c1 |x^_i|^2 with c1 = log2(e)/2 (0 for the padding rows).
-__global__ void prescale_tc_kernel(const float* __restrict__ xhat, int DP, int d, long long n,
-                                   long long ld, float* __restrict__ bneg) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < ld;
-       i += (long long)gridDim.x * blockDim.x) {
-    double s2 = 0.0;
-    if (i < n)
-      for (int q = 0; q < d; ++q) {
-        const double v = xhat[i * DP + q];
-        s2 += v * v;
-      }
-    bneg[i] = (float)(-0.5 * 1.4426950408889634 * s2);
-  }
-}
-
 // V columns vmap[0..R) -> BF16 high and low parts, a K-major canonical image of N rows
 // (right-hand sides) x 32 points each, back to back per j-tile (one bulk copy); rows r >= R and
 // points >= n are zero.
@@ -440,13 +425,6 @@ cudaError_t launch_kmv_tc(TcLaunch& L, cudaStream_t s) {
     case 16: return tc_dispatch_n<16>(L, s);
     default: return cudaErrorInvalidValue;
   }
-}
-
-cudaError_t launch_prescale_tc(const float* xhat, int DP, int d, long long n, long long ld,
-                               float* bneg, int num_sms, cudaStream_t s) {
-  const int blocks = (int)std::min<long long>((ld + 255) / 256, 8LL * num_sms);
-  prescale_tc_kernel<<<blocks, 256, 0, s>>>(xhat, DP, d, n, ld, bneg);
-  return cudaGetLastError();
 }
 
 }  // namespace ulisse

@@ -44,6 +44,7 @@
 #include <vector>
 
 #include "kmv_kernel.cuh"
+#include "prescale.cuh"
 #include "tc_common.cuh"
 
 namespace ulisse {
@@ -53,43 +54,70 @@ constexpr int kT2BM = 128;
 constexpr int kT2Threads = 288;    // warp 0 copies and MMAs, warps 1-8 epilogue
 constexpr uint32_t kT2Cols = 128;  // tensor-memory columns per CTA
 
-// The rows A_j = [x^_j, 1, 0...] and B_j = [2 c1 x^_j, b_j, 0...] for j in [0, rows) as TF32
-// high part and remainder, K8 columns, in 32-row K-major canonical tiles; rows >= n are zero.
-// When K8 == DP there is no slot for the augmented column (A_j = x^_j, B_j = 2 c1 x^_j); the
-// batched launches leave it out for every d (aug = 0) and add b_j in the epilogue.
-// b_j = -c1 |x^_j|^2 is read from the row norms of launch_prescale_tc.  A's parts are two
-// arrays; B's tiles hold high part, remainder and the tile's 32 b_j back to back
-// (tc2_b_stride floats each), so that a tile is one bulk copy.
-__global__ void pack_x_tf32_kernel(const float* __restrict__ xhat, const float* __restrict__ bneg,
-                                   const DevParams* __restrict__ params, int DP, int K8, int aug,
-                                   long long n, long long rows, float* __restrict__ Ahi,
-                                   float* __restrict__ Alo, float* __restrict__ Bt) {
-  const float two_c1 = 2.f * params->c1f;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < rows * K8;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const long long j = idx / K8;
-    const int k = (int)(idx - j * K8);
-    float va = 0.f, vb = 0.f;
+// The prescale of the mixed path, one row per thread: x^_j, the row norm b_j = -c1 |x^_j|^2
+// (summed in FP64), and the rows A_j = [x^_j, 1, 0...] and B_j = [2 c1 x^_j, b_j, 0...] as TF32
+// high part and remainder, K8 columns, in 32-row K-major canonical tiles.  Rows j in [n, rows)
+// are zero (x^ itself is written for j < n only).  When K8 == DP there is no slot for the
+// augmented column (A_j = x^_j, B_j = 2 c1 x^_j); the batched launches leave it out for every d
+// (aug = 0) and add b_j in the epilogue.  A's parts are two arrays; B's tiles hold high part,
+// remainder and the tile's 32 b_j back to back (tc2_b_stride floats each), so that a tile is one
+// bulk copy.
+template <int DP>
+__global__ void __launch_bounds__(128) prescale_mixed_kernel(
+    const PsiArg pa, double* __restrict__ psi_dev, const float* __restrict__ X,
+    float* __restrict__ xhat, long long n, long long rows, int d, int aug,
+    DevParams* __restrict__ P, float* __restrict__ bneg, float* __restrict__ Ahi,
+    float* __restrict__ Alo, float* __restrict__ Bt) {
+  constexpr int K8 = DP >= 8 ? DP : 8;
+  __shared__ InvLength s;
+  unpack_params(pa, psi_dev, d, P, s);
+  const float two_c1 = 2.f * (float)(0.5 * 1.4426950408889634);   // 2 c1f
+  for (long long j = blockIdx.x * 128LL + threadIdx.x; j < rows; j += gridDim.x * 128LL) {
+    float x[K8];
+    double s2 = 0.0;
+#pragma unroll
+    for (int k = 0; k < K8; ++k) {
+      x[k] = (k < d && j < n) ? scale_by_pair(X[j * d + k], s, k) : 0.f;
+      if (k < d) s2 += (double)x[k] * (double)x[k];
+    }
     if (j < n) {
-      if (k < DP) {
-        va = xhat[j * DP + k];
-        vb = two_c1 * va;
-      } else if (k == DP && aug) {
-        va = 1.f;
-        vb = bneg[j];
+      if constexpr (DP >= 4) {
+#pragma unroll
+        for (int k = 0; k < DP; k += 4)
+          *reinterpret_cast<float4*>(xhat + j * DP + k) = make_float4(x[k], x[k + 1], x[k + 2], x[k + 3]);
+      } else {
+        *reinterpret_cast<float2*>(xhat + j * DP) = make_float2(x[0], x[1]);
       }
     }
+    const float b = (float)(-0.5 * 1.4426950408889634 * s2);
+    bneg[j] = b;
     const long long t = j / kT2BN;
     const int jj = (int)(j - t * kT2BN);
-    const uint32_t in_tile = tc::canon_offset(jj, k, 4, K8 / 4) / 4;
-    const long long off = t * kT2BN * K8 + in_tile;
-    const float ha = tc::tf32_round(va), hb = tc::tf32_round(vb);
-    Ahi[off] = ha;
-    Alo[off] = va - ha;
     float* bt = Bt + t * tc2_b_stride(K8);
-    bt[in_tile] = hb;
-    bt[kT2BN * K8 + in_tile] = vb - hb;
-    if (k == 0) bt[2 * kT2BN * K8 + jj] = bneg[j];
+    bt[2 * kT2BN * K8 + jj] = b;
+#pragma unroll
+    for (int k0 = 0; k0 < K8; k0 += 4) {
+      float ah[4], al[4], bh[4], bl[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int k = k0 + q;
+        float va = x[k], vb = two_c1 * x[k];
+        if (DP < K8 && k == DP && aug && j < n) {
+          va = 1.f;
+          vb = b;
+        }
+        ah[q] = tc::tf32_round(va);
+        al[q] = va - ah[q];
+        bh[q] = tc::tf32_round(vb);
+        bl[q] = vb - bh[q];
+      }
+      const uint32_t in_tile = tc::canon_offset(jj, k0, 4, K8 / 4) / 4;
+      const long long off = t * kT2BN * K8 + in_tile;
+      *reinterpret_cast<float4*>(Ahi + off) = make_float4(ah[0], ah[1], ah[2], ah[3]);
+      *reinterpret_cast<float4*>(Alo + off) = make_float4(al[0], al[1], al[2], al[3]);
+      *reinterpret_cast<float4*>(bt + in_tile) = make_float4(bh[0], bh[1], bh[2], bh[3]);
+      *reinterpret_cast<float4*>(bt + kT2BN * K8 + in_tile) = make_float4(bl[0], bl[1], bl[2], bl[3]);
+    }
   }
 }
 
@@ -566,11 +594,6 @@ static cudaError_t tc2_dispatch_n(TcLaunch& L, cudaStream_t s) {
   return cudaErrorInvalidValue;
 }
 
-// K8, the TF32 MMA's K (a multiple of 8), from the padded d: padded d 2 and 4 take the
-// augmented column within one K step (K8 = 8); padded d 8 and 16 leave it to the epilogue
-// (K8 = d).
-static int tc2_k8(int DP) { return DP >= 8 ? DP : 8; }
-
 cudaError_t launch_kmv_tc2(TcLaunch& L, cudaStream_t s) {
   if (L.R < 1 || L.R > 64 || !L.X_hi || !L.X_lo || !L.X_b) return cudaErrorInvalidValue;
   switch (L.DP) {
@@ -582,14 +605,22 @@ cudaError_t launch_kmv_tc2(TcLaunch& L, cudaStream_t s) {
   }
 }
 
-cudaError_t launch_pack_x_tf32(const float* xhat, const float* bneg, const DevParams* params,
-                               int DP, long long n, long long ld128, float* X_hi, float* X_lo,
-                               float* X_b, int num_sms, cudaStream_t s, bool aug) {
-  const int K8 = tc2_k8(DP);
-  const long long total = ld128 * K8;
-  const int blocks = (int)std::min<long long>((total + 255) / 256, 8LL * num_sms);
-  pack_x_tf32_kernel<<<blocks, 256, 0, s>>>(xhat, bneg, params, DP, K8, aug ? 1 : 0, n, ld128,
-                                            X_hi, X_lo, X_b);
+cudaError_t launch_prescale_mixed(const PsiArg& pa, double* psi_dev, const float* X, float* xhat,
+                                  long long n, long long ld128, int d, int DP, bool aug,
+                                  DevParams* P, float* bneg, float* X_hi, float* X_lo, float* X_b,
+                                  int num_sms, cudaStream_t s) {
+  const int blocks = (int)std::min<long long>(ld128 / 128, 8LL * num_sms);
+  auto go = [&](auto kernel) {
+    kernel<<<blocks, 128, 0, s>>>(pa, psi_dev, X, xhat, n, ld128, d, aug ? 1 : 0, P, bneg, X_hi,
+                                  X_lo, X_b);
+  };
+  switch (DP) {
+    case 2: go(prescale_mixed_kernel<2>); break;
+    case 4: go(prescale_mixed_kernel<4>); break;
+    case 8: go(prescale_mixed_kernel<8>); break;
+    case 16: go(prescale_mixed_kernel<16>); break;
+    default: return cudaErrorInvalidValue;
+  }
   return cudaGetLastError();
 }
 

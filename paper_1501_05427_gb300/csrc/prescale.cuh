@@ -1,35 +1,123 @@
 // a1: parameter unpack and input prescale (shared by the context path and the
 // allocation-free K V entry point).
+//
+// What bounds it: latency and the FP64 pipe (1.7 lanes per clock per SM).  The 1 / l_k are
+// formed once per CTA, one exponential per thread; x^ = x / l in float is rounded once from
+// the product with 1 / l_k held as a pair of floats (48 bits), so that no element takes an FP64
+// multiply and two conversions.  With every thread forming all 1 / l_k and FP64 products the
+// launch took 10.7 us at n = 9,937, d = 4 and 27.5 us at n = 50,000, d = 8 (mixed precision:
+// then two more launches of 5 us for the row norms and the TF32 images, now the same launch).
+// A whole product call, which also loses the copies of psi, V and U, went from 45 to 25 us at
+// n = 1,030, d = 8, 5 columns (FP32) and from 840 to 795 us at n = 50,000 (mixed).
 #pragma once
 
+#include <cfloat>
+
+#include "tc_common.cuh"
 #include "ulisse_internal.cuh"
 
 namespace ulisse {
 
-// ------------------------------------------------------------------------------------
-// a1: parameters from psi, and x^ = x / l (rows >= n and dims >= d stay zero).
-// ------------------------------------------------------------------------------------
+// Parameters by value (a host call's psi needs no copy of its own), else from psi_dev.
+struct PsiArg {
+  double v[kMaxP];
+  int by_value;
+};
+
+// 1 / l_k as a double and as the pair hi + lo of floats.
+struct InvLength {
+  double inv[kMaxD];
+  float hi[kMaxD], lo[kMaxD];
+};
+
+// Every CTA: 1 / l_k into s; CTA 0 also writes the derived parameters (and psi when given by
+// value).  Ends with a barrier; needs at least kMaxP threads.
+__device__ inline void unpack_params(const PsiArg& pa, double* __restrict__ psi_dev, int d,
+                                     DevParams* __restrict__ P, InvLength& s) {
+  const int k = threadIdx.x;
+  if (k < d + 2) {
+    const double p = pa.by_value ? pa.v[k] : psi_dev[k];
+    const double e = exp(k < d ? -p : p);
+    if (k < d) {
+      s.inv[k] = e;
+      s.hi[k] = (float)e;
+      s.lo[k] = (float)(e - (double)s.hi[k]);
+    }
+    if (blockIdx.x == 0) {
+      P->psi[k] = p;
+      if (pa.by_value) psi_dev[k] = p;
+      if (k < d) P->inv_l[k] = e;
+      if (k == d) {
+        P->sigma2 = e;
+        P->c0f = (float)log2(e);
+        P->c1f = (float)(0.5 * 1.4426950408889634);  // log2(e) / 2
+      }
+      if (k == d + 1) {
+        P->lambda = e;
+        P->lambdaf = (float)e;
+      }
+    }
+  }
+  __syncthreads();
+}
+
+// (float)(x / l): x (hi + lo) with one rounding of the pair's sum where neither part nor the
+// product's error term can leave the normal range, else the FP64 product.
+__device__ __forceinline__ float scale_by_pair(float x, const InvLength& s, int k) {
+  const float hi = s.hi[k];
+  const float p = x * hi;
+  if (fabsf(p) < 1e30f && fabsf(p) > 1e-28f && hi > 1e-28f && hi < 1e30f)
+    return p + fmaf(x, s.lo[k], fmaf(x, hi, -p));
+  return x == 0.f ? x : (float)((double)x * s.inv[k]);
+}
+
 template <typename T>
-__global__ void prescale_kernel(const double* __restrict__ psi, const float* __restrict__ X,
-                                T* __restrict__ xhat, long long n, int d, int DP,
-                                DevParams* __restrict__ P) {
-  double inv_l[kMaxD];
-  for (int k = 0; k < d; ++k) inv_l[k] = exp(-psi[k]);
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    for (int k = 0; k < d + 2; ++k) P->psi[k] = psi[k];
-    for (int k = 0; k < d; ++k) P->inv_l[k] = inv_l[k];
-    const double s2 = exp(psi[d]), lam = exp(psi[d + 1]);
-    P->sigma2 = s2;
-    P->lambda = lam;
-    P->c0f = (float)log2(s2);
-    P->c1f = (float)(0.5 * 1.4426950408889634);  // log2(e) / 2
-    P->lambdaf = (float)lam;
+__device__ __forceinline__ T scaled(float x, const InvLength& s, int k) {
+  if constexpr (sizeof(T) == 4) return scale_by_pair(x, s, k);
+  else return (double)x * s.inv[k];
+}
+
+// x^ = x / l for rows [0, n) (rows >= n stay zero; dims >= d zero), one element per thread; the
+// CTAs from row_blocks on copy (and convert) R columns of V, leading dimension n, to D, leading
+// dimension ldn.
+template <typename T, typename TV>
+__global__ void __launch_bounds__(256) prescale_kernel(
+    const PsiArg pa, double* __restrict__ psi_dev, const float* __restrict__ X,
+    T* __restrict__ xhat, long long n, int d, int log2_dp, DevParams* __restrict__ P,
+    int row_blocks, const TV* __restrict__ V, T* __restrict__ D, long long ldn, int R) {
+  __shared__ InvLength s;
+  if ((int)blockIdx.x < row_blocks) {
+    unpack_params(pa, psi_dev, d, P, s);
+    const long long total = n << log2_dp;
+    for (long long idx = blockIdx.x * 256LL + threadIdx.x; idx < total; idx += row_blocks * 256LL) {
+      const int k = (int)(idx & ((1 << log2_dp) - 1));
+      const long long i = idx >> log2_dp;
+      xhat[idx] = k < d ? scaled<T>(X[i * d + k], s, k) : T(0);
+    }
+    return;
   }
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    for (int k = 0; k < DP; ++k)
-      xhat[i * DP + k] = (k < d) ? (T)((double)X[i * d + k] * inv_l[k]) : T(0);
+  const long long total = n * R, step = (gridDim.x - row_blocks) * 256LL;
+  for (long long idx = (blockIdx.x - row_blocks) * 256LL + threadIdx.x; idx < total; idx += step) {
+    const long long c = idx / n;
+    D[c * ldn + (idx - c * n)] = (T)V[idx];
   }
+}
+
+inline int log2_of(int dp) { return dp == 2 ? 1 : dp == 4 ? 2 : dp == 8 ? 3 : 4; }
+
+// Launch of prescale_kernel; V null: no columns to copy.
+template <typename T, typename TV>
+cudaError_t launch_prescale(const PsiArg& pa, double* psi_dev, const float* X, T* xhat, long long n,
+                            int d, int DP, DevParams* P, const TV* V, T* D, long long ldn, int R,
+                            int num_sms, cudaStream_t s) {
+  // four elements per thread, at most eight CTAs per SM for each of the two parts
+  auto blocks = [&](long long total) {
+    return (int)std::max<long long>(1, std::min<long long>((total + 1023) / 1024, 8LL * num_sms));
+  };
+  const int rb = blocks(n * DP);
+  prescale_kernel<T, TV><<<rb + (V ? blocks(n * R) : 0), 256, 0, s>>>(
+      pa, psi_dev, X, xhat, n, d, log2_of(DP), P, rb, V, D, ldn, R);
+  return cudaGetLastError();
 }
 
 }  // namespace ulisse

@@ -260,13 +260,13 @@ struct GradLaunch {
   int num_sms;
   size_t need_partials_len;  // set when partials_len is too small
   bool plan_only;            // only fill need_partials_len (no launch)
-  // tensor-core pass (launch_grad_tc) only: row norms (launch_prescale_tc) and BF16 scratch
+  // tensor-core pass (launch_grad_tc) only: row norms (launch_prescale_mixed) and BF16 scratch
   // for the packed operand blocks, 2 x kGtScratchRows elements per point (points rounded up to
   // 128): per tile the right operand (2M <= 128 factor slots) and the point features Z, each
   // high | low part
   const float* bneg;
   void* tc_tiles;
-  // padded d <= 8: the TF32 row images of launch_pack_x_tf32, from which the pass forms the
+  // padded d <= 8: the TF32 row images of launch_prescale_mixed, from which the pass forms the
   // exponent's cross term on the tensor cores; c_has_bj when they were packed with the
   // augmented column (b_j in C)
   const float* X_hi;
@@ -275,10 +275,10 @@ struct GradLaunch {
   bool c_has_bj;
 };
 
-// Mixed-precision (tcgen05) K V launch: operands prepared by launch_prescale_tc.
+// Mixed-precision (tcgen05) K V launch: operands prepared by launch_prescale_mixed.
 struct TcLaunch {
   const float* xhat;     // prescaled inputs, ld x DP row-major (the SIMT layout)
-  const float* bneg;     // -c1 |x^|^2 (launch_prescale_tc), ld128
+  const float* bneg;     // -c1 |x^|^2 (launch_prescale_mixed), ld128
   void* Vp;              // BF16 packed operand tiles, high | low part per tile (written by the
                          // launch), ld128 x 128
   const void* V;         // FP32 operand columns
@@ -305,7 +305,7 @@ struct TcLaunch {
   int need_counters;
   bool plan_only;        // only fill need_* (no launch): sizing scratch ahead of a capture
   // tensor-core cross term (launch_kmv_tc2): TF32 images of the augmented rows
-  // (launch_pack_x_tf32): A rows at X_hi / X_lo, B tiles at X_b
+  // (launch_prescale_mixed): A rows at X_hi / X_lo, B tiles at X_b
   const float* X_hi;
   const float* X_lo;
   const float* X_b;
@@ -329,11 +329,14 @@ void launch_pack_v(const TcLaunch& L, int N, long long ntiles, cudaStream_t s);
 // A rows: high part X_hi and remainder X_lo, ld128 x K8 floats each (K8 = max(8, DP)); B rows:
 // tiles of 32 points, high part | remainder | b_j, tc2_b_stride(K8) floats each, ld128 / 32 tiles.
 __host__ __device__ constexpr int tc2_b_stride(int K8) { return 2 * 32 * K8 + 32; }
-// aug: rows carry the column term b_j (padded d 2 and 4 of the single-problem launches);
-// false for the batched launches, whose epilogue adds it for every d.
-cudaError_t launch_pack_x_tf32(const float* xhat, const float* bneg, const DevParams* params,
-                               int DP, long long n, long long ld128, float* X_hi, float* X_lo,
-                               float* X_b, int num_sms, cudaStream_t s, bool aug);
+// The prescale of the mixed path with the row norms and the TF32 images (prescale.cuh,
+// kmv_tc2.cu).  aug: rows carry the column term b_j (padded d 2 and 4 of the single-problem
+// launches); false for the batched launches, whose epilogue adds it for every d.
+struct PsiArg;
+cudaError_t launch_prescale_mixed(const PsiArg& pa, double* psi_dev, const float* X, float* xhat,
+                                  long long n, long long ld128, int d, int DP, bool aug,
+                                  DevParams* P, float* bneg, float* X_hi, float* X_lo, float* X_b,
+                                  int num_sms, cudaStream_t s);
 // Batched tensor-core K V (padded d <= 8): per problem a TcLaunch with the operand pointers,
 // R or R_dev, and the forced split nsplit >= 1 (tiles per split <= kTcMaxSplitTiles);
 // items: (problem, 128-row block, split) per CTA; R_max: the largest live column count.
@@ -351,7 +354,5 @@ cudaError_t gt_batch_upload_args(const GradLaunch* L, const int* nsplit, int B, 
                                  cudaStream_t s);
 cudaError_t launch_grad_tc_batch(const void* args_dev, int B, const int4* items, int n_items,
                                  int DP, int M, cudaStream_t s, bool prime_only = false);
-cudaError_t launch_prescale_tc(const float* xhat, int DP, int d, long long n, long long ld,
-                               float* bneg, int num_sms, cudaStream_t s);
 
 }  // namespace ulisse

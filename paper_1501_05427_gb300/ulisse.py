@@ -186,6 +186,15 @@ def _colmajor(t):
     return t
 
 
+def _used_on(stream, *tensors):
+    """Tell the caching allocator that `tensors` are read or written on `stream` when that is not
+    the stream they live on (the products read V and write U in place)."""
+    import torch
+    if torch.cuda.current_stream() != stream:
+        for t in tensors:
+            t.record_stream(stream)
+
+
 class Context:
     """One GP regression problem on the current CUDA device (ulisse_create)."""
 
@@ -250,6 +259,7 @@ class Context:
             out = torch.empty((R, self.n), dtype=V.dtype, device=V.device).t()
         psi = _f64_host(psi, self.p)
         fn = self._lib.ulisse_kmv_f64 if f64 else self._lib.ulisse_kmv
+        _used_on(self.stream, Vc, out)
         self._check(fn(self._h, _hptr(psi), which, ctypes.c_void_p(Vc.data_ptr()), R,
                        ctypes.c_void_p(out.data_ptr())))
         return out[:, 0] if V.dim() == 1 else out
@@ -530,6 +540,7 @@ class BatchContext:
         vp = (ctypes.c_void_p * self.n_problems)(*[V.data_ptr() for V in Vc])
         up = (ctypes.c_void_p * self.n_problems)(*[U.data_ptr() for U in Us])
         psi = _f64_host(psi, self.n_params)
+        _used_on(self.stream, *Vc, *Us)
         self._check(self._lib.ulisse_batch_kmv(self._h, _hptr(psi), ctypes.cast(vp, ctypes.c_void_p),
                                                R, ctypes.cast(up, ctypes.c_void_p)))
         return Us
