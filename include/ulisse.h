@@ -136,6 +136,7 @@ ulisse_status ulisse_create_host(ulisse_ctx **out, const float *X, const float *
  *   psi  host, p = d+2 doubles.
  *   V    device, n x R column-major (leading dimension n), R >= 1.
  *   U    device, n x R column-major; must not overlap V.
+ * V may be read and U written in place: both stay valid until the stream's work is done.
  * In FP64 precision V and U are read and written as float and converted; use
  * ulisse_kmv_f64 for double data.  In mixed precision K V (which == -1) runs on the tensor
  * cores (each entry of U within 1e-4 of sum_j |K_ij| |V_jr|) and the derivative products in

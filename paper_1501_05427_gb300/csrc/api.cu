@@ -140,7 +140,7 @@ struct ulisse_ctx {
   int* b_h_rmax = nullptr;         // pinned
   double* b_psi = nullptr;         // device: packed parameters of all problems
   int b_np = 0;                    // packed parameter count
-  int b_maxch = 1;                 // largest chunk count of the batched CG launches
+  int b_cluster = 1;               // CTAs per column of the batched CG iterations
   // mixed-precision batches: the tensor-core K V over (problem, 128-row block, split) items
   bool tc_no_aug = false;          // sub-context of a mixed batch: rows packed without b_j
   int4* b_tc_items = nullptr;
@@ -672,19 +672,8 @@ static ulisse_status solve_core(ulisse_ctx* ctx, int R, int s0_cols, unsigned lo
     if (nl == 0) break;
     CKS(run_kmv(ctx, ctx->D, ctx->live, nl, ctx->KD, ctx->live, kModeK, -1));
     ctx->mvp_rounds += 1;
-    // Spread the live columns over about two waves of CTAs (at least 2048 rows each).
-    const long long target = std::max(1, (2 * ctx->num_sms + nl - 1) / nl);
-    long long ch = std::max<long long>((ctx->n + target - 1) / target, 2048);
-    ch = std::max<long long>(ch, (ctx->n + kMaxCgChunks - 1) / kMaxCgChunks);
-    ch = (ch + 255) / 256 * 256;
-    a.chunk = ch;
-    a.nchunk = (int)((ctx->n + ch - 1) / ch);
-    const dim3 grid(a.nchunk, nl);
-    cg_dot_kernel<T><<<grid, kCgChunkNT, 0, ctx->stream>>>(a);
-    cg_update_kernel<T><<<grid, kCgChunkNT, 0, ctx->stream>>>(a);
-    cg_finish_kernel<T><<<grid, kCgChunkNT, 0, ctx->stream>>>(a);
-    CK(cudaGetLastError());
-    ctx->launches += 3;
+    CK(launch_cg_round(a, nl, ctx->stream));
+    ctx->launches++;
     n_prev = nl;
   }
   return ULISSE_OK;
@@ -1500,20 +1489,6 @@ static void graph_release(ulisse_ctx* ctx) {
 
 extern "C++" {
 template <typename T>
-static void cg_round_launches(ulisse_ctx* ctx, CgArgs<T>& a, int nl) {
-  const long long target = std::max(1, (2 * ctx->num_sms + nl - 1) / nl);
-  long long ch = std::max<long long>((ctx->n + target - 1) / target, 2048);
-  ch = std::max<long long>(ch, (ctx->n + kMaxCgChunks - 1) / kMaxCgChunks);
-  ch = (ch + 255) / 256 * 256;
-  a.chunk = ch;
-  a.nchunk = (int)((ctx->n + ch - 1) / ch);
-  const dim3 grid(a.nchunk, nl);
-  cg_dot_kernel<T><<<grid, kCgChunkNT, 0, ctx->stream>>>(a);
-  cg_update_kernel<T><<<grid, kCgChunkNT, 0, ctx->stream>>>(a);
-  cg_finish_kernel<T><<<grid, kCgChunkNT, 0, ctx->stream>>>(a);
-}
-
-template <typename T>
 static ulisse_status graph_capture_body(ulisse_ctx* ctx, int s0_cols) {
   const int nr = ctx->cfg.n_probes, R = 1 + nr, p = ctx->d + 2;
   CKS(prescale(ctx));
@@ -1578,7 +1553,7 @@ static ulisse_status graph_capture_body(ulisse_ctx* ctx, int s0_cols) {
   const int per_chunk = ctx->mixed ? 2 : 1;
   compact_graph_kernel<<<1, 32, 0, ctx->cap_stream2>>>(
       ctx->st, ctx->st_next, R, ctx->live, ctx->n_live_dev, h_loop, h_branch, chunk_cols,
-      per_chunk, 3, ctx->cfg.max_iter + 2, ctx->gstat, ctx->status_dev);
+      per_chunk, 1, ctx->cfg.max_iter + 2, ctx->gstat, ctx->status_dev);
   cudaError_t e = cudaGetLastError();
   const cudaGraphNode_t* bdeps = nullptr;
   size_t nbdeps = 0;
@@ -1605,9 +1580,8 @@ static ulisse_status graph_capture_body(ulisse_ctx* ctx, int s0_cols) {
                                      nullptr, 0, cudaStreamCaptureModeThreadLocal));
     ctx->stream = ctx->cap_stream2;
     ulisse_status r = run_kmv(ctx, ctx->D, ctx->live, k + 1, ctx->KD, ctx->live, kModeK, -1);
-    if (r == ULISSE_OK) cg_round_launches<T>(ctx, a, k + 1);
     ctx->stream = outer;
-    const cudaError_t e3 = cudaGetLastError();
+    const cudaError_t e3 = r == ULISSE_OK ? launch_cg_round(a, k + 1, ctx->cap_stream2) : cudaSuccess;
     const cudaError_t e4 = cudaStreamEndCapture(ctx->cap_stream2, &tmp);
     CKS(r);
     CK(e3);
@@ -2494,18 +2468,18 @@ static ulisse_status batch_prepare(ulisse_ctx* ctx) {
   std::vector<BatchKmvDesc> kd(B), kd0(B);
   const std::vector<int> rcount(B, R);
   std::vector<BatchGradDesc> gd(B);
-  int slot0 = 0, maxch = 1;
+  // every column of the batch gets the cluster of the largest problem
+  long long n_max = 1;
+  for (ulisse_ctx* sub : ctx->subs) n_max = std::max(n_max, sub->n);
+  ctx->b_cluster = cg_cluster_size(n_max);
+  int slot0 = 0;
   for (int b = 0; b < B; ++b) {
     ulisse_ctx* sub = ctx->subs[b];
     CgArgs<float> a = cg_args<float>(sub, 0, 0);
     a.cs = ctx->chain;
-    // 4096 rows per CTA, more when the problem would need over kMaxCgChunks chunks
-    a.chunk = std::max<long long>(kBatchCgChunk,
-                                  ((sub->n + kMaxCgChunks - 1) / kMaxCgChunks + 255) / 256 * 256);
-    a.nchunk = (int)((sub->n + a.chunk - 1) / a.chunk);
+    a.chunk = cg_cluster_rows(sub->ldn, ctx->b_cluster);
     a.n_live = sub->n_live_dev;
     if (warm) a.warm_refresh = ctx->cfg.probe_refresh;
-    maxch = std::max(maxch, a.nchunk);
     args[b] = a;
     probs[b] = BatchCgProb{sub->st, sub->st_next, sub->live, sub->n_live_dev, R, sub->n};
     kd[b] = BatchKmvDesc{(const float*)sub->xhat, sub->n, sub->DP, 0, sub->params,
@@ -2522,7 +2496,6 @@ static ulisse_status batch_prepare(ulisse_ctx* ctx) {
                           ctx->b_g + (long long)b * kMaxP};
     slot0 += nslots;
   }
-  ctx->b_maxch = maxch;
   CK(cudaMemcpyAsync(ctx->b_cgargs, args.data(), sizeof(CgArgs<float>) * B, cudaMemcpyHostToDevice,
                      ctx->stream));
   CK(cudaMemcpyAsync(ctx->b_cgprob, probs.data(), sizeof(BatchCgProb) * B, cudaMemcpyHostToDevice,
@@ -2595,8 +2568,8 @@ static ulisse_status batch_prepare(ulisse_ctx* ctx) {
 
 // One batched step on ctx->stream: per problem its parameters from the packed vector, the
 // prescale, y and the probes, the CG start; then CG + ULISSE in lock-step rounds (one
-// batched compaction, one persistent K V over all live columns of all problems, three
-// batched CG launches per round); then the persistent gradient sweep and, with sgld, every
+// batched compaction, one persistent K V over all live columns of all problems, one batched
+// CG iteration per round); then the persistent gradient sweep and, with sgld, every
 // problem's update and the packed parameters back.  The host loop and the step graph run
 // exactly these launches; in the graph the round loop is a WHILE node whose compaction sets
 // the loop condition and a SWITCH over the K V width.
@@ -2632,17 +2605,15 @@ static ulisse_status batch_step_body(ulisse_ctx* ctx, bool sgld, bool in_graph) 
   }
   CK(cudaGetLastError());
   CK(cudaMemsetAsync(ctx->gstat + 3, 0, sizeof(long long), ctx->stream));
-  const dim3 cg_grid(ctx->b_maxch, R, B);
   auto cg_round = [&](cudaStream_t s) {
-    cg_dot_batch_kernel<float><<<cg_grid, kCgChunkNT, 0, s>>>(ctx->b_cgargs);
-    cg_update_batch_kernel<float><<<cg_grid, kCgChunkNT, 0, s>>>(ctx->b_cgargs);
-    cg_finish_batch_kernel<float><<<cg_grid, kCgChunkNT, 0, s>>>(ctx->b_cgargs);
-    return cudaGetLastError();
+    return launch_clustered(cg_round_batch_kernel<float>,
+                            dim3((unsigned)ctx->b_cluster, (unsigned)R, (unsigned)B), ctx->b_cluster,
+                            s, (const CgArgs<float>*)ctx->b_cgargs);
   };
   const int max_rounds = ctx->cfg.max_iter + 2;
   if (!in_graph) {
     for (int it = 0; it < max_rounds + 1; ++it) {
-      compact_batch_kernel<<<1, 256, 0, ctx->stream>>>(ctx->b_cgprob, B, ctx->b_rmax, 0, 0, 0,
+      compact_batch_kernel<<<1, kCompactBatchNT, 0, ctx->stream>>>(ctx->b_cgprob, B, ctx->b_rmax, 0, 0, 0,
                                                        max_rounds, ctx->gstat, ctx->status_dev);
       CK(cudaGetLastError());
       CK(cudaMemcpyAsync(ctx->b_h_rmax, ctx->b_rmax, sizeof(int), cudaMemcpyDeviceToHost,
@@ -2675,7 +2646,7 @@ static ulisse_status batch_step_body(ulisse_ctx* ctx, bool sgld, bool in_graph) 
     cudaStream_t s2 = ctx->cap_stream2;
     CK(cudaStreamBeginCaptureToGraph(s2, body, nullptr, nullptr, 0,
                                      cudaStreamCaptureModeThreadLocal));
-    compact_batch_kernel<<<1, 256, 0, s2>>>(ctx->b_cgprob, B, ctx->b_rmax, 1, h_loop, h_branch,
+    compact_batch_kernel<<<1, kCompactBatchNT, 0, s2>>>(ctx->b_cgprob, B, ctx->b_rmax, 1, h_loop, h_branch,
                                             max_rounds, ctx->gstat, ctx->status_dev);
     cudaError_t e = cudaGetLastError();
     const cudaGraphNode_t* bdeps = nullptr;

@@ -4,12 +4,14 @@
 // e^T e, d^T K d, alpha, beta, the early-stop test and the ULISSE weights -- is FP64.
 #pragma once
 
+#include <cooperative_groups.h>
+
 #include "prescale.cuh"
 #include "ulisse_internal.cuh"
 
 namespace ulisse {
 
-constexpr int kCgChunkNT = 256;   // threads of the chunked CG kernels
+constexpr int kCgChunkNT = 256;   // threads of the CG start
 
 // ------------------------------------------------------------------------------------
 // a2: probes r_j (column j = 1..nr of B): +-1 from the top bit, or N(0,1) by Box-Muller,
@@ -54,9 +56,9 @@ struct CgArgs {
   ColState* st;
   ColState* st_next;     // state written by an iteration, committed by compact_kernel
   const int* live;
-  double* part1;         // per (column, chunk) partial d^T K d
-  double* part2;         // per (column, chunk) partial e^T e
-  int nchunk;            // CTAs per column
+  double* part1;         // the CG start's partial sums per (column, chunk): residual
+  double* part2;         // ... and right-hand side
+  int nchunk;            // CTAs per column of the CG start
   long long chunk;       // rows per CTA
   double alpha_thr, eps, beta;
   int max_iter;
@@ -218,98 +220,137 @@ __global__ void __launch_bounds__(kCgChunkNT) cg_init_kernel(const CgArgs<T> a) 
   }
 }
 
-// One CG iteration (Algorithm 1) on every live column, with the ULISSE bookkeeping, in
-// three launches over a (chunk, live column) grid so that every column is spread over
-// several CTAs:
-//   cg_dot_kernel     partial d^T K d per chunk
-//   cg_update_kernel  alpha = e^T e / d^T K d (partials summed in chunk order), s += alpha d,
-//                     e -= alpha K d, the ULISSE tail term, partial e'^T e' per chunk
-//   cg_finish_kernel  e'^T e' (chunk order), the early-stop / convergence / max_iter
-//                     decisions (every CTA of a column reaches the same ones), the copy of
-//                     s_l into the estimators at the early stop, d = e' + beta d, and the
-//                     new column state (into st_next; compact_kernel commits it).
+// One CG iteration (Algorithm 1) on every live column, with the ULISSE bookkeeping, in one
+// launch: a cluster of CTAs per column (grid (CTAs of the column, live column)), each on its
+// range of rows, with two sums over the cluster:
+//   d^T K d         -> alpha = e^T e / d^T K d
+//   s += alpha d, e -= alpha K d, the ULISSE tail term; e'^T e'
+//   the early-stop / convergence / max_iter decisions (every CTA of a column reaches the same
+//   ones), the copy of s_l into the estimators at the early stop, d = e' + beta d, and the new
+//   column state (into st_next; the compaction commits it).
 // The increment delta_{m+1} = alpha_m d_m is added with weight prod_{r<=j} w_r to every
 // estimator whose J >= j (j = m+1-l) once the early stop at l has been reached.
+//
+// What bounds it: latency (cluster barriers, L2 round trips) and, per scalar, the FP64 pipe (64
+// clocks per warp instruction and SM quarter): the scalars are formed by one warp of each CTA
+// and read from shared memory, not by every thread.  As three launches that exchanged their
+// sums through global memory, with every thread forming the scalars, an iteration took 49 us at
+// n = 50,000, 17 columns, and 26 us at n = 1,030, 101 columns in FP64.
+constexpr int kCgNT = 512;
+constexpr int kCgMaxCluster = 8;
 
-// The bodies below take the chunk (ch) and the live-list index (li) of the CTA: the
-// single-problem kernels pass their grid coordinates, the batched ones add the problem.
+// 16 bytes of a vector.
 template <typename T>
-__device__ inline void cg_dot_body(const CgArgs<T>& a, int ch, int li) {
-  __shared__ double red[kCgChunkNT / 32];
+struct alignas(16) CgVec {
+  static constexpr int N = 16 / (int)sizeof(T);
+  T v[N];
+};
+
+// The padding rows [n, ld) of every column hold zeros (the products read whole tiles) and stay
+// zero whatever the scalars: an infinite step would make 0 * inf of them.
+template <typename T>
+__device__ __forceinline__ void cg_keep_padding(CgVec<T>& x, long long i, long long n) {
+  if ((i + 1) * CgVec<T>::N > n) {
+#pragma unroll
+    for (int q = 0; q < CgVec<T>::N; ++q)
+      if (i * CgVec<T>::N + q >= n) x.v[q] = T(0);
+  }
+}
+
+// Sum of v over the cluster's CTAs, in a fixed order, valid in warp 0.  slot: this use's shared
+// double (the peers read it: one slot per use within a launch).
+__device__ inline double cluster_sum_warp0(double v, double* red, double* slot) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  v = warp_sum(v);
+  if (lane == 0) red[warp] = v;
+  __syncthreads();
+  if (warp == 0) {
+    v = warp_sum(lane < kCgNT / 32 ? red[lane] : 0.0);
+    if (lane == 0) *slot = v;
+  }
+  cl.sync();
+  if (warp == 0) {
+    const int nc = (int)cl.num_blocks();
+    v = lane < nc ? *cl.map_shared_rank(slot, lane) : 0.0;
+#pragma unroll
+    for (int o = kCgMaxCluster / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    v = __shfl_sync(0xffffffffu, v, 0);
+  }
+  return v;
+}
+
+// The scalars warp 0 hands to the CTA.
+template <typename T>
+struct CgShared {
+  double red[kCgNT / 32];
+  double slot[2];
+  T al, w0, w1, bt;
+  int breakdown, copy_s, better, done;
+};
+
+// One column's iteration; ch: this CTA's rank in the column's cluster, li: its live-list index.
+template <typename T>
+__device__ inline void cg_round_body(const CgArgs<T>& a, int ch, int li, CgShared<T>& sh) {
+  using V = CgVec<T>;
+  constexpr int VN = V::N;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const bool warp0 = tid < 32;
   const int c = a.live[li];
-  const T* d = a.D + c * a.ld;
-  const T* kd = a.KD + c * a.ld;
-  long long i0, i1;
-  chunk_range(a, ch, &i0, &i1);
+  const ColState st = a.st[c];
+  const long long col = c * a.ld;
+  // rows in vectors of 16 bytes, the last one padded
+  const long long nv = (a.n + VN - 1) / VN, per = a.chunk / VN;
+  const long long v0 = min(nv, ch * per), v1 = min(nv, v0 + per);
+  V* s = reinterpret_cast<V*>(a.S + col);
+  V* e = reinterpret_cast<V*>(a.E + col);
+  V* d = reinterpret_cast<V*>(a.D + col);
+  const V* kd = reinterpret_cast<const V*>(a.KD + col);
+  V* se0 = reinterpret_cast<V*>(a.SE + (long long)st.est_off * a.ld);
+  V* se1 = se0 + a.ld / VN;
+
   double p = 0.0;
-  for (long long i = i0 + threadIdx.x; i < i1; i += kCgChunkNT) p += (double)d[i] * (double)kd[i];
-  p = block_sum<kCgChunkNT>(p, red);
-  if (threadIdx.x == 0) a.part1[(long long)c * a.nchunk + ch] = p;
-}
-
-template <typename T>
-__device__ inline void cg_update_body(const CgArgs<T>& a, int ch, int li) {
-  __shared__ double red[kCgChunkNT / 32];
-  const int c = a.live[li];
-  const ColState& st = a.st[c];
-  double dKd = 0.0;
-  for (int k = 0; k < a.nchunk; ++k) dKd += a.part1[(long long)c * a.nchunk + k];
-  if (!(dKd > 0.0) || !isfinite(dKd)) return;  // breakdown: handled in cg_finish_kernel
-  T* s = a.S + c * a.ld;
-  T* e = a.E + c * a.ld;
-  const T* d = a.D + c * a.ld;
-  const T* kd = a.KD + c * a.ld;
-  const double al = st.ee / dKd;
-  const T alT = (T)al;
-  T w0 = T(0), w1 = T(0);
-  if (st.phase == kTail) {
+#pragma unroll 4
+  for (long long i = v0 + tid; i < v1; i += kCgNT) {
+    const V di = d[i], ki = kd[i];
+#pragma unroll
+    for (int q = 0; q < VN; ++q) p += (double)di.v[q] * (double)ki.v[q];
+  }
+  const double dKd = cluster_sum_warp0(p, sh.red, &sh.slot[0]);
+  if (warp0) {
+    const bool bad = !(dKd > 0.0) || !isfinite(dKd);
+    const double al = bad ? 0.0 : st.ee / dKd;
+    T w0 = T(0), w1 = T(0);
     const int j = st.m + 1 - st.l;
-    const double Wa = weight_product(j, a.beta) * al;
-    if (st.J[0] >= j) w0 = (T)Wa;
-    if (st.n_est > 1 && st.J[1] >= j) w1 = (T)Wa;
+    if (!bad && st.phase == kTail && (st.J[0] >= j || (st.n_est > 1 && st.J[1] >= j))) {
+      // prod_{r <= j} exp(beta r) in the order of weight_product, the exponentials one per lane
+      double W = 1.0;
+      if (j < 32) {
+        const double w = exp(a.beta * (double)lane);
+        for (int r = 0; r <= j; ++r) W *= __shfl_sync(0xffffffffu, w, r);
+      } else {
+        W = weight_product(j, a.beta);
+      }
+      const double Wa = W * al;
+      if (st.J[0] >= j) w0 = (T)Wa;
+      if (st.n_est > 1 && st.J[1] >= j) w1 = (T)Wa;
+    }
+    if (lane == 0) {
+      sh.breakdown = bad;
+      sh.al = (T)al;
+      sh.w0 = w0;
+      sh.w1 = w1;
+    }
   }
-  T* se0 = a.SE + (long long)st.est_off * a.ld;
-  T* se1 = se0 + a.ld;
-  long long i0, i1;
-  chunk_range(a, ch, &i0, &i1);
-  double p2 = 0.0;
-  for (long long i = i0 + threadIdx.x; i < i1; i += kCgChunkNT) {
-    const T di = d[i];
-    s[i] = fma(alT, di, s[i]);
-    const T ei = fma(-alT, kd[i], e[i]);
-    e[i] = ei;
-    p2 += (double)ei * (double)ei;
-    if (w0 != T(0)) se0[i] = fma(w0, di, se0[i]);
-    if (w1 != T(0)) se1[i] = fma(w1, di, se1[i]);
-  }
-  p2 = block_sum<kCgChunkNT>(p2, red);
-  if (threadIdx.x == 0) a.part2[(long long)c * a.nchunk + ch] = p2;
-}
-
-template <typename T>
-__device__ inline void cg_finish_body(const CgArgs<T>& a, int ch, int li) {
-  const int c = a.live[li];
-  const ColState& st = a.st[c];
-  const int phase = st.phase, l = st.l, m = st.m, n_est = st.n_est;
-  const int J0 = st.J[0], J1 = st.J[1];
-  T* s = a.S + c * a.ld;
-  T* e = a.E + c * a.ld;
-  T* d = a.D + c * a.ld;
-  T* se0 = a.SE + (long long)st.est_off * a.ld;
-  long long i0, i1;
-  chunk_range(a, ch, &i0, &i1);
-  double dKd = 0.0, ee1 = 0.0;
-  for (int k = 0; k < a.nchunk; ++k) {
-    dKd += a.part1[(long long)c * a.nchunk + k];
-    ee1 += a.part2[(long long)c * a.nchunk + k];
-  }
-  ColState nx = st;
-  if (!(dKd > 0.0) || !isfinite(dKd)) {
-    // Breakdown: K is not positive definite along d, or a value is not finite.
-    if (phase == kPre)
-      for (int t = 0; t < n_est; ++t)
-        for (long long i = i0 + threadIdx.x; i < i1; i += kCgChunkNT) se0[t * a.ld + i] = s[i];
-    if (ch == 0 && threadIdx.x == 0) {
+  __syncthreads();
+  if (sh.breakdown) {
+    // K is not positive definite along d, or a value is not finite
+    if (st.phase == kPre)
+      for (int t = 0; t < st.n_est; ++t)
+        for (long long i = v0 + tid; i < v1; i += kCgNT) (t == 0 ? se0 : se1)[i] = s[i];
+    if (ch == 0 && tid == 0) {
+      ColState nx = st;
       nx.outcome = 3;
       nx.phase = kDone;
       a.st_next[c] = nx;
@@ -317,98 +358,197 @@ __device__ inline void cg_finish_body(const CgArgs<T>& a, int ch, int li) {
     }
     return;
   }
-  const int m1 = m + 1;
-  int ph = phase, l1 = l, outcome = st.outcome;
-  bool copy_s = false, done = false;
-  const int jmax = (n_est > 1 && J1 > J0) ? J1 : J0;
-  if (ph == kPre && sqrt(ee1) < a.alpha_thr) {
-    l1 = m1;
-    ph = kTail;
-    copy_s = true;
+
+  const T al = sh.al, w0 = sh.w0, w1 = sh.w1;
+  double p2 = 0.0;
+#pragma unroll 2
+  for (long long i = v0 + tid; i < v1; i += kCgNT) {
+    const V di = d[i], ki = kd[i];
+    V si = s[i], ei = e[i];
+#pragma unroll
+    for (int q = 0; q < VN; ++q) {
+      si.v[q] = fma(al, di.v[q], si.v[q]);
+      ei.v[q] = fma(-al, ki.v[q], ei.v[q]);
+    }
+    cg_keep_padding(si, i, a.n);
+    cg_keep_padding(ei, i, a.n);
+    s[i] = si;
+    e[i] = ei;
+#pragma unroll
+    for (int q = 0; q < VN; ++q) p2 += (double)ei.v[q] * (double)ei.v[q];
+    if (w0 != T(0)) {
+      V x = se0[i];
+#pragma unroll
+      for (int q = 0; q < VN; ++q) x.v[q] = fma(w0, di.v[q], x.v[q]);
+      cg_keep_padding(x, i, a.n);
+      se0[i] = x;
+    }
+    if (w1 != T(0)) {
+      V x = se1[i];
+#pragma unroll
+      for (int q = 0; q < VN; ++q) x.v[q] = fma(w1, di.v[q], x.v[q]);
+      cg_keep_padding(x, i, a.n);
+      se1[i] = x;
+    }
   }
-  const bool conv = sqrt(ee1) < a.eps;
-  if (ph == kPre && conv) {
-    copy_s = true;
-    done = true;
-  } else if (ph == kTail && (m1 - l1 >= jmax || conv)) {
-    done = true;
-  } else if (m1 >= a.max_iter) {
-    if (ph == kPre) copy_s = true;
-    outcome = 4;
-    done = true;
+  const double ee1 = cluster_sum_warp0(p2, sh.red, &sh.slot[1]);
+  if (warp0) {
+    const int m1 = st.m + 1;
+    int ph = st.phase, l1 = st.l, outcome = st.outcome;
+    bool copy_s = false, done = false;
+    const int jmax = (st.n_est > 1 && st.J[1] > st.J[0]) ? st.J[1] : st.J[0];
+    const double norm = sqrt(ee1);
+    if (ph == kPre && norm < a.alpha_thr) {
+      l1 = m1;
+      ph = kTail;
+      copy_s = true;
+    }
+    const bool conv = norm < a.eps;
+    if (ph == kPre && conv) {
+      copy_s = true;
+      done = true;
+    } else if (ph == kTail && (m1 - l1 >= jmax || conv)) {
+      done = true;
+    } else if (m1 >= a.max_iter) {
+      if (ph == kPre) copy_s = true;
+      outcome = 4;
+      done = true;
+    }
+    // warm-started solves: remember the iterate of smallest residual
+    const bool better = a.warm_refresh > 0 && ee1 < st.best_ee;
+    if (lane == 0) {
+      sh.copy_s = copy_s;
+      sh.better = better;
+      sh.done = done;
+      sh.bt = done ? T(0) : (T)(ee1 / st.ee);
+      if (ch == 0) {
+        ColState nx = st;
+        nx.ee = ee1;
+        if (better) nx.best_ee = ee1;
+        nx.m = m1;
+        nx.l = l1;
+        nx.outcome = outcome;
+        nx.phase = done ? kDone : ph;
+        a.st_next[c] = nx;
+        if (outcome == 4) atomicOr(a.status, kStatusMaxIter);
+      }
+    }
   }
-  if (copy_s)
-    for (int t = 0; t < n_est; ++t)
-      for (long long i = i0 + threadIdx.x; i < i1; i += kCgChunkNT) se0[t * a.ld + i] = s[i];
-  // warm-started solves: remember the iterate of smallest residual (same decision in every
-  // CTA of the column)
-  const bool better = a.warm_refresh > 0 && ee1 < st.best_ee;
-  if (better) {
-    T* sb = a.Sbest + c * a.ld;
-    for (long long i = i0 + threadIdx.x; i < i1; i += kCgChunkNT) sb[i] = s[i];
+  __syncthreads();
+  if (sh.copy_s || sh.better) {
+    V* sb = sh.better ? reinterpret_cast<V*>(a.Sbest + col) : nullptr;
+    for (long long i = v0 + tid; i < v1; i += kCgNT) {
+      const V si = s[i];
+      if (sh.copy_s) {
+        se0[i] = si;
+        if (st.n_est > 1) se1[i] = si;
+      }
+      if (sb) sb[i] = si;
+    }
   }
-  if (!done) {
-    const T btT = (T)(ee1 / st.ee);
-    for (long long i = i0 + threadIdx.x; i < i1; i += kCgChunkNT) d[i] = fma(btT, d[i], e[i]);
-  }
-  if (ch == 0 && threadIdx.x == 0) {
-    nx.ee = ee1;
-    if (better) nx.best_ee = ee1;
-    nx.m = m1;
-    nx.l = l1;
-    nx.outcome = outcome;
-    nx.phase = done ? kDone : ph;
-    a.st_next[c] = nx;
-    if (outcome == 4) atomicOr(a.status, kStatusMaxIter);
+  if (!sh.done) {
+    const T bt = sh.bt;
+#pragma unroll 4
+    for (long long i = v0 + tid; i < v1; i += kCgNT) {
+      V di = d[i];
+      const V ei = e[i];
+#pragma unroll
+      for (int q = 0; q < VN; ++q) di.v[q] = fma(bt, di.v[q], ei.v[q]);
+      cg_keep_padding(di, i, a.n);
+      d[i] = di;
+    }
   }
 }
 
+// The peers read this CTA's shared slots: nobody leaves before all have.
 template <typename T>
-__global__ void __launch_bounds__(kCgChunkNT) cg_dot_kernel(const CgArgs<T> a) {
-  cg_dot_body(a, blockIdx.x, blockIdx.y);
-}
-template <typename T>
-__global__ void __launch_bounds__(kCgChunkNT) cg_update_kernel(const CgArgs<T> a) {
-  cg_update_body(a, blockIdx.x, blockIdx.y);
-}
-template <typename T>
-__global__ void __launch_bounds__(kCgChunkNT) cg_finish_kernel(const CgArgs<T> a) {
-  cg_finish_body(a, blockIdx.x, blockIdx.y);
+__global__ void __launch_bounds__(kCgNT) cg_round_kernel(const CgArgs<T> a) {
+  __shared__ CgShared<T> sh;
+  cg_round_body(a, blockIdx.x, blockIdx.y, sh);
+  cooperative_groups::this_cluster().sync();
 }
 
-// Batched forms: grid (chunk, live-list index, problem) over all problems of a batch; a
-// CTA past its problem's chunk count or live count returns at once.
+// Batched form: grid (CTAs of a column, live-list index, problem); a cluster past its problem's
+// live count returns at once.
 template <typename T>
-__global__ void __launch_bounds__(kCgChunkNT) cg_dot_batch_kernel(const CgArgs<T>* __restrict__ args) {
+__global__ void __launch_bounds__(kCgNT) cg_round_batch_kernel(const CgArgs<T>* __restrict__ args) {
+  __shared__ CgShared<T> sh;
   const CgArgs<T>& a = args[blockIdx.z];
-  if ((int)blockIdx.y >= *a.n_live || (int)blockIdx.x >= a.nchunk) return;
-  cg_dot_body(a, blockIdx.x, blockIdx.y);
-}
-template <typename T>
-__global__ void __launch_bounds__(kCgChunkNT) cg_update_batch_kernel(const CgArgs<T>* __restrict__ args) {
-  const CgArgs<T>& a = args[blockIdx.z];
-  if ((int)blockIdx.y >= *a.n_live || (int)blockIdx.x >= a.nchunk) return;
-  cg_update_body(a, blockIdx.x, blockIdx.y);
-}
-template <typename T>
-__global__ void __launch_bounds__(kCgChunkNT) cg_finish_batch_kernel(const CgArgs<T>* __restrict__ args) {
-  const CgArgs<T>& a = args[blockIdx.z];
-  if ((int)blockIdx.y >= *a.n_live || (int)blockIdx.x >= a.nchunk) return;
-  cg_finish_body(a, blockIdx.x, blockIdx.y);
+  if ((int)blockIdx.y >= *a.n_live) return;
+  cg_round_body(a, blockIdx.x, blockIdx.y, sh);
+  cooperative_groups::this_cluster().sync();
 }
 
-// Commit the state of the columns that just iterated (the first n_prev entries of the
-// live list), then rebuild the live list in column order; count to *n_live.
+// CTAs per column: about 1,024 rows each, a power of two up to kCgMaxCluster.
+inline int cg_cluster_size(long long n) {
+  int c = 1;
+  while (c < kCgMaxCluster && n > 1024LL * c) c *= 2;
+  return c;
+}
+
+// Rows per CTA of a column of leading dimension ld (a multiple of 64) over c CTAs.
+inline long long cg_cluster_rows(long long ld, int c) {
+  return ((ld + c - 1) / c + 63) / 64 * 64;
+}
+
+template <typename... Params, typename... Args>
+cudaError_t launch_clustered(void (*kernel)(Params...), dim3 grid, int cluster, cudaStream_t s,
+                             Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(kCgNT);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)cluster;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// One CG iteration of nl live columns.
+template <typename T>
+cudaError_t launch_cg_round(CgArgs<T> a, int nl, cudaStream_t s) {
+  const int c = cg_cluster_size(a.n);
+  a.chunk = cg_cluster_rows(a.ld, c);
+  return launch_clustered(cg_round_kernel<T>, dim3((unsigned)c, (unsigned)nl), c, s, a);
+}
+
+// Commit the state of the first n_prev columns of the live list, then rebuild the list in column
+// order; returns the live count.  One warp, a lane per column: as one thread it took 39 us for
+// 101 columns (each column's state a dependent chain of global loads), now 3 us.
+__device__ inline int commit_and_compact(ColState* __restrict__ st,
+                                         const ColState* __restrict__ st_next, int R, int n_prev,
+                                         int* __restrict__ live) {
+  const int lane = threadIdx.x & 31;
+  for (int k = lane; k < n_prev; k += 32) {
+    const int c = live[k];
+    st[c] = st_next[c];
+  }
+  __syncwarp();
+  int n = 0;
+  for (int c0 = 0; c0 < R; c0 += 32) {
+    const int c = c0 + lane;
+    const bool alive = c < R && st[c].phase != kDone;
+    const unsigned mask = __ballot_sync(0xffffffffu, alive);
+    if (alive) live[n + __popc(mask & ((1u << lane) - 1u))] = c;
+    n += __popc(mask);
+  }
+  __syncwarp();
+  return n;
+}
+
+// The compaction of one solve (one warp); count to *n_live.
 __global__ void compact_kernel(ColState* __restrict__ st, const ColState* __restrict__ st_next,
                                int R, int n_prev, int* __restrict__ live,
                                int* __restrict__ n_live) {
-  if (threadIdx.x != 0) return;
-  for (int k = 0; k < n_prev; ++k) st[live[k]] = st_next[live[k]];
-  int k = 0;
-  for (int c = 0; c < R; ++c)
-    if (st[c].phase != kDone) live[k++] = c;
-  *n_live = k;
+  const int k = commit_and_compact(st, st_next, R, n_prev, live);
+  if (threadIdx.x == 0) *n_live = k;
 }
+
+constexpr int kCompactBatchNT = 1024;
 
 // Column bookkeeping of one problem of a batch (compact_batch_kernel).
 struct BatchCgProb {
@@ -426,36 +566,36 @@ __host__ __device__ inline int batch_width_bucket(int r) {
   return r <= 2 ? 0 : r <= 4 ? 1 : r <= 9 ? 2 : r <= 17 ? 3 : 4;
 }
 
-// compact_kernel for every problem of a batch in one launch (one thread per problem; the
+// compact_kernel for every problem of a batch in one launch (a warp per problem; the
 // live lists and counts are those of the previous round, the counts 0 before the first):
 // commit, rebuild, and the largest live count to *rmax.  Inside a step graph it also sets
 // the loop condition (another round while any column is live) and the branch (the width
 // bucket of rmax; none when 0).  A round cap stops a loop that would not end.
 // stat (may be null): [rounds, sum of n_b^2 x live columns, launches, rounds this call].
-__global__ void __launch_bounds__(256) compact_batch_kernel(
+__global__ void __launch_bounds__(kCompactBatchNT) compact_batch_kernel(
     const BatchCgProb* __restrict__ probs, int B, int* __restrict__ rmax, int in_graph,
     cudaGraphConditionalHandle h_loop, cudaGraphConditionalHandle h_branch, int max_rounds,
     long long* __restrict__ stat, int* __restrict__ status) {
-  __shared__ int s_max[256];
-  __shared__ long long s_ent[256];
+  constexpr int NW = kCompactBatchNT / 32;
+  __shared__ int s_max[NW];
+  __shared__ long long s_ent[NW];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int mx = 0;
   long long ent = 0;
-  for (int b = threadIdx.x; b < B; b += blockDim.x) {
+  for (int b = warp; b < B; b += NW) {
     const BatchCgProb P = probs[b];
-    const int n_prev = *P.n_live;
-    for (int k = 0; k < n_prev; ++k) P.st[P.live[k]] = P.st_next[P.live[k]];
-    int k = 0;
-    for (int c = 0; c < P.R; ++c)
-      if (P.st[c].phase != kDone) P.live[k++] = c;
-    *P.n_live = k;
+    const int k = commit_and_compact(P.st, P.st_next, P.R, *P.n_live, P.live);
+    if (lane == 0) *P.n_live = k;
     mx = max(mx, k);
     ent += P.n * P.n * (long long)k;
   }
-  s_max[threadIdx.x] = mx;
-  s_ent[threadIdx.x] = ent;
+  if (lane == 0) {
+    s_max[warp] = mx;
+    s_ent[warp] = ent;
+  }
   __syncthreads();
   if (threadIdx.x != 0) return;
-  for (int t = 1; t < (int)blockDim.x; ++t) {
+  for (int t = 1; t < NW; ++t) {
     mx = max(mx, s_max[t]);
     ent += s_ent[t];
   }
@@ -471,7 +611,7 @@ __global__ void __launch_bounds__(256) compact_batch_kernel(
     if (mx > 0) {
       stat[0] += 1;
       stat[1] += ent;
-      stat[2] += 4;   // the batched K V and the three batched CG launches
+      stat[2] += 2;   // the batched K V and the batched CG iteration
     }
   }
   *rmax = mx;
@@ -580,12 +720,8 @@ __global__ void compact_graph_kernel(ColState* __restrict__ st, const ColState* 
                                      cudaGraphConditionalHandle h_branch, int chunk_cols,
                                      int launches_per_chunk, int launches_fixed, int max_rounds,
                                      long long* __restrict__ stat, int* __restrict__ status) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  const int n_prev = *n_live;
-  for (int k = 0; k < n_prev; ++k) st[live[k]] = st_next[live[k]];
-  int k = 0;
-  for (int c = 0; c < R; ++c)
-    if (st[c].phase != kDone) live[k++] = c;
+  int k = commit_and_compact(st, st_next, R, *n_live, live);
+  if (threadIdx.x != 0) return;
   const long long it = stat[3]++;
   if (k > 0 && it >= max_rounds) {
     atomicOr(status, kStatusMaxIter);

@@ -190,7 +190,7 @@ def _used_on(stream, *tensors):
     """Tell the caching allocator that `tensors` are read or written on `stream` when that is not
     the stream they live on (the products read V and write U in place)."""
     import torch
-    if torch.cuda.current_stream() != stream:
+    if torch._C._cuda_getCurrentRawStream(tensors[0].get_device()) != stream.cuda_stream:
         for t in tensors:
             t.record_stream(stream)
 
