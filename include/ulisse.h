@@ -53,7 +53,9 @@ typedef enum {
 } ulisse_status;
 
 typedef enum {
-    ULISSE_PREC_FP32 = 0,     /* FP32 vectors and SIMT products, FP64 scalar recurrences */
+    ULISSE_PREC_FP32 = 0,     /* FP32 vectors and products, FP64 scalar recurrences (larger
+                                 products contract on the tensor cores through an exact
+                                 three-way BF16 split of each float, FP32 accumulation) */
     ULISSE_PREC_MIXED = 1,    /* tensor-core (tcgen05) products, FP32 vectors: K V with the
                                  exponent's dot product by three TF32 products and the
                                  contraction by three BF16 products, the gradient's bilinear

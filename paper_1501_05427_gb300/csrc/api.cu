@@ -38,6 +38,7 @@ struct ulisse_ctx {
   void* y = nullptr;          // labels, ldn (element type T)
   void* xhat = nullptr;       // prescaled inputs, ldn x DP
   DevParams* params = nullptr;
+  void* v3 = nullptr;         // FP32: operand scratch of the tensor-core contraction
   double* exp_tab = nullptr;  // FP64: table of the exponential (exp64.cuh)
   double* psi_dev = nullptr;  // kMaxP
   PsiArg psi_arg{};           // by_value: psi of a host call, handed to the next prescale launch
@@ -101,8 +102,12 @@ struct ulisse_ctx {
   int last_nsplit = 1;        // split count of the last K V launch (or plan)
 
   // CUDA graph of one SGLD step (ulisse_sgld_chain)
+  bool simt = false;          // FP32 products by the SIMT kernel (the autotuner's candidates)
   bool planning = false;      // launch helpers only size their scratch
   bool capturing = false;     // launch helpers are being captured: no host-side counting
+  long long cap_launches = 0; // ... but of the K V launches captured
+  int kv_launches[kMaxM] = {};        // kernels of a CG iteration's K V, per live column count
+  int* kv_launches_dev = nullptr;
   bool graph_enabled = true;
   cudaStream_t cap_stream = nullptr, cap_stream2 = nullptr;
   cudaGraph_t step_graph = nullptr;
@@ -114,6 +119,7 @@ struct ulisse_ctx {
   double* eps_one = nullptr;  // device step size of a single graph step
   bool m_identity = false;    // M_dev holds the identity (the graph's default M)
   bool prior_zero = false;    // prior_dev holds zeros
+  long long graph_init_launches = 0;   // kernels of the product K s_0
   long long graph_launches_fixed = 0;  // kernel launches per step outside the CG loop
   double graph_entries_fixed = 0.0;    // entries x right-hand sides per step outside the loop
   long long graph_rounds_fixed = 0;
@@ -150,6 +156,8 @@ struct ulisse_ctx {
   int* b_tc_cnt = nullptr;         // split counters of all problems (zero between launches)
   std::vector<int> b_tc_nsplit;
   std::vector<size_t> b_tc_part_off, b_tc_cnt_off;
+  void* b_v3 = nullptr;            // FP32: operand scratch of the tensor-core contraction
+  std::vector<size_t> b_v3_off;    // per problem, bytes
   // ... and the tensor-core gradient pass, one launch per padded input width (group)
   std::vector<std::vector<int>> b_gt_groups;   // problem indices of each width
   std::vector<int> b_gt_dp, b_gt_item_off, b_gt_item_n;
@@ -436,7 +444,7 @@ static ulisse_status run_kmv_tc(ulisse_ctx* ctx, const void* V, const int* vmap,
           ctx->free_events.push_back({ea, eb});
       }
       if (e == cudaSuccess) {
-        if (!ctx->capturing) ctx->launches += 2;
+        (ctx->capturing ? ctx->cap_launches : ctx->launches) += 2;   // the packing of V first
         break;
       }
       if (e != cudaErrorMemoryAllocation || attempt == 1 || ctx->capturing)
@@ -468,11 +476,14 @@ static ulisse_status run_kmv(ulisse_ctx* ctx, const void* V, const int* vmap, in
     L.ldv = ldv;
     L.vmap = vmap + c0;
     L.R = std::min(kMaxRChunk, R - c0);
+    L.launches = 1;
     L.U = U;
     L.ldu = ldu;
     L.umap = umap + c0;
     L.params = ctx->params;
     L.exp_tab = ctx->exp_tab;
+    L.v3 = ctx->v3;
+    L.simt = ctx->simt || ctx->cfg.kmv_rows_per_thread != 0;
     L.mode = mode;
     L.which = which;
     L.tm = ctx->cfg.kmv_rows_per_thread;
@@ -508,7 +519,7 @@ static ulisse_status run_kmv(ulisse_ctx* ctx, const void* V, const int* vmap, in
           ctx->free_events.push_back({ea, eb});
       }
       if (e == cudaSuccess) {
-        if (!ctx->capturing) ctx->launches++;
+        (ctx->capturing ? ctx->cap_launches : ctx->launches) += L.launches;
         break;
       }
       if (e != cudaErrorMemoryAllocation || attempt == 1 || ctx->capturing)
@@ -1008,7 +1019,7 @@ static ulisse_status check_cfg(const ulisse_config* c) {
 
 static ulisse_status create_impl(ulisse_ctx** out, const float* X, const float* y, long long n,
                                  int d, const ulisse_config* cfg, void* stream,
-                                 cudaMemcpyKind kind) {
+                                 cudaMemcpyKind kind, bool in_batch = false) {
   if (!out) return fail(nullptr, ULISSE_ERR_ARG, "out is null");
   *out = nullptr;
   if (!X || !y) return fail(nullptr, ULISSE_ERR_ARG, "X or y is null");
@@ -1064,6 +1075,9 @@ static ulisse_status create_impl(ulisse_ctx** out, const float* X, const float* 
                        4 * (ctx->ld128 / 32) * tc2_b_stride(16))))
       return bail(s);
   }
+  if (!ctx->f64 && !ctx->mixed && !in_batch && n >= kF32TcMinN &&
+      (s = dev_alloc(ctx, &ctx->v3, 2 * 3 * kMaxRChunk * ctx->ldn)))
+    return bail(s);
   if (ctx->f64) {
     if ((s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->exp_tab), sizeof(double) * kExpTabN)))
       return bail(s);
@@ -1188,15 +1202,24 @@ static ulisse_status kmv_common(ulisse_ctx* ctx, const double* psi, int which, c
   probe.R = std::min(R, kMaxRChunk);
   probe.mode = mode;
   probe.exp_tab = ctx->exp_tab;
+  probe.v3 = ctx->v3;
+  probe.simt = ctx->cfg.kmv_rows_per_thread != 0;
   const char *vb = (const char*)V, *ub = (const char*)U;
   const size_t bytes = (size_t)n * R * ue;
   const bool overlap = ub < vb + bytes && vb < ub + bytes;
-  const bool reads_direct = (ctx->mixed && mode == kModeK) ||
-                            (f64_data && kmv_f64_sym_applies(probe));
+  bool reads_direct = (ctx->mixed && mode == kModeK) || (f64_data && kmv_f64_sym_applies(probe));
+  if (!ctx->f64 && !ctx->mixed && ctx->tune.empty()) {
+    // FP32: every launch of kMaxRChunk columns and that of the rest
+    reads_direct = kmv_f32_tc_applies(probe);
+    if (R > kMaxRChunk && R % kMaxRChunk != 0) {
+      probe.R = R % kMaxRChunk;
+      reads_direct = reads_direct && kmv_f32_tc_applies(probe);
+    }
+  }
   const bool in_place = reads_direct && !overlap;
   if (in_place) {
     CKS(prescale(ctx));
-  } else if (ctx->mixed) {
+  } else if (ctx->mixed) {   // (its prescale copies nothing)
     CKS(prescale(ctx));
     CK(cudaMemcpy2DAsync(ctx->D, ctx->ldn * 4, V, n * 4, n * 4, R, cudaMemcpyDeviceToDevice,
                          ctx->stream));
@@ -1491,6 +1514,7 @@ extern "C++" {
 template <typename T>
 static ulisse_status graph_capture_body(ulisse_ctx* ctx, int s0_cols) {
   const int nr = ctx->cfg.n_probes, R = 1 + nr, p = ctx->d + 2;
+  ctx->cap_launches = 0;
   CKS(prescale(ctx));
   CK(cudaMemcpyAsync(ctx->B, ctx->y, ctx->ldn * ctx->esz, cudaMemcpyDeviceToDevice,
                      ctx->stream));
@@ -1515,6 +1539,7 @@ static ulisse_status graph_capture_body(ulisse_ctx* ctx, int s0_cols) {
   if (warm)
     CKS(run_kmv(ctx, ctx->S, ctx->warm_map + (s0_cols > 0 ? ctx->cap : 0), R, ctx->KD,
                 ctx->iota, kModeK, -1));
+  ctx->graph_init_launches = ctx->cap_launches;   // the product K s_0, if any
   CgArgs<T> a = cg_args<T>(ctx, s0_cols > 0 && !warm, 0);
   a.cs = ctx->chain;
   if (warm) {
@@ -1549,11 +1574,9 @@ static ulisse_status graph_capture_body(ulisse_ctx* ctx, int s0_cols) {
   cudaStream_t outer = ctx->stream;
   CK(cudaStreamBeginCaptureToGraph(ctx->cap_stream2, body, nullptr, nullptr, 0,
                                    cudaStreamCaptureModeThreadLocal));
-  const int chunk_cols = ctx->mixed ? 64 : kMaxRChunk;
-  const int per_chunk = ctx->mixed ? 2 : 1;
   compact_graph_kernel<<<1, 32, 0, ctx->cap_stream2>>>(
-      ctx->st, ctx->st_next, R, ctx->live, ctx->n_live_dev, h_loop, h_branch, chunk_cols,
-      per_chunk, 1, ctx->cfg.max_iter + 2, ctx->gstat, ctx->status_dev);
+      ctx->st, ctx->st_next, R, ctx->live, ctx->n_live_dev, h_loop, h_branch,
+      ctx->kv_launches_dev, ctx->cfg.max_iter + 2, ctx->gstat, ctx->status_dev);
   cudaError_t e = cudaGetLastError();
   const cudaGraphNode_t* bdeps = nullptr;
   size_t nbdeps = 0;
@@ -1579,7 +1602,9 @@ static ulisse_status graph_capture_body(ulisse_ctx* ctx, int s0_cols) {
     CK(cudaStreamBeginCaptureToGraph(ctx->cap_stream2, sp.conditional.phGraph_out[k], nullptr,
                                      nullptr, 0, cudaStreamCaptureModeThreadLocal));
     ctx->stream = ctx->cap_stream2;
+    ctx->cap_launches = 0;
     ulisse_status r = run_kmv(ctx, ctx->D, ctx->live, k + 1, ctx->KD, ctx->live, kModeK, -1);
+    ctx->kv_launches[k] = (int)ctx->cap_launches;
     ctx->stream = outer;
     const cudaError_t e3 = r == ULISSE_OK ? launch_cg_round(a, k + 1, ctx->cap_stream2) : cudaSuccess;
     const cudaError_t e4 = cudaStreamEndCapture(ctx->cap_stream2, &tmp);
@@ -1658,14 +1683,15 @@ static ulisse_status graph_build(ulisse_ctx* ctx, int s0_cols) {
   }
   ctx->step_graph = graph;
   CK(cudaGraphInstantiate(&ctx->step_exec, graph, 0));
+  CK(cudaMemcpyAsync(ctx->kv_launches_dev, ctx->kv_launches, sizeof(ctx->kv_launches),
+                     cudaMemcpyHostToDevice, ctx->stream));
   // what one launch does outside the CG loop (the loop's share is counted on the device)
-  const long long kmv_per = ctx->mixed ? 2 : 1, kmv_cols = ctx->mixed ? 64 : kMaxRChunk;
   const int init_cols = warm ? R : s0_cols;   // columns of the product K s_0
   // prescale, probes, the CG start, the gradient pass (+ its
   // operand images), the update, the learned start's two kernels, the product K s_0
   ctx->graph_launches_fixed = 1 + 1 + cg_init_launch_count(ctx->n, R, ctx->num_sms) +
       (ctx->mixed ? 2 : 1) + 1 + (s0_cols > 0 ? 2 : 0) +
-      (init_cols > 0 ? kmv_per * ((init_cols + kmv_cols - 1) / kmv_cols) : 0);
+      ctx->graph_init_launches;
   ctx->graph_entries_fixed = (double)ctx->n * (double)ctx->n * (double)(R + init_cols);
   ctx->graph_rounds_fixed = init_cols > 0 ? 1 : 0;
   ctx->graph_key = s0_cols;
@@ -1681,6 +1707,7 @@ static ulisse_status graph_alloc(ulisse_ctx* ctx) {
   CKS(dev_alloc(ctx, reinterpret_cast<void**>(&ctx->chain), sizeof(ChainSlot)));
   CKS(dev_alloc(ctx, reinterpret_cast<void**>(&ctx->gstat), sizeof(long long) * 4));
   CKS(dev_alloc(ctx, reinterpret_cast<void**>(&ctx->eps_one), sizeof(double)));
+  CKS(dev_alloc(ctx, reinterpret_cast<void**>(&ctx->kv_launches_dev), sizeof(ctx->kv_launches)));
   if (cudaMallocHost(&ctx->h_gstat, sizeof(long long) * 4) != cudaSuccess)
     return fail(ctx, ULISSE_ERR_NOMEM, "cudaMallocHost failed");
   return ULISSE_OK;
@@ -2093,7 +2120,7 @@ ulisse_status ulisse_create_batched(ulisse_ctx** out, int n_problems, const long
     sc.seed = cfg->seed + (unsigned long long)b;   // problem b draws from its own streams
     ulisse_ctx* sub = nullptr;
     const ulisse_status s = create_impl(&sub, X[b], y[b], n[b], d[b], &sc, stream,
-                                        cudaMemcpyDeviceToDevice);
+                                        cudaMemcpyDeviceToDevice, true);
     if (s != ULISSE_OK) {
       ctx->err = "problem " + std::to_string(b) + ": " + g_create_error;
       return bail(s);
@@ -2127,9 +2154,10 @@ ulisse_status ulisse_create_batched(ulisse_ctx** out, int n_problems, const long
       (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->b_g), sizeof(double) * kMaxP * n_problems)) ||
       (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->status_dev), sizeof(int))))
     return bail(s);
-  if (cfg->precision == ULISSE_PREC_MIXED) {
-    // tensor-core K V work list: per problem its 128-row blocks times a split of the j range
-    // into ranges of about kTcBatchTiles 32-point tiles; the longest ranges first
+  {
+    // tensor-core K V work list (mixed products; FP32 products from kF32TcMinR columns on): per
+    // problem its 128-row blocks times a split of the j range into ranges of about kTcBatchTiles
+    // 32-point tiles; the longest ranges first
     constexpr long long kTcBatchTiles = 256;
     std::vector<int4> tci;
     std::vector<std::pair<long long, int>> order;
@@ -2137,6 +2165,7 @@ ulisse_status ulisse_create_batched(ulisse_ctx** out, int n_problems, const long
     for (int b = 0; b < n_problems; ++b) {
       const long long nt = (n[b] + 31) / 32, nrb = (n[b] + 127) / 128;
       int ns = (int)std::min<long long>(64, (nt + kTcBatchTiles - 1) / kTcBatchTiles);
+      if (cfg->precision == ULISSE_PREC_FP32) ns = f3_nsplit(n[b], ctx->num_sms);
       const long long tps = (nt + ns - 1) / ns;
       ns = (int)((nt + tps - 1) / tps);
       ctx->b_tc_nsplit.push_back(ns);
@@ -2157,13 +2186,15 @@ ulisse_status ulisse_create_batched(ulisse_ctx** out, int n_problems, const long
         for (int sp = 0; sp < ctx->b_tc_nsplit[b]; ++sp) tci.push_back(make_int4(b, rb, sp, 0));
     }
     ctx->b_tc_n_items = (int)tci.size();
-    // gradient pass: per width group the (problem, row block, split) items, most tiles first
+    const bool mixed = cfg->precision == ULISSE_PREC_MIXED;
+    // gradient pass (mixed): per width group the (problem, row block, split) items, most tiles first
     // (row block rb visits the tiles [4 rb, ntiles): the symmetric pass)
     std::vector<int4> gti;
     size_t gpart = 0;
     ctx->b_gt_nsplit.assign(n_problems, 1);
     ctx->b_gt_part_off.assign(n_problems, 0);
     for (int dp : {2, 4, 8}) {
+      if (!mixed) break;
       std::vector<int> grp;
       for (int b = 0; b < n_problems; ++b)
         if ((d[b] <= 2 ? 2 : d[b] <= 4 ? 4 : 8) == dp) grp.push_back(b);
@@ -2194,19 +2225,25 @@ ulisse_status ulisse_create_batched(ulisse_ctx** out, int n_problems, const long
       ctx->b_gt_item_n.push_back((int)its.size());
       for (const auto& e : its) gti.push_back(e.second);
     }
+    size_t v3 = 0;
+    for (int b = 0; b < n_problems; ++b) {
+      ctx->b_v3_off.push_back(v3);
+      v3 += (size_t)((n[b] + 31) / 32) * 32 * 3 * kMaxRChunk * 2;
+    }
     if ((s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->b_tc_items), sizeof(int4) * tci.size())) ||
-        (s = dev_alloc(ctx, &ctx->b_tc_args, 3 * tc2_batch_args_bytes(n_problems))) ||
+        (s = dev_alloc(ctx, &ctx->b_tc_args,
+                       3 * (mixed ? tc2_batch_args_bytes(n_problems) : f3_batch_args_bytes(n_problems)))) ||
         (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->b_tc_part), sizeof(float) * std::max<size_t>(part, 1))) ||
         (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->b_tc_cnt), sizeof(int) * cnt)) ||
-        (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->b_gt_items), sizeof(int4) * gti.size())) ||
-        (s = dev_alloc(ctx, &ctx->b_gt_args, gt_batch_args_bytes(n_problems))) ||
-        (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->b_gt_part), sizeof(double) * gpart)) ||
-        (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->b_gt_cnt), sizeof(int) * n_problems)))
+        (!mixed && (s = dev_alloc(ctx, &ctx->b_v3, v3))) ||
+        (mixed &&
+         ((s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->b_gt_items), sizeof(int4) * gti.size())) ||
+          (s = dev_alloc(ctx, &ctx->b_gt_args, gt_batch_args_bytes(n_problems))) ||
+          (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->b_gt_part), sizeof(double) * gpart)) ||
+          (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->b_gt_cnt), sizeof(int) * n_problems)))))
       return bail(s);
-    if (cudaMemsetAsync(ctx->b_tc_cnt, 0, sizeof(int) * cnt, ctx->stream) != cudaSuccess ||
-        cudaMemsetAsync(ctx->b_gt_cnt, 0, sizeof(int) * n_problems, ctx->stream) != cudaSuccess ||
-        cudaMemcpyAsync(ctx->b_gt_items, gti.data(), sizeof(int4) * gti.size(),
-                        cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess ||
+    if ((mixed && cudaMemcpyAsync(ctx->b_gt_items, gti.data(), sizeof(int4) * gti.size(),
+                                  cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess) ||
         cudaMemcpyAsync(ctx->b_tc_items, tci.data(), sizeof(int4) * tci.size(),
                         cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess ||
         cudaStreamSynchronize(ctx->stream) != cudaSuccess) {
@@ -2321,17 +2358,44 @@ static ulisse_status batch_tc_upload(ulisse_ctx* ctx, int k, Fn cols) {
   return ULISSE_OK;
 }
 
-// One batched K V over all problems: the tensor-core launch (slot of its arguments) or the
-// persistent FP32 launch (its descriptor array), for at most r_max live columns.
+// Kernels of one batched K V for at most r_max live columns (packing, tensor cores, SIMT).
+static int batch_kv_launches(const ulisse_ctx* ctx, int r_max) {
+  if (ctx->cfg.precision == ULISSE_PREC_MIXED) return 2;
+  return r_max >= kF32TcMinR ? 3 : 1;
+}
+
+// One batched K V over all problems: the tensor-core launch (slot of its arguments) and, in
+// FP32, the persistent SIMT launch (its descriptor array), for at most r_max live columns.
 static cudaError_t batch_kv_launch(ulisse_ctx* ctx, int slot, BatchKmvDesc* desc, int r_max,
                                    cudaStream_t st) {
   const int B = (int)ctx->subs.size();
   if (ctx->cfg.precision == ULISSE_PREC_MIXED)
     return launch_kmv_tc2_batch((char*)ctx->b_tc_args + slot * tc2_batch_args_bytes(B), B,
                                 ctx->b_tc_items, ctx->b_tc_n_items, r_max, st);
+  // FP32: the tensor-core contraction takes the problems with enough live columns, the persistent
+  // SIMT launch the others
+  if (r_max >= kF32TcMinR) {
+    const cudaError_t e = launch_kmv_f32_tc_batch(
+        (char*)ctx->b_tc_args + slot * f3_batch_args_bytes(B), B, ctx->b_tc_items, ctx->b_tc_n_items,
+        kBatchWidths[batch_width_bucket(r_max)], st);
+    if (e != cudaSuccess) return e;
+  }
   return launch_kmv_batch(desc, ctx->b_items, ctx->b_n_items, ctx->b_queue,
                           kBatchWidths[batch_width_bucket(r_max)], ctx->num_sms,
                           ctx->status_dev, st);
+}
+
+// FP32: arguments of the tensor-core launches for the products described by desc, slot k.
+static ulisse_status batch_f3_upload(ulisse_ctx* ctx, int k, const std::vector<BatchKmvDesc>& desc) {
+  const int B = (int)ctx->subs.size();
+  std::vector<F3Problem> P((size_t)B);
+  for (int b = 0; b < B; ++b)
+    P[b] = F3Problem{desc[b], (char*)ctx->b_v3 + ctx->b_v3_off[b], ctx->b_tc_nsplit[b],
+                     ctx->b_tc_part + ctx->b_tc_part_off[b], ctx->b_tc_cnt + ctx->b_tc_cnt_off[b],
+                     ctx->status_dev};
+  CK(f3_batch_upload_args(P.data(), B, (char*)ctx->b_tc_args + k * f3_batch_args_bytes(B),
+                          ctx->stream));
+  return ULISSE_OK;
 }
 
 }  // extern "C++"
@@ -2376,7 +2440,7 @@ ulisse_status ulisse_batch_kmv(ulisse_ctx* ctx, const double* psi, const float* 
     if (mixed && !in_place)
       CK(cudaMemcpy2DAsync(sub->D, sub->ldn * 4, V[b], sub->n * 4, sub->n * 4, R,
                            cudaMemcpyDeviceToDevice, ctx->stream));
-    desc[b] = BatchKmvDesc{(const float*)sub->xhat, sub->n, sub->DP, 0, sub->params,
+    desc[b] = BatchKmvDesc{(const float*)sub->xhat, sub->n, sub->DP, 1, sub->params,
                            (const float*)sub->D, sub->ldn, sub->iota, U[b], sub->n,
                            sub->iota, ctx->b_rcount + b};
     entries += (double)sub->n * (double)sub->n * R;
@@ -2397,10 +2461,10 @@ ulisse_status ulisse_batch_kmv(ulisse_ctx* ctx, const double* psi, const float* 
                        ctx->stream));
     CK(cudaMemcpyAsync(ctx->b_rcount, rc.data(), sizeof(int) * B, cudaMemcpyHostToDevice,
                        ctx->stream));
-    CK(launch_kmv_batch(ctx->b_kdesc, ctx->b_items, ctx->b_n_items, ctx->b_queue, R,
-                        ctx->num_sms, ctx->status_dev, ctx->stream));
+    CKS(batch_f3_upload(ctx, 2, desc));
+    CK(batch_kv_launch(ctx, 2, ctx->b_kdesc, R, ctx->stream));
   }
-  ctx->launches++;
+  ctx->launches += batch_kv_launches(ctx, R);
   ctx->mvp_rounds++;
   ctx->entry_rhs += entries;
   int st = 0;
@@ -2482,11 +2546,11 @@ static ulisse_status batch_prepare(ulisse_ctx* ctx) {
     if (warm) a.warm_refresh = ctx->cfg.probe_refresh;
     args[b] = a;
     probs[b] = BatchCgProb{sub->st, sub->st_next, sub->live, sub->n_live_dev, R, sub->n};
-    kd[b] = BatchKmvDesc{(const float*)sub->xhat, sub->n, sub->DP, 0, sub->params,
+    kd[b] = BatchKmvDesc{(const float*)sub->xhat, sub->n, sub->DP, 1, sub->params,
                          (const float*)sub->D, sub->ldn, sub->live, (float*)sub->KD, sub->ldn,
                          sub->live, sub->n_live_dev};
     // K s_0 of warm-started solves: s_0 from Sbest (cap columns after S)
-    kd0[b] = BatchKmvDesc{(const float*)sub->xhat, sub->n, sub->DP, 0, sub->params,
+    kd0[b] = BatchKmvDesc{(const float*)sub->xhat, sub->n, sub->DP, 1, sub->params,
                           (const float*)sub->S, sub->ldn, sub->warm_map, (float*)sub->KD,
                           sub->ldn, sub->iota, ctx->b_rcount + b};
     const int nslots = (int)((sub->n + kBatchBM - 1) / kBatchBM);
@@ -2508,6 +2572,11 @@ static ulisse_status batch_prepare(ulisse_ctx* ctx) {
                      ctx->stream));
   CK(cudaMemcpyAsync(ctx->b_gdesc, gd.data(), sizeof(BatchGradDesc) * B, cudaMemcpyHostToDevice,
                      ctx->stream));
+  if (ctx->cfg.precision == ULISSE_PREC_FP32) {
+    CKS(batch_f3_upload(ctx, 0, kd));
+    CKS(batch_f3_upload(ctx, 1, kd0));
+    CK(launch_kmv_f32_tc_batch(nullptr, 0, nullptr, 0, 0, ctx->stream, true));
+  }
   if (ctx->cfg.precision == ULISSE_PREC_MIXED) {
     prime_kmv_tc2_batch();
     CKS(batch_tc_upload(ctx, 0, [](int, ulisse_ctx* sub, TcLaunch& l) {
@@ -2611,10 +2680,14 @@ static ulisse_status batch_step_body(ulisse_ctx* ctx, bool sgld, bool in_graph) 
                             s, (const CgArgs<float>*)ctx->b_cgargs);
   };
   const int max_rounds = ctx->cfg.max_iter + 2;
+  // K V kernels beyond the first, from how many live columns on (the counters')
+  const bool fp32 = ctx->cfg.precision == ULISSE_PREC_FP32;
+  const int tc_from = fp32 ? kF32TcMinR : 1, tc_launches = batch_kv_launches(ctx, 32) - 1;
   if (!in_graph) {
     for (int it = 0; it < max_rounds + 1; ++it) {
       compact_batch_kernel<<<1, kCompactBatchNT, 0, ctx->stream>>>(ctx->b_cgprob, B, ctx->b_rmax, 0, 0, 0,
-                                                       max_rounds, ctx->gstat, ctx->status_dev);
+                                                       max_rounds, tc_from, tc_launches, ctx->gstat,
+                                                       ctx->status_dev);
       CK(cudaGetLastError());
       CK(cudaMemcpyAsync(ctx->b_h_rmax, ctx->b_rmax, sizeof(int), cudaMemcpyDeviceToHost,
                          ctx->stream));
@@ -2647,7 +2720,8 @@ static ulisse_status batch_step_body(ulisse_ctx* ctx, bool sgld, bool in_graph) 
     CK(cudaStreamBeginCaptureToGraph(s2, body, nullptr, nullptr, 0,
                                      cudaStreamCaptureModeThreadLocal));
     compact_batch_kernel<<<1, kCompactBatchNT, 0, s2>>>(ctx->b_cgprob, B, ctx->b_rmax, 1, h_loop, h_branch,
-                                            max_rounds, ctx->gstat, ctx->status_dev);
+                                            max_rounds, tc_from, tc_launches, ctx->gstat,
+                                            ctx->status_dev);
     cudaError_t e = cudaGetLastError();
     const cudaGraphNode_t* bdeps = nullptr;
     size_t nbdeps = 0;
@@ -2735,7 +2809,7 @@ static void batch_count_fixed(ulisse_ctx* ctx, int steps, bool sgld) {
   long long init_launches = 0;   // the CG starts' (cg_init_launch_count) beyond one per problem
   for (ulisse_ctx* sub : ctx->subs) init_launches += cg_init_launch_count(sub->n, R, ctx->num_sms) - 1;
   ctx->launches += (long long)steps * (3LL * B + init_launches + grad_launches +
-                                       (sgld ? B + 1 : 0) + (warm ? (mixed ? 2 : 1) : 0));
+                                       (sgld ? B + 1 : 0) + (warm ? batch_kv_launches(ctx, R) : 0));
   ctx->entry_rhs += steps * ent * (warm ? 2.0 : 1.0);
   if (warm) ctx->mvp_rounds += steps;
 }
@@ -2747,8 +2821,6 @@ static ulisse_status batch_fold_gstat(ulisse_ctx* ctx) {
   ctx->mvp_rounds += ctx->h_gstat[0];
   ctx->entry_rhs += (double)ctx->h_gstat[1];
   ctx->launches += ctx->h_gstat[2];
-  // the device counts one K V launch per round; the mixed path also packs V each round
-  if (ctx->cfg.precision == ULISSE_PREC_MIXED) ctx->launches += ctx->h_gstat[0];
   CK(cudaMemsetAsync(ctx->gstat, 0, sizeof(long long) * 3, ctx->stream));
   return ULISSE_OK;
 }
@@ -2893,6 +2965,7 @@ static ulisse_status time_kmv_config(ulisse_ctx* ctx, int nl, int width, int tm,
     ctx->tune.resize((size_t)nl, ulisse_ctx::KmvTune{0, 0, 0, 0.f, 0.f, 0});
   const ulisse_ctx::KmvTune saved = ctx->tune[nl - 1];
   ctx->tune[nl - 1] = ulisse_ctx::KmvTune{width, tm, nsplit, 0.f, 0.f, cross};
+  ctx->simt = !ctx->mixed && width > 0;   // FP32: a given shape means the SIMT kernel
   ctx->planning = true;
   ulisse_status r = run_kmv(ctx, ctx->D, ctx->iota, nl, ctx->KD, ctx->iota, kModeK, -1);
   ctx->planning = false;
@@ -2919,6 +2992,7 @@ static ulisse_status time_kmv_config(ulisse_ctx* ctx, int nl, int width, int tm,
   if (a) cudaEventDestroy(a);
   if (b) cudaEventDestroy(b);
   ctx->tune[nl - 1] = saved;
+  ctx->simt = false;
   if (r != ULISSE_OK) return r;
   std::sort(t.begin(), t.end());
   *ms_out = t[t.size() / 2];
@@ -2971,7 +3045,9 @@ ulisse_status ulisse_autotune(ulisse_ctx* ctx, const double* psi, int max_cols, 
           int sp = 1;
           r = time_kmv_config(ctx, nl, wd, tm, 0, cr, reps, &ms, &sp);
           if (r != ULISSE_OK) break;
-          if (ms < best.ms) best = ulisse_ctx::KmvTune{wd, tm, 0, ms, ms_def, cr};
+          // FP32: an entry without a split count leaves the kernel to the dispatch (tensor
+          // cores or SIMT by size), so a SIMT winner carries its planned one
+          if (ms < best.ms) best = ulisse_ctx::KmvTune{wd, tm, ctx->mixed ? 0 : sp, ms, ms_def, cr};
         }
         if (r != ULISSE_OK) break;
       }
@@ -2992,7 +3068,8 @@ ulisse_status ulisse_autotune(ulisse_ctx* ctx, const double* psi, int max_cols, 
     }
     if (r != ULISSE_OK) break;
     if (best.width == 0) best.width = nl;
-    if (best.tm == 0) best.tm = ctx->cfg.kmv_rows_per_thread;
+    if (best.tm == 0) best.tm = ctx->mixed || ctx->cfg.kmv_rows_per_thread != 0
+                                    ? ctx->cfg.kmv_rows_per_thread : 2;
     table[nl - 1] = best;
   }
   ctx->prof = prof;
@@ -3098,7 +3175,7 @@ void ulisse_destroy(ulisse_ctx* ctx) {
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
   for (void** p : {reinterpret_cast<void**>(&ctx->st_next), reinterpret_cast<void**>(&ctx->part1),
                    reinterpret_cast<void**>(&ctx->part2), reinterpret_cast<void**>(&ctx->bneg),
-                   &ctx->Vt, &ctx->Gt,
+                   &ctx->Vt, &ctx->Gt, &ctx->v3, reinterpret_cast<void**>(&ctx->kv_launches_dev),
                    reinterpret_cast<void**>(&ctx->Xt_hi), reinterpret_cast<void**>(&ctx->Xt_lo),
                    reinterpret_cast<void**>(&ctx->Xt_b), reinterpret_cast<void**>(&ctx->exp_tab),
                    reinterpret_cast<void**>(&ctx->q_map), &ctx->q_sa, &ctx->pcg_buf, &ctx->pred_xs,
@@ -3137,7 +3214,7 @@ void ulisse_destroy(ulisse_ctx* ctx) {
                    reinterpret_cast<void**>(&ctx->b_gdesc), reinterpret_cast<void**>(&ctx->b_queue),
                    reinterpret_cast<void**>(&ctx->b_nlive), reinterpret_cast<void**>(&ctx->b_rcount),
                    reinterpret_cast<void**>(&ctx->b_gpart), reinterpret_cast<void**>(&ctx->b_g),
-                   reinterpret_cast<void**>(&ctx->b_tc_items), &ctx->b_tc_args,
+                   reinterpret_cast<void**>(&ctx->b_tc_items), &ctx->b_tc_args, &ctx->b_v3,
                    reinterpret_cast<void**>(&ctx->b_tc_part), reinterpret_cast<void**>(&ctx->b_tc_cnt),
                    reinterpret_cast<void**>(&ctx->b_gt_items), &ctx->b_gt_args,
                    reinterpret_cast<void**>(&ctx->b_gt_part), reinterpret_cast<void**>(&ctx->b_gt_cnt)})

@@ -30,7 +30,7 @@ struct BatchKmvDesc {
   const float* xhat;     // ldn x DP prescaled inputs (padding rows zero)
   long long n;
   int DP;
-  int pad0;
+  int tc;                // skip while f32_tc_columns holds (the tensor-core launch's)
   const DevParams* params;
   const float* V;        // column-major, leading dimension ldv (padding rows zero)
   long long ldv;
@@ -40,6 +40,24 @@ struct BatchKmvDesc {
   const int* umap;
   const int* nlive;      // live column count (device), 0 = skip the problem
 };
+
+// The same product by the tensor-core contraction (kmv_f32_tc.cu): its operand scratch (96 BF16
+// values per point, points rounded up to 32), the split of its j range, partial sums and counters.
+struct F3Problem {
+  BatchKmvDesc k;
+  void* v3;
+  int nsplit;
+  float* partials;
+  int* counters;
+  int* status;
+};
+int f3_nsplit(long long n, int num_sms);
+size_t f3_batch_args_bytes(int B);
+cudaError_t f3_batch_upload_args(const F3Problem* P, int B, void* args_dev, cudaStream_t s);
+// items: (problem, 128-row block, split) per CTA; R_max: the largest live column count.
+// prime_only: set the kernel attributes (ahead of a capture) and launch nothing.
+cudaError_t launch_kmv_f32_tc_batch(const void* args_dev, int B, const int4* items, int n_items,
+                                    int R_max, cudaStream_t s, bool prime_only = false);
 
 // Fused gradient for one problem (Eq. gradient:unbiased), as the single-problem pass.
 struct BatchGradDesc {

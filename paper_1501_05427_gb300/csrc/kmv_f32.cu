@@ -5,6 +5,7 @@ namespace ulisse {
 
 cudaError_t launch_kmv_f32(KmvLaunch& L, cudaStream_t s) {
   if (L.R < 1 || L.R > kMaxRChunk) return cudaErrorInvalidValue;
+  if (kmv_f32_tc_applies(L)) return launch_kmv_f32_tc(L, s);
   switch (L.DP) {
     case 2: return launch_kmv_f32_dp2(L, s);
     case 4: return launch_kmv_f32_dp4(L, s);

@@ -188,6 +188,7 @@ cudaError_t sym_launch(KmvLaunch& L, cudaStream_t s) {
   a.partials = static_cast<double*>(L.partials);
   const long long pairs = (long long)a.nb * (a.nb + 1) / 2;
   const size_t smem = sizeof(double) * (size_t)(T * (T + 1) + DP * T + 2 * L.R * T);
+  L.launches = 2;
   fn<<<(unsigned)pairs, NT, smem, s>>>(a);
   kmv_f64_sym_reduce_kernel<T, MODE>
       <<<dim3((unsigned)((4 * L.R * T + kSymRedNT - 1) / kSymRedNT), (unsigned)a.nb), kSymRedNT, 0, s>>>(a);

@@ -575,7 +575,7 @@ __host__ __device__ inline int batch_width_bucket(int r) {
 __global__ void __launch_bounds__(kCompactBatchNT) compact_batch_kernel(
     const BatchCgProb* __restrict__ probs, int B, int* __restrict__ rmax, int in_graph,
     cudaGraphConditionalHandle h_loop, cudaGraphConditionalHandle h_branch, int max_rounds,
-    long long* __restrict__ stat, int* __restrict__ status) {
+    int tc_from, int tc_launches, long long* __restrict__ stat, int* __restrict__ status) {
   constexpr int NW = kCompactBatchNT / 32;
   __shared__ int s_max[NW];
   __shared__ long long s_ent[NW];
@@ -611,7 +611,8 @@ __global__ void __launch_bounds__(kCompactBatchNT) compact_batch_kernel(
     if (mx > 0) {
       stat[0] += 1;
       stat[1] += ent;
-      stat[2] += 2;   // the batched K V and the batched CG iteration
+      // the batched K V, its tensor-core launches from tc_from columns on, the CG iteration
+      stat[2] += 2 + (mx >= tc_from ? tc_launches : 0);
     }
   }
   *rmax = mx;
@@ -717,8 +718,8 @@ __global__ void chain_advance_kernel(ChainSlot* __restrict__ cs) {
 __global__ void compact_graph_kernel(ColState* __restrict__ st, const ColState* __restrict__ st_next,
                                      int R, int* __restrict__ live, int* __restrict__ n_live,
                                      cudaGraphConditionalHandle h_loop,
-                                     cudaGraphConditionalHandle h_branch, int chunk_cols,
-                                     int launches_per_chunk, int launches_fixed, int max_rounds,
+                                     cudaGraphConditionalHandle h_branch,
+                                     const int* __restrict__ kv_launches, int max_rounds,
                                      long long* __restrict__ stat, int* __restrict__ status) {
   int k = commit_and_compact(st, st_next, R, *n_live, live);
   if (threadIdx.x != 0) return;
@@ -732,7 +733,7 @@ __global__ void compact_graph_kernel(ColState* __restrict__ st, const ColState* 
   if (k > 0) {
     stat[0] += 1;
     stat[1] += k;
-    stat[2] += launches_fixed + (long long)launches_per_chunk * ((k + chunk_cols - 1) / chunk_cols);
+    stat[2] += 1 + kv_launches[k - 1];   // the CG iteration, and the K V of k columns
   }
   cudaGraphSetConditional(h_loop, k > 0 ? 1u : 0u);
   cudaGraphSetConditional(h_branch, k > 0 ? (unsigned)(k - 1) : (unsigned)R);

@@ -222,10 +222,14 @@ struct KmvLaunch {
   int mode;              // KmvMode
   int which;             // dimension for kModeDLen
   const double* exp_tab; // FP64: the exponential's table (exp64.cuh)
+  void* v3;              // FP32: scratch of the tensor-core contraction's operand (kmv_f32_tc.cu),
+                         // 96 BF16 values per point (null: SIMT kernel)
+  bool simt;             // FP32: the SIMT kernel whatever the sizes
   int tm;                // rows per thread for K (0 = default)
   int r_min;             // compiled column count at least this (0: the smallest >= R)
   int nsplit;            // j-range split count (0: the launch plan's choice)
   int planned_nsplit;    // out: the split count used (or planned)
+  int launches;          // out: kernels launched (the caller sets 1)
   void* partials;        // split-j scratch
   size_t partials_bytes;
   int* counters;         // one per row block, zero between launches
@@ -318,6 +322,14 @@ cudaError_t launch_kmv_f32_dp4(KmvLaunch& L, cudaStream_t s);
 cudaError_t launch_kmv_f32_dp8(KmvLaunch& L, cudaStream_t s);
 cudaError_t launch_kmv_f32_dp16(KmvLaunch& L, cudaStream_t s);
 cudaError_t launch_kmv_f64(KmvLaunch& L, cudaStream_t s);
+// FP32 products with the contraction on the tensor cores (kmv_f32_tc.cu).
+constexpr long long kF32TcMinN = 256;
+constexpr int kF32TcMinR = 5;   // no problem takes this form below so many columns
+__host__ __device__ constexpr bool f32_tc_columns(long long n, int R) {
+  return n >= kF32TcMinN && R >= (n <= 10000 ? kF32TcMinR : 7);
+}
+bool kmv_f32_tc_applies(const KmvLaunch& L);
+cudaError_t launch_kmv_f32_tc(KmvLaunch& L, cudaStream_t s);
 bool kmv_f64_sym_applies(const KmvLaunch& L);
 cudaError_t launch_kmv_f64_sym(KmvLaunch& L, cudaStream_t s);
 cudaError_t launch_grad_f32(GradLaunch& L, cudaStream_t s);
