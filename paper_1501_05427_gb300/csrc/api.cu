@@ -43,6 +43,8 @@ struct ulisse_ctx {
   double* psi_dev = nullptr;  // kMaxP
   PsiArg psi_arg{};           // by_value: psi of a host call, handed to the next prescale launch
 
+  void* fixed_block = nullptr;   // the allocation of the buffers of fixed size
+  void* col_block = nullptr;     // ... and of the column buffers
   int cap = 0;                // column capacity of B, S, E, D, KD
   int cap_est = 0;            // column capacity of SE
   void *B = nullptr, *S = nullptr, *E = nullptr, *D = nullptr, *KD = nullptr, *SE = nullptr;
@@ -265,6 +267,32 @@ static ulisse_status dev_alloc(ulisse_ctx* ctx, void** p, size_t bytes) {
   return ULISSE_OK;
 }
 
+// Several buffers in one zeroed allocation, each on a 256-byte boundary (*block; the pointers lie
+// within it): an allocation costs tens of microseconds, whatever its size.
+struct Carve {
+  std::vector<std::pair<void**, size_t>> parts;
+  template <typename T>
+  void add(T*& p, size_t bytes) {
+    parts.push_back({reinterpret_cast<void**>(&p), bytes});
+  }
+};
+
+static size_t carve_round(size_t bytes) { return (bytes + 255) / 256 * 256; }
+
+static ulisse_status carve_alloc(ulisse_ctx* ctx, const Carve& c, void** block) {
+  size_t total = 0;
+  for (const auto& q : c.parts) total += carve_round(q.second);
+  for (const auto& q : c.parts) *q.first = nullptr;
+  const ulisse_status s = dev_alloc(ctx, block, total);
+  if (s != ULISSE_OK) return s;
+  char* at = static_cast<char*>(*block);
+  for (const auto& q : c.parts) {
+    *q.first = at;
+    at += carve_round(q.second);
+  }
+  return ULISSE_OK;
+}
+
 static void dev_free(void*& p) {
   if (p) cudaFree(p);
   p = nullptr;
@@ -276,34 +304,33 @@ static ulisse_status ensure_columns(ulisse_ctx* ctx, int R, int R_est) {
   ctx->graph_key = -1;   // a captured step graph holds the old buffers
   const int cap = std::max(R, ctx->cap), cap_est = std::max(R_est, ctx->cap_est);
   CK(cudaStreamSynchronize(ctx->stream));
-  for (void** p : {&ctx->B, &ctx->S, &ctx->E, &ctx->D, &ctx->KD, &ctx->SE}) dev_free(*p);
-  dev_free(reinterpret_cast<void*&>(ctx->st));
-  dev_free(reinterpret_cast<void*&>(ctx->st_next));
-  dev_free(reinterpret_cast<void*&>(ctx->part1));
-  dev_free(reinterpret_cast<void*&>(ctx->part2));
-  dev_free(reinterpret_cast<void*&>(ctx->live));
-  dev_free(reinterpret_cast<void*&>(ctx->iota));
-  dev_free(reinterpret_cast<void*&>(ctx->warm_map));
+  dev_free(ctx->col_block);
   const size_t col = (size_t)ctx->ldn * ctx->esz;
-  for (void** p : {&ctx->B, &ctx->E, &ctx->D, &ctx->KD})
-    CKS(dev_alloc(ctx, p, col * cap));
-  CKS(dev_alloc(ctx, &ctx->S, col * cap * 2));   // S, then Sbest
-  ctx->Sbest = (char*)ctx->S + col * cap;
-  CKS(dev_alloc(ctx, &ctx->SE, col * cap_est));
-  CKS(dev_alloc(ctx, reinterpret_cast<void**>(&ctx->st), sizeof(ColState) * cap));
-  CKS(dev_alloc(ctx, reinterpret_cast<void**>(&ctx->st_next), sizeof(ColState) * cap));
-  CKS(dev_alloc(ctx, reinterpret_cast<void**>(&ctx->part1), sizeof(double) * cap * kMaxCgChunks));
-  CKS(dev_alloc(ctx, reinterpret_cast<void**>(&ctx->part2), sizeof(double) * cap * kMaxCgChunks));
-  CKS(dev_alloc(ctx, reinterpret_cast<void**>(&ctx->live), sizeof(int) * cap));
   const int ni = std::max(cap, cap_est);
-  CKS(dev_alloc(ctx, reinterpret_cast<void**>(&ctx->iota), sizeof(int) * ni));
+  Carve cv;
+  cv.add(ctx->B, col * cap);
+  cv.add(ctx->E, col * cap);
+  cv.add(ctx->D, col * cap);
+  cv.add(ctx->KD, col * cap);
+  cv.add(ctx->S, col * cap * 2);   // S, then Sbest
+  cv.add(ctx->SE, col * cap_est);
+  cv.add(ctx->st, sizeof(ColState) * cap);
+  cv.add(ctx->st_next, sizeof(ColState) * cap);
+  cv.add(ctx->part1, sizeof(double) * cap * kMaxCgChunks);
+  cv.add(ctx->part2, sizeof(double) * cap * kMaxCgChunks);
+  cv.add(ctx->live, sizeof(int) * cap);
+  cv.add(ctx->iota, sizeof(int) * ni);
+  cv.add(ctx->warm_map, sizeof(int) * 2 * cap);
+  ctx->cap = ctx->cap_est = 0;   // until the buffers are there again
+  ctx->meta_grad_R = -1;         // the column metadata goes with them
+  CKS(carve_alloc(ctx, cv, &ctx->col_block));
+  ctx->Sbest = (char*)ctx->S + col * cap;
   std::vector<int> io(ni);
   for (int i = 0; i < ni; ++i) io[i] = i;
   CK(cudaMemcpyAsync(ctx->iota, io.data(), sizeof(int) * ni, cudaMemcpyHostToDevice,
                      ctx->stream));
   // warm-started solves read s_0 from Sbest (column cap + c); with the learned warm start
   // column 0 comes from S
-  CKS(dev_alloc(ctx, reinterpret_cast<void**>(&ctx->warm_map), sizeof(int) * 2 * cap));
   std::vector<int> wm(2 * cap);
   for (int c = 0; c < cap; ++c) wm[c] = wm[cap + c] = cap + c;
   wm[cap] = 0;
@@ -1049,42 +1076,37 @@ static ulisse_status create_impl(ulisse_ctx** out, const float* X, const float* 
     return bail(ULISSE_ERR_CUDA);
   }
   ulisse_status s;
-  if ((s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->X), sizeof(float) * n * d)) ||
-      (s = dev_alloc(ctx, &ctx->y, ctx->ldn * ctx->esz)) ||
-      (s = dev_alloc(ctx, &ctx->xhat, ctx->ldn * ctx->DP * ctx->esz)) ||
-      (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->params), sizeof(DevParams))) ||
-      (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->psi_dev), sizeof(double) * kMaxP)) ||
-      (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->n_live_dev), sizeof(int))) ||
-      (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->gcounter), sizeof(int))) ||
-      (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->g_dev), sizeof(double) * kMaxP)) ||
-      (s = dev_alloc(ctx, &ctx->sa_dev, sizeof(double) * kMaxM)) ||
-      (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->amap), sizeof(int) * kMaxM)) ||
-      (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->bmap), sizeof(int) * kMaxM)) ||
-      (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->M_dev), sizeof(double) * kMaxP * kMaxP)) ||
-      (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->prior_dev), sizeof(double) * kMaxP)) ||
-      (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->status_dev), sizeof(int))) ||
-      (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->warm_valid), sizeof(int))))
-    return bail(s);
+  Carve cv;
+  cv.add(ctx->X, sizeof(float) * n * d);
+  cv.add(ctx->y, ctx->ldn * ctx->esz);
+  cv.add(ctx->xhat, ctx->ldn * ctx->DP * ctx->esz);
+  cv.add(ctx->params, sizeof(DevParams));
+  cv.add(ctx->psi_dev, sizeof(double) * kMaxP);
+  cv.add(ctx->n_live_dev, sizeof(int));
+  cv.add(ctx->gcounter, sizeof(int));
+  cv.add(ctx->g_dev, sizeof(double) * kMaxP);
+  cv.add(ctx->sa_dev, sizeof(double) * kMaxM);
+  cv.add(ctx->amap, sizeof(int) * kMaxM);
+  cv.add(ctx->bmap, sizeof(int) * kMaxM);
+  cv.add(ctx->M_dev, sizeof(double) * kMaxP * kMaxP);
+  cv.add(ctx->prior_dev, sizeof(double) * kMaxP);
+  cv.add(ctx->status_dev, sizeof(int));
+  cv.add(ctx->warm_valid, sizeof(int));
   if (ctx->mixed) {
-    if ((s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->bneg), sizeof(float) * ctx->ld128)) ||
-        (s = dev_alloc(ctx, &ctx->Vt, 2 * 2 * ctx->ld128 * 64)) ||
-        (s = dev_alloc(ctx, &ctx->Gt, 2 * 2 * ctx->ld128 * kGtScratchRows)) ||
-        (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->Xt_hi), 4 * ctx->ld128 * 16)) ||
-        (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->Xt_lo), 4 * ctx->ld128 * 16)) ||
-        (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->Xt_b),
-                       4 * (ctx->ld128 / 32) * tc2_b_stride(16))))
-      return bail(s);
+    cv.add(ctx->bneg, sizeof(float) * ctx->ld128);
+    cv.add(ctx->Vt, 2 * 2 * ctx->ld128 * 64);
+    cv.add(ctx->Gt, 2 * 2 * ctx->ld128 * kGtScratchRows);
+    cv.add(ctx->Xt_hi, 4 * ctx->ld128 * 16);
+    cv.add(ctx->Xt_lo, 4 * ctx->ld128 * 16);
+    cv.add(ctx->Xt_b, 4 * (ctx->ld128 / 32) * tc2_b_stride(16));
   }
-  if (!ctx->f64 && !ctx->mixed && !in_batch && n >= kF32TcMinN &&
-      (s = dev_alloc(ctx, &ctx->v3, 2 * 3 * kMaxRChunk * ctx->ldn)))
-    return bail(s);
-  if (ctx->f64) {
-    if ((s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->exp_tab), sizeof(double) * kExpTabN)))
-      return bail(s);
-    if (launch_fill_exp_tab(ctx->exp_tab, ctx->stream) != cudaSuccess) {
-      ctx->err = "table launch failed";
-      return bail(ULISSE_ERR_CUDA);
-    }
+  if (!ctx->f64 && !ctx->mixed && !in_batch && n >= kF32TcMinN)
+    cv.add(ctx->v3, 2 * 3 * kMaxRChunk * ctx->ldn);
+  if (ctx->f64) cv.add(ctx->exp_tab, sizeof(double) * kExpTabN);
+  if ((s = carve_alloc(ctx, cv, &ctx->fixed_block))) return bail(s);
+  if (ctx->f64 && launch_fill_exp_tab(ctx->exp_tab, ctx->stream) != cudaSuccess) {
+    ctx->err = "table launch failed";
+    return bail(ULISSE_ERR_CUDA);
   }
   if (cudaMallocHost(&ctx->h_n_live, sizeof(int)) != cudaSuccess ||
       cudaMallocHost(&ctx->h_status, sizeof(int)) != cudaSuccess) {
@@ -1102,16 +1124,13 @@ static ulisse_status create_impl(ulisse_ctx** out, const float* X, const float* 
       return bail(ULISSE_ERR_CUDA);
     }
   } else {
-    float* tmp = nullptr;
-    if (cudaMalloc(&tmp, sizeof(float) * n) != cudaSuccess) {
-      ctx->err = "cudaMalloc failed";
-      return bail(ULISSE_ERR_NOMEM);
+    // by way of x^, which the first prescale writes
+    if (cudaMemcpyAsync(ctx->xhat, y, sizeof(float) * n, kind, ctx->stream) != cudaSuccess) {
+      ctx->err = "copy of y failed";
+      return bail(ULISSE_ERR_CUDA);
     }
-    cudaMemcpyAsync(tmp, y, sizeof(float) * n, kind, ctx->stream);
     convert_cols_kernel<float, double><<<dim3(64, 1), 256, 0, ctx->stream>>>(
-        tmp, n, (double*)ctx->y, ctx->ldn, n);
-    cudaStreamSynchronize(ctx->stream);
-    cudaFree(tmp);
+        (const float*)ctx->xhat, n, (double*)ctx->y, ctx->ldn, n);
   }
   if ((s = ensure_columns(ctx, 1 + cfg->n_probes, 2 + cfg->n_probes))) return bail(s);
   if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) {
@@ -3173,27 +3192,14 @@ const char* ulisse_last_error(const ulisse_ctx* ctx) {
 void ulisse_destroy(ulisse_ctx* ctx) {
   if (!ctx) return;
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
-  for (void** p : {reinterpret_cast<void**>(&ctx->st_next), reinterpret_cast<void**>(&ctx->part1),
-                   reinterpret_cast<void**>(&ctx->part2), reinterpret_cast<void**>(&ctx->bneg),
-                   &ctx->Vt, &ctx->Gt, &ctx->v3, reinterpret_cast<void**>(&ctx->kv_launches_dev),
-                   reinterpret_cast<void**>(&ctx->Xt_hi), reinterpret_cast<void**>(&ctx->Xt_lo),
-                   reinterpret_cast<void**>(&ctx->Xt_b), reinterpret_cast<void**>(&ctx->exp_tab),
+  for (void** p : {&ctx->fixed_block, &ctx->col_block,
+                   reinterpret_cast<void**>(&ctx->kv_launches_dev),
                    reinterpret_cast<void**>(&ctx->q_map), &ctx->q_sa, &ctx->pcg_buf, &ctx->pred_xs,
-                   reinterpret_cast<void**>(&ctx->pcg_aux), reinterpret_cast<void**>(&ctx->pcg_live)})
-    dev_free(*p);
-  for (void** p : {reinterpret_cast<void**>(&ctx->X), &ctx->y, &ctx->xhat,
-                   reinterpret_cast<void**>(&ctx->params), reinterpret_cast<void**>(&ctx->psi_dev),
-                   &ctx->B, &ctx->S, &ctx->E, &ctx->D, &ctx->KD, &ctx->SE,
-                   reinterpret_cast<void**>(&ctx->st), reinterpret_cast<void**>(&ctx->live),
-                   reinterpret_cast<void**>(&ctx->n_live_dev), reinterpret_cast<void**>(&ctx->iota),
+                   reinterpret_cast<void**>(&ctx->pcg_aux), reinterpret_cast<void**>(&ctx->pcg_live),
                    &ctx->partials, reinterpret_cast<void**>(&ctx->counters),
-                   reinterpret_cast<void**>(&ctx->gpart), reinterpret_cast<void**>(&ctx->gcounter),
-                   reinterpret_cast<void**>(&ctx->g_dev), &ctx->sa_dev,
-                   reinterpret_cast<void**>(&ctx->amap), reinterpret_cast<void**>(&ctx->bmap),
-                   reinterpret_cast<void**>(&ctx->M_dev), reinterpret_cast<void**>(&ctx->prior_dev),
-                   reinterpret_cast<void**>(&ctx->status_dev),
-                   reinterpret_cast<void**>(&ctx->warm_valid)})
+                   reinterpret_cast<void**>(&ctx->gpart)})
     dev_free(*p);
+  if (ctx->batched) dev_free(reinterpret_cast<void*&>(ctx->status_dev));   // its own allocation
   for (void* p : ctx->ws_allocs) cudaFree(p);
   ctx->ws_allocs.clear();
   for (ulisse_ctx* sub : ctx->subs) ulisse_destroy(sub);

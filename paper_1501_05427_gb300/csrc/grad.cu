@@ -217,12 +217,9 @@ __global__ void __launch_bounds__(NT) grad_kernel(const GradDevArgs<T> a) {
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  if (tid < a.d + 2) {
-    double v = 0.0;
-    for (unsigned b = 0; b < gridDim.x; ++b) v += __ldcg(a.partials + (long long)b * kMaxP + tid);
-    if (tid == a.d + 1) v *= a.params->lambda;
-    a.g_out[tid] = v;
-  }
+  __shared__ double s_sum[NT];
+  const double v = sum_partial_rows<NT>(a.partials, (int)gridDim.x, a.d + 2, s_sum);
+  if (tid < a.d + 2) a.g_out[tid] = tid == a.d + 1 ? v * a.params->lambda : v;
   if (tid == 0) *a.counter = 0;
 }
 

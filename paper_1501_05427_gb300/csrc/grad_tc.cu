@@ -226,7 +226,7 @@ __device__ __forceinline__ void gt_body(const GtDevArgs& a, const int rb, const 
   constexpr int ST = S::ST, K1 = S::K1, N2 = S::N2;
   constexpr int NACC = DP + 2;
   extern __shared__ __align__(1024) unsigned char smem[];
-  __shared__ double s_red[4 * kGtSets][NACC];
+  __shared__ double s_red[4][NACC];
   unsigned char* sAh = smem;
   unsigned char* sAl = smem + S::A_BYTES;
   const uint32_t smem0 = smem_u32(smem);
@@ -563,18 +563,22 @@ __device__ __forceinline__ void gt_body(const GtDevArgs& a, const int rb, const 
     }
     return;
   }
-  if (warp >= 1) {
+  // set 0 holds the lengthscale and sigma^2 sums, set 1 the diagonal's
+  if (warp >= 1 && warp <= 4) {
 #pragma unroll
-    for (int k = 0; k < NACC; ++k) {
+    for (int k = 0; k <= DP; ++k) {
       const double v = warp_sum(acc[k]);
       if (lane == 0) s_red[warp - 1][k] = v;
     }
+  } else if (warp >= 5 && warp <= 8) {
+    const double v = sp == 0 ? warp_sum(acc[DP + 1]) : 0.0;
+    if (lane == 0) s_red[warp - 5][DP + 1] = v;
   }
   __syncthreads();
   double* part = a.partials + slot * kMaxP;
   if (tid < NACC) {
     double v = 0.0;
-    for (int ww = 0; ww < 4 * kGtSets; ++ww) v += s_red[ww][tid];
+    for (int ww = 0; ww < 4; ++ww) v += s_red[ww][tid];
     // slots: lengthscales 0..d-1, then sigma^2 at d, lambda at d+1
     if (tid < a.d) part[tid] = v;
     else if (tid == DP) part[a.d] = v;
@@ -586,12 +590,9 @@ __device__ __forceinline__ void gt_body(const GtDevArgs& a, const int rb, const 
   __syncthreads();
   if (!*s_last) return;
   __threadfence();
-  if (tid < a.d + 2) {
-    double v = 0.0;
-    for (int b = 0; b < a.n_cta; ++b) v += __ldcg(a.partials + (long long)b * kMaxP + tid);
-    if (tid == a.d + 1) v *= a.params->lambda;
-    a.g_out[tid] = v;
-  }
+  __shared__ double s_sum[kGtThreads];
+  const double v = sum_partial_rows<kGtThreads>(a.partials, a.n_cta, a.d + 2, s_sum);
+  if (tid < a.d + 2) a.g_out[tid] = tid == a.d + 1 ? v * a.params->lambda : v;
   if (tid == 0) *a.counter = 0;
 }
 

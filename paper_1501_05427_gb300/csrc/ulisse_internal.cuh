@@ -197,6 +197,42 @@ __device__ inline double block_sum(double v, double* scratch /* >= NT/32 */) {
   return t;
 }
 
+// Sums over `count` rows of partial sums (kMaxP doubles each, the first `comps` in use), by a whole
+// CTA of NT threads in a fixed order; the sum of component k is returned to thread k < comps (the
+// others get 0).  red: NT doubles of shared memory.  Every thread takes a component of every
+// (NT / comps)th row, eight loads in flight: with one thread per component walking all rows (an
+// L2 round trip and a 64-clock FP64 add each) the last CTA of a gradient pass held up its end by
+// 100 us for 1,000 rows.
+template <int NT>
+__device__ inline double sum_partial_rows(const double* __restrict__ part, int count, int comps,
+                                          double* red) {
+  const int tid = threadIdx.x;
+  const int S = NT / comps, s = tid / comps, k = tid - s * comps;
+  double v = 0.0;
+  if (s < S)
+    for (int b = s; b < count; b += 8 * S) {
+      double x[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        x[q] = b + q * S < count ? __ldcg(part + (long long)(b + q * S) * kMaxP + k) : 0.0;
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        if (b + q * S < count) v += x[q];
+    }
+  red[tid] = v;
+  __syncthreads();
+  // the S sums of a component in four quarters, then the quarters
+  v = 0.0;
+  const int per = (S + 3) / 4;
+  if (tid < 4 * comps)
+    for (int q = s * per; q < min(S, (s + 1) * per); ++q) v += red[q * comps + k];
+  __syncthreads();
+  red[tid] = v;
+  __syncthreads();
+  if (tid >= comps) return 0.0;
+  return (red[tid] + red[comps + tid]) + (red[2 * comps + tid] + red[3 * comps + tid]);
+}
+
 // ------------------------------------------------------------------------------------
 // Launch descriptors.
 // ------------------------------------------------------------------------------------
