@@ -105,6 +105,7 @@ struct ulisse_ctx {
 
   // CUDA graph of one SGLD step (ulisse_sgld_chain)
   bool simt = false;          // FP32 products by the SIMT kernel (the autotuner's candidates)
+  bool v_packed = false;      // the prescale launch packed the coming product's operand
   bool planning = false;      // launch helpers only size their scratch
   bool capturing = false;     // launch helpers are being captured: no host-side counting
   long long cap_launches = 0; // ... but of the K V launches captured
@@ -365,23 +366,23 @@ static ulisse_status psi_to_device(ulisse_ctx* ctx) {
   return ULISSE_OK;
 }
 
-// The prescale launch (a1); TV columns of V (leading dimension n, may be null) are copied into D
-// by the same launch (FP32 and FP64 contexts).
+// The prescale launch (a1); R columns of V (leading dimension n, may be null) are copied into D by
+// the same launch (FP32 and FP64 contexts), or the operand pv of a tensor-core product is packed.
 template <typename TV>
-static ulisse_status prescale_and_copy(ulisse_ctx* ctx, const TV* V, int R) {
+static ulisse_status prescale_and_copy(ulisse_ctx* ctx, const TV* V, int R, PackV pv = PackV{}) {
   PsiArg pa = ctx->psi_arg;
   if (ctx->capturing) pa.by_value = 0;   // a captured step reads psi_dev
   if (ctx->mixed)
     CK(launch_prescale_mixed(pa, ctx->psi_dev, ctx->X, (float*)ctx->xhat, ctx->n, ctx->ld128, ctx->d,
                              ctx->DP, !ctx->tc_no_aug, ctx->params, ctx->bneg, ctx->Xt_hi,
-                             ctx->Xt_lo, ctx->Xt_b, ctx->num_sms, ctx->stream));
+                             ctx->Xt_lo, ctx->Xt_b, pv, ctx->num_sms, ctx->stream));
   else if (ctx->f64)
     CK((launch_prescale<double, TV>(pa, ctx->psi_dev, ctx->X, (double*)ctx->xhat, ctx->n, ctx->d,
-                                    ctx->DP, ctx->params, V, (double*)ctx->D, ctx->ldn, R,
+                                    ctx->DP, ctx->params, V, (double*)ctx->D, ctx->ldn, R, pv,
                                     ctx->num_sms, ctx->stream)));
   else
     CK((launch_prescale<float, TV>(pa, ctx->psi_dev, ctx->X, (float*)ctx->xhat, ctx->n, ctx->d,
-                                   ctx->DP, ctx->params, V, (float*)ctx->D, ctx->ldn, R,
+                                   ctx->DP, ctx->params, V, (float*)ctx->D, ctx->ldn, R, pv,
                                    ctx->num_sms, ctx->stream)));
   ctx->psi_arg.by_value = 0;
   if (!ctx->capturing) ctx->launches++;
@@ -421,6 +422,7 @@ static ulisse_status run_kmv_tc(ulisse_ctx* ctx, const void* V, const int* vmap,
     L.xhat = (const float*)ctx->xhat;
     L.bneg = ctx->bneg;
     L.Vp = ctx->Vt;
+    L.v_packed = ctx->v_packed;
     L.V = V;
     L.ldv = ldv;
     L.vmap = vmap + c0;
@@ -471,7 +473,7 @@ static ulisse_status run_kmv_tc(ulisse_ctx* ctx, const void* V, const int* vmap,
           ctx->free_events.push_back({ea, eb});
       }
       if (e == cudaSuccess) {
-        (ctx->capturing ? ctx->cap_launches : ctx->launches) += 2;   // the packing of V first
+        (ctx->capturing ? ctx->cap_launches : ctx->launches) += L.v_packed ? 1 : 2;   // packing V
         break;
       }
       if (e != cudaErrorMemoryAllocation || attempt == 1 || ctx->capturing)
@@ -511,6 +513,7 @@ static ulisse_status run_kmv(ulisse_ctx* ctx, const void* V, const int* vmap, in
     L.exp_tab = ctx->exp_tab;
     L.v3 = ctx->v3;
     L.simt = ctx->simt || ctx->cfg.kmv_rows_per_thread != 0;
+    L.v_packed = ctx->v_packed;
     L.mode = mode;
     L.which = which;
     L.tm = ctx->cfg.kmv_rows_per_thread;
@@ -1236,8 +1239,17 @@ static ulisse_status kmv_common(ulisse_ctx* ctx, const double* psi, int which, c
     }
   }
   const bool in_place = reads_direct && !overlap;
+  // One launch of at most 32 (mixed: 64) columns: its operand is packed by the prescale launch.
+  PackV pv{};
+  if (in_place && !ctx->f64 && ctx->tune.empty() && R <= (ctx->mixed ? 64 : kMaxRChunk)) {
+    pv.V = (const float*)V;
+    pv.R = R;
+    pv.N = R <= 16 ? 16 : R <= 32 ? 32 : 64;
+    pv.Vp = ctx->mixed ? ctx->Vt : ctx->v3;
+  }
+  ctx->v_packed = pv.V != nullptr;
   if (in_place) {
-    CKS(prescale(ctx));
+    CKS(prescale_and_copy<float>(ctx, nullptr, 0, pv));
   } else if (ctx->mixed) {   // (its prescale copies nothing)
     CKS(prescale(ctx));
     CK(cudaMemcpy2DAsync(ctx->D, ctx->ldn * 4, V, n * 4, n * 4, R, cudaMemcpyDeviceToDevice,
@@ -1248,8 +1260,10 @@ static ulisse_status kmv_common(ulisse_ctx* ctx, const double* psi, int which, c
     CKS(prescale_and_copy(ctx, (const float*)V, R));
   }
   const bool out_direct = ctx->esz == ue;
-  CKS(run_kmv(ctx, in_place ? V : ctx->D, ctx->iota, R, out_direct ? U : ctx->KD, ctx->iota, mode, w,
-              in_place ? n : 0, out_direct ? n : 0));
+  const ulisse_status kv = run_kmv(ctx, in_place ? V : ctx->D, ctx->iota, R, out_direct ? U : ctx->KD,
+                                   ctx->iota, mode, w, in_place ? n : 0, out_direct ? n : 0);
+  ctx->v_packed = false;
+  CKS(kv);
   if (!out_direct) {
     convert_cols_kernel<double, float><<<dim3(64, R), 256, 0, ctx->stream>>>(
         (const double*)ctx->KD, ctx->ldn, (float*)U, n, n);

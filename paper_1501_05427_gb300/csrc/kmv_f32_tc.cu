@@ -30,6 +30,7 @@
 
 #include "batch.cuh"
 #include "kmv_kernel.cuh"
+#include "pack_v.cuh"
 #include "tc_common.cuh"
 
 namespace ulisse {
@@ -87,36 +88,10 @@ struct F3Shape {
   static_assert(2 * (SMEM + 2048) <= 228 * 1024, "two CTAs per SM");
 };
 
-// V columns vmap[0..R) -> the three BF16 parts, a K-major canonical image of N rows (right-hand
-// sides) x 32 points each, back to back per tile; rows r >= R and points >= n are zero.  A value
-// that is not finite keeps it in the high part.
-__device__ inline void pack_v3(const float* __restrict__ V, long long ldv,
-                               const int* __restrict__ vmap, int R, int N, long long n,
-                               long long ntiles, __nv_bfloat16* __restrict__ Vp) {
-  const int per = N * kF3BN;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < ntiles * per;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const long long t = idx / per;
-    const int rem = (int)(idx - t * per);
-    const int r = rem / kF3BN, jj = rem - r * kF3BN;
-    const long long j = t * kF3BN + jj;
-    const float v = (r < R && j < n) ? V[(long long)vmap[r] * ldv + j] : 0.f;
-    const __nv_bfloat16 h = __float2bfloat16_rn(v);
-    const bool split = isfinite(__bfloat162float(h));
-    const float v1 = split ? v - __bfloat162float(h) : 0.f;
-    const __nv_bfloat16 m = __float2bfloat16_rn(v1);
-    const __nv_bfloat16 l = __float2bfloat16_rn(v1 - __bfloat162float(m));
-    __nv_bfloat16* o = Vp + t * 3LL * per + tc::canon_offset(r, jj, 2, kF3BN / 8) / 2;
-    o[0] = h;
-    o[per] = m;
-    o[2 * per] = l;
-  }
-}
-
 __global__ void pack_v3_kernel(const float* __restrict__ V, long long ldv,
                                const int* __restrict__ vmap, int R, int N, long long n,
                                long long ntiles, __nv_bfloat16* __restrict__ Vp) {
-  pack_v3(V, ldv, vmap, R, N, n, ntiles, Vp);
+  pack_v3(V, ldv, vmap, R, N, n, ntiles, Vp, blockIdx.x, gridDim.x);
 }
 
 // One problem per grid row; problems below the line are the SIMT launch's.
@@ -124,7 +99,8 @@ __global__ void pack_v3_batch_kernel(const F3Args* __restrict__ args, int N) {
   const F3Args& a = args[blockIdx.y];
   const int R = a.R_dev ? *a.R_dev : a.R;
   if (!f32_tc_columns(a.n, R)) return;
-  pack_v3(a.V, a.ldv, a.vmap, R, N, a.n, a.ntiles, const_cast<__nv_bfloat16*>(a.Vp));
+  pack_v3(a.V, a.ldv, a.vmap, R, N, a.n, a.ntiles, const_cast<__nv_bfloat16*>(a.Vp), blockIdx.x,
+          gridDim.x);
 }
 
 // Kernel values (j, j + 1) of a row against two points of the tile: xj points at point j.
@@ -456,7 +432,7 @@ cudaError_t f3_launch(KmvLaunch& L, cudaStream_t s) {
     cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   });
   __nv_bfloat16* Vp = static_cast<__nv_bfloat16*>(L.v3);
-  {
+  if (!L.v_packed) {
     const long long total = ntiles * N * kF3BN;
     const int blocks = (int)std::min<long long>((total + 255) / 256, 8LL * L.num_sms);
     pack_v3_kernel<<<blocks, 256, 0, s>>>(static_cast<const float*>(L.V), L.ldv, L.vmap, L.R, N,
@@ -484,7 +460,7 @@ cudaError_t f3_launch(KmvLaunch& L, cudaStream_t s) {
   a.partials = static_cast<float*>(L.partials);
   a.counters = L.counters;
   a.status = L.status;
-  L.launches = 2;
+  L.launches = L.v_packed ? 1 : 2;
   fn<<<p.n_rb * a.nsplit, kF3Threads, S::SMEM, s>>>(a);
   return cudaGetLastError();
 }

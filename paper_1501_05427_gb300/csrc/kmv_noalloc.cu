@@ -147,7 +147,7 @@ extern "C" ulisse_status ulisse_kmv_noalloc(const float* X, long long n, int d, 
   for (int i = 0; i < d + 2; ++i) pa.v[i] = psi[i];
   pa.by_value = 1;
   if ((st = ck(launch_prescale<float, float>(pa, psi_dev, X, xhat, n, d, DP, params, V, Vpad, ldn, R,
-                                             sc->num_sms, s),
+                                             PackV{}, sc->num_sms, s),
                "prescale launch failed")) != ULISSE_OK)
     return st;
 

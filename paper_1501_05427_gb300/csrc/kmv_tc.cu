@@ -24,6 +24,7 @@
 #include <mutex>
 
 #include "kmv_kernel.cuh"
+#include "pack_v.cuh"
 #include "tc_common.cuh"
 
 namespace ulisse {
@@ -36,26 +37,10 @@ constexpr uint32_t kTcCols = 128;  // tensor-memory columns per CTA (layout in T
 // ------------------------------------------------------------------------------------
 // Operand preparation
 // ------------------------------------------------------------------------------------
-// V columns vmap[0..R) -> BF16 high and low parts, a K-major canonical image of N rows
-// (right-hand sides) x 32 points each, back to back per j-tile (one bulk copy); rows r >= R and
-// points >= n are zero.
 __global__ void pack_v_kernel(const float* __restrict__ V, long long ldv,
                               const int* __restrict__ vmap, int R, int N, long long n,
                               long long ntiles, __nv_bfloat16* __restrict__ Vp) {
-  const long long per_tile = (long long)N * kTcBN;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < ntiles * per_tile;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const long long t = idx / per_tile;
-    const int rem = (int)(idx - t * per_tile);
-    const int r = rem / kTcBN, jj = rem - r * kTcBN;
-    const long long j = t * kTcBN + jj;
-    const float v = (r < R && j < n) ? V[(long long)vmap[r] * ldv + j] : 0.f;
-    const __nv_bfloat16 h = __float2bfloat16_rn(v);
-    const __nv_bfloat16 l = __float2bfloat16_rn(v - __bfloat162float(h));
-    const long long off = t * 2 * per_tile + tc::canon_offset(r, jj, 2, kTcBN / 8) / 2;
-    Vp[off] = h;
-    Vp[off + per_tile] = l;
-  }
+  pack_v2(V, ldv, vmap, R, N, n, ntiles, Vp, blockIdx.x, gridDim.x);
 }
 
 // ------------------------------------------------------------------------------------
@@ -379,7 +364,7 @@ struct TcInst {
       return cudaErrorMemoryAllocation;
     }
     const long long ntiles = (L.n + kTcBN - 1) / kTcBN;
-    launch_pack_v(L, N, ntiles, s);
+    if (!L.v_packed) launch_pack_v(L, N, ntiles, s);
     TcDevArgs a;
     a.xhat = L.xhat;
     a.bneg = L.bneg;

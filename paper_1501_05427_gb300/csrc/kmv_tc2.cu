@@ -17,26 +17,30 @@
 //      store them over C's own columns (tcgen05.st);
 //   3. U_I += K_IJ V_J on the tensor cores with V split into BF16 high + low parts (three
 //      products), FP32 accumulation in tensor memory, as in the FP32-pipe variant.
-// The TF32 images of A and B (high and low parts, K-major canonical, 32-point tiles back to
-// back so that four tiles form the 128-row A operand) are written once per parameter value by
-// pack_x_tf32_kernel; B's tiles and V's tiles each lie contiguously with all their parts, so
-// that a tile is two bulk copies.  Roles: warp 0 copies (the A image once, then B_J, b_J and
-// V_J into a ring of 3 to 8 stages) and issues the MMAs; eight epilogue warps make the kernel
-// values, in two sets of four (one per tensor-memory lane quadrant) that take alternate tiles
-// whole, so that each wait and hand-off covers 32 entries per thread.  Three C/K buffers (two
-// when the accumulator takes 64 columns); a buffer is refilled only after the MMAs that read it
-// have completed, and the stage of that tile is refilled at the same moment, so the copies need
-// no barrier and no warp of their own.  Every wait is bounded.  The split j range, the
-// fixed-order fix-up of the partial sums and the FP32 diagonal term lambda V are those of the
-// FP32-pipe variant.
+// The TF32 images of A and B (high and low parts, K-major canonical, 32-point tiles) are written
+// once per parameter value by the prescale launch; B's tiles and V's tiles each lie contiguously
+// with all their parts, so that a unit of tiles is two bulk copies.  A_I goes into tensor memory
+// once per CTA, and every MMA reads its A operand there (from shared memory the 4 KB take 40 clocks
+// per MMA, against 16 for the product itself at N = 32).  Roles: warp 0 copies (B_J, b_J and V_J
+// into a ring of stages) and issues the exponent's MMAs; warp 1 issues the contraction's; the
+// epilogue warps make the kernel values in sets of four (one per tensor-memory lane quadrant).  A
+// set takes a unit of G consecutive tiles whole, so that each wait and hand-off covers 32 G
+// entries per thread: three sets and units of two tiles up to N = 32, four sets and units of one
+// where the accumulator takes 64 columns.  A buffer is refilled only after the MMAs that read it
+// have completed, and the stage of that unit is refilled at the same moment.  Every wait is
+// bounded.  The split j range, the fixed-order fix-up of the partial sums and the FP32 diagonal
+// term lambda V are those of the FP32-pipe variant.
 //
-// What bounds it: the issue slots of the epilogue's instruction stream and, next to them, the
-// chain C -> epilogue -> contraction -> refill, whose middle is one warp's instructions.  That
-// warp runs its loop warp-uniformly and elects a lane only for the issuing instructions: the
-// descriptors then live in uniform registers.  With a separate copying warp and one divergent
-// lane issuing (moving every descriptor to uniform registers per MMA) a product at n = 50,000,
-// d = 8, 17 columns took 1.046 ms; nine warps instead of ten also raise the register budget from
-// 48 to 56, so that the high and low parts get registers of their own.  Now 0.78 ms.
+// What bounds it: the epilogue's issue slots (ncu at n = 50,000, d = 8, N = 32: 7.6 thread
+// instructions per entry, schedulers 77% busy), at N = 64 the tensor pipe (74% busy).  The issuing
+// warps come next: a tile takes about a hundred of their instructions, which wait their turn
+// among the epilogue's.  Times of the kernel at n = 50,000, d = 8, 17 columns: 1.046 ms with a
+// copying warp and one divergent lane issuing for four CTAs of eight epilogue warps per SM; 0.777
+// ms with one warp-uniform warp doing both (a lane elected for the issuing instructions keeps the
+// descriptors in uniform registers; 56 registers instead of 48); 0.677 ms with A in tensor memory,
+// two CTAs of twelve epilogue warps per SM, units of two tiles and the two issuing warps (with
+// one: 0.75 ms; units of one tile and four sets: 0.77 ms).  n = 200,000, d = 16, 64 columns: 19.2,
+// 15.6 and 14.6 ms per call.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -44,6 +48,7 @@
 #include <vector>
 
 #include "kmv_kernel.cuh"
+#include "pack_v.cuh"
 #include "prescale.cuh"
 #include "tc_common.cuh"
 
@@ -51,8 +56,7 @@ namespace ulisse {
 
 constexpr int kT2BN = 32;
 constexpr int kT2BM = 128;
-constexpr int kT2Threads = 288;    // warp 0 copies and MMAs, warps 1-8 epilogue
-constexpr uint32_t kT2Cols = 128;  // tensor-memory columns per CTA
+constexpr uint32_t kT2Cols = 256;  // tensor-memory columns per CTA (two CTAs per SM)
 
 // The prescale of the mixed path, one row per thread: x^_j, the row norm b_j = -c1 |x^_j|^2
 // (summed in FP64), and the rows A_j = [x^_j, 1, 0...] and B_j = [2 c1 x^_j, b_j, 0...] as TF32
@@ -67,12 +71,17 @@ __global__ void __launch_bounds__(128) prescale_mixed_kernel(
     const PsiArg pa, double* __restrict__ psi_dev, const float* __restrict__ X,
     float* __restrict__ xhat, long long n, long long rows, int d, int aug,
     DevParams* __restrict__ P, float* __restrict__ bneg, float* __restrict__ Ahi,
-    float* __restrict__ Alo, float* __restrict__ Bt) {
+    float* __restrict__ Alo, float* __restrict__ Bt, const PackV pv) {
   constexpr int K8 = DP >= 8 ? DP : 8;
   __shared__ InvLength s;
+  if ((int)blockIdx.x >= pv.first_cta) {   // a product's operand rides along
+    pack_v2(pv.V, n, nullptr, pv.R, pv.N, n, (n + kT2BN - 1) / kT2BN,
+            static_cast<__nv_bfloat16*>(pv.Vp), blockIdx.x - pv.first_cta, gridDim.x - pv.first_cta);
+    return;
+  }
   unpack_params(pa, psi_dev, d, P, s);
   const float two_c1 = 2.f * (float)(0.5 * 1.4426950408889634);   // 2 c1f
-  for (long long j = blockIdx.x * 128LL + threadIdx.x; j < rows; j += gridDim.x * 128LL) {
+  for (long long j = blockIdx.x * 128LL + threadIdx.x; j < rows; j += pv.first_cta * 128LL) {
     float x[K8];
     double s2 = 0.0;
 #pragma unroll
@@ -146,32 +155,35 @@ struct Tc2DevArgs {
 // BJ: the epilogue adds b_j (the rows are not augmented); the stage then carries b_J.
 template <int K8, int N, bool BJ>
 struct Tc2Shape {
-  static constexpr uint32_t A_BYTES = kT2BM * K8 * 4;   // one part of the A_I image
-  static constexpr uint32_t XB_BYTES = kT2BN * K8 * 4;  // one part of the B_J image
-  static constexpr uint32_t V_BYTES = N * kT2BN * 2;    // one part of the BF16 V_J tile
-  static constexpr uint32_t BN_BYTES = BJ ? kT2BN * 4 : 0;   // b_J
-  static constexpr uint32_t X_COPY = 2 * XB_BYTES + BN_BYTES;   // B_J high | remainder | b_J
-  static constexpr uint32_t OFF_BN = 2 * XB_BYTES;              // within a stage
-  static constexpr uint32_t OFF_V = X_COPY;
-  static constexpr uint32_t STAGE_BYTES = X_COPY + 2 * V_BYTES;
-  // as many stages (at most 8) as let four CTAs fit in shared memory (~54 KB each), at least 3
-  static constexpr int ST_FIT = (int)((54u * 1024u - 2 * A_BYTES) / STAGE_BYTES);
-  static constexpr int ST = ST_FIT > 8 ? 8 : ST_FIT < 3 ? 3 : ST_FIT;
-  static constexpr uint32_t OFF_STAGES = 2 * A_BYTES;
-  static constexpr uint32_t OFF_BARS = OFF_STAGES + ST * STAGE_BYTES;
-  // C/K buffers of 32 columns: three while they fit beside the accumulator, else two
-  static constexpr int NB = (3 * 32 + N <= (int)kT2Cols) ? 3 : 2;
-  // full per stage; a_full; c_full per tile mod 6 (so that each barrier serves one
-  // epilogue set and its phases are waited in order); k_full, b_free per buffer; done
-  static constexpr int NCF = 6;
-  static constexpr int NBARS = ST + 1 + NCF + 2 * NB + 1;
+  // A unit is G consecutive tiles handed over together: one wait, fence and arrival per unit.
+  // The accumulator and the A rows (high part and remainder, K8 columns each) leave room for
+  // three units of two tiles up to N = 32 (three sets of epilogue warps); with N = 64 for five
+  // units of one tile (four sets).
+  static constexpr int G = N <= 32 ? 2 : 1;
+  static constexpr int NBUF = N <= 32 ? 3 : 5;
+  static constexpr int SETS = N <= 32 ? 3 : 4;
+  static constexpr int THREADS = 32 * (2 + 4 * SETS);   // copies and C, contraction, the sets
+  static constexpr uint32_t XB_BYTES = kT2BN * K8 * 4;  // one part of a B tile
+  static constexpr uint32_t V_BYTES = N * kT2BN * 2;    // one part of a BF16 V tile
+  static constexpr uint32_t BN_BYTES = kT2BN * 4;       // a tile's b_j
+  static constexpr uint32_t X_COPY = 2 * XB_BYTES + BN_BYTES;   // B high | remainder | b
+  static constexpr uint32_t OFF_BN = 2 * XB_BYTES;              // within a tile
+  static constexpr uint32_t OFF_V = G * X_COPY;                 // within a stage
+  static constexpr uint32_t STAGE_BYTES = OFF_V + G * 2 * V_BYTES;
+  // as many stages (units) as let two CTAs fit in shared memory, at most 8
+  static constexpr int ST_FIT = (int)((108u * 1024u) / STAGE_BYTES);
+  static constexpr int ST = ST_FIT > 8 ? 8 : ST_FIT;
+  static_assert(ST > NBUF, "a stage beyond those in flight");
+  static constexpr uint32_t OFF_BARS = ST * STAGE_BYTES;
+  // full per stage; c_full, k_full, b_free per buffer; done
+  static constexpr int NBARS = ST + 3 * NBUF + 1;
   static constexpr uint32_t SMEM = OFF_BARS + NBARS * 8 + 64;
-  static constexpr uint32_t COL_U = NB * 32;   // after the C/K buffers
-  static_assert(COL_U + N <= kT2Cols, "tensor memory layout exceeds the allocation");
-  static_assert(STAGE_BYTES % 16 == 0 && A_BYTES % 16 == 0 && XB_BYTES % 16 == 0 &&
-                    X_COPY % 16 == 0,
+  // tensor-memory columns: the C/K buffers, the accumulator, A's two parts
+  static constexpr uint32_t COL_U = NBUF * G * 32;
+  static constexpr uint32_t COL_A = COL_U + N;
+  static_assert(COL_A + 2 * K8 <= kT2Cols, "tensor memory layout exceeds the allocation");
+  static_assert(STAGE_BYTES % 16 == 0 && XB_BYTES % 16 == 0 && X_COPY % 16 == 0 && OFF_V % 16 == 0,
                 "bulk copies and descriptors need 16-byte alignment");
-  static_assert(NCF % NB == 0, "a c_full barrier belongs to one buffer");
 };
 
 template <int NH>
@@ -199,18 +211,16 @@ template <int K8, int N, bool BJ>
 __device__ __forceinline__ void tc2_body(const Tc2DevArgs& a, const int rb, const int sp,
                                          const int R) {
   using S = Tc2Shape<K8, N, BJ>;
-  constexpr int ST = S::ST;
-  constexpr int NB = S::NB;
+  constexpr int ST = S::ST, G = S::G, NBUF = S::NBUF, SETS = S::SETS;
   constexpr int NH = N / 2;
   extern __shared__ __align__(1024) unsigned char smem[];
   const uint32_t smem0 = smem_u32(smem);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S::OFF_BARS);
   uint64_t* full = bars;
-  uint64_t* a_full = bars + ST;
-  uint64_t* c_full = a_full + 1;
-  uint64_t* k_full = c_full + S::NCF;
-  uint64_t* b_free = k_full + NB;
-  uint64_t* done = b_free + NB;
+  uint64_t* c_full = bars + ST;
+  uint64_t* k_full = c_full + NBUF;
+  uint64_t* b_free = k_full + NBUF;
+  uint64_t* done = b_free + NBUF;
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + S::OFF_BARS + S::NBARS * 8);
   volatile int* s_fail = reinterpret_cast<volatile int*>(s_tmem + 1);
   int* s_last = reinterpret_cast<int*>(s_tmem + 2);
@@ -223,13 +233,13 @@ __device__ __forceinline__ void tc2_body(const Tc2DevArgs& a, const int rb, cons
   const long long row0 = (long long)rb * kT2BM;
   const int tile_begin = sp * a.tiles_per_split;
   const int nt = max(0, min(tile_begin + a.tiles_per_split, a.ntiles) - tile_begin);
+  const int nu = (nt + G - 1) / G;   // units; the last may hold fewer tiles
 
   if (tid == 0) {
     for (int s = 0; s < ST; ++s) mbar_init(&full[s], 1);
-    mbar_init(a_full, 1);
-    for (int c = 0; c < S::NCF; ++c) mbar_init(&c_full[c], 1);
-    for (int b = 0; b < NB; ++b) {
-      mbar_init(&k_full[b], 4);   // the four epilogue warps of the tile's set
+    for (int b = 0; b < NBUF; ++b) {
+      mbar_init(&c_full[b], 1);
+      mbar_init(&k_full[b], 4);   // the four epilogue warps of the unit's set
       mbar_init(&b_free[b], 1);
     }
     mbar_init(done, 1);
@@ -241,176 +251,215 @@ __device__ __forceinline__ void tc2_body(const Tc2DevArgs& a, const int rb, cons
   __syncthreads();
   tc::fence_after();
   const uint32_t tbase = __shfl_sync(0xffffffffu, *s_tmem, 0);
-  int issued = 0;   // tiles whose copies were started (warp 0)
+  if (warp >= 2 && warp <= 5) {
+    // A_I into tensor memory, a row per thread: the cross term's A operand is then read there
+    // (an MMA whose A comes from shared memory takes 40 clocks for its 4 KB, from tensor memory 16)
+    const int eq = warp & 3;
+    const long long i = row0 + eq * 32 + lane;
+    const long long off = (i / 32) * 32 * K8 + tc::canon_offset((int)(i % 32), 0, 4, K8 / 4) / 4;
+    const uint32_t dst = tbase + ((uint32_t)(eq * 32) << 16) + S::COL_A;
+#pragma unroll
+    for (int part = 0; part < 2; ++part) {
+      const float* src = (part == 0 ? a.A_hi : a.A_lo) + off;
+#pragma unroll
+      for (int k = 0; k < K8; k += 8) {
+        const uint4 x = *reinterpret_cast<const uint4*>(src + k / 4 * 32);
+        const uint4 y = *reinterpret_cast<const uint4*>(src + (k / 4 + 1) * 32);
+        const uint32_t v[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+        tc::tmem_st8(dst + (uint32_t)(part * K8 + k), v);
+      }
+    }
+    tc::tmem_wait_st();
+  }
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  int issued = 0;   // units whose copies were started (warp 0)
 
   if (warp == 0) {
-    // ------ copies and MMAs: C = x^_I x^_J^T, then U += K V; one elected lane issues, the
+    // ------ copies and MMAs of the cross term, C = x^_I x^_J^T; one elected lane issues, the
     //        whole warp runs the loop, so that descriptors and addresses stay warp-uniform ------
     constexpr uint32_t idesc_c = tc::instr_desc(2, kT2BM, kT2BN);   // TF32
-    constexpr uint32_t idesc_u = tc::instr_desc(1, kT2BM, N);       // BF16
     constexpr uint32_t sbo_x = (K8 / 4) * 128;
-    const uint64_t dAh = tc::smem_desc(smem0, 128, sbo_x);
-    const uint64_t dAl = tc::smem_desc(smem0 + S::A_BYTES, 128, sbo_x);
-    const uint64_t dB0 = tc::smem_desc(smem0 + S::OFF_STAGES, 128, sbo_x);
-    const uint64_t dV0 = tc::smem_desc(smem0 + S::OFF_STAGES + S::OFF_V, 128, 512);
+    const uint64_t dB0 = tc::smem_desc(smem0, 128, sbo_x);
     const float* srcX = a.B + (long long)tile_begin * tc2_b_stride(K8);
     const __nv_bfloat16* srcV = a.Vp + (long long)tile_begin * 2 * N * kT2BN;
-    auto copy_tile = [&](int p, int s) {   // elected lane: tile p's B_J (with b_J) and V_J
-      unsigned char* st = smem + S::OFF_STAGES + s * S::STAGE_BYTES;
-      mbar_arrive_expect_tx(&full[s], S::STAGE_BYTES);
-      bulk_g2s(st, srcX + (long long)p * tc2_b_stride(K8), S::X_COPY, &full[s]);
-      bulk_g2s(st + S::OFF_V, srcV + (long long)p * 2 * N * kT2BN, 2 * S::V_BYTES, &full[s]);
+    auto copy_unit = [&](int u, int s) {   // elected lane: the unit's B (with b) and V tiles
+      const uint32_t m = (uint32_t)min(G, nt - u * G);
+      unsigned char* st = smem + s * S::STAGE_BYTES;
+      mbar_arrive_expect_tx(&full[s], m * (S::X_COPY + 2 * S::V_BYTES));
+      bulk_g2s(st, srcX + (long long)u * G * tc2_b_stride(K8), m * S::X_COPY, &full[s]);
+      bulk_g2s(st + S::OFF_V, srcV + (long long)u * G * 2 * N * kT2BN, m * 2 * S::V_BYTES, &full[s]);
     };
-    auto mma_c = [&](int s, int b, int cf) {   // elected lane: C into buffer b
-      const uint64_t dBh = dB0 + (uint64_t)s * (S::STAGE_BYTES >> 4), dBl = dBh + (S::XB_BYTES >> 4);
-      const uint32_t dC = tbase + (uint32_t)(b * 32);
+    auto mma_c = [&](int u, int s, int b) {   // elected lane: the unit's C into buffer b
 #pragma unroll
-      for (int term = 0; term < 3; ++term) {
-        const uint64_t A = term == 2 ? dAl : dAh;
-        const uint64_t B = term == 1 ? dBl : dBh;
+      for (int g = 0; g < G; ++g) {
+        if (g > 0 && u * G + g >= nt) break;
+        const uint64_t dBh = dB0 + (uint64_t)((s * S::STAGE_BYTES + g * S::X_COPY) >> 4);
+        const uint32_t dC = tbase + (uint32_t)(b * G * 32 + g * 32);
 #pragma unroll
-        for (int ks = 0; ks < K8 / 8; ++ks)
-          tc::mma_tf32(dC, A + 16u * ks, B + 16u * ks, idesc_c, (term | ks) != 0);
+        for (int term = 0; term < 3; ++term) {
+          const uint32_t A = tbase + S::COL_A + (term == 2 ? (uint32_t)K8 : 0u);
+          const uint64_t B = term == 1 ? dBh + (S::XB_BYTES >> 4) : dBh;
+#pragma unroll
+          for (int ks = 0; ks < K8 / 8; ++ks)
+            tc::mma_tf32_ts(dC, A + 8u * ks, B + 16u * ks, idesc_c, (term | ks) != 0);
+        }
       }
-      tc::commit(&c_full[cf]);
+      tc::commit(&c_full[b]);
     };
-    const int pre = min(ST, nt);
-    if (tc::elect_one()) {
-      mbar_arrive_expect_tx(a_full, 2 * S::A_BYTES);
-      bulk_g2s(smem, a.A_hi + row0 * K8, S::A_BYTES, a_full);
-      bulk_g2s(smem + S::A_BYTES, a.A_lo + row0 * K8, S::A_BYTES, a_full);
-      for (int p = 0; p < pre; ++p) copy_tile(p, p);
-    }
+    const int pre = min(ST, nu);
+    if (tc::elect_one())
+      for (int u = 0; u < pre; ++u) copy_unit(u, u);
+    __syncwarp();
     issued = pre;
-    bool ok = tc::warp_wait_uniform(smem_u32(a_full), 0);
-    // s_c, cf: stage and c_full barrier of the next tile whose C is issued; s, b: stage and
-    // buffer of tile p
-    int s_c = 0, ph_c = 0, cf = 0;
-    for (int p = 0; p < NB && p < nt && ok; ++p) {
+    bool ok = true;
+    int s_c = 0, ph_c = 0;   // stage of the next unit whose C is issued
+    for (int u = 0; u < NBUF && u < nu && ok; ++u) {
       ok = tc::warp_wait_uniform(full0 + 8u * s_c, ph_c);
       tc::fence_after();
-      if (ok && tc::elect_one()) mma_c(s_c, p, cf);
+      if (ok && tc::elect_one()) mma_c(u, s_c, u);
       __syncwarp();
       if (++s_c == ST) { s_c = 0; ph_c ^= 1; }
-      if (++cf == S::NCF) cf = 0;
     }
+    // the buffer and the stage of unit v are refilled once its contraction has read them
     int s = 0, b = 0, ph_b = 0;
 #pragma unroll 1
-    for (int p = 0; p < nt && ok; ++p) {
+    for (int v = 0; ok && v + min(NBUF, ST) < nu; ++v) {
+      ok = tc::warp_wait_uniform(b_free0 + 8u * b, ph_b);
+      if (ok && v + NBUF < nu) {
+        ok = tc::warp_wait_uniform(full0 + 8u * s_c, ph_c);
+        tc::fence_after();
+        if (ok && tc::elect_one()) mma_c(v + NBUF, s_c, b);
+        __syncwarp();
+        if (++s_c == ST) { s_c = 0; ph_c ^= 1; }
+      }
+      if (ok && v + ST < nu) {
+        if (tc::elect_one()) copy_unit(v + ST, s);
+        __syncwarp();
+        issued = v + ST + 1;
+      }
+      if (++s == ST) s = 0;
+      if (++b == NBUF) { b = 0; ph_b ^= 1; }
+    }
+    if (!ok) *s_fail = 1;
+  } else if (warp == 1) {
+    // ------ MMAs of the contraction: U += K V; a warp of their own, so that neither stream of
+    //        issuing instructions (about a hundred per tile, in turn with the epilogue's) and
+    //        waits holds up the other ------
+    constexpr uint32_t idesc_u = tc::instr_desc(1, kT2BM, N);       // BF16
+    const uint64_t dV0 = tc::smem_desc(smem0 + S::OFF_V, 128, 512);
+    bool ok = true;
+    int s = 0, b = 0, ph_b = 0;
+#pragma unroll 1
+    for (int u = 0; u < nu; ++u) {
       ok = tc::warp_wait_uniform(k_full0 + 8u * b, ph_b);
       if (!ok) break;
       tc::fence_after();
-      const bool more_c = p + NB < nt, more_v = p + ST < nt;
       if (tc::elect_one()) {
-        const uint64_t dVh = dV0 + (uint64_t)s * (S::STAGE_BYTES >> 4), dVl = dVh + (S::V_BYTES >> 4);
-        const uint32_t kcol = tbase + (uint32_t)(b * 32);
 #pragma unroll
-        for (int term = 0; term < 3; ++term) {
-          const uint32_t A = kcol + (term == 2 ? 8u : 0u);   // K high | K low per 16 points
-          const uint64_t B = term == 1 ? dVl : dVh;
+        for (int g = 0; g < G; ++g) {
+          if (g > 0 && u * G + g >= nt) break;
+          const uint64_t dVh = dV0 + (uint64_t)((s * S::STAGE_BYTES + g * 2 * S::V_BYTES) >> 4);
+          const uint32_t kcol = tbase + (uint32_t)(b * G * 32 + g * 32);
 #pragma unroll
-          for (int ks = 0; ks < kT2BN / 16; ++ks)
-            tc::mma_bf16_ts(tbase + S::COL_U, A + ks * 16, B + 16u * ks, idesc_u, (p | term | ks) != 0);
+          for (int term = 0; term < 3; ++term) {
+            const uint32_t A = kcol + (term == 2 ? 8u : 0u);   // K high | K low per 16 points
+            const uint64_t B = term == 1 ? dVh + (S::V_BYTES >> 4) : dVh;
+#pragma unroll
+            for (int ks = 0; ks < kT2BN / 16; ++ks)
+              tc::mma_bf16_ts(tbase + S::COL_U, A + ks * 16, B + 16u * ks, idesc_u,
+                              (u | g | term | ks) != 0);
+          }
         }
-        // buffer b takes tile p + NB's C, and stage s tile p + ST's operands, only after these
-        // MMAs have read its K and V
-        if (more_c || more_v) tc::commit(&b_free[b]);
+        // buffer b takes unit u + NBUF's C, and stage s unit u + ST's operands, only after
+        // these MMAs have read its K and V
+        tc::commit(&b_free[b]);
       }
       __syncwarp();
-      if (more_c || more_v) {
-        ok = tc::warp_wait_uniform(b_free0 + 8u * b, ph_b);
-        if (ok && more_c) {
-          ok = tc::warp_wait_uniform(full0 + 8u * s_c, ph_c);
-          tc::fence_after();
-          if (ok && tc::elect_one()) mma_c(s_c, b, cf);
-          __syncwarp();
-          if (++s_c == ST) { s_c = 0; ph_c ^= 1; }
-          if (++cf == S::NCF) cf = 0;
-        }
-        if (ok && more_v) {
-          if (tc::elect_one()) copy_tile(p + ST, s);
-          __syncwarp();
-          issued = p + ST + 1;
-        }
-      }
       if (++s == ST) s = 0;
-      if (++b == NB) { b = 0; ph_b ^= 1; }
+      if (++b == NBUF) { b = 0; ph_b ^= 1; }
     }
     if (!ok) *s_fail = 1;
     if (tc::elect_one()) tc::commit(done);
     __syncwarp();
   } else {
-    // ------ epilogue: 8 warps; warp (lane quadrant eq, set h) takes the tiles h, h + 2, ...
-    //        with all 32 of their columns ------
+    // ------ epilogue: warp (lane quadrant eq, set h) takes the units h, h + SETS, ... whole ------
     const int eq = warp & 3;
-    const int half = (warp - 1) >> 2;   // tile set; also the half of U it reads back
+    const int set = (warp - 2) >> 2;
+    const int half = set;   // sets 0 and 1 read back the two halves of U
     const int il = eq * 32 + lane;
     const long long i = row0 + il;
     const uint32_t lane_base = (uint32_t)(eq * 32) << 16;
     const float ai = a.params->c0f + a.bneg[i];   // bneg covers the padded rows (zero there)
+    // two entries per packed FP32x2 instruction (FADD2 / FFMA2, the same rounding as the
+    // scalar forms)
+    const float2 ai2 = make_float2(ai, ai);
+    const float2 minus1 = make_float2(-1.f, -1.f);
     bool ok = true;
-    int s = half % ST, ph_s = 0, b = half % NB, cf = half, ph_cf = 0;
+    int s = set, ph_s = 0, b = set, ph_b = 0;   // set < NBUF < ST
 #pragma unroll 1
-    for (int lt = half; lt < nt; lt += 2) {
-      ok = tc::warp_wait_uniform(c_full0 + 8u * cf, ph_cf);
+    for (int u = set; u < nu; u += SETS) {
+      // A wait for the unit's use of its buffer cannot see the use before last: that one's C was
+      // committed before the C of unit u - SETS, which this set has finished.
+      ok = tc::warp_wait_uniform(c_full0 + 8u * b, ph_b);
       // b_J is read from the stage: wait for its copy too (the stage is refilled only after
-      // this tile's contraction, which waits for this warp's K)
+      // this unit's contraction, which waits for this warp's K)
       if constexpr (BJ) ok = ok && tc::warp_wait_uniform(full0 + 8u * s, ph_s);
       if (!ok) break;
       tc::fence_after();
-      const float4* bj = reinterpret_cast<const float4*>(smem + S::OFF_STAGES + s * S::STAGE_BYTES +
-                                                         S::OFF_BN);
-      // all 32 columns of C in one tensor-memory round trip; each pair's K high and low parts
-      // are written back into the pair's own registers (no extra registers live)
-      const uint32_t ccol = tbase + lane_base + (uint32_t)(b * 32);
-      uint32_t c[32];
-      tc::tmem_ld16x2(ccol, c);
-      // two entries per packed FP32x2 instruction (FADD2 / FFMA2, the same rounding as the
-      // scalar forms)
-      const float2 ai2 = make_float2(ai, ai);
-      const float2 minus1 = make_float2(-1.f, -1.f);
+      const int m = G == 1 ? 1 : min(G, nt - u * G);
+#pragma unroll 1
+      for (int g = 0; g < m; ++g) {
+        const float4* bj = reinterpret_cast<const float4*>(smem + s * S::STAGE_BYTES +
+                                                           g * S::X_COPY + S::OFF_BN);
+        // all 32 columns of a tile's C in one tensor-memory round trip
+        const uint32_t ccol = tbase + lane_base + (uint32_t)(b * G * 32 + g * 32);
+        uint32_t c[32];
+        tc::tmem_ld16x2(ccol, c);
 #pragma unroll
-      for (int hh = 0; hh < 2; ++hh) {
-        uint32_t hi[8], lo[8];
+        for (int hh = 0; hh < 2; ++hh) {
+          uint32_t hi[8], lo[8];
 #pragma unroll
-        for (int g = 0; g < 4; ++g) {
-          float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
-          if constexpr (BJ) b4 = bj[4 * hh + g];
+          for (int g4 = 0; g4 < 4; ++g4) {
+            float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
+            if constexpr (BJ) b4 = bj[4 * hh + g4];
 #pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            const int e0 = 16 * hh + 4 * g + 2 * q;
-            // the exponent is <= log2 sigma^2 up to rounding (about 1e-6 relative in k)
-            float2 e = ai2;
-            if constexpr (BJ) e = __fadd2_rn(e, q == 0 ? make_float2(b4.x, b4.y) : make_float2(b4.z, b4.w));
-            e = __fadd2_rn(e, make_float2(__uint_as_float(c[e0]), __uint_as_float(c[e0 + 1])));
-            const float2 k = make_float2(ex2_approx(e.x), ex2_approx(e.y));
-            const __nv_bfloat162 h = __floats2bfloat162_rn(k.x, k.y);
-            const float2 r = __ffma2_rn(__bfloat1622float2(h), minus1, k);   // k - high part
-            const __nv_bfloat162 l = __floats2bfloat162_rn(r.x, r.y);
-            hi[2 * g + q] = *reinterpret_cast<const uint32_t*>(&h);
-            lo[2 * g + q] = *reinterpret_cast<const uint32_t*>(&l);
+            for (int q = 0; q < 2; ++q) {
+              const int e0 = 16 * hh + 4 * g4 + 2 * q;
+              // the exponent is <= log2 sigma^2 up to rounding (about 1e-6 relative in k)
+              float2 e = ai2;
+              if constexpr (BJ) e = __fadd2_rn(e, q == 0 ? make_float2(b4.x, b4.y) : make_float2(b4.z, b4.w));
+              e = __fadd2_rn(e, make_float2(__uint_as_float(c[e0]), __uint_as_float(c[e0 + 1])));
+              const float2 k = make_float2(ex2_approx(e.x), ex2_approx(e.y));
+              const __nv_bfloat162 h = __floats2bfloat162_rn(k.x, k.y);
+              const float2 r = __ffma2_rn(__bfloat1622float2(h), minus1, k);   // k - high part
+              const __nv_bfloat162 l = __floats2bfloat162_rn(r.x, r.y);
+              hi[2 * g4 + q] = *reinterpret_cast<const uint32_t*>(&h);
+              lo[2 * g4 + q] = *reinterpret_cast<const uint32_t*>(&l);
+            }
           }
+          // columns [16 hh, 16 hh + 16): high parts, then low parts (the A operand of the
+          // contraction's k-step hh)
+          tc::tmem_st8(ccol + 16 * hh, hi);
+          tc::tmem_st8(ccol + 16 * hh + 8, lo);
         }
-        // columns [16 hh, 16 hh + 16): high parts, then low parts (the A operand of the
-        // contraction's k-step hh)
-        tc::tmem_st8(ccol + 16 * hh, hi);
-        tc::tmem_st8(ccol + 16 * hh + 8, lo);
       }
       tc::tmem_wait_st();
       tc::fence_before();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&k_full[b]);
-      s += 2;
+      s += SETS;
       if (s >= ST) { s -= ST; ph_s ^= 1; }
-      b += 2;
-      if (b >= NB) b -= NB;
-      cf += 2;
-      if (cf >= S::NCF) { cf -= S::NCF; ph_cf ^= 1; }
+      b += SETS;
+      if (b >= NBUF) { b -= NBUF; ph_b ^= 1; }
     }
     if (!ok) *s_fail = 1;
     const bool fin = ok && tc::warp_wait_uniform(smem_u32(done), 0);
     ok = __all_sync(0xffffffffu, fin && !*s_fail);
-    if (ok && nt > 0) {
+    if (half > 1) {
+      // the other sets have nothing to read back
+    } else if (ok && nt > 0) {
       tc::fence_after();
       float u[NH];
       t2_ld_cols<NH>(tbase + lane_base + S::COL_U + (uint32_t)(half * NH), u);
@@ -447,7 +496,6 @@ __device__ __forceinline__ void tc2_body(const Tc2DevArgs& a, const int rb, cons
     if (tid == 0) {
       atomicOr(a.status, kStatusTimeout);
       // let the copies still in flight land before the CTA's shared memory goes away
-      (void)mbar_wait_bounded(a_full, 0);
       for (int lt2 = max(0, issued - ST); lt2 < issued; ++lt2)
         (void)mbar_wait_bounded(&full[lt2 % ST], (uint32_t)((lt2 / ST) & 1));
     }
@@ -462,7 +510,7 @@ __device__ __forceinline__ void tc2_body(const Tc2DevArgs& a, const int rb, cons
   __threadfence();
   const float* base = a.partials + (long long)rb * a.nsplit * N * kT2BM;
   const float lam = (float)a.params->lambda;
-  for (int idx = tid; idx < R * kT2BM; idx += kT2Threads) {
+  for (int idx = tid; idx < R * kT2BM; idx += S::THREADS) {
     const int r = idx / kT2BM, il = idx - r * kT2BM;
     const long long i = row0 + il;
     if (i >= a.n) continue;
@@ -474,7 +522,7 @@ __device__ __forceinline__ void tc2_body(const Tc2DevArgs& a, const int rb, cons
 }
 
 template <int K8, int N, bool BJ>
-__global__ void __launch_bounds__(kT2Threads, 4) kmv_tc2_kernel(const Tc2DevArgs a) {
+__global__ void __launch_bounds__(Tc2Shape<K8, N, BJ>::THREADS, 2) kmv_tc2_kernel(const Tc2DevArgs a) {
   const int rb = blockIdx.x / a.nsplit;
   tc2_body<K8, N, BJ>(a, rb, blockIdx.x - rb * a.nsplit, a.R);
 }
@@ -482,7 +530,7 @@ __global__ void __launch_bounds__(kT2Threads, 4) kmv_tc2_kernel(const Tc2DevArgs
 // Many problems in one launch: CTA b takes work item items[b] = (problem, row block, split)
 // with that problem's arguments; a problem with no live columns is skipped.
 template <int K8, int N, bool BJ>
-__global__ void __launch_bounds__(kT2Threads, 4) kmv_tc2_batch_kernel(
+__global__ void __launch_bounds__(Tc2Shape<K8, N, BJ>::THREADS, 2) kmv_tc2_batch_kernel(
     const Tc2DevArgs* __restrict__ args, const int4* __restrict__ items) {
   __shared__ Tc2DevArgs s_a;
   const int4 it = items[blockIdx.x];
@@ -499,48 +547,27 @@ __global__ void pack_v_batch_kernel(const Tc2DevArgs* __restrict__ args, int N) 
   const Tc2DevArgs& a = args[blockIdx.y];
   const int R = a.R_dev ? *a.R_dev : a.R;
   if (R <= 0) return;
-  const long long ntiles = a.ntiles;
-  const long long per_tile = (long long)N * kT2BN;
-  __nv_bfloat16* Vp = const_cast<__nv_bfloat16*>(a.Vp);
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < ntiles * per_tile;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const long long t = idx / per_tile;
-    const int rem = (int)(idx - t * per_tile);
-    const int r = rem / kT2BN, jj = rem - r * kT2BN;
-    const long long j = t * kT2BN + jj;
-    const float v = (r < R && j < a.n) ? a.V[(long long)a.vmap[r] * a.ldv + j] : 0.f;
-    const __nv_bfloat16 h = __float2bfloat16_rn(v);
-    const __nv_bfloat16 l = __float2bfloat16_rn(v - __bfloat162float(h));
-    const long long off = t * 2 * per_tile + tc::canon_offset(r, jj, 2, kT2BN / 8) / 2;
-    Vp[off] = h;
-    Vp[off + per_tile] = l;
-  }
+  pack_v2(a.V, a.ldv, a.vmap, R, N, a.n, a.ntiles, const_cast<__nv_bfloat16*>(a.Vp), blockIdx.x,
+          gridDim.x);
 }
 
 template <int K8, int N, bool BJ>
 struct Tc2Inst {
   using S = Tc2Shape<K8, N, BJ>;
-  // CTAs per SM: shared memory, tensor memory (512 columns) and the launch bound.
-  static int occupancy() {
-    static int occ = -1;
+  // The split plan counts four CTAs' worth of work per SM.  The ranges it gives also set the
+  // rounding of the sums, which tensor memory accumulates with truncation (kTcMaxSplitTiles).
+  static constexpr int kPlanOcc = 4;
+  static void prime() {
     static std::once_flag once;
     std::call_once(once, [] {
       auto fn = kmv_tc2_kernel<K8, N, BJ>;
       cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
       cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-      int dev = 0, smem_sm = 0;
-      cudaGetDevice(&dev);
-      if (cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) !=
-          cudaSuccess)
-        smem_sm = 228 * 1024;
-      const int by_smem = smem_sm / (int)(S::SMEM + 1024);
-      occ = std::max(1, std::min({by_smem, (int)(512 / kT2Cols), 4}));
     });
-    return occ;
   }
   static cudaError_t launch(TcLaunch& L, cudaStream_t s) {
     KmvPlan p = L.nsplit > 0 ? plan_split_forced(L.n, kT2BM, N, 4, L.nsplit)
-                             : plan_split(L.n, kT2BM, N, 4, L.num_sms * occupancy());
+                             : plan_split(L.n, kT2BM, N, 4, L.num_sms * kPlanOcc);
     p = tc_bound_split(p, L.n, kT2BM, N, kT2BN);
     const size_t pbytes = p.nsplit > 1 ? (size_t)p.n_rb * p.nsplit * N * kT2BM * 4 : 0;
     L.planned_nsplit = p.nsplit;
@@ -555,7 +582,7 @@ struct Tc2Inst {
       return cudaErrorMemoryAllocation;
     }
     const long long ntiles = (L.n + kT2BN - 1) / kT2BN;
-    launch_pack_v(L, N, ntiles, s);
+    if (!L.v_packed) launch_pack_v(L, N, ntiles, s);
     Tc2DevArgs a;
     a.A_hi = L.X_hi;
     a.A_lo = L.X_lo;
@@ -578,9 +605,9 @@ struct Tc2Inst {
     a.partials = static_cast<float*>(L.partials);
     a.counters = L.counters;
     a.status = L.status;
-    (void)occupancy();
+    prime();
     const int nrb = (int)((L.n + kT2BM - 1) / kT2BM);
-    kmv_tc2_kernel<K8, N, BJ><<<nrb * a.nsplit, kT2Threads, S::SMEM, s>>>(a);
+    kmv_tc2_kernel<K8, N, BJ><<<nrb * a.nsplit, S::THREADS, S::SMEM, s>>>(a);
     return cudaGetLastError();
   }
 };
@@ -608,11 +635,13 @@ cudaError_t launch_kmv_tc2(TcLaunch& L, cudaStream_t s) {
 cudaError_t launch_prescale_mixed(const PsiArg& pa, double* psi_dev, const float* X, float* xhat,
                                   long long n, long long ld128, int d, int DP, bool aug,
                                   DevParams* P, float* bneg, float* X_hi, float* X_lo, float* X_b,
-                                  int num_sms, cudaStream_t s) {
+                                  PackV pv, int num_sms, cudaStream_t s) {
   const int blocks = (int)std::min<long long>(ld128 / 128, 8LL * num_sms);
+  pv.first_cta = blocks;
+  const int more = pv.V ? pack_v_ctas(n, pv.N, 128, num_sms) : 0;
   auto go = [&](auto kernel) {
-    kernel<<<blocks, 128, 0, s>>>(pa, psi_dev, X, xhat, n, ld128, d, aug ? 1 : 0, P, bneg, X_hi,
-                                  X_lo, X_b);
+    kernel<<<blocks + more, 128, 0, s>>>(pa, psi_dev, X, xhat, n, ld128, d, aug ? 1 : 0, P, bneg,
+                                         X_hi, X_lo, X_b, pv);
   };
   switch (DP) {
     case 2: go(prescale_mixed_kernel<2>); break;
@@ -686,7 +715,8 @@ static cudaError_t tc2_batch_launch(const Tc2DevArgs* args, int B, const int4* i
   tc2_batch_prime<N>();
   pack_v_batch_kernel<<<dim3(64, (unsigned)B), 256, 0, s>>>(args, N);
   if (n_items > 0)
-    kmv_tc2_batch_kernel<8, N, true><<<n_items, kT2Threads, Tc2Shape<8, N, true>::SMEM, s>>>(
+    kmv_tc2_batch_kernel<8, N, true><<<n_items, Tc2Shape<8, N, true>::THREADS,
+                                       Tc2Shape<8, N, true>::SMEM, s>>>(
         args, items);
   return cudaGetLastError();
 }

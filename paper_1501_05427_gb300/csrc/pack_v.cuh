@@ -1,0 +1,56 @@
+// The operand images of the tensor-core contractions: columns vmap[0..R) of V (vmap null: 0, 1, ...)
+// as K-major canonical BF16 images of N rows (right-hand sides) x 32 points per tile, the parts of
+// a tile back to back (one bulk copy); rows r >= R and points >= n are zero.  The CTAs
+// cta = 0..ctas-1 share the work.
+#pragma once
+
+#include <cuda_bf16.h>
+
+#include "tc_common.cuh"
+
+namespace ulisse {
+
+// High and low part (mixed precision).
+__device__ inline void pack_v2(const float* __restrict__ V, long long ldv,
+                               const int* __restrict__ vmap, int R, int N, long long n,
+                               long long ntiles, __nv_bfloat16* __restrict__ Vp, int cta, int ctas) {
+  const int per = N * 32;
+  for (long long idx = cta * (long long)blockDim.x + threadIdx.x; idx < ntiles * per;
+       idx += (long long)ctas * blockDim.x) {
+    const long long t = idx / per;
+    const int rem = (int)(idx - t * per);
+    const int r = rem / 32, jj = rem - r * 32;
+    const long long j = t * 32 + jj;
+    const float v = (r < R && j < n) ? V[(long long)(vmap ? vmap[r] : r) * ldv + j] : 0.f;
+    const __nv_bfloat16 h = __float2bfloat16_rn(v);
+    __nv_bfloat16* o = Vp + t * 2LL * per + tc::canon_offset(r, jj, 2, 4) / 2;
+    o[0] = h;
+    o[per] = __float2bfloat16_rn(v - __bfloat162float(h));
+  }
+}
+
+// High, middle and low part: a float exactly (FP32 products).  A value that is not finite stays
+// in the high part.
+__device__ inline void pack_v3(const float* __restrict__ V, long long ldv,
+                               const int* __restrict__ vmap, int R, int N, long long n,
+                               long long ntiles, __nv_bfloat16* __restrict__ Vp, int cta, int ctas) {
+  const int per = N * 32;
+  for (long long idx = cta * (long long)blockDim.x + threadIdx.x; idx < ntiles * per;
+       idx += (long long)ctas * blockDim.x) {
+    const long long t = idx / per;
+    const int rem = (int)(idx - t * per);
+    const int r = rem / 32, jj = rem - r * 32;
+    const long long j = t * 32 + jj;
+    const float v = (r < R && j < n) ? V[(long long)(vmap ? vmap[r] : r) * ldv + j] : 0.f;
+    const __nv_bfloat16 h = __float2bfloat16_rn(v);
+    const bool split = isfinite(__bfloat162float(h));
+    const float v1 = split ? v - __bfloat162float(h) : 0.f;
+    const __nv_bfloat16 m = __float2bfloat16_rn(v1);
+    __nv_bfloat16* o = Vp + t * 3LL * per + tc::canon_offset(r, jj, 2, 4) / 2;
+    o[0] = h;
+    o[per] = m;
+    o[2 * per] = __float2bfloat16_rn(v1 - __bfloat162float(m));
+  }
+}
+
+}  // namespace ulisse

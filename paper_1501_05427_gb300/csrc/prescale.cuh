@@ -11,8 +11,9 @@
 // n = 1,030, d = 8, 5 columns (FP32) and from 840 to 795 us at n = 50,000 (mixed).
 #pragma once
 
-#include <cfloat>
+#include <algorithm>
 
+#include "pack_v.cuh"
 #include "tc_common.cuh"
 #include "ulisse_internal.cuh"
 
@@ -23,6 +24,20 @@ struct PsiArg {
   double v[kMaxP];
   int by_value;
 };
+
+// A product's operand V (R columns, leading dimension n) packed by the prescale launch (V null: no).
+struct PackV {
+  const float* V;
+  int R, N;        // columns, MMA columns
+  void* Vp;
+  int first_cta;   // the CTAs from here on pack (set by the launcher)
+};
+
+inline int pack_v_ctas(long long n, int N, int threads, int num_sms) {
+  const long long total = (n + 31) / 32 * 32 * N;
+  return (int)std::max<long long>(1, std::min<long long>((total + 4 * threads - 1) / (4 * threads),
+                                                         8LL * num_sms * 256 / threads));
+}
 
 // 1 / l_k as a double and as the pair hi + lo of floats.
 struct InvLength {
@@ -79,12 +94,13 @@ __device__ __forceinline__ T scaled(float x, const InvLength& s, int k) {
 
 // x^ = x / l for rows [0, n) (rows >= n stay zero; dims >= d zero), one element per thread; the
 // CTAs from row_blocks on copy (and convert) R columns of V, leading dimension n, to D, leading
-// dimension ldn.
+// dimension ldn, or pack pv.
 template <typename T, typename TV>
 __global__ void __launch_bounds__(256) prescale_kernel(
     const PsiArg pa, double* __restrict__ psi_dev, const float* __restrict__ X,
     T* __restrict__ xhat, long long n, int d, int log2_dp, DevParams* __restrict__ P,
-    int row_blocks, const TV* __restrict__ V, T* __restrict__ D, long long ldn, int R) {
+    int row_blocks, const TV* __restrict__ V, T* __restrict__ D, long long ldn, int R,
+    const PackV pv) {
   __shared__ InvLength s;
   if ((int)blockIdx.x < row_blocks) {
     unpack_params(pa, psi_dev, d, P, s);
@@ -96,6 +112,11 @@ __global__ void __launch_bounds__(256) prescale_kernel(
     }
     return;
   }
+  if (pv.V) {   // FP32 tensor-core products
+    pack_v3(pv.V, n, nullptr, pv.R, pv.N, n, (n + 31) / 32, static_cast<__nv_bfloat16*>(pv.Vp),
+            blockIdx.x - row_blocks, gridDim.x - row_blocks);
+    return;
+  }
   const long long total = n * R, step = (gridDim.x - row_blocks) * 256LL;
   for (long long idx = (blockIdx.x - row_blocks) * 256LL + threadIdx.x; idx < total; idx += step) {
     const long long c = idx / n;
@@ -105,18 +126,19 @@ __global__ void __launch_bounds__(256) prescale_kernel(
 
 inline int log2_of(int dp) { return dp == 2 ? 1 : dp == 4 ? 2 : dp == 8 ? 3 : 4; }
 
-// Launch of prescale_kernel; V null: no columns to copy.
+// Launch of prescale_kernel; V and pv.V null: no columns to copy or pack.
 template <typename T, typename TV>
 cudaError_t launch_prescale(const PsiArg& pa, double* psi_dev, const float* X, T* xhat, long long n,
                             int d, int DP, DevParams* P, const TV* V, T* D, long long ldn, int R,
-                            int num_sms, cudaStream_t s) {
+                            PackV pv, int num_sms, cudaStream_t s) {
   // four elements per thread, at most eight CTAs per SM for each of the two parts
   auto blocks = [&](long long total) {
     return (int)std::max<long long>(1, std::min<long long>((total + 1023) / 1024, 8LL * num_sms));
   };
   const int rb = blocks(n * DP);
-  prescale_kernel<T, TV><<<rb + (V ? blocks(n * R) : 0), 256, 0, s>>>(
-      pa, psi_dev, X, xhat, n, d, log2_of(DP), P, rb, V, D, ldn, R);
+  const int more = pv.V ? pack_v_ctas(n, pv.N, 256, num_sms) : V ? blocks(n * R) : 0;
+  prescale_kernel<T, TV><<<rb + more, 256, 0, s>>>(pa, psi_dev, X, xhat, n, d, log2_of(DP), P, rb, V,
+                                                   D, ldn, R, pv);
   return cudaGetLastError();
 }
 

@@ -261,6 +261,7 @@ struct KmvLaunch {
   void* v3;              // FP32: scratch of the tensor-core contraction's operand (kmv_f32_tc.cu),
                          // 96 BF16 values per point (null: SIMT kernel)
   bool simt;             // FP32: the SIMT kernel whatever the sizes
+  bool v_packed;         // v3 already holds the operand (packed by the prescale launch)
   int tm;                // rows per thread for K (0 = default)
   int r_min;             // compiled column count at least this (0: the smallest >= R)
   int nsplit;            // j-range split count (0: the launch plan's choice)
@@ -321,6 +322,7 @@ struct TcLaunch {
   const float* bneg;     // -c1 |x^|^2 (launch_prescale_mixed), ld128
   void* Vp;              // BF16 packed operand tiles, high | low part per tile (written by the
                          // launch), ld128 x 128
+  bool v_packed;         // ... already, by the prescale launch
   const void* V;         // FP32 operand columns
   long long ldv;
   const int* vmap;
@@ -381,10 +383,11 @@ __host__ __device__ constexpr int tc2_b_stride(int K8) { return 2 * 32 * K8 + 32
 // kmv_tc2.cu).  aug: rows carry the column term b_j (padded d 2 and 4 of the single-problem
 // launches); false for the batched launches, whose epilogue adds it for every d.
 struct PsiArg;
+struct PackV;
 cudaError_t launch_prescale_mixed(const PsiArg& pa, double* psi_dev, const float* X, float* xhat,
                                   long long n, long long ld128, int d, int DP, bool aug,
                                   DevParams* P, float* bneg, float* X_hi, float* X_lo, float* X_b,
-                                  int num_sms, cudaStream_t s);
+                                  PackV pv, int num_sms, cudaStream_t s);
 // Batched tensor-core K V (padded d <= 8): per problem a TcLaunch with the operand pointers,
 // R or R_dev, and the forced split nsplit >= 1 (tiles per split <= kTcMaxSplitTiles);
 // items: (problem, 128-row block, split) per CTA; R_max: the largest live column count.
