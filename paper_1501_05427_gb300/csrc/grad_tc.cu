@@ -29,20 +29,23 @@
 //   3. [S | G | H]_I += P_IJ Z_J on the tensor cores, Z_j = [x^_j, x^_j^2, 1] split the same
 //      way, accumulated in tensor memory across all tiles of the CTA's j range.
 // The per-row combination and the diagonal sum run in FP64 at the end; CTA partials are summed
-// in a fixed order by the last CTA to arrive (as in the SIMT gradient kernel).  Roles: warp 0
-// copies (B_J's TF32 image with b_J, or x^_J and b_J for d = 16, then B^_J and Z_J as one
-// block, into a ring of 3 to 6 stages) and issues the MMAs, its loop warp-uniform with a lane
-// elected for the issuing instructions; twelve epilogue warps make P in three sets of four (one
-// warp per tensor-memory lane quadrant): set h takes the tiles h, h + 3, ... whole and owns
-// the W/P and C buffers h, so that each wait and hand-off covers 32 entries per thread.  A
-// buffer pair is refilled, and the tile's stage with it, only after the MMAs that read P have
-// completed.  Every wait is bounded.
+// in a fixed order by the last CTA to arrive (as in the SIMT gradient kernel).  The left operands
+// [A^ | B]_I and A_I lie in tensor memory (in shared memory where 128 factor slots leave no room).
+// Roles: three issuing warps, one per stream of MMAs (warp 0: C; warp 1: W; warp 2: P Z and the
+// copies of B_J's TF32 image with b_J, or x^_J and b_J for d = 16, then B^_J and Z_J as one block,
+// into a ring of 4 to 8 stages), their loops warp-uniform with a lane elected for the issuing
+// instructions; twelve epilogue warps (eight for d = 16) make P in sets of four (one warp per
+// tensor-memory lane quadrant): set h takes the tiles h, h + 3, ... whole and owns the W/P buffer
+// h, so that each wait and hand-off covers 32 entries per thread; C has two buffers (one with 64
+// factor slots), given back as soon as they are read.  A W/P buffer is refilled, and the tile's
+// stage, only after the MMAs that read P have completed.  Every wait is bounded.
 //
-// What bounds it: the issue slots and the chain W, C -> epilogue -> P Z -> refill of each set.
-// Two CTAs per SM of three sets (256 tensor-memory columns each) took the place of three CTAs
-// whose eight epilogue warps shared every tile by column halves behind one C buffer: the waits,
-// fences and hand-offs are then paid once per 32 entries of a thread instead of once per 16, and
-// no set waits for another to read C.  n = 50,000, d = 8, M = 17: 1.224 -> 0.99 ms.
+// What bounds it: the epilogue's issue slots and the chain W, C -> epilogue -> P Z -> refill of
+// each set.  n = 50,000, d = 8, M = 17 (kernel alone): 1.224 ms with eight epilogue warps that
+// shared every tile by column halves behind one C buffer and one divergent issuing lane (three
+// CTAs per SM); 0.976 ms with the sets and one uniform issuing warp (two CTAs of 256
+// tensor-memory columns); 0.64 ms with the left operands in tensor memory (an MMA with A in shared
+// memory takes 40 clocks, 16 otherwise) and an issuing warp per stream.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -56,8 +59,7 @@ namespace ulisse {
 
 constexpr int kGtBN = 32;
 constexpr int kGtBM = 128;
-constexpr int kGtSets = 3;         // epilogue sets of four warps
-constexpr int kGtThreads = 32 * (1 + 4 * kGtSets);   // warp 0 copies and MMAs, then the epilogue
+constexpr int kGtIssuers = 3;      // warps 0-2: C; W; P Z and the copies
 constexpr uint32_t kGtCols = 256;  // tensor-memory columns per CTA (two CTAs per SM)
 static_assert(16 * 8 + 48 <= kGtScratchRows, "operand images exceed the gradient scratch");
 
@@ -159,11 +161,17 @@ struct GtDevArgs {
 template <int DP, int KS>
 struct GtShape {
   static constexpr bool XC = DP <= 8;
+  // epilogue sets of four warps: three; two for padded d = 16, whose cross term needs registers
+  static constexpr int SETS = XC ? 3 : 2;
+  static constexpr int THREADS = 32 * (kGtIssuers + 4 * SETS);
+  // the left operands [A^ | B]_I and A_I in tensor memory (128 factor slots leave no room: then
+  // they stay in shared memory)
+  static constexpr bool TS = KS <= 4;
   static constexpr int K1 = 16 * KS;                   // factor slots (2M), padded
   static constexpr int N2 = (2 * DP + 1 + 15) / 16 * 16;
   static constexpr int K8 = 8;                         // columns of the TF32 row images
-  static constexpr uint32_t A_BYTES = kGtBM * K1 * 2;  // one part of A^_I
-  static constexpr uint32_t XA_BYTES = XC ? kGtBM * K8 * 4 : 0;   // one part of A_I (TF32)
+  static constexpr uint32_t A_BYTES = TS ? 0 : kGtBM * K1 * 2;           // one part of A^_I
+  static constexpr uint32_t XA_BYTES = XC && !TS ? kGtBM * K8 * 4 : 0;   // one part of A_I (TF32)
   static constexpr uint32_t X_BYTES = XC ? 2 * kGtBN * K8 * 4 : kGtBN * DP * 4;
   static constexpr uint32_t XB_BYTES = kGtBN * K8 * 4;  // one part of B_J (TF32)
   static constexpr uint32_t BN_BYTES = kGtBN * 4;
@@ -175,27 +183,34 @@ struct GtShape {
   static constexpr uint32_t OFF_BT = OFF_BN + BN_BYTES;
   static constexpr uint32_t OFF_Z = OFF_BT + 2 * BT_BYTES;
   static constexpr uint32_t STAGE_BYTES = OFF_Z + 2 * Z_BYTES;
-  // cw_full, p_full, b_free per set; done
-  static constexpr int NBARS_FIXED = 3 * kGtSets + 1;
-  static constexpr uint32_t FIXED = 2 * A_BYTES + 2 * XA_BYTES + (6 + NBARS_FIXED) * 8 + 64;
-  // as many stages (3 to 6) as let two CTAs share the SM's 228 KB, else as fit one
+  // C buffers: two while they fit beside the left operands, else one
+  static constexpr int NC = !XC ? 0 : KS == 4 ? 1 : 2;
+  // c_full per tile mod 6: each barrier then serves one set, whose waits visit its phases in
+  // order whatever the number of buffers
+  static constexpr int NCF = 2 * SETS;
+  // w_full, p_full, b_free per set; c_full; c_free per buffer; done
+  static constexpr int NBARS_FIXED = 3 * SETS + NCF + 2 + 1;
+  static constexpr uint32_t FIXED = 2 * A_BYTES + 2 * XA_BYTES + (8 + NBARS_FIXED) * 8 + 64;
+  // as many stages (3 to 8) as let two CTAs share the SM's 228 KB, else as fit one
   static constexpr int fit(uint32_t budget) { return (int)((budget - FIXED) / STAGE_BYTES); }
-  static constexpr uint32_t kHalfSm = 110u * 1024u, kWholeSm = 222u * 1024u;
+  static constexpr uint32_t kHalfSm = 108u * 1024u, kWholeSm = 220u * 1024u;
   static constexpr int ST_HALF = FIXED < kHalfSm ? fit(kHalfSm) : 0;
-  static constexpr int OCC = ST_HALF >= kGtSets ? 2 : 1;   // CTAs per SM
+  static constexpr int OCC = ST_HALF > SETS ? 2 : 1;   // CTAs per SM
   static constexpr int ST_ANY = OCC == 2 ? ST_HALF : fit(kWholeSm);
-  static constexpr int ST = ST_ANY > 6 ? 6 : ST_ANY;
-  static_assert(ST >= kGtSets, "each set's next tile needs a stage");
+  static constexpr int ST = ST_ANY > 8 ? 8 : ST_ANY;
+  static_assert(ST > SETS, "a stage beyond those in flight");
   static constexpr uint32_t OFF_XA = 2 * A_BYTES;
   static constexpr uint32_t OFF_STAGES = OFF_XA + 2 * XA_BYTES;
   static constexpr uint32_t OFF_BARS = OFF_STAGES + ST * STAGE_BYTES;
   static constexpr int NBARS = ST + NBARS_FIXED;    // full per stage, then the fixed ones
   static constexpr uint32_t SMEM = OFF_BARS + NBARS * 8 + 64;
-  // tensor-memory columns: the sets' W/P buffers of 32, their C buffers of 32 (XC), then the
-  // [G | H | S] accumulator
-  static constexpr uint32_t COL_C = 32 * kGtSets;
-  static constexpr uint32_t COL_D2 = XC ? 64 * kGtSets : 32 * kGtSets;
-  static_assert(COL_D2 + N2 <= kGtCols, "tensor memory layout exceeds the allocation");
+  // tensor-memory columns: the sets' W/P buffers of 32, the C buffers of 32, the [G | H | S]
+  // accumulator, then the left operands' high and low parts
+  static constexpr uint32_t COL_C = 32 * SETS;
+  static constexpr uint32_t COL_D2 = COL_C + 32 * NC;
+  static constexpr uint32_t COL_A = COL_D2 + N2;             // two BF16 per column
+  static constexpr uint32_t COL_XA = COL_A + (TS ? K1 : 0);
+  static_assert(COL_XA + (TS && XC ? 2 * K8 : 0) <= kGtCols, "tensor memory layout exceeds the allocation");
   static_assert(X_BYTES % 16 == 0 && STAGE_BYTES % 16 == 0 && A_BYTES % 16 == 0 &&
                     OFF_BT % 16 == 0 && OFF_Z % 16 == 0 && OFF_STAGES % 16 == 0,
                 "bulk copies and descriptors need 16-byte alignment");
@@ -223,7 +238,7 @@ __device__ inline void gt_tmem_ld16_two(uint32_t ta, uint32_t tb, uint32_t (&r)[
 template <int DP, int KS>
 __device__ __forceinline__ void gt_body(const GtDevArgs& a, const int rb, const int sp) {
   using S = GtShape<DP, KS>;
-  constexpr int ST = S::ST, K1 = S::K1, N2 = S::N2;
+  constexpr int ST = S::ST, K1 = S::K1, N2 = S::N2, SETS = S::SETS;
   constexpr int NACC = DP + 2;
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ double s_red[4][NACC];
@@ -232,15 +247,17 @@ __device__ __forceinline__ void gt_body(const GtDevArgs& a, const int rb, const 
   const uint32_t smem0 = smem_u32(smem);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S::OFF_BARS);
   uint64_t* full = bars;
-  uint64_t* cw_full = bars + ST;           // W (and C) of the set's tile formed (MMA commit)
-  uint64_t* p_full = cw_full + kGtSets;    // P written by the set's four warps
-  uint64_t* b_free = p_full + kGtSets;     // P Z of the set's tile done (MMA commit)
-  uint64_t* done = b_free + kGtSets;
+  uint64_t* w_full = bars + ST;            // W of the set's tile formed (MMA commit)
+  uint64_t* p_full = w_full + SETS;     // P written by the set's four warps
+  uint64_t* b_free = p_full + SETS;     // P Z of the set's tile done (MMA commit)
+  uint64_t* c_full = b_free + SETS;     // C of the tile formed (MMA commit), tile mod NCF
+  uint64_t* c_free = c_full + S::NCF;      // C read by the set's four warps, per buffer
+  uint64_t* done = c_free + 2;
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + S::OFF_BARS + S::NBARS * 8);
   volatile int* s_fail = reinterpret_cast<volatile int*>(s_tmem + 1);
   int* s_last = reinterpret_cast<int*>(s_tmem + 2);
-  const uint32_t full0 = smem_u32(full), cw_full0 = smem_u32(cw_full),
-                 p_full0 = smem_u32(p_full), b_free0 = smem_u32(b_free);
+  const uint32_t full0 = smem_u32(full), w_full0 = smem_u32(w_full), p_full0 = smem_u32(p_full),
+                 b_free0 = smem_u32(b_free), c_full0 = smem_u32(c_full), c_free0 = smem_u32(c_free);
 
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform for the compiler
@@ -256,39 +273,42 @@ __device__ __forceinline__ void gt_body(const GtDevArgs& a, const int rb, const 
   const int nt = max(0, min(tile_begin + per, a.ntiles) - tile_begin);
 
   // [A^_I | B_I]: slot m < M holds sa[m] a_m[i], slot M + m holds b_m[i]; split into BF16
-  // high and low parts (K-major canonical image).
-  for (int idx = tid; idx < kGtBM * K1; idx += kGtThreads) {
-    const int m = idx / kGtBM, il = idx - m * kGtBM;
-    const long long i = row0 + il;
-    float v = 0.f;
-    if (i < a.n) {
-      if (m < a.M) v = a.sa[m] * a.A[(long long)a.amap[m] * a.ld + i];
-      else if (m < 2 * a.M) v = a.B[(long long)a.bmap[m - a.M] * a.ld + i];
+  // high and low parts
+  auto left = [&](int m, long long i) -> float {
+    if (i >= a.n) return 0.f;
+    if (m < a.M) return a.sa[m] * a.A[(long long)a.amap[m] * a.ld + i];
+    return m < 2 * a.M ? a.B[(long long)a.bmap[m - a.M] * a.ld + i] : 0.f;
+  };
+  if constexpr (!S::TS) {   // K-major canonical images in shared memory
+    for (int idx = tid; idx < kGtBM * K1; idx += S::THREADS) {
+      const int m = idx / kGtBM, il = idx - m * kGtBM;
+      __nv_bfloat16 h, l;
+      split_bf16(left(m, row0 + il), h, l);
+      const uint32_t off = tc::canon_offset(il, m, 2, K1 / 8);
+      *reinterpret_cast<__nv_bfloat16*>(sAh + off) = h;
+      *reinterpret_cast<__nv_bfloat16*>(sAl + off) = l;
     }
-    __nv_bfloat16 h, l;
-    split_bf16(v, h, l);
-    const uint32_t off = tc::canon_offset(il, m, 2, K1 / 8);
-    *reinterpret_cast<__nv_bfloat16*>(sAh + off) = h;
-    *reinterpret_cast<__nv_bfloat16*>(sAl + off) = l;
+    if constexpr (S::XC) {
+      // A_I's TF32 image (high part, then remainder): 128 rows of the packed images, which
+      // are zero beyond n
+      constexpr int kQ = kGtBM * S::K8 / 4;   // float4 per part
+      float4* sx = reinterpret_cast<float4*>(smem + S::OFF_XA);
+      const float4* gh = reinterpret_cast<const float4*>(a.XA_hi + row0 * S::K8);
+      const float4* gl = reinterpret_cast<const float4*>(a.XA_lo + row0 * S::K8);
+      for (int idx = tid; idx < 2 * kQ; idx += S::THREADS)
+        sx[idx] = idx < kQ ? gh[idx] : gl[idx - kQ];
+    }
+    tc::fence_async_smem();
   }
-  if constexpr (S::XC) {
-    // A_I's TF32 image (high part, then remainder): 128 rows of the packed images, which
-    // are zero beyond n
-    constexpr int kQ = kGtBM * S::K8 / 4;   // float4 per part
-    float4* sx = reinterpret_cast<float4*>(smem + S::OFF_XA);
-    const float4* gh = reinterpret_cast<const float4*>(a.XA_hi + row0 * S::K8);
-    const float4* gl = reinterpret_cast<const float4*>(a.XA_lo + row0 * S::K8);
-    for (int idx = tid; idx < 2 * kQ; idx += kGtThreads)
-      sx[idx] = idx < kQ ? gh[idx] : gl[idx - kQ];
-  }
-  tc::fence_async_smem();
   if (tid == 0) {
     for (int s = 0; s < ST; ++s) mbar_init(&full[s], 1);
-    for (int h = 0; h < kGtSets; ++h) {
-      mbar_init(&cw_full[h], 1);
+    for (int h = 0; h < SETS; ++h) {
+      mbar_init(&w_full[h], 1);
       mbar_init(&p_full[h], 4);
       mbar_init(&b_free[h], 1);
     }
+    for (int c = 0; c < S::NCF; ++c) mbar_init(&c_full[c], 1);
+    for (int c = 0; c < 2; ++c) mbar_init(&c_free[c], 4);
     mbar_init(done, 1);
     fence_barrier_init();
     *s_fail = 0;
@@ -298,25 +318,131 @@ __device__ __forceinline__ void gt_body(const GtDevArgs& a, const int rb, const 
   __syncthreads();
   tc::fence_after();
   const uint32_t tbase = __shfl_sync(0xffffffffu, *s_tmem, 0);
-  int issued = 0;   // tiles whose copies were started (warp 0)
+  if (S::TS && warp >= kGtIssuers && warp < kGtIssuers + 4) {
+    // the left operands into tensor memory, a row per thread (an MMA whose A comes from shared
+    // memory takes 40 clocks for its 4 KB, from tensor memory 16)
+    const int eq = warp & 3;
+    const long long i = row0 + eq * 32 + lane;
+    const uint32_t dst = tbase + ((uint32_t)(eq * 32) << 16);
+#pragma unroll 1
+    for (int ks = 0; ks < KS; ++ks) {
+      uint32_t hi[8], lo[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const float v0 = left(16 * ks + 2 * q, i), v1 = left(16 * ks + 2 * q + 1, i);
+        const __nv_bfloat162 h = __floats2bfloat162_rn(v0, v1);
+        const float2 hf = __bfloat1622float2(h);
+        const __nv_bfloat162 l = __floats2bfloat162_rn(v0 - hf.x, v1 - hf.y);
+        hi[q] = *reinterpret_cast<const uint32_t*>(&h);
+        lo[q] = *reinterpret_cast<const uint32_t*>(&l);
+      }
+      tc::tmem_st8(dst + S::COL_A + 8u * ks, hi);
+      tc::tmem_st8(dst + S::COL_A + (uint32_t)(K1 / 2) + 8u * ks, lo);
+    }
+    if constexpr (S::XC) {
+      const long long off =
+          (i / 32) * 32 * S::K8 + tc::canon_offset((int)(i % 32), 0, 4, S::K8 / 4) / 4;
+#pragma unroll
+      for (int part = 0; part < 2; ++part) {
+        const float* src = (part == 0 ? a.XA_hi : a.XA_lo) + off;
+        const uint4 x = *reinterpret_cast<const uint4*>(src);
+        const uint4 y = *reinterpret_cast<const uint4*>(src + 32);
+        const uint32_t v[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+        tc::tmem_st8(dst + S::COL_XA + (uint32_t)(part * S::K8), v);
+      }
+    }
+    tc::tmem_wait_st();
+  }
+  if constexpr (S::TS) {
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+  }
+  int issued = 0;   // tiles whose copies were started (warp 2)
 
   double acc[NACC];
 #pragma unroll
   for (int k = 0; k < NACC; ++k) acc[k] = 0.0;
 
+  // Three issuing warps, so that no stream of MMAs and waits holds up another: the loops run
+  // warp-uniformly, one elected lane issues.
   if (warp == 0) {
-    // ------ copies and MMAs: W = A^ B^T and C = A B^T, then [G | H | S] += P Z ------
+    // ------ C_J = A_I B_J^T (three TF32 products, K = 8) ------
+    if constexpr (S::XC) {
+      constexpr uint32_t idesc_c = tc::instr_desc(2, kGtBM, kGtBN);   // TF32
+      constexpr uint32_t sbo_x = (S::K8 / 4) * 128;
+      const uint64_t dXA0 = tc::smem_desc(smem0 + S::OFF_XA, 128, sbo_x);
+      const uint64_t dXB0 = tc::smem_desc(smem0 + S::OFF_STAGES, 128, sbo_x);
+      bool ok = true;
+      int s = 0, ph_s = 0, c = 0, ph_c = 1, cf = 0;   // ph_c: parity of the buffer's last release
+#pragma unroll 1
+      for (int p = 0; p < nt; ++p) {
+        ok = tc::warp_wait_uniform(full0 + 8u * s, ph_s) &&
+             (p < S::NC || tc::warp_wait_uniform(c_free0 + 8u * c, ph_c));
+        if (!ok) break;
+        tc::fence_after();
+        if (tc::elect_one()) {
+          const uint64_t so = (uint64_t)s * (S::STAGE_BYTES >> 4);
+          const uint32_t dC = tbase + S::COL_C + (uint32_t)(c * 32);
+#pragma unroll
+          for (int term = 0; term < 3; ++term) {
+            const uint64_t B = dXB0 + so + (term == 1 ? (S::XB_BYTES >> 4) : 0u);
+            if constexpr (S::TS)
+              tc::mma_tf32_ts(dC, tbase + S::COL_XA + (term == 2 ? (uint32_t)S::K8 : 0u), B, idesc_c,
+                              term != 0);
+            else
+              tc::mma_tf32(dC, dXA0 + (term == 2 ? (S::XA_BYTES >> 4) : 0u), B, idesc_c, term != 0);
+          }
+          tc::commit(&c_full[cf]);
+        }
+        __syncwarp();
+        if (++s == ST) { s = 0; ph_s ^= 1; }
+        if (++c == S::NC) { c = 0; ph_c ^= 1; }
+        if (++cf == S::NCF) cf = 0;
+      }
+      if (!ok) *s_fail = 1;
+    }
+  } else if (warp == 1) {
+    // ------ W = A^ B^T ------
     constexpr uint32_t idesc_w = tc::instr_desc(1, kGtBM, kGtBN);
-    constexpr uint32_t idesc_g = tc::instr_desc(1, kGtBM, N2);
-    constexpr uint32_t idesc_c = tc::instr_desc(2, kGtBM, kGtBN);   // TF32
     constexpr uint32_t sbo_k1 = (K1 / 8) * 128;
-    constexpr uint32_t sbo_x = (S::K8 / 4) * 128;
-    const uint64_t dAh = tc::smem_desc(smem0, 128, sbo_k1);
-    const uint64_t dAl = tc::smem_desc(smem0 + S::A_BYTES, 128, sbo_k1);
-    const uint64_t dXAh = tc::smem_desc(smem0 + S::OFF_XA, 128, sbo_x);
-    const uint64_t dXAl = tc::smem_desc(smem0 + S::OFF_XA + S::XA_BYTES, 128, sbo_x);
-    const uint64_t dXB0 = tc::smem_desc(smem0 + S::OFF_STAGES, 128, sbo_x);
+    const uint64_t dA0 = tc::smem_desc(smem0, 128, sbo_k1);
     const uint64_t dBT0 = tc::smem_desc(smem0 + S::OFF_STAGES + S::OFF_BT, 128, sbo_k1);
+    bool ok = true;
+    int s = 0, ph_s = 0, h = 0, ph_h = 1;   // ph_h: parity of the buffer's last release
+#pragma unroll 1
+    for (int p = 0; p < nt; ++p) {
+      ok = tc::warp_wait_uniform(full0 + 8u * s, ph_s) &&
+           (p < SETS || tc::warp_wait_uniform(b_free0 + 8u * h, ph_h));
+      if (!ok) break;
+      tc::fence_after();
+      if (tc::elect_one()) {
+        const uint64_t dBT = dBT0 + (uint64_t)s * (S::STAGE_BYTES >> 4);
+        const uint32_t dW = tbase + (uint32_t)(h * 32);
+#pragma unroll
+        for (int term = 0; term < 3; ++term) {
+          const uint64_t B = dBT + (term == 1 ? (S::BT_BYTES >> 4) : 0u);
+#pragma unroll
+          for (int ks = 0; ks < KS; ++ks) {
+            if constexpr (S::TS)
+              tc::mma_bf16_ts(dW, tbase + S::COL_A + (term == 2 ? (uint32_t)(K1 / 2) : 0u) + 8u * ks,
+                              B + 16u * ks, idesc_w, (term | ks) != 0);
+            else
+              tc::mma_bf16(dW, dA0 + (term == 2 ? (S::A_BYTES >> 4) : 0u) + 16u * ks, B + 16u * ks,
+                           idesc_w, (term | ks) != 0);
+          }
+        }
+        tc::commit(&w_full[h]);
+      }
+      __syncwarp();
+      if (++s == ST) { s = 0; ph_s ^= 1; }
+      if (++h == SETS) { h = 0; ph_h ^= 1; }
+    }
+    if (!ok) *s_fail = 1;
+  } else if (warp == 2) {
+    // ------ [G | H | S] += P Z, and the copies: a stage is refilled once its tile's P Z, the
+    //        last to read it, is complete (looked at one tile late, when it is) ------
+    constexpr uint32_t idesc_g = tc::instr_desc(1, kGtBM, N2);
     const uint64_t dZ0 = tc::smem_desc(smem0 + S::OFF_STAGES + S::OFF_Z, 128, 512);
     auto copy_tile = [&](int p, int s) {   // elected lane
       const long long t = tile_begin + p;
@@ -330,47 +456,18 @@ __device__ __forceinline__ void gt_body(const GtDevArgs& a, const int rb, const 
       }
       bulk_g2s(st + S::OFF_BT, a.tiles + t * (S::TILE_BYTES / 2), S::TILE_BYTES, &full[s]);
     };
-    auto mma_cw = [&](int s, int h) {   // elected lane: W and C of the tile in stage s
-      const uint64_t so = (uint64_t)s * (S::STAGE_BYTES >> 4);
-#pragma unroll
-      for (int term = 0; term < 3; ++term) {
-        const uint64_t A = term == 2 ? dAl : dAh;
-        const uint64_t B = dBT0 + so + (term == 1 ? (S::BT_BYTES >> 4) : 0u);
-#pragma unroll
-        for (int ks = 0; ks < KS; ++ks)
-          tc::mma_bf16(tbase + (uint32_t)(h * 32), A + 16u * ks, B + 16u * ks, idesc_w,
-                       (term | ks) != 0);
-      }
-      if constexpr (S::XC) {
-        // C_J = A_I B_J^T (three TF32 products, K = 8)
-#pragma unroll
-        for (int term = 0; term < 3; ++term)
-          tc::mma_tf32(tbase + S::COL_C + (uint32_t)(h * 32), term == 2 ? dXAl : dXAh,
-                       dXB0 + so + (term == 1 ? (S::XB_BYTES >> 4) : 0u), idesc_c, term != 0);
-      }
-      tc::commit(&cw_full[h]);
-    };
     const int pre = min(ST, nt);
     if (tc::elect_one())
       for (int p = 0; p < pre; ++p) copy_tile(p, p);
     __syncwarp();
     issued = pre;
     bool ok = true;
-    int s_c = 0, ph_c = 0;   // stage of the next tile whose W and C are issued
-    for (int p = 0; p < kGtSets && p < nt && ok; ++p) {
-      ok = tc::warp_wait_uniform(full0 + 8u * s_c, ph_c);
-      tc::fence_after();
-      if (ok && tc::elect_one()) mma_cw(s_c, p);
-      __syncwarp();
-      if (++s_c == ST) { s_c = 0; ph_c ^= 1; }
-    }
     int s = 0, h = 0, ph_h = 0;
 #pragma unroll 1
-    for (int p = 0; p < nt && ok; ++p) {
+    for (int p = 0; p < nt; ++p) {
       ok = tc::warp_wait_uniform(p_full0 + 8u * h, ph_h);
       if (!ok) break;
       tc::fence_after();
-      const bool more_w = p + kGtSets < nt, more_t = p + ST < nt;
       if (tc::elect_one()) {
         const uint64_t dZ = dZ0 + (uint64_t)s * (S::STAGE_BYTES >> 4);
         const uint32_t pcol = tbase + (uint32_t)(h * 32);
@@ -383,28 +480,19 @@ __device__ __forceinline__ void gt_body(const GtDevArgs& a, const int rb, const 
             tc::mma_bf16_ts(tbase + S::COL_D2, A + ks * 16, B + 16u * ks, idesc_g,
                             (p | term | ks) != 0);
         }
-        // the set's buffers take tile p + 3's W and C, and stage s tile p + ST's operands, only
-        // after these MMAs have read P and Z
-        if (more_w || more_t) tc::commit(&b_free[h]);
+        tc::commit(&b_free[h]);
       }
       __syncwarp();
-      if (more_w || more_t) {
-        ok = tc::warp_wait_uniform(b_free0 + 8u * h, ph_h);
-        if (ok && more_w) {
-          ok = tc::warp_wait_uniform(full0 + 8u * s_c, ph_c);
-          tc::fence_after();
-          if (ok && tc::elect_one()) mma_cw(s_c, h);
-          __syncwarp();
-          if (++s_c == ST) { s_c = 0; ph_c ^= 1; }
-        }
-        if (ok && more_t) {
-          if (tc::elect_one()) copy_tile(p + ST, s);
-          __syncwarp();
-          issued = p + ST + 1;
-        }
+      if (p >= 1 && p - 1 + ST < nt) {
+        const int hp = h == 0 ? SETS - 1 : h - 1, s1 = s == 0 ? ST - 1 : s - 1;
+        ok = tc::warp_wait_uniform(b_free0 + 8u * hp, (uint32_t)(((p - 1) / SETS) & 1));
+        if (!ok) break;
+        if (tc::elect_one()) copy_tile(p - 1 + ST, s1);
+        __syncwarp();
+        issued = p + ST;
       }
       if (++s == ST) s = 0;
-      if (++h == kGtSets) { h = 0; ph_h ^= 1; }
+      if (++h == SETS) { h = 0; ph_h ^= 1; }
     }
     if (!ok) *s_fail = 1;
     // a CTA with an empty range issues nothing and waits on nothing
@@ -413,7 +501,7 @@ __device__ __forceinline__ void gt_body(const GtDevArgs& a, const int rb, const 
   } else {
     // ------ epilogue: warp (lane quadrant eq, set h) takes the tiles h, h + 3, ... whole ------
     const int eq = warp & 3;
-    const int set = (warp - 1) >> 2;
+    const int set = (warp - kGtIssuers) >> 2;
     const int il = eq * 32 + lane;
     const long long i = row0 + il;
     const uint32_t lane_base = (uint32_t)(eq * 32) << 16;
@@ -430,12 +518,14 @@ __device__ __forceinline__ void gt_body(const GtDevArgs& a, const int rb, const 
     const float2 ai2 = make_float2(ai, ai);
     bool ok = true;
     int s = set, ph_s = 0, ph = 0;   // set < ST
+    int c = S::NC > 0 ? set % S::NC : 0, cf = set, ph_cf = 0;
 #pragma unroll 1
-    for (int lt = set; lt < nt; lt += kGtSets) {
+    for (int lt = set; lt < nt; lt += SETS) {
       // b_J (and x^_J) are read from the stage: wait for its copy too (the stage is refilled
       // only after this tile's P Z, which waits for this warp's P)
-      ok = tc::warp_wait_uniform(cw_full0 + 8u * set, ph) &&
+      ok = tc::warp_wait_uniform(w_full0 + 8u * set, ph) &&
            tc::warp_wait_uniform(full0 + 8u * s, ph_s);
+      if constexpr (S::XC) ok = ok && tc::warp_wait_uniform(c_full0 + 8u * cf, ph_cf);
       if (!ok) break;
       tc::fence_after();
       const bool own = tile_begin + lt < diag_end;   // a tile of I itself: weight 1/2
@@ -448,7 +538,12 @@ __device__ __forceinline__ void gt_body(const GtDevArgs& a, const int rb, const 
         float w[16], cx[S::XC ? 16 : 1];
         if constexpr (S::XC) {
           uint32_t r[32];
-          gt_tmem_ld16_two(wcol, wcol + S::COL_C, r);
+          gt_tmem_ld16_two(wcol, tbase + lane_base + S::COL_C + (uint32_t)(c * 32 + half * 16), r);
+          if (half == 1) {   // the C buffer may take its next tile
+            tc::fence_before();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&c_free[c]);
+          }
 #pragma unroll
           for (int q = 0; q < 16; ++q) {
             w[q] = __uint_as_float(r[q]);
@@ -511,8 +606,13 @@ __device__ __forceinline__ void gt_body(const GtDevArgs& a, const int rb, const 
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&p_full[set]);
       ph ^= 1;
-      s += kGtSets;
+      s += SETS;
       if (s >= ST) { s -= ST; ph_s ^= 1; }
+      if constexpr (S::XC) {
+        c = (c + SETS) % S::NC;
+        cf += SETS;
+        if (cf >= S::NCF) { cf -= S::NCF; ph_cf ^= 1; }
+      }
     }
     if (!ok) *s_fail = 1;
     const bool fin = ok && (nt == 0 || tc::warp_wait_uniform(smem_u32(done), 0));
@@ -564,15 +664,16 @@ __device__ __forceinline__ void gt_body(const GtDevArgs& a, const int rb, const 
     return;
   }
   // set 0 holds the lengthscale and sigma^2 sums, set 1 the diagonal's
-  if (warp >= 1 && warp <= 4) {
+  const int ew = warp - kGtIssuers;
+  if (ew >= 0 && ew < 4) {
 #pragma unroll
     for (int k = 0; k <= DP; ++k) {
       const double v = warp_sum(acc[k]);
-      if (lane == 0) s_red[warp - 1][k] = v;
+      if (lane == 0) s_red[ew][k] = v;
     }
-  } else if (warp >= 5 && warp <= 8) {
+  } else if (ew >= 4 && ew < 8) {
     const double v = sp == 0 ? warp_sum(acc[DP + 1]) : 0.0;
-    if (lane == 0) s_red[warp - 5][DP + 1] = v;
+    if (lane == 0) s_red[ew - 4][DP + 1] = v;
   }
   __syncthreads();
   double* part = a.partials + slot * kMaxP;
@@ -590,14 +691,14 @@ __device__ __forceinline__ void gt_body(const GtDevArgs& a, const int rb, const 
   __syncthreads();
   if (!*s_last) return;
   __threadfence();
-  __shared__ double s_sum[kGtThreads];
-  const double v = sum_partial_rows<kGtThreads>(a.partials, a.n_cta, a.d + 2, s_sum);
+  __shared__ double s_sum[S::THREADS];
+  const double v = sum_partial_rows<S::THREADS>(a.partials, a.n_cta, a.d + 2, s_sum);
   if (tid < a.d + 2) a.g_out[tid] = tid == a.d + 1 ? v * a.params->lambda : v;
   if (tid == 0) *a.counter = 0;
 }
 
 template <int DP, int KS>
-__global__ void __launch_bounds__(kGtThreads, GtShape<DP, KS>::OCC) grad_tc_kernel(const GtDevArgs a) {
+__global__ void __launch_bounds__(GtShape<DP, KS>::THREADS, GtShape<DP, KS>::OCC) grad_tc_kernel(const GtDevArgs a) {
   const int rb = blockIdx.x / a.nsplit;
   gt_body<DP, KS>(a, rb, blockIdx.x - rb * a.nsplit);
 }
@@ -605,7 +706,7 @@ __global__ void __launch_bounds__(kGtThreads, GtShape<DP, KS>::OCC) grad_tc_kern
 // Many problems of one input width in one launch: CTA b takes work item items[b] =
 // (problem, row block, split) with that problem's arguments.
 template <int DP, int KS>
-__global__ void __launch_bounds__(kGtThreads, GtShape<DP, KS>::OCC) grad_tc_batch_kernel(
+__global__ void __launch_bounds__(GtShape<DP, KS>::THREADS, GtShape<DP, KS>::OCC) grad_tc_batch_kernel(
     const GtDevArgs* __restrict__ args, const int4* __restrict__ items) {
   __shared__ GtDevArgs s_a;
   const int4 it = items[blockIdx.x];
@@ -718,7 +819,7 @@ struct GtInst {
     a.counter = L.counter;
     a.g_out = L.g_out;
     a.status = L.status;
-    grad_tc_kernel<DP, KS><<<n_rb * nsplit, kGtThreads, S::SMEM, s>>>(a);
+    grad_tc_kernel<DP, KS><<<n_rb * nsplit, S::THREADS, S::SMEM, s>>>(a);
     return cudaGetLastError();
   }
 };
@@ -795,7 +896,7 @@ static cudaError_t gt_batch_launch(const GtDevArgs* args, int B, const int4* ite
   if (prime_only) return cudaSuccess;
   pack_gt_batch_kernel<DP, KS><<<dim3(64, (unsigned)B), 256, 0, s>>>(args);
   if (n_items > 0)
-    grad_tc_batch_kernel<DP, KS><<<n_items, kGtThreads, GtShape<DP, KS>::SMEM, s>>>(args, items);
+    grad_tc_batch_kernel<DP, KS><<<n_items, GtShape<DP, KS>::THREADS, GtShape<DP, KS>::SMEM, s>>>(args, items);
   return cudaGetLastError();
 }
 
