@@ -17,6 +17,15 @@
 
 using namespace ulisse;
 
+// What a call hands back to the host, in one block on the device and one in pinned memory: one
+// copy and one synchronisation return all of it.
+struct ResultBlock {
+  double psi[kMaxP];
+  double g[kMaxP];
+  int status;
+  int n_live;
+};
+
 struct ulisse_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
@@ -43,6 +52,8 @@ struct ulisse_ctx {
   double* psi_dev = nullptr;  // kMaxP
   PsiArg psi_arg{};           // by_value: psi of a host call, handed to the next prescale launch
 
+  ResultBlock* result = nullptr;     // device; psi_dev, g_dev, status_dev, n_live_dev lie in it
+  ResultBlock* h_result = nullptr;   // pinned
   void* fixed_block = nullptr;   // the allocation of the buffers of fixed size
   void* col_block = nullptr;     // ... and of the column buffers
   int cap = 0;                // column capacity of B, S, E, D, KD
@@ -61,6 +72,8 @@ struct ulisse_ctx {
   size_t partials_bytes = 0;
   int* counters = nullptr;
   int counters_len = 0;
+  void* fixed_partials = nullptr;   // the first ones, part of fixed_block
+  int* fixed_counters = nullptr;
 
   double* gpart = nullptr;
   size_t gpart_len = 0;
@@ -70,7 +83,6 @@ struct ulisse_ctx {
   int* amap = nullptr;        // gradient left-factor columns
   int* bmap = nullptr;        // gradient right-factor columns
   int grad_nr = -1;           // probe count the maps were built for
-  int* q_map = nullptr;       // ulisse_dk_bilinear: identity column map (kMaxM)
   void* q_sa = nullptr;       // ulisse_dk_bilinear: scales (T), kMaxM
 
   double* M_dev = nullptr;
@@ -400,13 +412,15 @@ static ulisse_status grow_kmv_scratch(ulisse_ctx* ctx, size_t need_bytes, int ne
   ctx->graph_key = -1;
   CK(cudaStreamSynchronize(ctx->stream));
   if (need_bytes > ctx->partials_bytes) {
-    dev_free(ctx->partials);
+    if (ctx->partials != ctx->fixed_partials) dev_free(ctx->partials);
+    ctx->partials = nullptr;
     ctx->partials_bytes = 0;
     CKS(dev_alloc(ctx, &ctx->partials, need_bytes));
     ctx->partials_bytes = need_bytes;
   }
   if (need_counters > ctx->counters_len) {
-    dev_free(reinterpret_cast<void*&>(ctx->counters));
+    if (ctx->counters != ctx->fixed_counters) dev_free(reinterpret_cast<void*&>(ctx->counters));
+    ctx->counters = nullptr;
     ctx->counters_len = 0;
     CKS(dev_alloc(ctx, reinterpret_cast<void**>(&ctx->counters), sizeof(int) * need_counters));
     ctx->counters_len = need_counters;
@@ -569,6 +583,16 @@ static ulisse_status read_status(ulisse_ctx* ctx, int* status) {
   CK(cudaStreamSynchronize(ctx->stream));
   prof_drain(ctx);
   *status = *ctx->h_status;
+  return ULISSE_OK;
+}
+
+// As read_status, with psi and g in h_result.
+static ulisse_status read_result(ulisse_ctx* ctx, int* status) {
+  CK(cudaMemcpyAsync(ctx->h_result, ctx->result, sizeof(ResultBlock), cudaMemcpyDeviceToHost,
+                     ctx->stream));
+  CK(cudaStreamSynchronize(ctx->stream));
+  prof_drain(ctx);
+  *status = ctx->h_result->status;
   return ULISSE_OK;
 }
 
@@ -895,21 +919,23 @@ static void set_grad_images(GradLaunch& L, const ulisse_ctx* c) {
 }
 
 // The fused gradient pass over the columns of SE (left factors, scaled) and B (right factors);
-// the maps and scales default to the gradient's own.
+// the maps and scales default to the gradient's own, the columns (leading dimension ld; the
+// tensor-core pass takes any) to the context's.
 static ulisse_status run_grad(ulisse_ctx* ctx, int M, const int* amap = nullptr,
-                              const void* sa = nullptr, const int* bmap = nullptr) {
+                              const void* sa = nullptr, const int* bmap = nullptr,
+                              const void* A = nullptr, const void* B = nullptr, long long ld = 0) {
   GradLaunch L{};
   L.xhat = ctx->xhat;
   L.n = ctx->n;
   L.ldn = ctx->ldn;
   L.d = ctx->d;
   L.DP = ctx->DP;
-  L.A = ctx->SE;
+  L.A = A ? A : ctx->SE;
   L.amap = amap ? amap : ctx->amap;
   L.sa = sa ? sa : ctx->sa_dev;
-  L.B = ctx->B;
+  L.B = B ? B : ctx->B;
   L.bmap = bmap ? bmap : ctx->bmap;
-  L.ld = ctx->ldn;
+  L.ld = ld > 0 ? ld : ctx->ldn;
   L.M = M;
   L.params = ctx->params;
   L.exp_tab = ctx->exp_tab;
@@ -1047,6 +1073,14 @@ static ulisse_status check_cfg(const ulisse_config* c) {
   return ULISSE_OK;
 }
 
+// Split-j scratch to begin with: what a product of at most 32 columns takes (FP64: the pair form
+// of a gradient's columns), where that is at most 64 MiB.
+static size_t initial_partials(const ulisse_ctx* ctx) {
+  const size_t b = ctx->f64 ? kmv_f64_sym_bytes(ctx->n, std::min(1 + ctx->cfg.n_probes, kMaxRChunk))
+                            : kmv_tile_partial_bytes(ctx->n, ctx->num_sms, ctx->mixed);
+  return b <= (64u << 20) ? b : 0;
+}
+
 static ulisse_status create_impl(ulisse_ctx** out, const float* X, const float* y, long long n,
                                  int d, const ulisse_config* cfg, void* stream,
                                  cudaMemcpyKind kind, bool in_batch = false) {
@@ -1084,16 +1118,14 @@ static ulisse_status create_impl(ulisse_ctx** out, const float* X, const float* 
   cv.add(ctx->y, ctx->ldn * ctx->esz);
   cv.add(ctx->xhat, ctx->ldn * ctx->DP * ctx->esz);
   cv.add(ctx->params, sizeof(DevParams));
-  cv.add(ctx->psi_dev, sizeof(double) * kMaxP);
-  cv.add(ctx->n_live_dev, sizeof(int));
+  cv.add(ctx->result, sizeof(ResultBlock));
+  cv.add(ctx->q_sa, sizeof(double) * kMaxM);
   cv.add(ctx->gcounter, sizeof(int));
-  cv.add(ctx->g_dev, sizeof(double) * kMaxP);
   cv.add(ctx->sa_dev, sizeof(double) * kMaxM);
   cv.add(ctx->amap, sizeof(int) * kMaxM);
   cv.add(ctx->bmap, sizeof(int) * kMaxM);
   cv.add(ctx->M_dev, sizeof(double) * kMaxP * kMaxP);
   cv.add(ctx->prior_dev, sizeof(double) * kMaxP);
-  cv.add(ctx->status_dev, sizeof(int));
   cv.add(ctx->warm_valid, sizeof(int));
   if (ctx->mixed) {
     cv.add(ctx->bneg, sizeof(float) * ctx->ld128);
@@ -1106,16 +1138,29 @@ static ulisse_status create_impl(ulisse_ctx** out, const float* X, const float* 
   if (!ctx->f64 && !ctx->mixed && !in_batch && n >= kF32TcMinN)
     cv.add(ctx->v3, 2 * 3 * kMaxRChunk * ctx->ldn);
   if (ctx->f64) cv.add(ctx->exp_tab, sizeof(double) * kExpTabN);
+  // split-j scratch for the widest usual product, so that no first call has to allocate it (a
+  // batch's launches have their own)
+  ctx->partials_bytes = in_batch ? 0 : initial_partials(ctx);
+  ctx->counters_len = (int)((n + 31) / 32);
+  cv.add(ctx->partials, ctx->partials_bytes);
+  cv.add(ctx->counters, sizeof(int) * ctx->counters_len);
   if ((s = carve_alloc(ctx, cv, &ctx->fixed_block))) return bail(s);
+  ctx->fixed_partials = ctx->partials;
+  ctx->fixed_counters = ctx->counters;
+  ctx->psi_dev = ctx->result->psi;   // device addresses
+  ctx->g_dev = ctx->result->g;
+  ctx->status_dev = &ctx->result->status;
+  ctx->n_live_dev = &ctx->result->n_live;
   if (ctx->f64 && launch_fill_exp_tab(ctx->exp_tab, ctx->stream) != cudaSuccess) {
     ctx->err = "table launch failed";
     return bail(ULISSE_ERR_CUDA);
   }
-  if (cudaMallocHost(&ctx->h_n_live, sizeof(int)) != cudaSuccess ||
-      cudaMallocHost(&ctx->h_status, sizeof(int)) != cudaSuccess) {
+  if (cudaMallocHost(&ctx->h_result, sizeof(ResultBlock)) != cudaSuccess) {
     ctx->err = "cudaMallocHost failed";
     return bail(ULISSE_ERR_NOMEM);
   }
+  ctx->h_status = &ctx->h_result->status;
+  ctx->h_n_live = &ctx->h_result->n_live;
   // Inputs: X as given (row-major float); y into the context's element type.
   if (cudaMemcpyAsync(ctx->X, X, sizeof(float) * n * d, kind, ctx->stream) != cudaSuccess) {
     ctx->err = "copy of X failed";
@@ -1339,11 +1384,10 @@ ulisse_status ulisse_grad(ulisse_ctx* ctx, const double* psi, unsigned long long
   CKS(set_psi_host(ctx, psi));
   CK(cudaMemsetAsync(ctx->status_dev, 0, sizeof(int), ctx->stream));
   CKS(grad_core(ctx, step));
-  CK(cudaMemcpyAsync(g, ctx->g_dev, sizeof(double) * (ctx->d + 2), cudaMemcpyDeviceToHost,
-                     ctx->stream));
   CKS(copy_stats(ctx, stats, 1 + ctx->cfg.n_probes));
   int st = 0;
-  CKS(read_status(ctx, &st));
+  CKS(read_result(ctx, &st));
+  std::memcpy(g, ctx->h_result->g, sizeof(double) * (ctx->d + 2));
   return status_to_result(ctx, st);
 }
 
@@ -1412,46 +1456,32 @@ ulisse_status ulisse_dk_bilinear(ulisse_ctx* ctx, const double* psi, const float
     for (int m = 0; m < M; ++m)
       if (!std::isfinite(scale[m])) return fail(ctx, ULISSE_ERR_ARG, "scale not finite");
   CKS(set_psi_host(ctx, psi));
-  CKS(prescale(ctx));
   CKS(ensure_columns(ctx, M, M));
-  if (!ctx->q_map) {
-    std::vector<int> id(kMaxM);
-    for (int m = 0; m < kMaxM; ++m) id[m] = m;
-    CKS(dev_alloc(ctx, reinterpret_cast<void**>(&ctx->q_map), sizeof(int) * kMaxM));
-    CKS(dev_alloc(ctx, &ctx->q_sa, sizeof(double) * kMaxM));
-    CK(cudaMemcpy(ctx->q_map, id.data(), sizeof(int) * kMaxM, cudaMemcpyHostToDevice));
-  }
-  CK(cudaStreamSynchronize(ctx->stream));   // the scale upload below reuses a host buffer
-  std::vector<double> sd(M, 1.0);
-  std::vector<float> sf(M, 1.f);
-  for (int m = 0; m < M; ++m) {
-    if (scale) sd[m] = scale[m];
-    sf[m] = (float)sd[m];
-  }
-  if (ctx->f64)
-    CK(cudaMemcpy(ctx->q_sa, sd.data(), sizeof(double) * M, cudaMemcpyHostToDevice));
-  else
-    CK(cudaMemcpy(ctx->q_sa, sf.data(), sizeof(float) * M, cudaMemcpyHostToDevice));
-  CK(cudaMemsetAsync(ctx->status_dev, 0, sizeof(int), ctx->stream));
+  CKS(prescale(ctx));
+  // One launch for the scales (by value), the status word and, for the SIMT passes, which copy
+  // whole tiles, the padded factor columns; the tensor-core pass reads A and B in place.
+  BilinearScales sc{};
+  for (int m = 0; m < M; ++m) sc.v[m] = scale ? scale[m] : 1.0;
   const long long n = ctx->n;
-  auto in_cols = [&](const float* src, void* dst) -> ulisse_status {
-    if (!ctx->f64) {
-      CK(cudaMemcpy2DAsync(dst, ctx->ldn * 4, src, n * 4, n * 4, M, cudaMemcpyDeviceToDevice,
-                           ctx->stream));
-    } else {
-      convert_cols_kernel<float, double><<<dim3(64, M), 256, 0, ctx->stream>>>(
-          src, n, (double*)dst, ctx->ldn, n);
-      CK(cudaGetLastError());
-    }
-    return ULISSE_OK;
-  };
-  CKS(in_cols(A, ctx->SE));
-  CKS(in_cols(B, ctx->B));
-  CKS(run_grad(ctx, M, ctx->q_map, ctx->q_sa, ctx->q_map));
-  CK(cudaMemcpyAsync(out, ctx->g_dev, sizeof(double) * (ctx->d + 2), cudaMemcpyDeviceToHost,
-                     ctx->stream));
+  const dim3 grid(ctx->mixed ? 1u : (unsigned)std::min<long long>((n + 1023) / 1024, 64),
+                  ctx->mixed ? 1u : 2u * M);
+  if (ctx->f64)
+    bilinear_prepare_kernel<double><<<grid, 256, 0, ctx->stream>>>(
+        sc, M, (double*)ctx->q_sa, ctx->status_dev, A, (double*)ctx->SE, B, (double*)ctx->B, n,
+        ctx->ldn);
+  else
+    bilinear_prepare_kernel<float><<<grid, 256, 0, ctx->stream>>>(
+        sc, M, (float*)ctx->q_sa, ctx->status_dev, ctx->mixed ? nullptr : A, (float*)ctx->SE, B,
+        (float*)ctx->B, n, ctx->ldn);
+  CK(cudaGetLastError());
+  ctx->launches++;
+  if (ctx->mixed)
+    CKS(run_grad(ctx, M, ctx->iota, ctx->q_sa, ctx->iota, A, B, n));
+  else
+    CKS(run_grad(ctx, M, ctx->iota, ctx->q_sa, ctx->iota));
   int st = 0;
-  CKS(read_status(ctx, &st));
+  CKS(read_result(ctx, &st));
+  std::memcpy(out, ctx->h_result->g, sizeof(double) * (ctx->d + 2));
   return status_to_result(ctx, st);
 }
 
@@ -1497,16 +1527,12 @@ ulisse_status ulisse_sgld_step(ulisse_ctx* ctx, double* psi_inout, double eps_t,
     CK(cudaMemcpyAsync(ctx->h_gstat, ctx->gstat, sizeof(long long) * 4, cudaMemcpyDeviceToHost,
                        ctx->stream));
     int st = 0;
-    CKS(read_status(ctx, &st));
+    CKS(read_result(ctx, &st));
     graph_fold_counters(ctx, 1);
     ulisse_status r = status_to_result(ctx, st);
     if (r == ULISSE_ERR_ARG) return r;
-    CK(cudaMemcpyAsync(psi_inout, ctx->psi_dev, sizeof(double) * (ctx->d + 2),
-                       cudaMemcpyDeviceToHost, ctx->stream));
-    if (g_out)
-      CK(cudaMemcpyAsync(g_out, ctx->g_dev, sizeof(double) * (ctx->d + 2),
-                         cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
+    std::memcpy(psi_inout, ctx->h_result->psi, sizeof(double) * (ctx->d + 2));
+    if (g_out) std::memcpy(g_out, ctx->h_result->g, sizeof(double) * (ctx->d + 2));
     return r;
   }
   CKS(grad_core(ctx, step));
@@ -1516,15 +1542,11 @@ ulisse_status ulisse_sgld_step(ulisse_ctx* ctx, double* psi_inout, double eps_t,
   CK(cudaGetLastError());
   ctx->launches++;
   int st = 0;
-  CKS(read_status(ctx, &st));
+  CKS(read_result(ctx, &st));
   ulisse_status r = status_to_result(ctx, st);
   if (r == ULISSE_ERR_ARG) return r;
-  CK(cudaMemcpyAsync(psi_inout, ctx->psi_dev, sizeof(double) * (ctx->d + 2),
-                     cudaMemcpyDeviceToHost, ctx->stream));
-  if (g_out)
-    CK(cudaMemcpyAsync(g_out, ctx->g_dev, sizeof(double) * (ctx->d + 2), cudaMemcpyDeviceToHost,
-                       ctx->stream));
-  CK(cudaStreamSynchronize(ctx->stream));
+  std::memcpy(psi_inout, ctx->h_result->psi, sizeof(double) * (ctx->d + 2));
+  if (g_out) std::memcpy(g_out, ctx->h_result->g, sizeof(double) * (ctx->d + 2));
   return r;
 }
 
@@ -3208,11 +3230,12 @@ void ulisse_destroy(ulisse_ctx* ctx) {
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
   for (void** p : {&ctx->fixed_block, &ctx->col_block,
                    reinterpret_cast<void**>(&ctx->kv_launches_dev),
-                   reinterpret_cast<void**>(&ctx->q_map), &ctx->q_sa, &ctx->pcg_buf, &ctx->pred_xs,
+                   &ctx->pcg_buf, &ctx->pred_xs,
                    reinterpret_cast<void**>(&ctx->pcg_aux), reinterpret_cast<void**>(&ctx->pcg_live),
-                   &ctx->partials, reinterpret_cast<void**>(&ctx->counters),
                    reinterpret_cast<void**>(&ctx->gpart)})
     dev_free(*p);
+  if (ctx->partials != ctx->fixed_partials) dev_free(ctx->partials);
+  if (ctx->counters != ctx->fixed_counters) dev_free(reinterpret_cast<void*&>(ctx->counters));
   if (ctx->batched) dev_free(reinterpret_cast<void*&>(ctx->status_dev));   // its own allocation
   for (void* p : ctx->ws_allocs) cudaFree(p);
   ctx->ws_allocs.clear();
@@ -3246,8 +3269,8 @@ void ulisse_destroy(ulisse_ctx* ctx) {
     cudaEventDestroy(e.first);
     cudaEventDestroy(e.second);
   }
-  if (ctx->h_n_live) cudaFreeHost(ctx->h_n_live);
-  if (ctx->h_status) cudaFreeHost(ctx->h_status);
+  if (ctx->h_result) cudaFreeHost(ctx->h_result);
+  else if (ctx->h_status) cudaFreeHost(ctx->h_status);   // a batch has a status word alone
   delete ctx;
 }
 

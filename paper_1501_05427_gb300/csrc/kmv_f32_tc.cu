@@ -43,6 +43,13 @@ int f3_nsplit(long long n, int num_sms) {
   return (int)((ntiles + tps - 1) / tps);
 }
 
+size_t kmv_tile_partial_bytes(long long n, int num_sms, bool mixed) {
+  const size_t nrb = ((size_t)n + 127) / 128;
+  size_t ns = f3_nsplit(n, num_sms);
+  if (mixed) ns = tc_bound_split(plan_split(n, 128, 32, 4, 4 * num_sms), n, 128, 32, 32).nsplit;
+  return ns > 1 ? nrb * ns * 32 * 128 * 4 : 0;
+}
+
 namespace {
 
 constexpr int kF3BN = 32;

@@ -212,19 +212,22 @@ cudaError_t sym_dp(KmvLaunch& L, cudaStream_t s) {
 
 }  // namespace
 
+size_t kmv_f64_sym_bytes(long long n, int R) {
+  const size_t T = (size_t)sym_tile(n), nb = ((size_t)n + T - 1) / T;
+  return nb * nb * T * R * 8;
+}
+
 // The pair form's scratch grows as n^2 R / T doubles; it is used while that is at most 256 MiB
 // (n = 10,000 with 16 columns, 5,700 with 32), beyond which the row-block kernel runs.  A forced
 // configuration (an installed launch table) means the row-block kernel, and dK/dlog lambda has
 // no pairs.
 bool kmv_f64_sym_applies(const KmvLaunch& L) {
   if (L.mode == kModeDLam || L.nsplit > 0 || L.r_min > 0 || !L.exp_tab) return false;
-  const long long T = sym_tile(L.n), nb = (L.n + T - 1) / T;
-  return nb * nb * T * L.R * 8 <= kSymMaxPartialBytes;
+  return kmv_f64_sym_bytes(L.n, L.R) <= (size_t)kSymMaxPartialBytes;
 }
 
 cudaError_t launch_kmv_f64_sym(KmvLaunch& L, cudaStream_t s) {
-  const long long T = sym_tile(L.n), nb = (L.n + T - 1) / T;
-  const size_t need = (size_t)(nb * nb * T * L.R * 8);
+  const size_t need = kmv_f64_sym_bytes(L.n, L.R);
   L.planned_nsplit = 1;
   if (L.plan_only || need > L.partials_bytes) {
     L.need_partials_bytes = need;

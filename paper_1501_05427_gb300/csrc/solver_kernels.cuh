@@ -739,6 +739,31 @@ __global__ void compact_graph_kernel(ColState* __restrict__ st, const ColState* 
   cudaGraphSetConditional(h_branch, k > 0 ? (unsigned)(k - 1) : (unsigned)R);
 }
 
+// ulisse_dk_bilinear's scales by value.
+struct BilinearScales {
+  double v[kMaxM];
+};
+
+// Scales to sa, the status word to 0, and (A not null) columns 0..M-1 of A and B, leading
+// dimension n, to the context's buffers, leading dimension ld: column c of A, then of B, per grid
+// row.
+template <typename T>
+__global__ void __launch_bounds__(256) bilinear_prepare_kernel(
+    const BilinearScales sc, int M, T* __restrict__ sa, int* __restrict__ status,
+    const float* __restrict__ A, T* __restrict__ Ad, const float* __restrict__ B,
+    T* __restrict__ Bd, long long n, long long ld) {
+  if (blockIdx.x == 0 && blockIdx.y == 0) {
+    if ((int)threadIdx.x < M) sa[threadIdx.x] = (T)sc.v[threadIdx.x];
+    if (threadIdx.x == 0) *status = 0;
+  }
+  if (!A) return;
+  const int c = (int)blockIdx.y < M ? blockIdx.y : blockIdx.y - M;
+  const float* src = ((int)blockIdx.y < M ? A : B) + c * n;
+  T* dst = ((int)blockIdx.y < M ? Ad : Bd) + c * ld;
+  for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += gridDim.x * 256LL)
+    dst[i] = (T)src[i];
+}
+
 // Element-type conversion between caller buffers and the context's (FP64 contexts).
 template <typename S, typename D>
 __global__ void convert_cols_kernel(const S* __restrict__ src, long long lds, D* __restrict__ dst,

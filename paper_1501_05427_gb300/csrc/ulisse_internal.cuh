@@ -370,6 +370,10 @@ bool kmv_f32_tc_applies(const KmvLaunch& L);
 cudaError_t launch_kmv_f32_tc(KmvLaunch& L, cudaStream_t s);
 bool kmv_f64_sym_applies(const KmvLaunch& L);
 cudaError_t launch_kmv_f64_sym(KmvLaunch& L, cudaStream_t s);
+// Partial sums of one launch: FP64 pairs with R columns; the 128-row tensor-core products with up
+// to 32 (mixed or FP32).
+size_t kmv_f64_sym_bytes(long long n, int R);
+size_t kmv_tile_partial_bytes(long long n, int num_sms, bool mixed);
 cudaError_t launch_grad_f32(GradLaunch& L, cudaStream_t s);
 cudaError_t launch_grad_f64(GradLaunch& L, cudaStream_t s);
 cudaError_t launch_kmv_tc(TcLaunch& L, cudaStream_t s);
