@@ -138,6 +138,42 @@ __device__ __forceinline__ uint32_t f3_bits(const __nv_bfloat162& v) {
   return *reinterpret_cast<const uint32_t*>(&v);
 }
 
+// Rows whose sum came out as NaN, once more: a column of V that holds an infinity meets zeros and
+// both signs among the parts of K, where k_ij > 0 itself gives that infinity.  The terms that are
+// not finite decide such a sum, so only they are formed (a column without any stays as it is).
+// Not reached by finite results; a scan of V per entry otherwise.
+template <int MODE>
+__device__ __noinline__ void f3_not_finite(const F3Args& a, const long long row0, const int R) {
+  const float c0 = a.params->c0f, c1 = a.params->c1f;
+  for (int idx = threadIdx.x; idx < R * kF3BM; idx += kF3Threads) {
+    const int r = idx / kF3BM;
+    const long long i = row0 + (idx - r * kF3BM);
+    if (i >= a.n) continue;
+    float* out = a.U + (long long)a.umap[r] * a.ldu + i;
+    if (!isnan(*out)) continue;
+    const float* v = a.V + (long long)a.vmap[r] * a.ldv;
+    const float* xi = a.xhat + i * a.DP;
+    float u = 0.f;
+    bool any = false;
+    for (long long j = 0; j < a.n && !isnan(u); ++j) {
+      if (isfinite(v[j])) continue;
+      const float* xj = a.xhat + j * a.DP;
+      float dist = 0.f;
+      for (int k = 0; k < a.DP; ++k) dist = fmaf(xi[k] - xj[k], xi[k] - xj[k], dist);
+      float kv = ex2_approx(fmaf(-c1, dist, c0));
+      if constexpr (MODE == kModeDLen) {
+        const float dw = xi[a.which] - xj[a.which];
+        kv *= dw * dw;
+      }
+      u = fmaf(kv, v[j], u);
+      any = true;
+    }
+    if (!any) continue;
+    if (a.add_diag) u = fmaf((float)a.params->lambda, v[i], u);
+    *out = u;
+  }
+}
+
 // One CTA's work: row block rb, j-range split sp, R columns.  Shared by the single-problem kernel
 // and the batched one.
 template <int DP, int N, int MODE>
@@ -155,6 +191,7 @@ __device__ __forceinline__ void f3_body(const F3Args& a, const int rb, const int
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* s_fail = reinterpret_cast<volatile int*>(s_tmem + 1);
   int* s_last = reinterpret_cast<int*>(s_tmem + 2);
+  volatile int* s_nan = reinterpret_cast<volatile int*>(s_tmem + 3);   // a sum came out as NaN
   const uint32_t full0 = smem_u32(full), k_full0 = smem_u32(k_full), b_free0 = smem_u32(b_free),
                  u_full0 = smem_u32(u_full), u_free0 = smem_u32(u_free);
 
@@ -178,6 +215,7 @@ __device__ __forceinline__ void f3_body(const F3Args& a, const int rb, const int
     mbar_init(done, 1);
     fence_barrier_init();
     *s_fail = 0;
+    *s_nan = 0;
   }
   if (warp == 0) tc::tmem_alloc(s_tmem, kF3Cols);
   tc::fence_before();
@@ -344,6 +382,7 @@ __device__ __forceinline__ void f3_body(const F3Args& a, const int rb, const int
             float u = r & 1 ? acc[r / 2].y : acc[r / 2].x;
             if (a.add_diag) u = fmaf(lam, a.V[(long long)a.vmap[r] * a.ldv + i], u);
             a.U[(long long)a.umap[r] * a.ldu + i] = u;
+            if (isnan(u)) *s_nan = 1;
           }
       }
     } else {
@@ -368,7 +407,10 @@ __device__ __forceinline__ void f3_body(const F3Args& a, const int rb, const int
     }
     return;
   }
-  if (a.nsplit == 1) return;
+  if (a.nsplit == 1) {
+    if (*s_nan) f3_not_finite<MODE>(a, row0, R);
+    return;
+  }
   __threadfence();
   __syncthreads();
   if (tid == 0) *s_last = (atomicAdd(&a.counters[rb], 1) == a.nsplit - 1);
@@ -385,8 +427,11 @@ __device__ __forceinline__ void f3_body(const F3Args& a, const int rb, const int
     for (int s2 = 0; s2 < a.nsplit; ++s2) u += __ldcg(base + ((long long)s2 * N + r) * kF3BM + il);
     if (a.add_diag) u = fmaf(lam, a.V[(long long)a.vmap[r] * a.ldv + i], u);
     a.U[(long long)a.umap[r] * a.ldu + i] = u;
+    if (isnan(u)) *s_nan = 1;
   }
   if (tid == 0) a.counters[rb] = 0;
+  __syncthreads();
+  if (*s_nan) f3_not_finite<MODE>(a, row0, R);
 }
 
 template <int DP, int N, int MODE>

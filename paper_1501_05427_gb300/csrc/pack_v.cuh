@@ -29,8 +29,9 @@ __device__ inline void pack_v2(const float* __restrict__ V, long long ldv,
   }
 }
 
-// High, middle and low part: a float exactly (FP32 products).  A value that is not finite stays
-// in the high part.
+// High, middle and low part: a float exactly (FP32 products).  The high part of the largest floats
+// is rounded towards zero, as to nearest it is infinite; a value that is not finite stays whole in
+// the high part.
 __device__ inline void pack_v3(const float* __restrict__ V, long long ldv,
                                const int* __restrict__ vmap, int R, int N, long long n,
                                long long ntiles, __nv_bfloat16* __restrict__ Vp, int cta, int ctas) {
@@ -42,9 +43,9 @@ __device__ inline void pack_v3(const float* __restrict__ V, long long ldv,
     const int r = rem / 32, jj = rem - r * 32;
     const long long j = t * 32 + jj;
     const float v = (r < R && j < n) ? V[(long long)(vmap ? vmap[r] : r) * ldv + j] : 0.f;
-    const __nv_bfloat16 h = __float2bfloat16_rn(v);
-    const bool split = isfinite(__bfloat162float(h));
-    const float v1 = split ? v - __bfloat162float(h) : 0.f;
+    __nv_bfloat16 h = __float2bfloat16_rn(v);
+    if (isinf(__bfloat162float(h))) h = __float2bfloat16_rz(v);
+    const float v1 = isfinite(v) ? v - __bfloat162float(h) : 0.f;
     const __nv_bfloat16 m = __float2bfloat16_rn(v1);
     __nv_bfloat16* o = Vp + t * 3LL * per + tc::canon_offset(r, jj, 2, 4) / 2;
     o[0] = h;

@@ -81,3 +81,31 @@ def test_not_finite():
     keep = [0, 2, 3, 5]
     assert np.array_equal(U[:, keep], U0[:, keep])
     assert not np.isfinite(U[10, 1]) and np.all(np.isnan(U[:, 4]))
+
+
+@pytest.mark.parametrize("n", [300, 700, 5001])
+@pytest.mark.parametrize("which", [-1, 1])
+def test_infinities(n, which):
+    # k_ij > 0 at these distances: one infinity is every row's, both signs are NaN, and the
+    # SIMT kernel says the same (the derivative's k_jj is 0: NaN in the infinity's own row)
+    X, psi, V, _ = _problem(n, 2, 6, 11)
+    V[5, 0], V[n - 1, 2], V[7, 3], V[n - 2, 3], V[9, 4] = np.inf, -np.inf, np.inf, -np.inf, np.nan
+    a, b = _run(X, psi, V, which), _run(X, psi, V, which, rows_per_thread=2)
+    bad = [0, 2, 3, 4]
+    assert np.array_equal(a[:, bad], b[:, bad], equal_nan=True)
+    assert np.all(np.isfinite(a[:, [1, 5]]))
+    if which == -1:
+        assert np.all(a[:, 0] == np.inf) and np.all(a[:, 2] == -np.inf)
+        assert np.all(np.isnan(a[:, 3])) and np.all(np.isnan(a[:, 4]))
+
+
+def test_largest_floats():
+    # the largest floats are beyond the largest BF16 value, and finite times k_ij < 1
+    X, psi, V, rows = _problem(700, 2, 6, 13)
+    psi[2] = -1.0
+    V[10, 1], V[20, 4] = np.finfo(np.float32).max, -np.finfo(np.float32).max
+    U = _run(X, psi, V)[rows]
+    Xd, Vd = X.astype(np.float64), V.astype(np.float64)
+    ref = oracle.kmv_rows(Xd, psi, Vd, rows)
+    scale = oracle.kmv_rows(Xd, psi, Vd, rows, absolute=True)
+    assert np.max(np.abs(U - ref) / scale) <= 1e-5
