@@ -17,7 +17,8 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libulisse.so")
 SOURCES = ["api.cu", "kmv_f32.cu", "kmv_f32_dp2.cu", "kmv_f32_dp4.cu", "kmv_f32_dp8.cu",
-           "kmv_f32_dp16.cu", "kmv_f32_tc.cu", "kmv_f64.cu", "kmv_f64_sym.cu", "grad.cu", "kmv_noalloc.cu", "kmv_tc.cu",
+           "kmv_f32_dp16.cu", "kmv_f32_tc.cu", "kmv_f64.cu", "kmv_f64_sym.cu", "kmv_f64_dense.cu",
+           "grad.cu", "kmv_noalloc.cu", "kmv_tc.cu",
            "warm_start.cu", "batch_kmv.cu", "batch_grad.cu", "grad_tc.cu", "kmv_tc2.cu", "calib.cu",
            "predict.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

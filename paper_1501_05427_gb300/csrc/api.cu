@@ -49,6 +49,9 @@ struct ulisse_ctx {
   DevParams* params = nullptr;
   void* v3 = nullptr;         // FP32: operand scratch of the tensor-core contraction
   double* exp_tab = nullptr;  // FP64: table of the exponential (exp64.cuh)
+  double* kmat = nullptr;     // FP64: the kernel values of a solve (kmat_ld(n)^2)
+  bool kmat_tried = false;    // its allocation was attempted
+  bool kmat_formed = false;   // it holds the values of the current psi (or will, when captured)
   double* psi_dev = nullptr;  // kMaxP
   PsiArg psi_arg{};           // by_value: psi of a host call, handed to the next prescale launch
 
@@ -382,6 +385,7 @@ static ulisse_status psi_to_device(ulisse_ctx* ctx) {
 // the same launch (FP32 and FP64 contexts), or the operand pv of a tensor-core product is packed.
 template <typename TV>
 static ulisse_status prescale_and_copy(ulisse_ctx* ctx, const TV* V, int R, PackV pv = PackV{}) {
+  ctx->kmat_formed = false;
   PsiArg pa = ctx->psi_arg;
   if (ctx->capturing) pa.by_value = 0;   // a captured step reads psi_dev
   if (ctx->mixed)
@@ -403,6 +407,30 @@ static ulisse_status prescale_and_copy(ulisse_ctx* ctx, const TV* V, int R, Pack
 
 static ulisse_status prescale(ulisse_ctx* ctx) {
   return prescale_and_copy<float>(ctx, nullptr, 0);
+}
+
+// Buffer of an FP64 solve's kernel values, with the first solve.  Without the memory for it every
+// round makes the values anew.
+static void ensure_kmat(ulisse_ctx* ctx) {
+  if (!ctx->f64 || ctx->n > kKmatMaxN || ctx->kmat_tried) return;
+  ctx->kmat_tried = true;
+  const size_t ld = (size_t)kmat_ld(ctx->n);
+  if (cudaMalloc(reinterpret_cast<void**>(&ctx->kmat), ld * ld * sizeof(double)) != cudaSuccess) {
+    ctx->kmat = nullptr;
+    cudaGetLastError();
+  }
+}
+
+// The kernel values of the psi just prescaled, for all rounds of the solve that follows: a round
+// then costs R FP64 operations per entry instead of (2d + 7) / 2 + R, and one product already pays
+// for the forming.
+static ulisse_status form_kmat(ulisse_ctx* ctx) {
+  if (!ctx->kmat || ctx->kmat_formed) return ULISSE_OK;
+  CK(launch_form_kmat((const double*)ctx->xhat, ctx->n, ctx->DP, ctx->exp_tab, ctx->kmat,
+                      kmat_ld(ctx->n), ctx->stream));
+  if (!ctx->capturing) ctx->launches++;
+  ctx->kmat_formed = true;
+  return ULISSE_OK;
 }
 
 // U[:, umap[r]] = A V[:, vmap[r]] for r < R (chunks of kMaxRChunk columns per launch).
@@ -525,6 +553,7 @@ static ulisse_status run_kmv(ulisse_ctx* ctx, const void* V, const int* vmap, in
     L.umap = umap + c0;
     L.params = ctx->params;
     L.exp_tab = ctx->exp_tab;
+    L.kmat = ctx->kmat_formed ? ctx->kmat : nullptr;
     L.v3 = ctx->v3;
     L.simt = ctx->simt || ctx->cfg.kmv_rows_per_thread != 0;
     L.v_packed = ctx->v_packed;
@@ -869,6 +898,8 @@ static ulisse_status pcg_core(ulisse_ctx* ctx, int R, unsigned long long step) {
 static ulisse_status solve_dispatch(ulisse_ctx* ctx, int R, int s0_cols,
                                     unsigned long long step, bool warm = false,
                                     bool y_learned = false) {
+  ensure_kmat(ctx);
+  CKS(form_kmat(ctx));
   if (ctx->cfg.pcg_delta > 0.0) {
     if (s0_cols > 0 || warm || y_learned)
       return fail(ctx, ULISSE_ERR_ARG, "preconditioned CG solves start from zero (no S0, "
@@ -1571,6 +1602,7 @@ static ulisse_status graph_capture_body(ulisse_ctx* ctx, int s0_cols) {
   const int nr = ctx->cfg.n_probes, R = 1 + nr, p = ctx->d + 2;
   ctx->cap_launches = 0;
   CKS(prescale(ctx));
+  CKS(form_kmat(ctx));
   CK(cudaMemcpyAsync(ctx->B, ctx->y, ctx->ldn * ctx->esz, cudaMemcpyDeviceToDevice,
                      ctx->stream));
   dim3 pg((unsigned)std::min<long long>((ctx->n + 255) / 256, 2LL * ctx->num_sms), nr);
@@ -1727,6 +1759,7 @@ static ulisse_status graph_build(ulisse_ctx* ctx, int s0_cols) {
   const cudaError_t e2 = e == cudaSuccess ? cudaStreamEndCapture(ctx->cap_stream, &graph) : e;
   ctx->stream = saved;
   ctx->capturing = false;
+  ctx->kmat_formed = false;   // only captured
   ctx->prof = prof;
   if (r != ULISSE_OK) {
     if (graph) cudaGraphDestroy(graph);
@@ -1742,9 +1775,9 @@ static ulisse_status graph_build(ulisse_ctx* ctx, int s0_cols) {
                      cudaMemcpyHostToDevice, ctx->stream));
   // what one launch does outside the CG loop (the loop's share is counted on the device)
   const int init_cols = warm ? R : s0_cols;   // columns of the product K s_0
-  // prescale, probes, the CG start, the gradient pass (+ its
+  // prescale (and an FP64 solve's kernel values), probes, the CG start, the gradient pass (+ its
   // operand images), the update, the learned start's two kernels, the product K s_0
-  ctx->graph_launches_fixed = 1 + 1 + cg_init_launch_count(ctx->n, R, ctx->num_sms) +
+  ctx->graph_launches_fixed = 1 + (ctx->kmat ? 1 : 0) + 1 + cg_init_launch_count(ctx->n, R, ctx->num_sms) +
       (ctx->mixed ? 2 : 1) + 1 + (s0_cols > 0 ? 2 : 0) +
       ctx->graph_init_launches;
   ctx->graph_entries_fixed = (double)ctx->n * (double)ctx->n * (double)(R + init_cols);
@@ -1786,6 +1819,7 @@ static ulisse_status graph_prepare(ulisse_ctx* ctx, const double* M, const doubl
     ctx->prior_zero = true;
   }
   CKS(graph_alloc(ctx));
+  ensure_kmat(ctx);
   const ChainSlot cs{0, step0, eps_dev, trace_dev};
   CK(cudaMemcpyAsync(ctx->chain, &cs, sizeof(ChainSlot), cudaMemcpyHostToDevice, ctx->stream));
   const int s0 = (ctx->ws_use && ctx->ws_trained) ? 1 : 0;
@@ -3230,6 +3264,7 @@ void ulisse_destroy(ulisse_ctx* ctx) {
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
   for (void** p : {&ctx->fixed_block, &ctx->col_block,
                    reinterpret_cast<void**>(&ctx->kv_launches_dev),
+                   reinterpret_cast<void**>(&ctx->kmat),
                    &ctx->pcg_buf, &ctx->pred_xs,
                    reinterpret_cast<void**>(&ctx->pcg_aux), reinterpret_cast<void**>(&ctx->pcg_live),
                    reinterpret_cast<void**>(&ctx->gpart)})

@@ -55,6 +55,7 @@ struct Sym64Args {
 
 constexpr long long kSymMaxPartialBytes = 256LL << 20;
 constexpr int kSymRedNT = 128;
+constexpr int kFillNT = 128;
 constexpr int sym_tile(long long n) { return n <= 2048 ? 32 : 64; }
 
 // U = sigma^2 (the block's nb partials in partner order) + lambda V.  Four lanes per element,
@@ -88,41 +89,33 @@ __global__ void __launch_bounds__(kSymRedNT) kmv_f64_sym_reduce_kernel(const Sym
   a.U[(long long)a.umap[r] * a.ldu + i] = u;
 }
 
-template <int DP, int T, int NT, int MODE>
-__global__ void __launch_bounds__(NT) kmv_f64_sym_kernel(const Sym64Args a) {
-  constexpr int LD = T + 1;   // padded row: the transposed pass reads columns
-  extern __shared__ __align__(16) double sm[];
-  double* sK = sm;                       // T x LD
-  double* sXI = sK + T * LD;             // DP x T
-  double* sVI = sXI + DP * T;            // R x T
-  double* sVJ = sVI + a.R * T;           // R x T
-  const int tid = threadIdx.x;
-  // pair p -> (bi, bj), bi <= bj: p = bj (bj + 1) / 2 + bi
-  const long long p = blockIdx.x;
-  long long bj = (long long)((sqrtf(8.f * (float)p + 1.f) - 1.f) * 0.5f);
+// pair p -> (bi, bj), bi <= bj: p = bj (bj + 1) / 2 + bi
+__device__ __forceinline__ void pair_blocks(long long p, int& bi, long long& bj) {
+  bj = (long long)((sqrtf(8.f * (float)p + 1.f) - 1.f) * 0.5f);
   while (bj * (bj + 1) / 2 > p) --bj;
   while ((bj + 1) * (bj + 2) / 2 <= p) ++bj;
-  const int bi = (int)(p - bj * (bj + 1) / 2);
-  const long long i0 = (long long)bi * T, j0 = bj * T;
-  const bool diag = bi == bj;
+  bi = (int)(p - bj * (bj + 1) / 2);
+}
 
+// The pair's T x T kernel values (sigma^2 left out) into sK, rows of T + 1; sXI holds DP x T.
+// Barriers before (the caller's own shared stores are then visible too) and after.
+template <int DP, int T, int NT, int MODE>
+__device__ __forceinline__ void form_pair(const double* __restrict__ xhat, long long n,
+                                          const double* __restrict__ exp_tab, int which,
+                                          long long i0, long long j0, double* sXI, double* sK) {
+  constexpr int LD = T + 1;   // padded row: the transposed pass reads columns
+  const int tid = threadIdx.x;
   for (int e = tid; e < DP * T; e += NT) {
     const int i = e / DP, k = e - i * DP;
-    sXI[k * T + i] = i0 + i < a.n ? a.xhat[(i0 + i) * DP + k] : 0.0;
-  }
-  for (int e = tid; e < a.R * T; e += NT) {
-    const int r = e / T, i = e - r * T;
-    const double* v = a.V + (long long)a.vmap[r] * a.ldv;
-    sVI[e] = i0 + i < a.n ? v[i0 + i] : 0.0;
-    sVJ[e] = j0 + i < a.n ? v[j0 + i] : 0.0;
+    sXI[k * T + i] = i0 + i < n ? xhat[(i0 + i) * DP + k] : 0.0;
   }
   // thread's column j is fixed (NT is a multiple of T)
   const int j = tid % T;
   double xj[DP];
 #pragma unroll
-  for (int k = 0; k < DP; ++k) xj[k] = j0 + j < a.n ? a.xhat[(j0 + j) * DP + k] : 0.0;
+  for (int k = 0; k < DP; ++k) xj[k] = j0 + j < n ? xhat[(j0 + j) * DP + k] : 0.0;
   double xjw = 0.0;
-  if constexpr (MODE == kModeDLen) xjw = j0 + j < a.n ? a.xhat[(j0 + j) * DP + a.which] : 0.0;
+  if constexpr (MODE == kModeDLen) xjw = j0 + j < n ? xhat[(j0 + j) * DP + which] : 0.0;
   __syncthreads();
 #pragma unroll 4
   for (int i = tid / T; i < T; i += NT / T) {
@@ -133,14 +126,38 @@ __global__ void __launch_bounds__(NT) kmv_f64_sym_kernel(const Sym64Args a) {
       const double df = sXI[k * T + i] - xj[k];
       dist = fma(df, df, dist);
     }
-    double kv = exp_neg_half(dist, a.exp_tab);
+    double kv = exp_neg_half(dist, exp_tab);
     if constexpr (MODE == kModeDLen) {
-      const double dw = sXI[a.which * T + i] - xjw;
+      const double dw = sXI[which * T + i] - xjw;
       kv *= dw * dw;
     }
     sK[i * LD + j] = kv;
   }
   __syncthreads();
+}
+
+template <int DP, int T, int NT, int MODE>
+__global__ void __launch_bounds__(NT) kmv_f64_sym_kernel(const Sym64Args a) {
+  constexpr int LD = T + 1;   // padded row: the transposed pass reads columns
+  extern __shared__ __align__(16) double sm[];
+  double* sK = sm;                       // T x LD
+  double* sXI = sK + T * LD;             // DP x T
+  double* sVI = sXI + DP * T;            // R x T
+  double* sVJ = sVI + a.R * T;           // R x T
+  const int tid = threadIdx.x;
+  int bi;
+  long long bj;
+  pair_blocks(blockIdx.x, bi, bj);
+  const long long i0 = (long long)bi * T, j0 = bj * T;
+  const bool diag = bi == bj;
+
+  for (int e = tid; e < a.R * T; e += NT) {
+    const int r = e / T, i = e - r * T;
+    const double* v = a.V + (long long)a.vmap[r] * a.ldv;
+    sVI[e] = i0 + i < a.n ? v[i0 + i] : 0.0;
+    sVJ[e] = j0 + i < a.n ? v[j0 + i] : 0.0;
+  }
+  form_pair<DP, T, NT, MODE>(a.xhat, a.n, a.exp_tab, a.which, i0, j0, sXI, sK);
   // rows of I: K V_J; rows of J: K^T V_I (a diagonal pair holds both orders itself)
   const int outs = a.R * T;
   double* partI = a.partials + ((long long)bi * a.nb + bj) * outs;
@@ -159,6 +176,27 @@ __global__ void __launch_bounds__(NT) kmv_f64_sym_kernel(const Sym64Args a) {
       u1 = fma(kp[(y + 1) * step], v[y + 1], u1);
     }
     (side_j ? partJ : partI)[q] = u0 + u1;
+  }
+}
+
+// The kernel values themselves (sigma^2 left out), both orders of every pair: K is ldk x ldk, ldk a
+// multiple of T.  Values of rows and columns past n are finite where x is, and unused.
+template <int DP>
+__global__ void __launch_bounds__(kFillNT) form_kmat_kernel(const double* __restrict__ xhat,
+                                                            long long n,
+                                                            const double* __restrict__ exp_tab,
+                                                            double* __restrict__ K, long long ldk) {
+  constexpr int T = 32, LD = T + 1;
+  __shared__ double sK[T * LD], sXI[DP * T];
+  int bi;
+  long long bj;
+  pair_blocks(blockIdx.x, bi, bj);
+  const long long i0 = (long long)bi * T, j0 = bj * T;
+  form_pair<DP, T, kFillNT, kModeK>(xhat, n, exp_tab, 0, i0, j0, sXI, sK);
+  const int j = threadIdx.x % T;
+  for (int i = threadIdx.x / T; i < T; i += kFillNT / T) {
+    K[(i0 + i) * ldk + j0 + j] = sK[i * LD + j];
+    if (bi != bj) K[(j0 + i) * ldk + i0 + j] = sK[j * LD + i];
   }
 }
 
@@ -211,6 +249,20 @@ cudaError_t sym_dp(KmvLaunch& L, cudaStream_t s) {
 }
 
 }  // namespace
+
+cudaError_t launch_form_kmat(const double* xhat, long long n, int DP, const double* exp_tab, double* K,
+                             long long ldk, cudaStream_t s) {
+  const long long nb = (n + 31) / 32;
+  const unsigned pairs = (unsigned)(nb * (nb + 1) / 2);
+  switch (DP) {
+    case 2: form_kmat_kernel<2><<<pairs, kFillNT, 0, s>>>(xhat, n, exp_tab, K, ldk); break;
+    case 4: form_kmat_kernel<4><<<pairs, kFillNT, 0, s>>>(xhat, n, exp_tab, K, ldk); break;
+    case 8: form_kmat_kernel<8><<<pairs, kFillNT, 0, s>>>(xhat, n, exp_tab, K, ldk); break;
+    case 16: form_kmat_kernel<16><<<pairs, kFillNT, 0, s>>>(xhat, n, exp_tab, K, ldk); break;
+    default: return cudaErrorInvalidValue;
+  }
+  return cudaGetLastError();
+}
 
 size_t kmv_f64_sym_bytes(long long n, int R) {
   const size_t T = (size_t)sym_tile(n), nb = ((size_t)n + T - 1) / T;

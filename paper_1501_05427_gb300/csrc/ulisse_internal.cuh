@@ -260,6 +260,7 @@ struct KmvLaunch {
   const double* exp_tab; // FP64: the exponential's table (exp64.cuh)
   void* v3;              // FP32: scratch of the tensor-core contraction's operand (kmv_f32_tc.cu),
                          // 96 BF16 values per point (null: SIMT kernel)
+  const double* kmat;    // FP64: the kernel values of this solve, n <= kKmatMaxN (null: not formed)
   bool simt;             // FP32: the SIMT kernel whatever the sizes
   bool v_packed;         // v3 already holds the operand (packed by the prescale launch)
   int tm;                // rows per thread for K (0 = default)
@@ -368,6 +369,13 @@ __host__ __device__ constexpr bool f32_tc_columns(long long n, int R) {
 }
 bool kmv_f32_tc_applies(const KmvLaunch& L);
 cudaError_t launch_kmv_f32_tc(KmvLaunch& L, cudaStream_t s);
+// FP64 solves form the kernel values once (kmat_ld(n)^2 doubles, at most 256 MiB) and read them in
+// every round.
+constexpr long long kKmatMaxN = 5792;
+constexpr long long kmat_ld(long long n) { return (n + 31) / 32 * 32; }
+cudaError_t launch_form_kmat(const double* xhat, long long n, int DP, const double* exp_tab, double* K,
+                             long long ldk, cudaStream_t s);
+cudaError_t launch_kmv_f64_dense(KmvLaunch& L, cudaStream_t s);
 bool kmv_f64_sym_applies(const KmvLaunch& L);
 cudaError_t launch_kmv_f64_sym(KmvLaunch& L, cudaStream_t s);
 // Partial sums of one launch: FP64 pairs with R columns; the 128-row tensor-core products with up
