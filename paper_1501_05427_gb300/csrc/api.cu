@@ -536,7 +536,9 @@ static ulisse_status run_kmv(ulisse_ctx* ctx, const void* V, const int* vmap, in
   if (ldv == 0) ldv = ctx->ldn;
   if (ldu == 0) ldu = ctx->ldn;
   if (ctx->mixed && mode == kModeK) return run_kmv_tc(ctx, V, vmap, R, U, umap, ldv, ldu);
-  for (int c0 = 0; c0 < R; c0 += kMaxRChunk) {
+  // a product from formed kernel values takes any number of columns in one launch
+  const int per = ctx->kmat_formed && mode == kModeK ? std::max(R, 1) : kMaxRChunk;
+  for (int c0 = 0; c0 < R; c0 += per) {
     KmvLaunch L{};
     L.xhat = ctx->xhat;
     L.n = ctx->n;
@@ -546,7 +548,7 @@ static ulisse_status run_kmv(ulisse_ctx* ctx, const void* V, const int* vmap, in
     L.V = V;
     L.ldv = ldv;
     L.vmap = vmap + c0;
-    L.R = std::min(kMaxRChunk, R - c0);
+    L.R = std::min(per, R - c0);
     L.launches = 1;
     L.U = U;
     L.ldu = ldu;
