@@ -50,6 +50,7 @@ struct ulisse_ctx {
   void* v3 = nullptr;         // FP32: operand scratch of the tensor-core contraction
   double* exp_tab = nullptr;  // FP64: table of the exponential (exp64.cuh)
   double* kmat = nullptr;     // FP64: the kernel values of a solve (kmat_ld(n)^2)
+  bool ordered = false;       // FP64, during a truncated solve and its gradient: see OrderedScope
   bool kmat_tried = false;    // its allocation was attempted
   bool kmat_formed = false;   // it holds the values of the current psi (or will, when captured)
   double* psi_dev = nullptr;  // kMaxP
@@ -409,6 +410,17 @@ static ulisse_status prescale(ulisse_ctx* ctx) {
   return prescale_and_copy<float>(ctx, nullptr, 0);
 }
 
+// A truncated solve in FP64 amplifies the rounding of its products and sums (2^-53 becomes 1e-3
+// within ten steps of a chain), so that rounding is part of its result: the library's exponential
+// and one order of additions, whatever kernel does them.  Products by themselves and predictions,
+// which solve to convergence, use the faster forms.
+struct OrderedScope {
+  ulisse_ctx* ctx;
+  bool was;
+  OrderedScope(ulisse_ctx* c) : ctx(c), was(c->ordered) { c->ordered = c->f64; }
+  ~OrderedScope() { ctx->ordered = was; }
+};
+
 // Buffer of an FP64 solve's kernel values, with the first solve.  Without the memory for it every
 // round makes the values anew.
 static void ensure_kmat(ulisse_ctx* ctx) {
@@ -426,8 +438,8 @@ static void ensure_kmat(ulisse_ctx* ctx) {
 // for the forming.
 static ulisse_status form_kmat(ulisse_ctx* ctx) {
   if (!ctx->kmat || ctx->kmat_formed) return ULISSE_OK;
-  CK(launch_form_kmat((const double*)ctx->xhat, ctx->n, ctx->DP, ctx->exp_tab, ctx->kmat,
-                      kmat_ld(ctx->n), ctx->stream));
+  CK(launch_form_kmat((const double*)ctx->xhat, ctx->n, ctx->DP, ctx->ordered ? nullptr : ctx->exp_tab,
+                      ctx->params, ctx->kmat, kmat_ld(ctx->n), ctx->stream));
   if (!ctx->capturing) ctx->launches++;
   ctx->kmat_formed = true;
   return ULISSE_OK;
@@ -537,7 +549,7 @@ static ulisse_status run_kmv(ulisse_ctx* ctx, const void* V, const int* vmap, in
   if (ldu == 0) ldu = ctx->ldn;
   if (ctx->mixed && mode == kModeK) return run_kmv_tc(ctx, V, vmap, R, U, umap, ldv, ldu);
   // a product from formed kernel values takes any number of columns in one launch
-  const int per = ctx->kmat_formed && mode == kModeK ? std::max(R, 1) : kMaxRChunk;
+  const int per = ctx->kmat_formed && mode == kModeK && !ctx->ordered ? std::max(R, 1) : kMaxRChunk;
   for (int c0 = 0; c0 < R; c0 += per) {
     KmvLaunch L{};
     L.xhat = ctx->xhat;
@@ -554,7 +566,8 @@ static ulisse_status run_kmv(ulisse_ctx* ctx, const void* V, const int* vmap, in
     L.ldu = ldu;
     L.umap = umap + c0;
     L.params = ctx->params;
-    L.exp_tab = ctx->exp_tab;
+    L.exp_tab = ctx->ordered ? nullptr : ctx->exp_tab;
+    L.ordered = ctx->ordered;
     L.kmat = ctx->kmat_formed ? ctx->kmat : nullptr;
     L.v3 = ctx->v3;
     L.simt = ctx->simt || ctx->cfg.kmv_rows_per_thread != 0;
@@ -681,6 +694,7 @@ static CgArgs<T> cg_args(ulisse_ctx* ctx, int has_s0, unsigned long long step) {
   a.y_learned = 0;
   a.Sbest = (T*)ctx->Sbest;
   a.status = ctx->status_dev;
+  a.ordered = ctx->ordered;
   return a;
 }
 
@@ -768,7 +782,7 @@ static ulisse_status solve_core(ulisse_ctx* ctx, int R, int s0_cols, unsigned lo
     if (nl == 0) break;
     CKS(run_kmv(ctx, ctx->D, ctx->live, nl, ctx->KD, ctx->live, kModeK, -1));
     ctx->mvp_rounds += 1;
-    CK(launch_cg_round(a, nl, ctx->stream));
+    CK(launch_cg_round(a, nl, ctx->num_sms, ctx->stream));
     ctx->launches++;
     n_prev = nl;
   }
@@ -971,7 +985,7 @@ static ulisse_status run_grad(ulisse_ctx* ctx, int M, const int* amap = nullptr,
   L.ld = ld > 0 ? ld : ctx->ldn;
   L.M = M;
   L.params = ctx->params;
-  L.exp_tab = ctx->exp_tab;
+  L.exp_tab = ctx->ordered ? nullptr : ctx->exp_tab;
   L.counter = ctx->gcounter;
   L.g_out = ctx->g_dev;
   L.status = ctx->status_dev;
@@ -1026,6 +1040,7 @@ static ulisse_status run_grad(ulisse_ctx* ctx, int M, const int* amap = nullptr,
 // solves and the gradient pass of all its problems together).
 static ulisse_status grad_core(ulisse_ctx* ctx, unsigned long long step,
                                bool prologue_only = false) {
+  const OrderedScope ordered(ctx);
   const int nr = ctx->cfg.n_probes, R = 1 + nr;
   CKS(ensure_columns(ctx, R, R + 1));
   CKS(ensure_grad_maps(ctx, nr));
@@ -1366,6 +1381,7 @@ ulisse_status ulisse_solve(ulisse_ctx* ctx, const double* psi, const float* B, i
   if (!ctx) return ULISSE_ERR_ARG;
   if (ctx->batched) return fail(ctx, ULISSE_ERR_ARG, "batched context: use the ulisse_batch_* calls");
   if (!B || !S_est || R < 1 || R > 1024) return fail(ctx, ULISSE_ERR_ARG, "B/S_est null or R out of range");
+  const OrderedScope ordered(ctx);
   int tot = 0;
   if (n_est)
     for (int c = 0; c < R; ++c) {
@@ -1695,7 +1711,7 @@ static ulisse_status graph_capture_body(ulisse_ctx* ctx, int s0_cols) {
     ulisse_status r = run_kmv(ctx, ctx->D, ctx->live, k + 1, ctx->KD, ctx->live, kModeK, -1);
     ctx->kv_launches[k] = (int)ctx->cap_launches;
     ctx->stream = outer;
-    const cudaError_t e3 = r == ULISSE_OK ? launch_cg_round(a, k + 1, ctx->cap_stream2) : cudaSuccess;
+    const cudaError_t e3 = r == ULISSE_OK ? launch_cg_round(a, k + 1, ctx->num_sms, ctx->cap_stream2) : cudaSuccess;
     const cudaError_t e4 = cudaStreamEndCapture(ctx->cap_stream2, &tmp);
     CKS(r);
     CK(e3);
@@ -1716,6 +1732,7 @@ static ulisse_status graph_capture_body(ulisse_ctx* ctx, int s0_cols) {
 }  // extern "C++"
 
 static ulisse_status graph_build(ulisse_ctx* ctx, int s0_cols) {
+  const OrderedScope ordered(ctx);
   graph_release(ctx);
   const int nr = ctx->cfg.n_probes, R = 1 + nr;
   CKS(ensure_columns(ctx, R, R + 1));

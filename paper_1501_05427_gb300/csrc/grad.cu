@@ -95,7 +95,9 @@ __device__ __forceinline__ void tile_pass_f32(const float* tX, const float* tB,
   }
 }
 
-template <typename T, int DP, int M, int TM, int NT>
+// TAB: FP64 by the table-driven exponential.  Without it FP64 keeps the rounding of the solves that
+// the gradient belongs to: the library's exponential and the partials added one by one.
+template <typename T, int DP, int M, int TM, int NT, bool TAB>
 __global__ void __launch_bounds__(NT) grad_kernel(const GradDevArgs<T> a) {
   constexpr int BM = NT * TM;
   constexpr int NW = NT / 32;
@@ -216,7 +218,7 @@ __global__ void __launch_bounds__(NT) grad_kernel(const GradDevArgs<T> a) {
               sq[k] = df * df;
               dist += sq[k];
             }
-            const T P = kernel_from_dist<T>(dist, c0, c1, sigma2, a.exp_tab) * W[t][q];
+            const T P = kernel_from_dist<T, TAB>(dist, c0, c1, sigma2, a.exp_tab) * W[t][q];
             gs += P;
 #pragma unroll
             for (int k = 0; k < DP; ++k) gl[k] = fma(P, sq[k], gl[k]);
@@ -277,13 +279,29 @@ __global__ void __launch_bounds__(NT) grad_kernel(const GradDevArgs<T> a) {
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  __shared__ double s_sum[NT];
-  const double v = sum_partial_rows<NT>(a.partials, (int)gridDim.x, a.d + 2, s_sum);
+  double v = 0.0;
+  if constexpr (sizeof(T) == 8 && !TAB) {
+    if (tid < a.d + 2) {
+      const double* part = a.partials + tid;
+      for (int b = 0; b < (int)gridDim.x; b += 16) {   // 16 loads in flight
+        double x[16];
+#pragma unroll
+        for (int q = 0; q < 16; ++q)
+          x[q] = b + q < (int)gridDim.x ? __ldcg(part + (long long)(b + q) * kMaxP) : 0.0;
+#pragma unroll
+        for (int q = 0; q < 16; ++q)
+          if (b + q < (int)gridDim.x) v += x[q];
+      }
+    }
+  } else {
+    __shared__ double s_sum[NT];
+    v = sum_partial_rows<NT>(a.partials, (int)gridDim.x, a.d + 2, s_sum);
+  }
   if (tid < a.d + 2) a.g_out[tid] = tid == a.d + 1 ? v * a.params->lambda : v;
   if (tid == 0) *a.counter = 0;
 }
 
-template <typename T, int DP, int M, int TM>
+template <typename T, int DP, int M, int TM, bool TAB>
 struct GradInst {
   static constexpr int BM = kGradNT * TM;
   static size_t smem_bytes() {
@@ -293,7 +311,7 @@ struct GradInst {
     static int occ = -1;
     static std::once_flag once;
     std::call_once(once, [] {
-      auto fn = grad_kernel<T, DP, M, TM, kGradNT>;
+      auto fn = grad_kernel<T, DP, M, TM, kGradNT, TAB>;
       cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes());
       int o = 0;
       if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, fn, kGradNT, smem_bytes()) !=
@@ -335,34 +353,38 @@ struct GradInst {
     a.counter = L.counter;
     a.g_out = L.g_out;
     a.status = L.status;
-    grad_kernel<T, DP, M, TM, kGradNT><<<p.n_rb * p.nsplit, kGradNT, smem_bytes(), s>>>(a);
+    grad_kernel<T, DP, M, TM, kGradNT, TAB><<<p.n_rb * p.nsplit, kGradNT, smem_bytes(), s>>>(a);
     return cudaGetLastError();
   }
 };
 
-template <typename T, int DP>
+template <typename T, int DP, bool TAB>
 static cudaError_t grad_dispatch_m(GradLaunch& L, cudaStream_t s) {
   constexpr int TMs = sizeof(T) == 4 ? 2 : 1;
-  if (L.M <= 5) return GradInst<T, DP, 5, TMs>::launch(L, s);
-  if (L.M <= 9) return GradInst<T, DP, 9, TMs>::launch(L, s);
-  if (L.M <= 17) return GradInst<T, DP, 17, TMs>::launch(L, s);
-  if (L.M <= 33) return GradInst<T, DP, 33, 1>::launch(L, s);
-  if (L.M <= 64) return GradInst<T, DP, 64, 1>::launch(L, s);
+  if (L.M <= 5) return GradInst<T, DP, 5, TMs, TAB>::launch(L, s);
+  if (L.M <= 9) return GradInst<T, DP, 9, TMs, TAB>::launch(L, s);
+  if (L.M <= 17) return GradInst<T, DP, 17, TMs, TAB>::launch(L, s);
+  if (L.M <= 33) return GradInst<T, DP, 33, 1, TAB>::launch(L, s);
+  if (L.M <= 64) return GradInst<T, DP, 64, 1, TAB>::launch(L, s);
   return cudaErrorInvalidValue;
 }
 
-template <typename T>
+template <typename T, bool TAB>
 static cudaError_t grad_dispatch(GradLaunch& L, cudaStream_t s) {
   switch (L.DP) {
-    case 2: return grad_dispatch_m<T, 2>(L, s);
-    case 4: return grad_dispatch_m<T, 4>(L, s);
-    case 8: return grad_dispatch_m<T, 8>(L, s);
-    case 16: return grad_dispatch_m<T, 16>(L, s);
+    case 2: return grad_dispatch_m<T, 2, TAB>(L, s);
+    case 4: return grad_dispatch_m<T, 4, TAB>(L, s);
+    case 8: return grad_dispatch_m<T, 8, TAB>(L, s);
+    case 16: return grad_dispatch_m<T, 16, TAB>(L, s);
     default: return cudaErrorInvalidValue;
   }
 }
 
-cudaError_t launch_grad_f32(GradLaunch& L, cudaStream_t s) { return grad_dispatch<float>(L, s); }
-cudaError_t launch_grad_f64(GradLaunch& L, cudaStream_t s) { return grad_dispatch<double>(L, s); }
+cudaError_t launch_grad_f32(GradLaunch& L, cudaStream_t s) {
+  return grad_dispatch<float, false>(L, s);
+}
+cudaError_t launch_grad_f64(GradLaunch& L, cudaStream_t s) {
+  return L.exp_tab ? grad_dispatch<double, true>(L, s) : grad_dispatch<double, false>(L, s);
+}
 
 }  // namespace ulisse

@@ -97,12 +97,13 @@ __device__ __forceinline__ void pair_blocks(long long p, int& bi, long long& bj)
   bi = (int)(p - bj * (bj + 1) / 2);
 }
 
-// The pair's T x T kernel values (sigma^2 left out) into sK, rows of T + 1; sXI holds DP x T.
+// The pair's T x T kernel values (sigma^2 left out; LIB: with it, by the library's exponential) into sK, rows of T + 1; sXI holds DP x T.
 // Barriers before (the caller's own shared stores are then visible too) and after.
-template <int DP, int T, int NT, int MODE>
+template <int DP, int T, int NT, int MODE, bool LIB = false>
 __device__ __forceinline__ void form_pair(const double* __restrict__ xhat, long long n,
                                           const double* __restrict__ exp_tab, int which,
-                                          long long i0, long long j0, double* sXI, double* sK) {
+                                          long long i0, long long j0, double* sXI, double* sK,
+                                          double sigma2 = 0.0) {
   constexpr int LD = T + 1;   // padded row: the transposed pass reads columns
   const int tid = threadIdx.x;
   for (int e = tid; e < DP * T; e += NT) {
@@ -126,7 +127,9 @@ __device__ __forceinline__ void form_pair(const double* __restrict__ xhat, long 
       const double df = sXI[k * T + i] - xj[k];
       dist = fma(df, df, dist);
     }
-    double kv = exp_neg_half(dist, exp_tab);
+    double kv;
+    if constexpr (LIB) kv = sigma2 * exp(-0.5 * dist);
+    else kv = exp_neg_half(dist, exp_tab);
     if constexpr (MODE == kModeDLen) {
       const double dw = sXI[which * T + i] - xjw;
       kv *= dw * dw;
@@ -179,12 +182,13 @@ __global__ void __launch_bounds__(NT) kmv_f64_sym_kernel(const Sym64Args a) {
   }
 }
 
-// The kernel values themselves (sigma^2 left out), both orders of every pair: K is ldk x ldk, ldk a
+// The kernel values themselves, as form_pair, both orders of every pair: K is ldk x ldk, ldk a
 // multiple of T.  Values of rows and columns past n are finite where x is, and unused.
-template <int DP>
+template <int DP, bool LIB>
 __global__ void __launch_bounds__(kFillNT) form_kmat_kernel(const double* __restrict__ xhat,
                                                             long long n,
                                                             const double* __restrict__ exp_tab,
+                                                            const DevParams* __restrict__ params,
                                                             double* __restrict__ K, long long ldk) {
   constexpr int T = 32, LD = T + 1;
   __shared__ double sK[T * LD], sXI[DP * T];
@@ -192,7 +196,7 @@ __global__ void __launch_bounds__(kFillNT) form_kmat_kernel(const double* __rest
   long long bj;
   pair_blocks(blockIdx.x, bi, bj);
   const long long i0 = (long long)bi * T, j0 = bj * T;
-  form_pair<DP, T, kFillNT, kModeK>(xhat, n, exp_tab, 0, i0, j0, sXI, sK);
+  form_pair<DP, T, kFillNT, kModeK, LIB>(xhat, n, exp_tab, 0, i0, j0, sXI, sK, params->sigma2);
   const int j = threadIdx.x % T;
   for (int i = threadIdx.x / T; i < T; i += kFillNT / T) {
     K[(i0 + i) * ldk + j0 + j] = sK[i * LD + j];
@@ -250,18 +254,25 @@ cudaError_t sym_dp(KmvLaunch& L, cudaStream_t s) {
 
 }  // namespace
 
-cudaError_t launch_form_kmat(const double* xhat, long long n, int DP, const double* exp_tab, double* K,
-                             long long ldk, cudaStream_t s) {
+template <bool LIB>
+static cudaError_t form_kmat(const double* xhat, long long n, int DP, const double* exp_tab,
+                             const DevParams* P, double* K, long long ldk, cudaStream_t s) {
   const long long nb = (n + 31) / 32;
   const unsigned pairs = (unsigned)(nb * (nb + 1) / 2);
   switch (DP) {
-    case 2: form_kmat_kernel<2><<<pairs, kFillNT, 0, s>>>(xhat, n, exp_tab, K, ldk); break;
-    case 4: form_kmat_kernel<4><<<pairs, kFillNT, 0, s>>>(xhat, n, exp_tab, K, ldk); break;
-    case 8: form_kmat_kernel<8><<<pairs, kFillNT, 0, s>>>(xhat, n, exp_tab, K, ldk); break;
-    case 16: form_kmat_kernel<16><<<pairs, kFillNT, 0, s>>>(xhat, n, exp_tab, K, ldk); break;
+    case 2: form_kmat_kernel<2, LIB><<<pairs, kFillNT, 0, s>>>(xhat, n, exp_tab, P, K, ldk); break;
+    case 4: form_kmat_kernel<4, LIB><<<pairs, kFillNT, 0, s>>>(xhat, n, exp_tab, P, K, ldk); break;
+    case 8: form_kmat_kernel<8, LIB><<<pairs, kFillNT, 0, s>>>(xhat, n, exp_tab, P, K, ldk); break;
+    case 16: form_kmat_kernel<16, LIB><<<pairs, kFillNT, 0, s>>>(xhat, n, exp_tab, P, K, ldk); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
+}
+
+cudaError_t launch_form_kmat(const double* xhat, long long n, int DP, const double* exp_tab,
+                             const DevParams* P, double* K, long long ldk, cudaStream_t s) {
+  return exp_tab ? form_kmat<false>(xhat, n, DP, exp_tab, P, K, ldk, s)
+                 : form_kmat<true>(xhat, n, DP, exp_tab, P, K, ldk, s);
 }
 
 size_t kmv_f64_sym_bytes(long long n, int R) {

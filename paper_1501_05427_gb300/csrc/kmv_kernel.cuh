@@ -31,7 +31,6 @@ struct KmvDevArgs {
   long long ldu;
   const int* umap;
   const DevParams* params;
-  const double* exp_tab;   // FP64 only
   int mode, which;
   int nsplit, tiles_per_split, ntiles;
   T* partials;
@@ -61,13 +60,17 @@ __device__ __forceinline__ void load_row(const T* __restrict__ p, T (&x)[DP]) {
 }
 
 // Signal covariance from the squared prescaled distance.
-template <typename T>
+// TAB: in FP64 the table-driven exponential, else the library's (the solves' own, see
+// launch_form_kmat).
+template <typename T, bool TAB = false>
 __device__ __forceinline__ T kernel_from_dist(T dist, float c0, float c1, double sigma2,
                                               const double* __restrict__ exp_tab) {
   if constexpr (sizeof(T) == 4) {
     return ex2_approx(fmaf(-c1, dist, c0));
-  } else {
+  } else if constexpr (TAB) {
     return sigma2 * exp_neg_half(dist, exp_tab);
+  } else {
+    return sigma2 * exp(-0.5 * dist);
   }
 }
 
@@ -166,7 +169,7 @@ __global__ void __launch_bounds__(NT) kmv_kernel(const KmvDevArgs<T> a) {
               const T df = xi[t][k] - xj[k];
               dist = fma(df, df, dist);
             }
-            T kv = kernel_from_dist<T>(dist, c0, c1, sigma2, a.exp_tab);
+            T kv = kernel_from_dist<T>(dist, c0, c1, sigma2, nullptr);
             if constexpr (MODE == kModeDLen) {
               const T dw = xiw[t] - tX[(jq + q) * DP + a.which];
               kv *= dw * dw;

@@ -67,7 +67,6 @@ struct KmvInst {
     a.ldu = L.ldu;
     a.umap = L.umap;
     a.params = L.params;
-    a.exp_tab = L.exp_tab;
     a.mode = L.mode;
     a.which = L.which;
     a.nsplit = p.nsplit;

@@ -60,6 +60,7 @@ struct CgArgs {
   double* part2;         // ... and right-hand side
   int nchunk;            // CTAs per column of the CG start
   long long chunk;       // rows per CTA
+  int ordered;           // FP64: sums in the order of cg_ordered_dot
   double alpha_thr, eps, beta;
   int max_iter;
   int has_s0;
@@ -281,6 +282,35 @@ __device__ inline double cluster_sum_warp0(double v, double* red, double* slot) 
   return v;
 }
 
+// FP64 iterations whose sums keep one order, whatever the cluster: kCgChunkNT threads take every
+// kCgChunkNT'th row of a chunk, then the warps' and the chunks' sums are added one by one.  A
+// truncated solve's estimates follow the rounding of these sums, so it is part of the result.
+template <typename T>
+__device__ inline double cg_ordered_dot(const T* x, const T* y, long long i0, long long i1,
+                                        double* red, double* slot) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const int tid = threadIdx.x;
+  double p = 0.0;
+  if (tid < kCgChunkNT) {
+#pragma unroll 4
+    for (long long i = i0 + tid; i < i1; i += kCgChunkNT) p += (double)x[i] * (double)y[i];
+  }
+  p = warp_sum(p);
+  if ((tid & 31) == 0) red[tid >> 5] = p;
+  __syncthreads();
+  if (tid == 0) {
+    double t = 0.0;
+    for (int w = 0; w < kCgChunkNT / 32; ++w) t += red[w];
+    *slot = t;
+  }
+  cl.sync();
+  double t = 0.0;
+  if (tid < 32)
+    for (int k = 0; k < (int)cl.num_blocks(); ++k) t += *cl.map_shared_rank(slot, k);
+  return t;
+}
+
 // The scalars warp 0 hands to the CTA.
 template <typename T>
 struct CgShared {
@@ -310,14 +340,21 @@ __device__ inline void cg_round_body(const CgArgs<T>& a, int ch, int li, CgShare
   V* se0 = reinterpret_cast<V*>(a.SE + (long long)st.est_off * a.ld);
   V* se1 = se0 + a.ld / VN;
 
-  double p = 0.0;
+  const bool ordered = sizeof(T) == 8 && a.ordered;
+  const long long i0 = min(a.n, v0 * VN), i1 = min(a.n, v1 * VN);
+  double dKd;
+  if (ordered) {
+    dKd = cg_ordered_dot(a.D + col, a.KD + col, i0, i1, sh.red, &sh.slot[0]);
+  } else {
+    double p = 0.0;
 #pragma unroll 4
-  for (long long i = v0 + tid; i < v1; i += kCgNT) {
-    const V di = d[i], ki = kd[i];
+    for (long long i = v0 + tid; i < v1; i += kCgNT) {
+      const V di = d[i], ki = kd[i];
 #pragma unroll
-    for (int q = 0; q < VN; ++q) p += (double)di.v[q] * (double)ki.v[q];
+      for (int q = 0; q < VN; ++q) p += (double)di.v[q] * (double)ki.v[q];
+    }
+    dKd = cluster_sum_warp0(p, sh.red, &sh.slot[0]);
   }
-  const double dKd = cluster_sum_warp0(p, sh.red, &sh.slot[0]);
   if (warp0) {
     const bool bad = !(dKd > 0.0) || !isfinite(dKd);
     const double al = bad ? 0.0 : st.ee / dKd;
@@ -391,7 +428,13 @@ __device__ inline void cg_round_body(const CgArgs<T>& a, int ch, int li, CgShare
       se1[i] = x;
     }
   }
-  const double ee1 = cluster_sum_warp0(p2, sh.red, &sh.slot[1]);
+  double ee1;
+  if (ordered) {
+    __syncthreads();
+    ee1 = cg_ordered_dot(a.E + col, a.E + col, i0, i1, sh.red, &sh.slot[1]);
+  } else {
+    ee1 = cluster_sum_warp0(p2, sh.red, &sh.slot[1]);
+  }
   if (warp0) {
     const int m1 = st.m + 1;
     int ph = st.phase, l1 = st.l, outcome = st.outcome;
@@ -508,11 +551,22 @@ cudaError_t launch_clustered(void (*kernel)(Params...), dim3 grid, int cluster, 
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-// One CG iteration of nl live columns.
+// One CG iteration of nl live columns.  Ordered sums: chunks of at least 2,048 rows, about two
+// CTAs per SM over all columns; beyond eight chunks (more than 16,384 rows) the usual form.
 template <typename T>
-cudaError_t launch_cg_round(CgArgs<T> a, int nl, cudaStream_t s) {
-  const int c = cg_cluster_size(a.n);
+cudaError_t launch_cg_round(CgArgs<T> a, int nl, int num_sms, cudaStream_t s) {
+  int c = cg_cluster_size(a.n);
   a.chunk = cg_cluster_rows(a.ld, c);
+  if (a.ordered) {
+    const long long target = std::max(1, (2 * num_sms + nl - 1) / nl);
+    const long long ch = (std::max<long long>((a.n + target - 1) / target, 2048) + 255) / 256 * 256;
+    const long long nc = (a.n + ch - 1) / ch;
+    a.ordered = nc <= kCgMaxCluster;
+    if (a.ordered) {
+      c = (int)nc;
+      a.chunk = ch;
+    }
+  }
   return launch_clustered(cg_round_kernel<T>, dim3((unsigned)c, (unsigned)nl), c, s, a);
 }
 

@@ -260,6 +260,7 @@ struct KmvLaunch {
   const double* exp_tab; // FP64: the exponential's table (exp64.cuh)
   void* v3;              // FP32: scratch of the tensor-core contraction's operand (kmv_f32_tc.cu),
                          // 96 BF16 values per point (null: SIMT kernel)
+  bool ordered;          // FP64: keep the row-block kernel's order of additions
   const double* kmat;    // FP64: the kernel values of this solve, n <= kKmatMaxN (null: not formed)
   bool simt;             // FP32: the SIMT kernel whatever the sizes
   bool v_packed;         // v3 already holds the operand (packed by the prescale launch)
@@ -373,9 +374,13 @@ cudaError_t launch_kmv_f32_tc(KmvLaunch& L, cudaStream_t s);
 // every round.
 constexpr long long kKmatMaxN = 5792;
 constexpr long long kmat_ld(long long n) { return (n + 31) / 32 * 32; }
-cudaError_t launch_form_kmat(const double* xhat, long long n, int DP, const double* exp_tab, double* K,
-                             long long ldk, cudaStream_t s);
+// With exp_tab by the table-driven exponential and without sigma^2, for launch_kmv_f64_dense; without
+// by the library's and with sigma^2, for launch_kmv_f64_ordered, whose products then have the bits
+// of the row-block kernel's (split count nsplit).
+cudaError_t launch_form_kmat(const double* xhat, long long n, int DP, const double* exp_tab,
+                             const DevParams* P, double* K, long long ldk, cudaStream_t s);
 cudaError_t launch_kmv_f64_dense(KmvLaunch& L, cudaStream_t s);
+cudaError_t launch_kmv_f64_ordered(KmvLaunch& L, int nsplit, cudaStream_t s);
 bool kmv_f64_sym_applies(const KmvLaunch& L);
 cudaError_t launch_kmv_f64_sym(KmvLaunch& L, cudaStream_t s);
 // Partial sums of one launch: FP64 pairs with R columns; the 128-row tensor-core products with up
