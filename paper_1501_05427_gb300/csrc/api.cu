@@ -412,12 +412,15 @@ static ulisse_status prescale(ulisse_ctx* ctx) {
 
 // A truncated solve in FP64 amplifies the rounding of its products and sums (2^-53 becomes 1e-3
 // within ten steps of a chain), so that rounding is part of its result: the library's exponential
-// and one order of additions, whatever kernel does them.  Products by themselves and predictions,
-// which solve to convergence, use the faster forms.
+// and one order of additions, whatever kernel does them.  Products by themselves and predictions
+// that solve to convergence (q = 0) use the faster forms; with q > 0 a prediction's columns are
+// the truncated estimates of ulisse_solve and keep its rounding.
 struct OrderedScope {
   ulisse_ctx* ctx;
   bool was;
-  OrderedScope(ulisse_ctx* c) : ctx(c), was(c->ordered) { c->ordered = c->f64; }
+  explicit OrderedScope(ulisse_ctx* c, bool on = true) : ctx(c), was(c->ordered) {
+    c->ordered = on && c->f64;
+  }
   ~OrderedScope() { ctx->ordered = was; }
 };
 
@@ -1444,6 +1447,7 @@ extern "C++" {
 template <typename T>
 static ulisse_status predict_core(ulisse_ctx* ctx, const float* Xs, long long m,
                                   unsigned long long step, float* mean, float* var) {
+  const OrderedScope ordered(ctx, ctx->cfg.q > 0.0);
   const int R = var ? 1 + (int)m : 1;
   CKS(ensure_columns(ctx, R, R));
   CK(cudaMemsetAsync(ctx->status_dev, 0, sizeof(int), ctx->stream));
