@@ -536,8 +536,9 @@ ulisse_status ulisse_set_tune(ulisse_ctx *ctx, const ulisse_tune_entry *table, i
  * that nothing completes.  The wait gives up after about half a second (2^30 SM cycles), the
  * kernel records the timeout in the context's status word as every kernel of the library
  * does when one of its bounded waits runs out, and this call reports it as any call would:
- * ULISSE_ERR_TIMEOUT (after zeroing the context's split counters, as every timeout does).
- * The context stays usable.  Synchronises the stream.
+ * ULISSE_ERR_TIMEOUT (after zeroing the split counters of the context, or of a batch and its
+ * problems, as every timeout does; the self-test first leaves counts in them that no launch
+ * would complete).  The context stays usable.  Synchronises the stream.
  */
 ulisse_status ulisse_selftest_wait_timeout(ulisse_ctx *ctx);
 

@@ -173,6 +173,7 @@ struct ulisse_ctx {
   void* b_tc_args = nullptr;       // 3 x problems kernel arguments: rounds, K s_0, batch K V
   float* b_tc_part = nullptr;      // split partial sums of all problems
   int* b_tc_cnt = nullptr;         // split counters of all problems (zero between launches)
+  size_t b_tc_cnt_len = 0;
   std::vector<int> b_tc_nsplit;
   std::vector<size_t> b_tc_part_off, b_tc_cnt_off;
   void* b_v3 = nullptr;            // FP32: operand scratch of the tensor-core contraction
@@ -643,13 +644,24 @@ static ulisse_status read_result(ulisse_ctx* ctx, int* status) {
   return ULISSE_OK;
 }
 
+// Every byte of the counters that count a launch's CTAs (split counters, the gradient passes' last
+// CTA), a batch's and its problems' too; zero between launches.
+static void fill_counters(ulisse_ctx* ctx, int byte) {
+  auto fill = [&](int* p, size_t len) {
+    if (p && len) cudaMemsetAsync(p, byte, sizeof(int) * len, ctx->stream);
+  };
+  fill(ctx->counters, (size_t)ctx->counters_len);
+  fill(ctx->gcounter, 1);
+  fill(ctx->b_tc_cnt, ctx->b_tc_cnt_len);
+  fill(ctx->b_gt_cnt, ctx->subs.size());
+  for (ulisse_ctx* sub : ctx->subs) fill_counters(sub, byte);
+}
+
 // A CTA whose bounded wait ran out returns before it counts itself in its row block's split
 // counter or the gradient's last-CTA counter (both reset themselves only when every CTA
 // arrives): zero them, so that the context's next launches pick their last CTA correctly.
 static void reset_counters_after_timeout(ulisse_ctx* ctx) {
-  if (ctx->counters && ctx->counters_len > 0)
-    cudaMemsetAsync(ctx->counters, 0, sizeof(int) * ctx->counters_len, ctx->stream);
-  if (ctx->gcounter) cudaMemsetAsync(ctx->gcounter, 0, sizeof(int), ctx->stream);
+  fill_counters(ctx, 0);
   cudaStreamSynchronize(ctx->stream);
 }
 
@@ -2342,6 +2354,7 @@ ulisse_status ulisse_create_batched(ulisse_ctx** out, int n_problems, const long
       ctx->b_v3_off.push_back(v3);
       v3 += (size_t)((n[b] + 31) / 32) * 32 * 3 * kMaxRChunk * 2;
     }
+    ctx->b_tc_cnt_len = cnt;
     if ((s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->b_tc_items), sizeof(int4) * tci.size())) ||
         (s = dev_alloc(ctx, &ctx->b_tc_args,
                        3 * (mixed ? tc2_batch_args_bytes(n_problems) : f3_batch_args_bytes(n_problems)))) ||
@@ -3243,6 +3256,7 @@ __global__ void selftest_wait_timeout_kernel(int* status) {
 ulisse_status ulisse_selftest_wait_timeout(ulisse_ctx* ctx) {
   if (!ctx) return ULISSE_ERR_ARG;
   CK(cudaMemsetAsync(ctx->status_dev, 0, sizeof(int), ctx->stream));
+  fill_counters(ctx, 1);   // counts that no launch completes
   selftest_wait_timeout_kernel<<<1, 32, 0, ctx->stream>>>(ctx->status_dev);
   CK(cudaGetLastError());
   int st = 0;
