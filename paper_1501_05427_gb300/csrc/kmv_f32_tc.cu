@@ -141,10 +141,12 @@ __device__ __forceinline__ uint32_t f3_bits(const __nv_bfloat162& v) {
 // Rows whose sum came out as NaN, once more: a column of V that holds an infinity meets zeros and
 // both signs among the parts of K, where k_ij > 0 itself gives that infinity.  The terms that are
 // not finite decide such a sum, so only they are formed (a column without any stays as it is).
+// From sigma^2 = 2^127 on, the kernel values' high parts can be infinite too: then all terms are.
 // Not reached by finite results; a scan of V per entry otherwise.
 template <int MODE>
 __device__ __noinline__ void f3_not_finite(const F3Args& a, const long long row0, const int R) {
   const float c0 = a.params->c0f, c1 = a.params->c1f;
+  const bool all = !(c0 < 127.f);
   for (int idx = threadIdx.x; idx < R * kF3BM; idx += kF3Threads) {
     const int r = idx / kF3BM;
     const long long i = row0 + (idx - r * kF3BM);
@@ -156,7 +158,7 @@ __device__ __noinline__ void f3_not_finite(const F3Args& a, const long long row0
     float u = 0.f;
     bool any = false;
     for (long long j = 0; j < a.n && !isnan(u); ++j) {
-      if (isfinite(v[j])) continue;
+      if (!all && isfinite(v[j])) continue;
       const float* xj = a.xhat + j * a.DP;
       float dist = 0.f;
       for (int k = 0; k < a.DP; ++k) dist = fmaf(xi[k] - xj[k], xi[k] - xj[k], dist);
