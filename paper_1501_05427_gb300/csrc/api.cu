@@ -1199,7 +1199,7 @@ static ulisse_status create_impl(ulisse_ctx** out, const float* X, const float* 
     cv.add(ctx->Xt_b, 4 * (ctx->ld128 / 32) * tc2_b_stride(16));
   }
   if (!ctx->f64 && !ctx->mixed && !in_batch && n >= kF32TcMinN)
-    cv.add(ctx->v3, 2 * 3 * kMaxRChunk * ctx->ldn);
+    cv.add(ctx->v3, pack_v3_bytes((n + 31) / 32, kMaxRChunk));
   if (ctx->f64) cv.add(ctx->exp_tab, sizeof(double) * kExpTabN);
   // split-j scratch for the widest usual product, so that no first call has to allocate it (a
   // batch's launches have their own)
@@ -2352,7 +2352,7 @@ ulisse_status ulisse_create_batched(ulisse_ctx** out, int n_problems, const long
     size_t v3 = 0;
     for (int b = 0; b < n_problems; ++b) {
       ctx->b_v3_off.push_back(v3);
-      v3 += (size_t)((n[b] + 31) / 32) * 32 * 3 * kMaxRChunk * 2;
+      v3 += pack_v3_bytes((n[b] + 31) / 32, kMaxRChunk);   // a multiple of 16 (bulk copies)
     }
     ctx->b_tc_cnt_len = cnt;
     if ((s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->b_tc_items), sizeof(int4) * tci.size())) ||

@@ -41,8 +41,8 @@ struct BatchKmvDesc {
   const int* nlive;      // live column count (device), 0 = skip the problem
 };
 
-// The same product by the tensor-core contraction (kmv_f32_tc.cu): its operand scratch (96 BF16
-// values per point, points rounded up to 32), the split of its j range, partial sums and counters.
+// The same product by the tensor-core contraction (kmv_f32_tc.cu): its operand scratch
+// (pack_v3_bytes), the split of its j range, partial sums and counters.
 struct F3Problem {
   BatchKmvDesc k;
   void* v3;

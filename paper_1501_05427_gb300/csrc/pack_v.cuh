@@ -29,6 +29,10 @@ __device__ inline void pack_v2(const float* __restrict__ V, long long ldv,
   }
 }
 
+// A tile of 32 points with N columns of V in three parts, and all tiles of a product: the tiles, then
+// per tile and column a word with a bit for every point whose value is not finite.
+constexpr size_t pack_v3_bytes(long long ntiles, int N) { return (size_t)ntiles * N * (3 * 32 * 2 + 4); }
+
 // High, middle and low part: a float exactly (FP32 products).  The high part of the largest floats
 // is rounded towards zero, as to nearest it is infinite; a value that is not finite stays whole in
 // the high part.
@@ -36,6 +40,7 @@ __device__ inline void pack_v3(const float* __restrict__ V, long long ldv,
                                const int* __restrict__ vmap, int R, int N, long long n,
                                long long ntiles, __nv_bfloat16* __restrict__ Vp, int cta, int ctas) {
   const int per = N * 32;
+  uint32_t* bad = reinterpret_cast<uint32_t*>(Vp + ntiles * 3LL * per);
   for (long long idx = cta * (long long)blockDim.x + threadIdx.x; idx < ntiles * per;
        idx += (long long)ctas * blockDim.x) {
     const long long t = idx / per;
@@ -51,6 +56,9 @@ __device__ inline void pack_v3(const float* __restrict__ V, long long ldv,
     o[0] = h;
     o[per] = m;
     o[2 * per] = __float2bfloat16_rn(v1 - __bfloat162float(m));
+    // a warp holds the 32 points of one tile and column
+    const uint32_t mask = __ballot_sync(0xffffffffu, !isfinite(v));
+    if (jj == 0) bad[t * N + r] = mask;
   }
 }
 
