@@ -494,7 +494,8 @@ ulisse_status ulisse_set_graph(ulisse_ctx *ctx, int enable);
 typedef struct {
     int live_cols;           /* columns of the product */
     int width;               /* compiled column count (SIMT) or MMA N (tensor cores) used */
-    int rows_per_thread;     /* SIMT rows per thread (0 on the tensor-core path) */
+    int rows_per_thread;     /* SIMT rows per thread; 0 in mixed precision, and in FP32 where the
+                                untuned choice (tensor cores or SIMT, by size) is the fastest */
     int nsplit;              /* j-range split count forced (0: the launch plan's choice) */
     float ms;                /* median time of the chosen configuration */
     float ms_default;        /* median time of the untuned configuration */
@@ -510,7 +511,7 @@ typedef struct {
  * fastest from then on (the untuned choice is always a candidate).  psi: host, the
  * parameters to tune at (they set the data layout only; any valid psi).  out: NULL or
  * max_cols entries.  The tuning launches are not counted as the method's work.  Results
- * change only in the summation order of the split j range (the last bits).
+ * change only in their last bits, as with ulisse_set_tune.
  * FP32 and mixed contexts. */
 ulisse_status ulisse_autotune(ulisse_ctx *ctx, const double *psi, int max_cols, int reps,
                               ulisse_tune_entry *out);
@@ -521,12 +522,15 @@ ulisse_status ulisse_autotune(ulisse_ctx *ctx, const double *psi, int max_cols, 
  * k + 1 columns.  Per entry (live_cols, ms and ms_default are ignored):
  *   width: k + 1 .. 64; the smallest compiled column count at least this wide is used
  *          (tensor cores: the MMA N 16, 32 or 64; SIMT: up to 32);
- *   rows_per_thread: SIMT 2 or 4 (ignored on the tensor-core path);
+ *   rows_per_thread: FP32 2 or 4: the SIMT kernel in this shape; 0: the untuned choice, the
+ *           tensor-core contraction or the SIMT kernel by size (width is then not used and
+ *           nsplit must be 0).  Ignored in mixed precision;
  *   nsplit: 0 (the launch plan's choice) or 1 .. 64 (the j range is still split further
  *           where a tensor-core CTA would exceed its accumulation bound);
  *   cross_term: tensor-core path 1 or 2, SIMT path 0.
- * Column counts beyond n keep the untuned choice.  Results differ from another table's only
- * in the summation order of the split j range.  n = 0 (table may be NULL) clears the table.
+ * Column counts beyond n keep the untuned choice.  Results differ from another table's in the
+ * summation order of the split j range, and in FP32 in the contraction's rounding where one
+ * table fixes the SIMT kernel and the other does not.  n = 0 (table may be NULL) clears the table.
  * Errors: ULISSE_ERR_ARG (FP64 or batched context, n out of range, an invalid entry; the
  * table in use is then unchanged). */
 ulisse_status ulisse_set_tune(ulisse_ctx *ctx, const ulisse_tune_entry *table, int n);

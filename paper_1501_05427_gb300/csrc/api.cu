@@ -120,7 +120,6 @@ struct ulisse_ctx {
   int last_nsplit = 1;        // split count of the last K V launch (or plan)
 
   // CUDA graph of one SGLD step (ulisse_sgld_chain)
-  bool simt = false;          // FP32 products by the SIMT kernel (the autotuner's candidates)
   bool v_packed = false;      // the prescale launch packed the coming product's operand
   bool planning = false;      // launch helpers only size their scratch
   bool capturing = false;     // launch helpers are being captured: no host-side counting
@@ -574,14 +573,17 @@ static ulisse_status run_kmv(ulisse_ctx* ctx, const void* V, const int* vmap, in
     L.ordered = ctx->ordered;
     L.kmat = ctx->kmat_formed ? ctx->kmat : nullptr;
     L.v3 = ctx->v3;
-    L.simt = ctx->simt || ctx->cfg.kmv_rows_per_thread != 0;
+    L.simt = ctx->cfg.kmv_rows_per_thread != 0;
     L.v_packed = ctx->v_packed;
     L.mode = mode;
     L.which = which;
     L.tm = ctx->cfg.kmv_rows_per_thread;
     L.status = ctx->status_dev;
     L.num_sms = ctx->num_sms;
-    if (mode == kModeK && (int)ctx->tune.size() >= L.R && ctx->tune[L.R - 1].width > 0) {
+    // a table entry with rows per thread fixes the SIMT kernel's shape; without, it means the
+    // untuned choice
+    if (mode == kModeK && (int)ctx->tune.size() >= L.R && ctx->tune[L.R - 1].tm > 0) {
+      L.simt = true;
       L.r_min = ctx->tune[L.R - 1].width;
       L.tm = ctx->tune[L.R - 1].tm;
       L.nsplit = ctx->tune[L.R - 1].nsplit;
@@ -3090,7 +3092,6 @@ static ulisse_status time_kmv_config(ulisse_ctx* ctx, int nl, int width, int tm,
     ctx->tune.resize((size_t)nl, ulisse_ctx::KmvTune{0, 0, 0, 0.f, 0.f, 0});
   const ulisse_ctx::KmvTune saved = ctx->tune[nl - 1];
   ctx->tune[nl - 1] = ulisse_ctx::KmvTune{width, tm, nsplit, 0.f, 0.f, cross};
-  ctx->simt = !ctx->mixed && width > 0;   // FP32: a given shape means the SIMT kernel
   ctx->planning = true;
   ulisse_status r = run_kmv(ctx, ctx->D, ctx->iota, nl, ctx->KD, ctx->iota, kModeK, -1);
   ctx->planning = false;
@@ -3117,7 +3118,6 @@ static ulisse_status time_kmv_config(ulisse_ctx* ctx, int nl, int width, int tm,
   if (a) cudaEventDestroy(a);
   if (b) cudaEventDestroy(b);
   ctx->tune[nl - 1] = saved;
-  ctx->simt = false;
   if (r != ULISSE_OK) return r;
   std::sort(t.begin(), t.end());
   *ms_out = t[t.size() / 2];
@@ -3170,9 +3170,7 @@ ulisse_status ulisse_autotune(ulisse_ctx* ctx, const double* psi, int max_cols, 
           int sp = 1;
           r = time_kmv_config(ctx, nl, wd, tm, 0, cr, reps, &ms, &sp);
           if (r != ULISSE_OK) break;
-          // FP32: an entry without a split count leaves the kernel to the dispatch (tensor
-          // cores or SIMT by size), so a SIMT winner carries its planned one
-          if (ms < best.ms) best = ulisse_ctx::KmvTune{wd, tm, ctx->mixed ? 0 : sp, ms, ms_def, cr};
+          if (ms < best.ms) best = ulisse_ctx::KmvTune{wd, tm, 0, ms, ms_def, cr};
         }
         if (r != ULISSE_OK) break;
       }
@@ -3180,21 +3178,23 @@ ulisse_status ulisse_autotune(ulisse_ctx* ctx, const double* psi, int max_cols, 
     }
     if (r != ULISSE_OK) break;
     const int wd = best.width > 0 ? best.width : nl;
+    // FP32 without a shape yet: the splits of the SIMT kernel's default shape
+    const int tm = ctx->mixed || best.tm != 0 ? best.tm
+                   : ctx->cfg.kmv_rows_per_thread != 0 ? ctx->cfg.kmv_rows_per_thread : 2;
     float ms_base = 0.f;
     int base = 1;
-    r = time_kmv_config(ctx, nl, wd, best.tm, 0, best.cross, 1, &ms_base, &base);   // its planned split
+    r = time_kmv_config(ctx, nl, wd, tm, 0, best.cross, 1, &ms_base, &base);   // its planned split
     for (int sp : {base / 2, base * 2}) {
       if (r != ULISSE_OK || sp < 1 || sp == base) continue;
       float ms = 0.f;
       int used = sp;
-      r = time_kmv_config(ctx, nl, wd, best.tm, sp, best.cross, reps, &ms, &used);
+      r = time_kmv_config(ctx, nl, wd, tm, sp, best.cross, reps, &ms, &used);
       if (r == ULISSE_OK && ms < best.ms)
-        best = ulisse_ctx::KmvTune{wd, best.tm, sp, ms, ms_def, best.cross};
+        best = ulisse_ctx::KmvTune{wd, tm, sp, ms, ms_def, best.cross};
     }
     if (r != ULISSE_OK) break;
     if (best.width == 0) best.width = nl;
-    if (best.tm == 0) best.tm = ctx->mixed || ctx->cfg.kmv_rows_per_thread != 0
-                                    ? ctx->cfg.kmv_rows_per_thread : 2;
+    if (best.tm == 0) best.tm = ctx->cfg.kmv_rows_per_thread;   // FP32: 0 is the untuned choice
     table[nl - 1] = best;
   }
   ctx->prof = prof;
@@ -3227,7 +3227,8 @@ ulisse_status ulisse_set_tune(ulisse_ctx* ctx, const ulisse_tune_entry* table, i
     if (ctx->mixed)
       ok = ok && (e.cross_term == kCrossPipe || e.cross_term == kCrossTensor);
     else
-      ok = ok && (e.rows_per_thread == 2 || e.rows_per_thread == 4) && e.cross_term == 0;
+      ok = ok && (e.rows_per_thread == 2 || e.rows_per_thread == 4 ||
+                  (e.rows_per_thread == 0 && e.nsplit == 0)) && e.cross_term == 0;
     if (!ok) return fail(ctx, ULISSE_ERR_ARG, "invalid K V table entry " + std::to_string(k));
     t[k] = ulisse_ctx::KmvTune{e.width, e.rows_per_thread, e.nsplit, e.ms, e.ms_default,
                                e.cross_term};

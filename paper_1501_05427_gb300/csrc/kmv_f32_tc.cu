@@ -548,7 +548,7 @@ cudaError_t f3_dp(KmvLaunch& L, cudaStream_t s) {
 // 6 columns 2,200 / 2,295, 7 columns 2,494 / 2,296, 32 columns 5,223 / 2,275.  (Error against 64
 // bits, relative: 1.7e-7 / 1.3e-7 at n = 1,030, 8.5e-7 / 2.8e-7 at n = 22,784, 17 columns.)
 bool kmv_f32_tc_applies(const KmvLaunch& L) {
-  return L.v3 && L.mode != kModeDLam && L.nsplit == 0 && !L.simt && f32_tc_columns(L.n, L.R);
+  return L.v3 && L.mode != kModeDLam && !L.simt && f32_tc_columns(L.n, L.R);
 }
 
 cudaError_t launch_kmv_f32_tc(KmvLaunch& L, cudaStream_t s) {
