@@ -259,7 +259,7 @@ struct KmvLaunch {
   int which;             // dimension for kModeDLen
   const double* exp_tab; // FP64: the exponential's table (exp64.cuh)
   void* v3;              // FP32: scratch of the tensor-core contraction's operand (kmv_f32_tc.cu),
-                         // pack_v3_bytes (null: SIMT kernel)
+                         // 96 BF16 values per point (null: SIMT kernel)
   bool ordered;          // FP64: keep the row-block kernel's order of additions
   const double* kmat;    // FP64: the kernel values of this solve, n <= kKmatMaxN (null: not formed)
   bool simt;             // FP32: the SIMT kernel whatever the sizes
