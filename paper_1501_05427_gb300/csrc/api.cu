@@ -206,7 +206,6 @@ struct ulisse_ctx {
 };
 
 static thread_local std::string g_create_error;
-static constexpr int kMaxCgChunks = 64;
 
 #define CK(call)                                                                     \
   do {                                                                               \
@@ -712,6 +711,7 @@ static CgArgs<T> cg_args(ulisse_ctx* ctx, int has_s0, unsigned long long step) {
   a.Sbest = (T*)ctx->Sbest;
   a.status = ctx->status_dev;
   a.ordered = ctx->ordered;
+  a.o_chunks = a.o_per = 0;
   return a;
 }
 

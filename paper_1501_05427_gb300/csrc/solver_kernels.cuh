@@ -12,6 +12,7 @@
 namespace ulisse {
 
 constexpr int kCgChunkNT = 256;   // threads of the CG start
+constexpr int kMaxCgChunks = 64;  // row ranges with a partial sum each, per column
 
 // ------------------------------------------------------------------------------------
 // a2: probes r_j (column j = 1..nr of B): +-1 from the top bit, or N(0,1) by Box-Muller,
@@ -60,7 +61,8 @@ struct CgArgs {
   double* part2;         // ... and right-hand side
   int nchunk;            // CTAs per column of the CG start
   long long chunk;       // rows per CTA
-  int ordered;           // FP64: sums in the order of cg_ordered_dot
+  int ordered;           // FP64: rows per chunk of cg_ordered_dot's sums, 0: sums in any order
+  int o_chunks, o_per;   // ... the column's chunks, and those of a CTA (chunk rows)
   double alpha_thr, eps, beta;
   int max_iter;
   int has_s0;
@@ -283,31 +285,52 @@ __device__ inline double cluster_sum_warp0(double v, double* red, double* slot) 
 }
 
 // FP64 iterations whose sums keep one order, whatever the cluster: kCgChunkNT threads take every
-// kCgChunkNT'th row of a chunk, then the warps' and the chunks' sums are added one by one.  A
-// truncated solve's estimates follow the rounding of these sums, so it is part of the result.
+// kCgChunkNT'th row of a chunk of a.ordered rows, then the warps' and the chunks' sums are added one
+// by one.  A CTA takes as many chunks as its rows hold, two at a time.  A truncated solve's estimates
+// follow the rounding of these sums, so it is part of the result.  parts: a shared double per chunk
+// of the CTA (the peers read them).  The sum is valid in warp 0.
 template <typename T>
-__device__ inline double cg_ordered_dot(const T* x, const T* y, long long i0, long long i1,
-                                        double* red, double* slot) {
+__device__ inline double cg_ordered_dot(const CgArgs<T>& a, const T* x, const T* y, int ch,
+                                        double* red, double* parts) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
-  const int tid = threadIdx.x;
-  double p = 0.0;
-  if (tid < kCgChunkNT) {
+  constexpr int kWarps = kCgChunkNT / 32, kGroups = kCgNT / kCgChunkNT;
+  const int tid = threadIdx.x, g = tid / kCgChunkNT, lane = tid & 31;
+  const int rows = a.ordered, per = a.o_per;
+  const long long at = (long long)ch * a.chunk;
+  x += at;
+  y += at;
+  const int left = (int)min(a.chunk, max(a.n - at, 0LL));   // the CTA's rows
+#pragma unroll 1
+  for (int q0 = 0; q0 < per; q0 += kGroups) {
+    const int q = q0 + g, end = min(left, (q + 1) * rows);
+    double p = 0.0;
 #pragma unroll 4
-    for (long long i = i0 + tid; i < i1; i += kCgChunkNT) p += (double)x[i] * (double)y[i];
-  }
-  p = warp_sum(p);
-  if ((tid & 31) == 0) red[tid >> 5] = p;
-  __syncthreads();
-  if (tid == 0) {
-    double t = 0.0;
-    for (int w = 0; w < kCgChunkNT / 32; ++w) t += red[w];
-    *slot = t;
+    for (int i = q * rows + tid % kCgChunkNT; i < end; i += kCgChunkNT)
+      p += (double)x[i] * (double)y[i];
+    p = warp_sum(p);
+    if (lane == 0) red[tid >> 5] = p;
+    __syncthreads();
+    if (tid % kCgChunkNT == 0 && q < per) {
+      double t = 0.0;
+      for (int w = 0; w < kWarps; ++w) t += red[g * kWarps + w];
+      parts[q] = t;
+    }
+    if (q0 + kGroups < per) __syncthreads();
   }
   cl.sync();
   double t = 0.0;
-  if (tid < 32)
-    for (int k = 0; k < (int)cl.num_blocks(); ++k) t += *cl.map_shared_rank(slot, k);
+  if (tid < 32) {
+    if (per == 1) {
+      for (int k = 0; k < a.o_chunks; ++k) t += *cl.map_shared_rank(parts, k);
+    } else {
+      for (int k0 = 0; k0 < a.o_chunks; k0 += 32) {
+        const int k = k0 + lane;
+        const double v = k < a.o_chunks ? *cl.map_shared_rank(parts + k % per, k / per) : 0.0;
+        for (int l = 0; l < min(32, a.o_chunks - k0); ++l) t += __shfl_sync(0xffffffffu, v, l);
+      }
+    }
+  }
   return t;
 }
 
@@ -316,6 +339,7 @@ template <typename T>
 struct CgShared {
   double red[kCgNT / 32];
   double slot[2];
+  double parts[2][kMaxCgChunks / kCgMaxCluster];   // ordered sums
   T al, w0, w1, bt;
   int breakdown, copy_s, better, done;
 };
@@ -340,11 +364,10 @@ __device__ inline void cg_round_body(const CgArgs<T>& a, int ch, int li, CgShare
   V* se0 = reinterpret_cast<V*>(a.SE + (long long)st.est_off * a.ld);
   V* se1 = se0 + a.ld / VN;
 
-  const bool ordered = sizeof(T) == 8 && a.ordered;
-  const long long i0 = min(a.n, v0 * VN), i1 = min(a.n, v1 * VN);
+  const bool ordered = sizeof(T) == 8 && a.ordered > 0;
   double dKd;
   if (ordered) {
-    dKd = cg_ordered_dot(a.D + col, a.KD + col, i0, i1, sh.red, &sh.slot[0]);
+    dKd = cg_ordered_dot(a, a.D + col, a.KD + col, ch, sh.red, sh.parts[0]);
   } else {
     double p = 0.0;
 #pragma unroll 4
@@ -431,7 +454,7 @@ __device__ inline void cg_round_body(const CgArgs<T>& a, int ch, int li, CgShare
   double ee1;
   if (ordered) {
     __syncthreads();
-    ee1 = cg_ordered_dot(a.E + col, a.E + col, i0, i1, sh.red, &sh.slot[1]);
+    ee1 = cg_ordered_dot(a, a.E + col, a.E + col, ch, sh.red, sh.parts[1]);
   } else {
     ee1 = cluster_sum_warp0(p2, sh.red, &sh.slot[1]);
   }
@@ -552,20 +575,22 @@ cudaError_t launch_clustered(void (*kernel)(Params...), dim3 grid, int cluster, 
 }
 
 // One CG iteration of nl live columns.  Ordered sums: chunks of at least 2,048 rows, about two
-// CTAs per SM over all columns; beyond eight chunks (more than 16,384 rows) the usual form.
+// CTAs' worth per SM over all columns and at most kMaxCgChunks, shared by up to kCgMaxCluster CTAs.
 template <typename T>
 cudaError_t launch_cg_round(CgArgs<T> a, int nl, int num_sms, cudaStream_t s) {
   int c = cg_cluster_size(a.n);
   a.chunk = cg_cluster_rows(a.ld, c);
   if (a.ordered) {
     const long long target = std::max(1, (2 * num_sms + nl - 1) / nl);
-    const long long ch = (std::max<long long>((a.n + target - 1) / target, 2048) + 255) / 256 * 256;
-    const long long nc = (a.n + ch - 1) / ch;
-    a.ordered = nc <= kCgMaxCluster;
-    if (a.ordered) {
-      c = (int)nc;
-      a.chunk = ch;
-    }
+    long long ch = std::max<long long>((a.n + target - 1) / target, 2048);
+    ch = std::max<long long>(ch, (a.n + kMaxCgChunks - 1) / kMaxCgChunks);
+    ch = (ch + 255) / 256 * 256;
+    const int nc = (int)((a.n + ch - 1) / ch), per = (nc + kCgMaxCluster - 1) / kCgMaxCluster;
+    c = (nc + per - 1) / per;
+    a.chunk = per * ch;
+    a.ordered = (int)ch;
+    a.o_chunks = nc;
+    a.o_per = per;
   }
   return launch_clustered(cg_round_kernel<T>, dim3((unsigned)c, (unsigned)nl), c, s, a);
 }
