@@ -120,7 +120,6 @@ struct ulisse_ctx {
   int last_nsplit = 1;        // split count of the last K V launch (or plan)
 
   // CUDA graph of one SGLD step (ulisse_sgld_chain)
-  bool v_packed = false;      // the prescale launch packed the coming product's operand
   bool planning = false;      // launch helpers only size their scratch
   bool capturing = false;     // launch helpers are being captured: no host-side counting
   long long cap_launches = 0; // ... but of the K V launches captured
@@ -472,13 +471,13 @@ static ulisse_status grow_kmv_scratch(ulisse_ctx* ctx, size_t need_bytes, int ne
 
 // U[:, umap[r]] = A V[:, vmap[r]] for r < R (chunks of 64 columns per launch).
 static ulisse_status run_kmv_tc(ulisse_ctx* ctx, const void* V, const int* vmap, int R, void* U,
-                                const int* umap, long long ldv, long long ldu) {
+                                const int* umap, long long ldv, long long ldu, bool v_packed) {
   for (int c0 = 0; c0 < R; c0 += 64) {
     TcLaunch L{};
     L.xhat = (const float*)ctx->xhat;
     L.bneg = ctx->bneg;
     L.Vp = ctx->Vt;
-    L.v_packed = ctx->v_packed;
+    L.v_packed = v_packed;
     L.V = V;
     L.ldv = ldv;
     L.vmap = vmap + c0;
@@ -543,13 +542,14 @@ static ulisse_status run_kmv_tc(ulisse_ctx* ctx, const void* V, const int* vmap,
 }
 
 // ldv, ldu: leading dimensions (0: the context's own, ldn); only the tensor-core products and
-// the FP64 pair form take a V that is not padded to whole tiles.
+// the FP64 pair form take a V that is not padded to whole tiles.  v_packed: the prescale launch
+// packed the operand.
 static ulisse_status run_kmv(ulisse_ctx* ctx, const void* V, const int* vmap, int R, void* U,
                              const int* umap, int mode, int which, long long ldv = 0,
-                             long long ldu = 0) {
+                             long long ldu = 0, bool v_packed = false) {
   if (ldv == 0) ldv = ctx->ldn;
   if (ldu == 0) ldu = ctx->ldn;
-  if (ctx->mixed && mode == kModeK) return run_kmv_tc(ctx, V, vmap, R, U, umap, ldv, ldu);
+  if (ctx->mixed && mode == kModeK) return run_kmv_tc(ctx, V, vmap, R, U, umap, ldv, ldu, v_packed);
   // a product from formed kernel values takes any number of columns in one launch
   const int per = ctx->kmat_formed && mode == kModeK && !ctx->ordered ? std::max(R, 1) : kMaxRChunk;
   for (int c0 = 0; c0 < R; c0 += per) {
@@ -573,7 +573,7 @@ static ulisse_status run_kmv(ulisse_ctx* ctx, const void* V, const int* vmap, in
     L.kmat = ctx->kmat_formed ? ctx->kmat : nullptr;
     L.v3 = ctx->v3;
     L.simt = ctx->cfg.kmv_rows_per_thread != 0;
-    L.v_packed = ctx->v_packed;
+    L.v_packed = v_packed;
     L.mode = mode;
     L.which = which;
     L.tm = ctx->cfg.kmv_rows_per_thread;
@@ -1357,7 +1357,6 @@ static ulisse_status kmv_common(ulisse_ctx* ctx, const double* psi, int which, c
     pv.N = R <= 16 ? 16 : R <= 32 ? 32 : 64;
     pv.Vp = ctx->mixed ? ctx->Vt : ctx->v3;
   }
-  ctx->v_packed = pv.V != nullptr;
   if (in_place) {
     CKS(prescale_and_copy<float>(ctx, nullptr, 0, pv));
   } else if (ctx->mixed) {   // (its prescale copies nothing)
@@ -1370,10 +1369,8 @@ static ulisse_status kmv_common(ulisse_ctx* ctx, const double* psi, int which, c
     CKS(prescale_and_copy(ctx, (const float*)V, R));
   }
   const bool out_direct = ctx->esz == ue;
-  const ulisse_status kv = run_kmv(ctx, in_place ? V : ctx->D, ctx->iota, R, out_direct ? U : ctx->KD,
-                                   ctx->iota, mode, w, in_place ? n : 0, out_direct ? n : 0);
-  ctx->v_packed = false;
-  CKS(kv);
+  CKS(run_kmv(ctx, in_place ? V : ctx->D, ctx->iota, R, out_direct ? U : ctx->KD, ctx->iota, mode, w,
+              in_place ? n : 0, out_direct ? n : 0, pv.V != nullptr));
   if (!out_direct) {
     convert_cols_kernel<double, float><<<dim3(64, R), 256, 0, ctx->stream>>>(
         (const double*)ctx->KD, ctx->ldn, (float*)U, n, n);
