@@ -77,6 +77,7 @@ struct ulisse_ctx {
   int* counters = nullptr;
   int counters_len = 0;
   void* fixed_partials = nullptr;   // the first ones, part of fixed_block
+  size_t fixed_partials_bytes = 0;
   int* fixed_counters = nullptr;
 
   double* gpart = nullptr;
@@ -454,9 +455,13 @@ static ulisse_status grow_kmv_scratch(ulisse_ctx* ctx, size_t need_bytes, int ne
   CK(cudaStreamSynchronize(ctx->stream));
   if (need_bytes > ctx->partials_bytes) {
     if (ctx->partials != ctx->fixed_partials) dev_free(ctx->partials);
-    ctx->partials = nullptr;
     ctx->partials_bytes = 0;
-    CKS(dev_alloc(ctx, &ctx->partials, need_bytes));
+    const ulisse_status s = dev_alloc(ctx, &ctx->partials, need_bytes);
+    if (s != ULISSE_OK) {   // back to the first ones
+      ctx->partials = ctx->fixed_partials;
+      ctx->partials_bytes = ctx->fixed_partials_bytes;
+      return s;
+    }
     ctx->partials_bytes = need_bytes;
   }
   if (need_counters > ctx->counters_len) {
@@ -467,6 +472,17 @@ static ulisse_status grow_kmv_scratch(ulisse_ctx* ctx, size_t need_bytes, int ne
     ctx->counters_len = need_counters;
   }
   return ULISSE_OK;
+}
+
+// Whether an FP64 product takes the pair form: where it applies and its scratch (up to 256 MiB, more
+// than the row-block kernel's) is there or can be had; else the row-block kernel runs.
+static bool f64_pairs(ulisse_ctx* ctx, const KmvLaunch& L) {
+  if (!ctx->f64 || !kmv_f64_sym_applies(L)) return false;
+  const size_t need = kmv_f64_sym_bytes(L.n, L.R);
+  if (need > ctx->partials_bytes && !ctx->capturing &&
+      grow_kmv_scratch(ctx, need, 0) == ULISSE_ERR_NOMEM)
+    cudaGetLastError();
+  return need <= ctx->partials_bytes;
 }
 
 // U[:, umap[r]] = A V[:, vmap[r]] for r < R (chunks of 64 columns per launch).
@@ -587,6 +603,7 @@ static ulisse_status run_kmv(ulisse_ctx* ctx, const void* V, const int* vmap, in
       L.tm = ctx->tune[L.R - 1].tm;
       L.nsplit = ctx->tune[L.R - 1].nsplit;
     }
+    if (ctx->f64 && !L.kmat && !f64_pairs(ctx, L)) L.r_min = 1;   // the row-block kernel
     if (ctx->planning) {
       L.plan_only = true;
       cudaError_t e = ctx->f64 ? launch_kmv_f64(L, ctx->stream) : launch_kmv_f32(L, ctx->stream);
@@ -1211,6 +1228,7 @@ static ulisse_status create_impl(ulisse_ctx** out, const float* X, const float* 
   cv.add(ctx->counters, sizeof(int) * ctx->counters_len);
   if ((s = carve_alloc(ctx, cv, &ctx->fixed_block))) return bail(s);
   ctx->fixed_partials = ctx->partials;
+  ctx->fixed_partials_bytes = ctx->partials_bytes;
   ctx->fixed_counters = ctx->counters;
   ctx->psi_dev = ctx->result->psi;   // device addresses
   ctx->g_dev = ctx->result->g;
@@ -1339,7 +1357,7 @@ static ulisse_status kmv_common(ulisse_ctx* ctx, const double* psi, int which, c
   const char *vb = (const char*)V, *ub = (const char*)U;
   const size_t bytes = (size_t)n * R * ue;
   const bool overlap = ub < vb + bytes && vb < ub + bytes;
-  bool reads_direct = (ctx->mixed && mode == kModeK) || (f64_data && kmv_f64_sym_applies(probe));
+  bool reads_direct = (ctx->mixed && mode == kModeK) || (f64_data && f64_pairs(ctx, probe));
   if (!ctx->f64 && !ctx->mixed && ctx->tune.empty()) {
     // FP32: every launch of kMaxRChunk columns and that of the rest
     reads_direct = kmv_f32_tc_applies(probe);
