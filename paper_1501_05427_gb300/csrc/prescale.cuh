@@ -2,13 +2,14 @@
 // allocation-free K V entry point).
 //
 // What bounds it: latency and the FP64 pipe (1.7 lanes per clock per SM).  The 1 / l_k are
-// formed once per CTA, one exponential per thread; x^ = x / l in float is rounded once from
-// the product with 1 / l_k held as a pair of floats (48 bits), so that no element takes an FP64
-// multiply and two conversions.  With every thread forming all 1 / l_k and FP64 products the
-// launch took 10.7 us at n = 9,937, d = 4 and 27.5 us at n = 50,000, d = 8 (mixed precision:
-// then two more launches of 5 us for the row norms and the TF32 images, now the same launch).
-// A whole product call, which also loses the copies of psi, V and U, went from 45 to 25 us at
-// n = 1,030, d = 8, 5 columns (FP32) and from 840 to 795 us at n = 50,000 (mixed).
+// formed once per CTA, one exponential per thread; x^ = x / l in float comes from the product with
+// 1 / l_k held as a pair of floats (48 bits) where that decides the rounding of the FP64 product,
+// so that hardly any element takes an FP64 multiply and two conversions.  With every thread
+// forming all 1 / l_k and FP64 products the launch took 10.7 us at n = 9,937, d = 4 and 27.5 us at
+// n = 50,000, d = 8 (mixed precision: then two more launches of 5 us for the row norms and the
+// TF32 images, now the same launch).  A whole product call, which also loses the copies of psi, V
+// and U, went from 45 to 25 us at n = 1,030, d = 8, 5 columns (FP32) and from 840 to 795 us at
+// n = 50,000 (mixed).
 #pragma once
 
 #include <algorithm>
@@ -76,13 +77,18 @@ __device__ inline void unpack_params(const PsiArg& pa, double* __restrict__ psi_
   __syncthreads();
 }
 
-// (float)(x / l): x (hi + lo) with one rounding of the pair's sum where neither part nor the
-// product's error term can leave the normal range, else the FP64 product.
+// (float)(x / l), rounded as the FP64 product is: x (hi + lo) from the pair, whose error (the pair's
+// 48 bits, the rounding of c) is below 2^-46 of it, where the ends of p + c (1 -+ 2^-44 p) round to
+// one float and neither part nor the product's error term can leave the normal range; else the
+// FP64 product (about one element in 2^19).
 __device__ __forceinline__ float scale_by_pair(float x, const InvLength& s, int k) {
   const float hi = s.hi[k];
   const float p = x * hi;
-  if (fabsf(p) < 1e30f && fabsf(p) > 1e-28f && hi > 1e-28f && hi < 1e30f)
-    return p + fmaf(x, s.lo[k], fmaf(x, hi, -p));
+  if (fabsf(p) < 1e30f && fabsf(p) > 1e-28f && hi > 1e-28f && hi < 1e30f) {
+    const float c = fmaf(x, s.lo[k], fmaf(x, hi, -p)), w = fabsf(p) * 0x1p-44f;
+    const float y = p + (c - w);
+    if (y == p + (c + w)) return y;
+  }
   return x == 0.f ? x : (float)((double)x * s.inv[k]);
 }
 
