@@ -36,11 +36,28 @@
 namespace ulisse {
 
 // The split of a problem's j range: by its size alone, so that a problem gives the same bits on
-// its own and in a batch (the tiles' sums are added in the same order).
+// its own and in a batch (the tiles' sums are added in the same order).  The other kernels' plan
+// stops at four waves of CTAs; from about 32,000 points on (several hundred row blocks on 304 places)
+// that leaves up to a quarter of the places empty in the last wave, and a product of 7 to 9 columns
+// took up to 19% longer than the SIMT kernel's (d = 2, n = 64,000: 2.70 against 2.28 ms).  There a
+// larger split is taken when it saves 5% of the waves' tiles (a CTA's start and end count as 8 tiles)
+// with partial sums of at most 64 MiB, which a context comes with.
 int f3_nsplit(long long n, int num_sms) {
-  const KmvPlan p = plan_split(n, 128, 32, 4, 2 * num_sms);
-  const long long ntiles = (n + 31) / 32, tps = (ntiles + p.nsplit - 1) / p.nsplit;
-  return (int)((ntiles + tps - 1) / tps);
+  const long long ntiles = (n + 31) / 32, nrb = (n + 127) / 128, slots = 2 * num_sms;
+  auto whole = [&](long long s) {   // without empty ranges
+    const long long tps = (ntiles + s - 1) / s;
+    return (ntiles + tps - 1) / tps;
+  };
+  auto cost = [&](long long s) {
+    return (nrb * s + slots - 1) / slots * ((ntiles + s - 1) / s + 8);
+  };
+  const long long plan = whole(plan_split(n, 128, 32, 4, (int)slots).nsplit);
+  if (2 * nrb <= slots) return (int)plan;
+  long long best = plan;
+  for (long long s = plan + 1; s <= 64 && nrb * s * (32 * 128 * 4) <= (64LL << 20); ++s)
+    if (cost(s) < cost(best)) best = s;
+  best = whole(best);
+  return (int)(100 * cost(best) < 95 * cost(plan) ? best : plan);
 }
 
 size_t kmv_tile_partial_bytes(long long n, int num_sms, bool mixed) {
@@ -542,11 +559,18 @@ cudaError_t f3_dp(KmvLaunch& L, cudaStream_t s) {
 }  // namespace
 
 // The time here does not depend on the column count up to 32; the SIMT kernel's grows with it.
-// Calls at d = 8, SIMT / here, us: n = 1,030: 1 column 18 / 19, 5 columns 26 / 21, 17 columns
-// 51 / 23; n = 9,937: 3 columns 101 / 114, 5 columns 113 / 115, 17 columns 208 / 121, 32 columns
-// 325 / 128; n = 22,784: 5 columns 454 / 491, 7 columns 586 / 492, 17 columns 760 / 490; n = 50,000:
-// 6 columns 2,200 / 2,295, 7 columns 2,494 / 2,296, 32 columns 5,223 / 2,275.  (Error against 64
-// bits, relative: 1.7e-7 / 1.3e-7 at n = 1,030, 8.5e-7 / 2.8e-7 at n = 22,784, 17 columns.)
+// Calls, SIMT / here, us (SIMT with two rows per thread, its default):
+//   d = 8, n = 1,030: 1 column 18 / 19, 5 columns 26 / 21, 17 columns 51 / 23; n = 9,937: 3 columns
+//   101 / 114, 5 columns 113 / 115, 17 columns 208 / 121, 32 columns 325 / 128; n = 50,000: 6 columns
+//   2,200 / 2,295, 7 columns 2,494 / 2,296, 32 columns 5,223 / 2,275.
+// By padded width, 5 columns at n = 8,000: d = 2 68 / 60, 4 78 / 65, 8 87 / 81, 16 125 / 116; 7 columns at
+// n = 10,100: 100 / 83, 118 / 92, 151 / 120, 199 / 175; at 31,000: 609 / 536, 712 / 630, 1,016 / 880,
+// 1,508 / 1,329; at 64,000: 2,285 / 2,210, 2,836 / 2,620, 3,989 / 3,701, 6,117 / 5,606; at 120,000: 7,680 /
+// 7,611, 10,137 / 9,085, 14,011 / 12,911, 22,269 / 19,606.  So one line for all widths; what it loses
+// most is 7 and 8 columns at d <= 2, n = 35,000, 725 / 773 (one wave of CTAs, nine tenths full; 3% at
+// most for the other widths there), and 4% at d <= 2, n = 75,000.
+// (Error against 64 bits, relative: 1.7e-7 / 1.3e-7 at n = 1,030, 8.5e-7 / 2.8e-7 at n = 22,784, 17
+// columns.)
 bool kmv_f32_tc_applies(const KmvLaunch& L) {
   return L.v3 && L.mode != kModeDLam && !L.simt && f32_tc_columns(L.n, L.R);
 }
