@@ -428,8 +428,10 @@ ulisse_status ulisse_ws_x0(ulisse_ctx *ctx, const double *psi, int bf16, float *
  * key is cfg->seed + b, so problem b reproduces a single context created with that seed).
  * The O(n^2) passes of all problems run as one launch each: every CG round's covariance
  * products over all live columns of all problems, and the fused gradient sweep.
- *   ULISSE_PREC_FP32: persistent SIMT launches over (problem, 256-row block) items, longest
- *     rows first;
+ *   ULISSE_PREC_FP32: products from five live columns on by the tensor-core contraction over
+ *     (problem, 128-row block, ranges of j) items, the sums those of the problem on its own; with
+ *     fewer columns, and the gradient sweep, persistent SIMT launches over (problem, 256-row
+ *     block) items; the longest first;
  *   ULISSE_PREC_MIXED: the tensor-core products (as ulisse_config.tc_cross_term = 2, the
  *     column term added in the epilogue for every d) over (problem, 128-row block, split)
  *     items, and the tensor-core gradient pass, one launch per padded input width (2, 4, 8).
@@ -472,9 +474,9 @@ ulisse_status ulisse_batch_sgld_step(ulisse_ctx *ctx, double *psi_inout, double 
  *   trace_dev device, NULL or n_steps x n_params (packed parameters after each step).
  * With the graph enabled (ulisse_set_graph, the default) each step is ONE launch of a CUDA
  * graph holding the whole batched step: every problem's prescale, probes and CG start, the
- * round loop as a conditional WHILE node (one batched compaction, the persistent K V over
- * all live columns of all problems with its compiled width chosen by a SWITCH node, three
- * batched CG launches), the persistent gradient sweep and the updates.  The host loop runs
+ * round loop as a conditional WHILE node (one batched compaction, the K V over
+ * all live columns of all problems with its compiled width chosen by a SWITCH node, one
+ * batched CG launch), the persistent gradient sweep and the updates.  The host loop runs
  * the same launches and gives the same results. */
 ulisse_status ulisse_batch_sgld_chain(ulisse_ctx *ctx, double *psi_dev, const double *eps_dev,
                                       int n_steps, unsigned long long step0, double *trace_dev);

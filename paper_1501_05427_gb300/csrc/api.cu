@@ -2296,13 +2296,18 @@ ulisse_status ulisse_create_batched(ulisse_ctx** out, int n_problems, const long
       (s = dev_alloc(ctx, reinterpret_cast<void**>(&ctx->status_dev), sizeof(int))))
     return bail(s);
   {
-    // tensor-core K V work list (mixed products; FP32 products from kF32TcMinR columns on): per
+    // tensor-core K V work list (mixed products; FP32 products from kBatchTcMinR columns on): per
     // problem its 128-row blocks times a split of the j range into ranges of about kTcBatchTiles
     // 32-point tiles; the longest ranges first
     constexpr long long kTcBatchTiles = 256;
     std::vector<int4> tci;
     std::vector<std::pair<long long, int>> order;
+    std::vector<int> per_cta;   // ranges that a CTA takes
     size_t part = 0, cnt = 0;
+    // FP32: tiles of a CTA at least, three waves of two CTAs per SM, at most 32
+    long long fill = 0;
+    for (int b = 0; b < n_problems; ++b) fill += (n[b] + 31) / 32 * ((n[b] + 127) / 128);
+    fill = std::min(32LL, fill / (6LL * ctx->num_sms));
     for (int b = 0; b < n_problems; ++b) {
       const long long nt = (n[b] + 31) / 32, nrb = (n[b] + 127) / 128;
       int ns = (int)std::min<long long>(64, (nt + kTcBatchTiles - 1) / kTcBatchTiles);
@@ -2314,17 +2319,19 @@ ulisse_status ulisse_create_batched(ulisse_ctx** out, int n_problems, const long
       ctx->b_tc_cnt_off.push_back(cnt);
       if (ns > 1) part += (size_t)nrb * ns * 32 * 128;
       cnt += (size_t)nrb;
-      order.push_back({tps, b});
+      per_cta.push_back(cfg->precision == ULISSE_PREC_FP32 ? f3_ranges_per_cta(n[b], ns, fill) : 1);
+      order.push_back({tps * per_cta[b], b});
     }
     std::stable_sort(order.begin(), order.end(),
                      [](const std::pair<long long, int>& a, const std::pair<long long, int>& c) {
                        return a.first > c.first;
                      });
     for (const auto& o : order) {
-      const int b = o.second;
+      const int b = o.second, ns = ctx->b_tc_nsplit[b];
       const int nrb = (int)((n[b] + 127) / 128);
       for (int rb = 0; rb < nrb; ++rb)
-        for (int sp = 0; sp < ctx->b_tc_nsplit[b]; ++sp) tci.push_back(make_int4(b, rb, sp, 0));
+        for (int sp = 0; sp < ns; sp += per_cta[b])
+          tci.push_back(make_int4(b, rb, sp, std::min(per_cta[b], ns - sp)));
     }
     ctx->b_tc_n_items = (int)tci.size();
     const bool mixed = cfg->precision == ULISSE_PREC_MIXED;
@@ -2503,7 +2510,7 @@ static ulisse_status batch_tc_upload(ulisse_ctx* ctx, int k, Fn cols) {
 // Kernels of one batched K V for at most r_max live columns (packing, tensor cores, SIMT).
 static int batch_kv_launches(const ulisse_ctx* ctx, int r_max) {
   if (ctx->cfg.precision == ULISSE_PREC_MIXED) return 2;
-  return r_max >= kF32TcMinR ? 3 : 1;
+  return r_max >= kBatchTcMinR ? 3 : 1;
 }
 
 // One batched K V over all problems: the tensor-core launch (slot of its arguments) and, in
@@ -2516,7 +2523,7 @@ static cudaError_t batch_kv_launch(ulisse_ctx* ctx, int slot, BatchKmvDesc* desc
                                 ctx->b_tc_items, ctx->b_tc_n_items, r_max, st);
   // FP32: the tensor-core contraction takes the problems with enough live columns, the persistent
   // SIMT launch the others
-  if (r_max >= kF32TcMinR) {
+  if (r_max >= kBatchTcMinR) {
     const cudaError_t e = launch_kmv_f32_tc_batch(
         (char*)ctx->b_tc_args + slot * f3_batch_args_bytes(B), B, ctx->b_tc_items, ctx->b_tc_n_items,
         kBatchWidths[batch_width_bucket(r_max)], st);
@@ -2824,7 +2831,7 @@ static ulisse_status batch_step_body(ulisse_ctx* ctx, bool sgld, bool in_graph) 
   const int max_rounds = ctx->cfg.max_iter + 2;
   // K V kernels beyond the first, from how many live columns on (the counters')
   const bool fp32 = ctx->cfg.precision == ULISSE_PREC_FP32;
-  const int tc_from = fp32 ? kF32TcMinR : 1, tc_launches = batch_kv_launches(ctx, 32) - 1;
+  const int tc_from = fp32 ? kBatchTcMinR : 1, tc_launches = batch_kv_launches(ctx, 32) - 1;
   if (!in_graph) {
     for (int it = 0; it < max_rounds + 1; ++it) {
       compact_batch_kernel<<<1, kCompactBatchNT, 0, ctx->stream>>>(ctx->b_cgprob, B, ctx->b_rmax, 0, 0, 0,

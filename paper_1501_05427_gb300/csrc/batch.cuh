@@ -30,7 +30,7 @@ struct BatchKmvDesc {
   const float* xhat;     // ldn x DP prescaled inputs (padding rows zero)
   long long n;
   int DP;
-  int tc;                // skip while f32_tc_columns holds (the tensor-core launch's)
+  int tc;                // skip while batch_tc_columns holds (the tensor-core launch's)
   const DevParams* params;
   const float* V;        // column-major, leading dimension ldv (padding rows zero)
   long long ldv;
@@ -40,6 +40,15 @@ struct BatchKmvDesc {
   const int* umap;
   const int* nlive;      // live column count (device), 0 = skip the problem
 };
+
+// Whether a problem's product is the tensor-core launch's.  One line of columns for all sizes, where a
+// product on its own has a higher one above n = 10,000: the persistent SIMT kernel takes 1.5 times
+// the single-problem kernel's time there, and a batch on both sides of a size is two launches with
+// a tail each.
+constexpr int kBatchTcMinR = 5;
+__host__ __device__ constexpr bool batch_tc_columns(long long n, int R) {
+  return n >= kF32TcMinN && R >= kBatchTcMinR;
+}
 
 // The same product by the tensor-core contraction (kmv_f32_tc.cu): its operand scratch
 // (pack_v3_bytes), the split of its j range, partial sums and counters.
@@ -52,9 +61,10 @@ struct F3Problem {
   int* status;
 };
 int f3_nsplit(long long n, int num_sms);
+int f3_ranges_per_cta(long long n, int nsplit, long long tiles);
 size_t f3_batch_args_bytes(int B);
 cudaError_t f3_batch_upload_args(const F3Problem* P, int B, void* args_dev, cudaStream_t s);
-// items: (problem, 128-row block, split) per CTA; R_max: the largest live column count.
+// items: (problem, 128-row block, first range, ranges) per CTA; R_max: the largest live column count.
 // prime_only: set the kernel attributes (ahead of a capture) and launch nothing.
 cudaError_t launch_kmv_f32_tc_batch(const void* args_dev, int B, const int4* items, int n_items,
                                     int R_max, cudaStream_t s, bool prime_only = false);

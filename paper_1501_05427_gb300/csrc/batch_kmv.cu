@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(kBatchNT) kmv_batch_kernel(const BatchKmvDesc*
     const BatchItem item = items[it];
     const BatchKmvDesc P = descs[item.prob];
     const int Ra = min(*P.nlive, R);
-    if (Ra > 0 && !(P.tc && f32_tc_columns(P.n, *P.nlive))) {
+    if (Ra > 0 && !(P.tc && batch_tc_columns(P.n, *P.nlive))) {
       if (tid < R) s_vcol[tid] = (tid < Ra) ? P.vmap[tid] : 0;
       // Column slots beyond the live count read as zero in every stage.
       for (int idx = tid; idx < kStages * (R - Ra) * kBN; idx += kBatchNT) {

@@ -60,6 +60,16 @@ int f3_nsplit(long long n, int num_sms) {
   return (int)(100 * cost(best) < 95 * cost(plan) ? best : plan);
 }
 
+// Consecutive ranges that a CTA of a batch takes one after the other, `tiles` tiles or more: the sums
+// are those of the product on its own, which has a CTA per range to fill the SMs by itself.  Many
+// problems fill them anyway, and with one or two tiles per CTA (n = 1,000) their starts and ends,
+// about 8 tiles' time each, were most of a launch: a round of 64 problems of 300 to 2,000 points,
+// 9 columns, 357 -> 295 us (the SIMT kernel 338); few problems keep a CTA per range.
+int f3_ranges_per_cta(long long n, int nsplit, long long tiles) {
+  const long long ntiles = (n + 31) / 32, tps = (ntiles + nsplit - 1) / nsplit;
+  return (int)std::max(1LL, std::min<long long>(nsplit, (tiles + tps - 1) / tps));
+}
+
 size_t kmv_tile_partial_bytes(long long n, int num_sms, bool mixed) {
   const size_t nrb = ((size_t)n + 127) / 128;
   size_t ns = f3_nsplit(n, num_sms);
@@ -122,7 +132,7 @@ __global__ void pack_v3_kernel(const float* __restrict__ V, long long ldv,
 __global__ void pack_v3_batch_kernel(const F3Args* __restrict__ args, int N) {
   const F3Args& a = args[blockIdx.y];
   const int R = a.R_dev ? *a.R_dev : a.R;
-  if (!f32_tc_columns(a.n, R)) return;
+  if (!batch_tc_columns(a.n, R)) return;
   pack_v3(a.V, a.ldv, a.vmap, R, N, a.n, a.ntiles, const_cast<__nv_bfloat16*>(a.Vp), blockIdx.x,
           gridDim.x);
 }
@@ -206,10 +216,11 @@ __device__ __noinline__ void f3_not_finite(const F3Args& a, const long long row0
   }
 }
 
-// One CTA's work: row block rb, j-range split sp, R columns.  Shared by the single-problem kernel
-// and the batched one.
-template <int DP, int N, int MODE>
-__device__ __forceinline__ void f3_body(const F3Args& a, const int rb, const int sp, const int R) {
+// One CTA's work: row block rb, the j ranges sp .. sp + nsp - 1 (one unless MULTI), R columns.  Shared by
+// the single-problem kernel and the batched one.
+template <int DP, int N, int MODE, bool MULTI>
+__device__ __forceinline__ void f3_body(const F3Args& a, const int rb, const int sp, const int nsp,
+                                        const int R) {
   using S = F3Shape<DP, N>;
   constexpr int ST = S::ST;
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -229,10 +240,10 @@ __device__ __forceinline__ void f3_body(const F3Args& a, const int rb, const int
 
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
-  const long long slot = (long long)rb * a.nsplit + sp;   // this CTA's partial-sum slot
+  const long long slot = (long long)rb * a.nsplit + sp;   // the first range's partial-sum slot
   const long long row0 = (long long)rb * kF3BM;
   const int tile_begin = sp * a.tiles_per_split;
-  const int nt = max(0, min(tile_begin + a.tiles_per_split, a.ntiles) - tile_begin);
+  const int nt = max(0, min(tile_begin + nsp * a.tiles_per_split, a.ntiles) - tile_begin);
 
   if (tid == 0) {
     for (int s = 0; s < ST; ++s) mbar_init(&full[s], 1);
@@ -385,6 +396,12 @@ __device__ __forceinline__ void f3_body(const F3Args& a, const int rb, const int
 #pragma unroll
     for (int q = 0; q < N / 2; ++q) acc[q] = make_float2(0.f, 0.f);
     bool ok = true;
+    auto put = [&](int range) {   // the CTA's range-th partial sums
+      float* part = a.partials + (slot + range) * N * kF3BM + il;
+#pragma unroll
+      for (int r = 0; r < N; ++r) part[r * kF3BM] = r & 1 ? acc[r / 2].y : acc[r / 2].x;
+    };
+    int end = MULTI ? a.tiles_per_split : nt;   // of the current range
 #pragma unroll 1
     for (int p = 0; p < nt; ++p) {
       const uint32_t ub = (uint32_t)(p & 1);
@@ -402,6 +419,12 @@ __device__ __forceinline__ void f3_body(const F3Args& a, const int rb, const int
       tc::fence_before();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&u_free[ub]);
+      if (MULTI && p + 1 == end && p + 1 < nt) {   // on to the next range
+        put(p / a.tiles_per_split);
+#pragma unroll
+        for (int q = 0; q < N / 2; ++q) acc[q] = make_float2(0.f, 0.f);
+        end += a.tiles_per_split;
+      }
     }
     if (!ok) {
       *s_fail = 1;
@@ -418,9 +441,7 @@ __device__ __forceinline__ void f3_body(const F3Args& a, const int rb, const int
           }
       }
     } else {
-      float* part = a.partials + slot * N * kF3BM;
-#pragma unroll
-      for (int r = 0; r < N; ++r) part[r * kF3BM + il] = r & 1 ? acc[r / 2].y : acc[r / 2].x;
+      put(MULTI ? (nt - 1) / a.tiles_per_split : 0);
     }
   }
 
@@ -445,7 +466,7 @@ __device__ __forceinline__ void f3_body(const F3Args& a, const int rb, const int
   }
   __threadfence();
   __syncthreads();
-  if (tid == 0) *s_last = (atomicAdd(&a.counters[rb], 1) == a.nsplit - 1);
+  if (tid == 0) *s_last = (atomicAdd(&a.counters[rb], nsp) == a.nsplit - nsp);
   __syncthreads();
   if (!*s_last) return;
   __threadfence();
@@ -469,11 +490,11 @@ __device__ __forceinline__ void f3_body(const F3Args& a, const int rb, const int
 template <int DP, int N, int MODE>
 __global__ void __launch_bounds__(kF3Threads, 2) kmv_f32_tc_kernel(const F3Args a) {
   const int rb = blockIdx.x / a.nsplit;
-  f3_body<DP, N, MODE>(a, rb, blockIdx.x - rb * a.nsplit, a.R);
+  f3_body<DP, N, MODE, false>(a, rb, blockIdx.x - rb * a.nsplit, 1, a.R);
 }
 
 // Many problems in one launch (mode K, padded d <= 8): CTA b takes work item items[b] = (problem,
-// row block, split) with that problem's arguments.
+// row block, first range, ranges) with that problem's arguments.
 template <int N>
 __global__ void __launch_bounds__(kF3Threads, 2) kmv_f32_tc_batch_kernel(
     const F3Args* __restrict__ args, const int4* __restrict__ items) {
@@ -482,11 +503,11 @@ __global__ void __launch_bounds__(kF3Threads, 2) kmv_f32_tc_batch_kernel(
   if (threadIdx.x == 0) s_a = args[it.x];
   __syncthreads();
   const int R = s_a.R_dev ? *s_a.R_dev : s_a.R;
-  if (!f32_tc_columns(s_a.n, R)) return;
+  if (!batch_tc_columns(s_a.n, R)) return;
   switch (s_a.DP) {
-    case 2: f3_body<2, N, kModeK>(s_a, it.y, it.z, R); break;
-    case 4: f3_body<4, N, kModeK>(s_a, it.y, it.z, R); break;
-    default: f3_body<8, N, kModeK>(s_a, it.y, it.z, R); break;
+    case 2: f3_body<2, N, kModeK, true>(s_a, it.y, it.z, it.w, R); break;
+    case 4: f3_body<4, N, kModeK, true>(s_a, it.y, it.z, it.w, R); break;
+    default: f3_body<8, N, kModeK, true>(s_a, it.y, it.z, it.w, R); break;
   }
 }
 
