@@ -41,7 +41,7 @@ struct ulisse_ctx {
   void* Vt = nullptr;         // BF16 operand tiles of K V, high | low part per tile
   void* Gt = nullptr;         // packed operand blocks of the tensor-core gradient
   float *Xt_hi = nullptr, *Xt_lo = nullptr;  // TF32 images of the A rows (tensor-core cross term)
-  float* Xt_b = nullptr;      // ... and the tiles of the B rows, see launch_pack_x_tf32
+  float* Xt_b = nullptr;      // ... and the tiles of the B rows, see launch_prescale_mixed
 
   float* X = nullptr;         // raw inputs, n x d row-major
   void* y = nullptr;          // labels, ldn (element type T)

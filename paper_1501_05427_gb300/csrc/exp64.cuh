@@ -32,7 +32,8 @@ __device__ __forceinline__ double exp_neg_half(double dist, const double* __rest
   constexpr double kStep = 2.0 * kExpLn2 / (double)kExpTabN;
   constexpr double kH = kExpLn2 / (2.0 * kExpTabN);
   constexpr double kC2 = 0.125 + 0.82842712474619009760 * kH * kH / 96.0;
-  // beyond 1400 the result leaves the normal range (and k its exact one); NaN comes here too
+  // beyond 1400 the result leaves the normal range (and k its exact one); a NaN comes here or, with
+  // its sign set, stays one below
   if (__double2hiint(dist) >= 0x4095E000) return exp(-0.5 * dist);
   const double z = fma(dist, kInv, kMagic);
   const int k = __double2loint(z);

@@ -182,49 +182,49 @@ __global__ void __launch_bounds__(NT) grad_kernel(const GradDevArgs<T> a) {
         tile_pass_f32<DP, M, TM>(tX, tB, xi, av, c0, c1, gl, gs);
       } else {
 #pragma unroll 1
-      for (int jq = 0; jq < kBN; jq += 4) {
-        T W[TM][4];
-#pragma unroll
-        for (int t = 0; t < TM; ++t)
-#pragma unroll
-          for (int q = 0; q < 4; ++q) W[t][q] = T(0);
-#pragma unroll
-        for (int m = 0; m < M; ++m) {
-          T b[4];
-          if constexpr (sizeof(T) == 4) {
-            const float4 b4 = *reinterpret_cast<const float4*>(tB + m * kBN + jq);
-            b[0] = b4.x; b[1] = b4.y; b[2] = b4.z; b[3] = b4.w;
-          } else {
-            const double2 b0 = *reinterpret_cast<const double2*>(tB + m * kBN + jq);
-            const double2 b1 = *reinterpret_cast<const double2*>(tB + m * kBN + jq + 2);
-            b[0] = b0.x; b[1] = b0.y; b[2] = b1.x; b[3] = b1.y;
-          }
+        for (int jq = 0; jq < kBN; jq += 4) {
+          T W[TM][4];
 #pragma unroll
           for (int t = 0; t < TM; ++t)
 #pragma unroll
-            for (int q = 0; q < 4; ++q) W[t][q] = fma(av[t][m], b[q], W[t][q]);
-        }
+            for (int q = 0; q < 4; ++q) W[t][q] = T(0);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          T xj[DP];
-          load_row<T, DP>(tX + (jq + q) * DP, xj);
-#pragma unroll
-          for (int t = 0; t < TM; ++t) {
-            T sq[DP];
-            T dist = T(0);
-#pragma unroll
-            for (int k = 0; k < DP; ++k) {
-              const T df = xi[t][k] - xj[k];
-              sq[k] = df * df;
-              dist += sq[k];
+          for (int m = 0; m < M; ++m) {
+            T b[4];
+            if constexpr (sizeof(T) == 4) {
+              const float4 b4 = *reinterpret_cast<const float4*>(tB + m * kBN + jq);
+              b[0] = b4.x; b[1] = b4.y; b[2] = b4.z; b[3] = b4.w;
+            } else {
+              const double2 b0 = *reinterpret_cast<const double2*>(tB + m * kBN + jq);
+              const double2 b1 = *reinterpret_cast<const double2*>(tB + m * kBN + jq + 2);
+              b[0] = b0.x; b[1] = b0.y; b[2] = b1.x; b[3] = b1.y;
             }
-            const T P = kernel_from_dist<T, TAB>(dist, c0, c1, sigma2, a.exp_tab) * W[t][q];
-            gs += P;
 #pragma unroll
-            for (int k = 0; k < DP; ++k) gl[k] = fma(P, sq[k], gl[k]);
+            for (int t = 0; t < TM; ++t)
+#pragma unroll
+              for (int q = 0; q < 4; ++q) W[t][q] = fma(av[t][m], b[q], W[t][q]);
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            T xj[DP];
+            load_row<T, DP>(tX + (jq + q) * DP, xj);
+#pragma unroll
+            for (int t = 0; t < TM; ++t) {
+              T sq[DP];
+              T dist = T(0);
+#pragma unroll
+              for (int k = 0; k < DP; ++k) {
+                const T df = xi[t][k] - xj[k];
+                sq[k] = df * df;
+                dist += sq[k];
+              }
+              const T P = kernel_from_dist<T, TAB>(dist, c0, c1, sigma2, a.exp_tab) * W[t][q];
+              gs += P;
+#pragma unroll
+              for (int k = 0; k < DP; ++k) gl[k] = fma(P, sq[k], gl[k]);
+            }
           }
         }
-      }
       }
 #pragma unroll
       for (int k = 0; k < DP; ++k) acc[k] += (double)gl[k];

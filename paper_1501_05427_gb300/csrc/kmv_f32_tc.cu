@@ -1,4 +1,4 @@
-// FP32 tile-generating K V with the contraction on the tensor cores and no loss to FP32.
+// FP32 tile-generating K V with the contraction on the tensor cores, from BF16 parts of each float.
 //
 // The kernel values are formed as the SIMT kernel forms them (distance from the differences of
 // the prescaled inputs, one FMA, one ex2, FP32 throughout).  The contraction U_I += K_IJ V_J runs
@@ -9,6 +9,14 @@
 // up over a long range; here a 32-point tile's product (12 MMAs) starts from zero and is added to
 // running FP32 sums in registers (round to nearest) by four draining warps, so that the rounding
 // is that of n / 32 FP32 additions instead of the SIMT kernel's n FMAs in sequence.
+//
+// Rounding, against 64 bits: the three products left out are below 2^-26 of a term; of the 12
+// truncations the last two, of the halves of h h, are of the tile's own size, so a tile's product
+// is off by 2.1 2^-23 at most and low by 1.1 2^-24 on average: sums come out low by 6e-8 of
+// themselves (the SIMT kernel's by 2e-8).  Errors of products are 0.3 to 0.8 of the SIMT
+// kernel's over n = 500 to 22,784, d = 1 to 16 at the lengthscales in use, where its chain of n
+// roundings counts; with K close to sigma^2 I (lengthscales 0.1 to 0.3 of those, n = 1,030, d = 4
+// to 16) one term makes a row and they are up to 1.09 of it (5.5e-8 / 6.1e-8).
 //
 // What bounds it: the FP32 pipe, 2 DP + 4 lanes per entry (distance, exponent, the split's
 // subtractions), whatever the column count, against 2 DP + 1 + R in the SIMT kernel; the BF16

@@ -281,11 +281,10 @@ size_t kmv_f64_sym_bytes(long long n, int R) {
 }
 
 // The pair form's scratch grows as n^2 R / T doubles; it is used while that is at most 256 MiB
-// (n = 10,000 with 16 columns, 5,700 with 32), beyond which the row-block kernel runs.  A forced
-// configuration (an installed launch table) means the row-block kernel, and dK/dlog lambda has
-// no pairs.
+// (n = 11,584 with 16 columns, 8,192 with 32) and can be had, else the row-block kernel runs, which
+// the caller asks for by r_min; dK/dlog lambda has no pairs.
 bool kmv_f64_sym_applies(const KmvLaunch& L) {
-  if (L.mode == kModeDLam || L.nsplit > 0 || L.r_min > 0 || !L.exp_tab) return false;
+  if (L.mode == kModeDLam || L.r_min > 0 || !L.exp_tab) return false;
   return kmv_f64_sym_bytes(L.n, L.R) <= (size_t)kSymMaxPartialBytes;
 }
 

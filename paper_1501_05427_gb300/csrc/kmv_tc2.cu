@@ -6,8 +6,8 @@
 //          A_i = [x^_i, 1],  B_j = [2 c1 x^_j, b_j],   b_j = -c1 |x^_j|^2, c1 = log2(e)/2,
 //      so that C_ij = 2 c1 x^_i . x^_j + b_j in one 8-wide K step; with padded d = 8 or 16
 //      the rows are A_i = x^_i, B_j = 2 c1 x^_j (K = d: the augmented column would cost a
-//      whole further K step, three MMAs per tile on the one issuing thread that paces the
-//      kernel) and the epilogue adds b_j.  Both sides split into a TF32 high part and the
+//      whole further K step, three MMAs per tile that warp 0 would issue and the tensor pipe
+//      run) and the epilogue adds b_j.  Both sides split into a TF32 high part and the
 //      remainder, three products (Ah Bh + Ah Bl + Al Bh), FP32 accumulation into a 32-column
 //      tensor-memory buffer;
 //   2. the epilogue warps read C back (tcgen05.ld) and form
@@ -193,7 +193,7 @@ __device__ inline void t2_ld_cols(uint32_t taddr, float (&v)[NH]) {
   } else if constexpr (NH == 16) {
     tc::tmem_ld16(taddr, v);
   } else {
-    // two 16-column loads: a 32-register load does not fit the 48-register budget
+    // two 16-column loads: the registers of one are free again before the other's arrive
     float v0[16], v1[16];
     tc::tmem_ld16(taddr, v0);
     tc::tmem_ld16(taddr + 16, v1);

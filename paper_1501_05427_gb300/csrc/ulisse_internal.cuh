@@ -153,17 +153,6 @@ __device__ inline bool mbar_wait_spin(uint64_t* bar, uint32_t parity) {
   return false;
 }
 
-// Bounded wait for a single thread with nothing else to do meanwhile (a producer or an MMA
-// issuer): it sleeps between polls so that polling takes no issue slots from the warps that
-// compute (about a second at most, then false).
-__device__ inline bool mbar_wait_backoff(uint64_t* bar, uint32_t parity) {
-  for (int it = 0; it < (1 << 24); ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
-    __nanosleep(64);
-  }
-  return false;
-}
-
 __device__ inline float ex2_approx(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -259,7 +248,7 @@ struct KmvLaunch {
   int which;             // dimension for kModeDLen
   const double* exp_tab; // FP64: the exponential's table (exp64.cuh)
   void* v3;              // FP32: scratch of the tensor-core contraction's operand (kmv_f32_tc.cu),
-                         // 96 BF16 values per point (null: SIMT kernel)
+                         // pack_v3_bytes (null: SIMT kernel)
   bool ordered;          // FP64: keep the row-block kernel's order of additions
   const double* kmat;    // FP64: the kernel values of this solve, n <= kKmatMaxN (null: not formed)
   bool simt;             // FP32: the SIMT kernel whatever the sizes
@@ -364,8 +353,8 @@ cudaError_t launch_kmv_f32_dp16(KmvLaunch& L, cudaStream_t s);
 cudaError_t launch_kmv_f64(KmvLaunch& L, cudaStream_t s);
 // FP32 products with the contraction on the tensor cores (kmv_f32_tc.cu).
 constexpr long long kF32TcMinN = 256;
-constexpr int kF32TcMinR = 5;   // no problem takes this form below so many columns
-__host__ __device__ constexpr bool f32_tc_columns(long long n, int R) {
+constexpr int kF32TcMinR = 5;   // no product takes this form below so many columns
+constexpr bool f32_tc_columns(long long n, int R) {
   return n >= kF32TcMinN && R >= (n <= 10000 ? kF32TcMinR : 7);
 }
 bool kmv_f32_tc_applies(const KmvLaunch& L);
