@@ -3206,7 +3206,7 @@ ulisse_status ulisse_autotune(ulisse_ctx* ctx, const double* psi, int max_cols, 
     float ms_base = 0.f;
     int base = 1;
     r = time_kmv_config(ctx, nl, wd, tm, 0, best.cross, 1, &ms_base, &base);   // its planned split
-    for (int sp : {base / 2, base * 2}) {
+    for (int sp : {base / 2, std::min(64, base * 2)}) {   // at most what ulisse_set_tune takes
       if (r != ULISSE_OK || sp < 1 || sp == base) continue;
       float ms = 0.f;
       int used = sp;

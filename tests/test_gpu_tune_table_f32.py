@@ -48,3 +48,13 @@ def test_installed_table_reproduces_the_tuned_context():
         ctx.set_tune(table)
         for V, ref in zip(Vs, outs):
             assert torch.equal(ctx.kmv(prob.psi_true, V), ref)
+
+
+def test_tuned_splits_can_be_installed():
+    # 50,000 points, one column: the plan's split is 49, its double beyond the 64 of a table
+    prob = w.census_like(n=50_000, seed=33)
+    with _ctx(prob) as ctx:
+        table = ctx.autotune(prob.psi_true, 2, reps=1)
+        ctx.set_tune(table)
+        ctx.set_tune([dict(e, rows_per_thread=2, nsplit=64) for e in table])
+    assert all(0 <= e["nsplit"] <= 64 for e in table)
