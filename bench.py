@@ -55,7 +55,7 @@ EX2_PEAK_DERIVED_TENTRIES = 152 * 32 * 2.070e9 / 1e12    # SMs x ex2 per clock x
 WORK_FILE = os.path.join(ROOT, "profiles", "census_like_step_work.txt")
 # per K V kernel: its ncu traffic summary and the sources whose hash it was taken for
 KMV_KERNELS = {
-    "fp32": ("kmv_kernel (tile-generating K V, FP32 SIMT)",
+    "fp32": ("kmv_kernel (tile-generating K V, FP32; from 7 columns on kmv_f32_tc_kernel)",
              os.path.join(ROOT, "profiles", "kmv_census_like_traffic.txt"),
              ["paper_1501_05427_gb300/csrc/kmv_kernel.cuh",
               "paper_1501_05427_gb300/csrc/kmv_launch.cuh",

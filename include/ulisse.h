@@ -123,6 +123,10 @@ void ulisse_config_default(ulisse_config *cfg);
  *   d      input dimension, 1 <= d <= 16.
  *   cfg    host; copied.  stream: cudaStream_t (as void*) for all later work.
  * The context selects the current CUDA device at creation and uses it for its lifetime.
+ * Device memory beyond the inputs and the columns: the split scratch of a usual product, up to
+ * 64 MiB, at creation; FP32 196 bytes and mixed about 1 KB per input; FP64 up to 256 MiB with
+ * the first product that wants it and, for n <= 5,792, up to 256 MiB with the first solve (both
+ * kept; without the memory the calls run a form that does without).
  * Errors: ULISSE_ERR_ARG (null pointers, n or d out of range, bad cfg), ULISSE_ERR_NOMEM.
  */
 ulisse_status ulisse_create(ulisse_ctx **out, const float *X, const float *y, long long n,
@@ -173,9 +177,8 @@ ulisse_status ulisse_kmv_f64(ulisse_ctx *ctx, const double *psi, int which, cons
  * R = 17, n <= 167,000); larger requests return ULISSE_ERR_ARG without touching the GPU.
  * The first call on a device looks up the array's device address (cudaGetSymbolAddress,
  * with that device current); make that first call before any stream capture.  Do not
- * capture this call in a CUDA graph at all: psi is copied from (possibly pageable) host
- * memory when the call is made, and a captured copy would read the host buffer again at each
- * replay.
+ * capture this call in a CUDA graph at all: psi is read when the call is made, so a replay
+ * would use that psi again, whatever the host array holds by then.
  * All calls share the array: each call clears the parts that must start at zero, but two
  * calls whose GPU work overlaps (different streams, or different host threads) race on it
  * and may return wrong results.  Serialise them.

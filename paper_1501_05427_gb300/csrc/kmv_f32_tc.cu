@@ -21,8 +21,8 @@
 // What bounds it: the FP32 pipe, 2 DP + 4 lanes per entry (distance, exponent, the split's
 // subtractions), whatever the column count, against 2 DP + 1 + R in the SIMT kernel; the BF16
 // conversions (three per two entries at 32 lanes per clock per SM) come next.  n = 22,784, d = 8:
-// 0.47 ms at any count up to 32 columns (ncu: issue 73%, FP32 pipe about 60% counting the packed
-// instructions twice); the SIMT kernel takes 0.74 ms at 17 columns and 1.12 ms at 32.
+// 0.47 ms at any count up to 32 columns (ncu: issue 73%, FMA pipe 68%); the SIMT kernel takes 0.74
+// ms at 17 columns and 1.12 ms at 32.
 //
 // Roles (544 threads, two CTAs per SM): warp 0 copies x^_J and V_J into a ring of stages and
 // issues the MMAs (warp-uniform, one lane elected); warps 1-12 make the kernel values in three
