@@ -124,7 +124,7 @@ void ulisse_config_default(ulisse_config *cfg);
  *   cfg    host; copied.  stream: cudaStream_t (as void*) for all later work.
  * The context selects the current CUDA device at creation and uses it for its lifetime.
  * Device memory beyond the inputs and the columns: the split scratch of a usual product, up to
- * 64 MiB, at creation; FP32 196 bytes and mixed about 1 KB per input; FP64 up to 256 MiB with
+ * 64 MiB, at creation; FP32 196 bytes and mixed about 1.2 KB per input; FP64 up to 256 MiB with
  * the first product that wants it and, for n <= 5,792, up to 256 MiB with the first solve (both
  * kept; without the memory the calls run a form that does without).
  * Errors: ULISSE_ERR_ARG (null pointers, n or d out of range, bad cfg), ULISSE_ERR_NOMEM.

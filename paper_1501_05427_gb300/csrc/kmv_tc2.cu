@@ -32,7 +32,7 @@
 // term lambda V are those of the FP32-pipe variant.
 //
 // What bounds it: the epilogue's issue slots (ncu at n = 50,000, d = 8, N = 32: 7.6 thread
-// instructions per entry, schedulers 77% busy), at N = 64 the tensor pipe (74% busy).  The issuing
+// instructions per entry, schedulers 77% busy), at N = 64 the tensor pipe (77% busy).  The issuing
 // warps come next: a tile takes about a hundred of their instructions, which wait their turn
 // among the epilogue's.  Times of the kernel at n = 50,000, d = 8, 17 columns: 1.046 ms with a
 // copying warp and one divergent lane issuing for four CTAs of eight epilogue warps per SM; 0.777
