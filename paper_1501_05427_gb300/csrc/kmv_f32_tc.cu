@@ -182,18 +182,18 @@ __device__ __forceinline__ uint32_t f3_bits(const __nv_bfloat162& v) {
 // inputs (every result a NaN) 0.52 ms, 9.6 with a scan of V per entry; with an infinity in one
 // column 0.72, then 2.2.
 template <int N, int MODE>
-__device__ __noinline__ void f3_not_finite(const F3Args& a, const long long row0, const int R) {
-  __shared__ unsigned s_cols;   // the columns with a value that is not finite
+__device__ __noinline__ void f3_not_finite(const F3Args& a, const long long row0, const int R,
+                                           unsigned* s_cols) {
   const uint32_t* bad =
       reinterpret_cast<const uint32_t*>(a.Vp + (long long)a.ntiles * 3 * N * kF3BN);
-  if (threadIdx.x == 0) s_cols = 0;
+  if (threadIdx.x == 0) *s_cols = 0;   // the columns with a value that is not finite
   __syncthreads();
   for (int e = threadIdx.x; e < a.ntiles * N; e += kF3Threads)
-    if (bad[e]) atomicOr(&s_cols, 1u << (e % N));
+    if (bad[e]) atomicOr(s_cols, 1u << (e % N));
   __syncthreads();
   const float c0 = a.params->c0f, c1 = a.params->c1f;
   const bool all = !(c0 < 127.f);
-  const unsigned cols = all ? ~0u : s_cols;
+  const unsigned cols = all ? ~0u : *s_cols;
   for (int idx = threadIdx.x; idx < R * kF3BM; idx += kF3Threads) {
     const int r = idx / kF3BM;
     const long long i = row0 + (idx - r * kF3BM);
@@ -469,7 +469,7 @@ __device__ __forceinline__ void f3_body(const F3Args& a, const int rb, const int
     return;
   }
   if (a.nsplit == 1) {
-    if (*s_nan) f3_not_finite<N, MODE>(a, row0, R);
+    if (*s_nan) f3_not_finite<N, MODE>(a, row0, R, s_tmem + 4);
     return;
   }
   __threadfence();
@@ -492,7 +492,7 @@ __device__ __forceinline__ void f3_body(const F3Args& a, const int rb, const int
   }
   if (tid == 0) a.counters[rb] = 0;
   __syncthreads();
-  if (*s_nan) f3_not_finite<N, MODE>(a, row0, R);
+  if (*s_nan) f3_not_finite<N, MODE>(a, row0, R, s_tmem + 4);
 }
 
 template <int DP, int N, int MODE>
